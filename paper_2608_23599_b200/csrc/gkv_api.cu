@@ -494,17 +494,20 @@ void build_descs(gkv_cache* c, LayerState& L, bool allow_split) {
   size_t total = 0;
   // A small workload leaves most warps of the GPU without work, and its launch then lasts as long
   // as its longest unit (an exact block: eight steps).  Such lists are cut finer: an exact block
-  // into its four tiles and, when the workload is smaller still, a quantised block into its two
-  // halves, a warp holding as little as one of them (more, finer units also mean more partial rows
-  // to merge at the end, which is why this stops at some size).
+  // into its four tiles and a quantised block into its two halves, a warp holding as little as one of
+  // them.  More, finer units also mean more partial rows to merge at the end, so it stops where the whole
+  // blocks fill the GPU's warps: half blocks take a call over 4001 tokens of 8 streams from 13.6 to 11.1 us,
+  // over 8000 tokens from 14.9 to 13.3, over 16000 tokens of 2 streams from 14.2 to 13.0 and, near the line,
+  // over 2000 tokens of 64 streams from 16.2 to 15.8.  (Exact blocks stop at half of that: the lists have room for
+  // three extra units of as many blocks.)
   bool split = false, split_all = false;
   if (allow_split) {
     size_t rough = 0;
     for (int s = 0; s < ns; ++s) rough += static_cast<size_t>(L.n_closed + 1) * 1000 + static_cast<size_t>(L.res_count_h[s] / 16) * 550;
     split = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost / 2;          // exact blocks only
-    split_all = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost / 8;      // quantised blocks too
+    split_all = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost;         // quantised blocks
   }
-  L.desc_split = split;
+  L.desc_split = allow_split;             // the tail's tiles at least
   for (int s = 0; s < ns; ++s) {
     const int8_t* lv = L.level.data() + static_cast<size_t>(s) * c->max_blocks;
     same_as[s] = s;
@@ -536,7 +539,9 @@ void build_descs(gkv_cache* c, LayerState& L, bool allow_split) {
       for (int j = 0; j < run; ++j) k += item_cost(c, L, s, i + j);
       const uint32_t base = static_cast<uint32_t>(i) | (static_cast<uint32_t>(run) << 24);
       const int8_t lvl = (run == 1 && i < L.n_closed) ? lv[i] : int8_t{0};
-      if (split && lvl == 16) {
+      // the tail's four tiles are units of their own (a tile that holds no row yet is skipped by the kernel): as
+      // one unit of up to eight steps it kept its warp 2 - 4 us beyond the others on small contexts
+      if ((split && lvl == 16) || (allow_split && i == L.n_closed)) {
         for (uint32_t t = 0; t < 4; ++t) u.push_back(Unit{base | ((1u << t) << 20), static_cast<uint32_t>(k / 4)});
       } else if (split_all && (lvl == 8 || lvl == 4 || lvl == 2)) {
         u.push_back(Unit{base | (3u << 20), static_cast<uint32_t>(k / 2)});

@@ -296,7 +296,6 @@ struct WarpCtx {
   int stream;                // the (sequence, KV head) stream whose cache is read
   int sparse_rank;           // page-list reads: this warp's number among the warps of its head group
   int head0;                 // first query head (within the KV head's group) of the warp's head group
-  bool has_tail;
   uint32_t stage0;           // shared-memory address of stage 0 (stage s at + s * kStageBytes)
   const uint8_t* stage_ptr0; // the same as a generic pointer
   uint32_t bar0;             // mbarrier of stage 0 (stage s at + 8 s)
@@ -359,8 +358,8 @@ __device__ __forceinline__ bool load_item_dense(WarpCtx& w, int pos, Cursor& c) 
         c.level = 16;
         c.ntok = p.n_tail;
         const int nt = (p.n_tail + 15) >> 4;
-        c.tmask = (1 << nt) - 1;
-        if (nt == 0) {
+        c.tmask = ((1 << nt) - 1) & mask;      // the unit's tiles that hold rows by now
+        if (c.tmask == 0) {
           ++pos;
           continue;
         }
@@ -443,8 +442,9 @@ __device__ __forceinline__ bool load_item_sparse(WarpCtx& w, int pos, Cursor& c)
     }
     return true;
   }
-  // pos == item_end (also after skipped entries): the tail
-  if (pos == w.item_end && w.has_tail && p.n_tail > 0) {
+  // pos == item_end (also after skipped entries): the tail, one 16-token tile each for the head group's last four warps
+  const int tail_tile = p.warps_per_stream - 1 - w.sparse_rank;
+  if (pos == w.item_end && tail_tile < 4 && 16 * tail_tile < p.n_tail) {
     const TableEntry e = w.table[p.n_closed];
     c.item = pos;
     c.sub = 0;
@@ -453,9 +453,8 @@ __device__ __forceinline__ bool load_item_sparse(WarpCtx& w, int pos, Cursor& c)
     c.resmask = 0;
     c.level = 16;
     c.ntok = p.n_tail;
-    const int nt = (p.n_tail + 15) >> 4;
-    c.tmask = (1 << nt) - 1;
-    c.nsub = 2 * nt;
+    c.tmask = 1 << tail_tile;
+    c.nsub = 2;
     return true;
   }
   // Positions past the tail: the stream's groups of 16 exact residual rows, dealt round-robin to
@@ -917,6 +916,38 @@ __device__ __forceinline__ void compute_step(const WarpCtx& w, const Cursor& c, 
   }
 }
 
+// The four query rows of the warp's head group into its second stage (idle until the first unit is under
+// way), zeros for heads that the group does not have.
+__device__ __forceinline__ void fetch_query(const WarpCtx& w) {
+  const DecodeParams& p = *w.p;
+  const uint16_t* q0 = p.q + (static_cast<size_t>(w.stream) * p.group + w.head0) * kD;      // [batch][n_q_heads], KV heads in order
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int piece = w.lane + 32 * i, j = piece >> 4, col = piece & 15;
+    const bool on = w.head0 + j < p.group;
+    cp_async16(w.stage0 + kStageBytes + j * kRowPitch + col * 16, q0 + (on ? j * kD + col * 8 : 0), on ? 16u : 0u);
+  }
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+// Query fragments: B operand Q^T[16 channels x 8 columns]; lane (r, c4) holds column r = the hi (r even)
+// or lo (r odd) column of head r / 2 of the head group, channels 16 s + 2 c4 (+1) and 16 s + 8 + 2 c4 (+1), in
+// bf16 (exact rows) and fp16 (quantised tiers).  Both columns of a head hold its query; the parts of the
+// scaled query are formed per key group.
+__device__ __forceinline__ void stage_query(const WarpCtx& w) {
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncwarp();
+  const uint32_t row = w.stage0 + kStageBytes + (w.lane >> 3) * kRowPitch + (w.lane & 3) * 4;
+#pragma unroll
+  for (int s = 0; s < 8; ++s) {
+    const uint32_t v0 = lds32(row + 32 * s), v1 = lds32(row + 32 * s + 16);
+    asm volatile("st.shared.v2.u32 [%0], {%1,%2};\n" ::"r"(w.qb_addr + s * 256), "r"(v0), "r"(v1) : "memory");
+    const uint32_t h0 = h2_as_u32(__floats2half2_rn(bf16lo_to_f32(v0), bf16hi_to_f32(v0)));
+    const uint32_t h1 = h2_as_u32(__floats2half2_rn(bf16lo_to_f32(v1), bf16hi_to_f32(v1)));
+    asm volatile("st.shared.v2.u32 [%0], {%1,%2};\n" ::"r"(w.qh_addr + s * 256), "r"(h0), "r"(h1) : "memory");
+  }
+  __syncwarp();
+}
+
 template <bool SPARSE, bool MASS>
 __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_kernel(const __grid_constant__ DecodeParams p) {
   static_assert(!(SPARSE && MASS), "block masses are observed by full reads only");
@@ -935,7 +966,6 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   w.head0 = 0;
   w.sparse_rank = 0;
   w.item_end = 0;
-  w.has_tail = false;
   // A warp works for one head group: up to four query heads of one KV head.  Head group hg of stream s
   // has the index s * head_groups + hg; partial rows, ranges of rows and tickets go by that index.
   int hgroup = -1, partial_row = 0, first = 0;
@@ -952,21 +982,21 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
       const int wi = gw - hgroup * wps;
       first = static_cast<int>((static_cast<long long>(wi) * p.n_sel) / wps);
       w.item_end = static_cast<int>((static_cast<long long>(wi + 1) * p.n_sel) / wps);
-      w.has_tail = (wi == wps - 1);
       w.sparse_rank = wi;
       partial_row = blockIdx.x;      // whole CTAs per head group: one partial row per CTA
     }
   }
-  // per-warp (head group, partial row) for the merge at the end
+  // per warp, for the merge at the end: head group, partial row, the head group's first and end row; then a flag
   int* s_group = reinterpret_cast<int*>(smem + kDecodeWarps * (kStages * kStageBytes + kStages * 8 + 2 * 2048));
   if (lane == 0) {
     s_group[warp] = hgroup;
     s_group[kDecodeWarps + warp] = partial_row;
+    if constexpr (!SPARSE) {
+      const StreamParts sp = hgroup >= 0 ? p.parts[hgroup] : StreamParts{0, 0};
+      s_group[2 * kDecodeWarps + warp] = sp.begin;
+      s_group[3 * kDecodeWarps + warp] = sp.end;
+    }
   }
-  if (hgroup >= 0) {
-  w.stream = hgroup / p.head_groups;
-  w.head0 = kHeadsPerWarp * (hgroup - w.stream * p.head_groups);
-  w.table = p.table + static_cast<size_t>(w.stream) * p.table_stride;
   uint8_t* sbase = smem + warp * (kStages * kStageBytes);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kDecodeWarps * kStages * kStageBytes) + warp * kStages;
   uint8_t* qb_smem = smem + kDecodeWarps * (kStages * kStageBytes + kStages * 8) + warp * 2048;
@@ -975,56 +1005,37 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   w.bar0 = smem_u32(bars);
   w.qb_addr = smem_u32(qb_smem) + lane * 8;       // word pair s at + 256 s (conflict-free 8-byte accesses)
   w.qh_addr = w.qb_addr + kDecodeWarps * 2048;
-  if (lane == 0) {
+  if (hgroup >= 0) {
+    w.stream = hgroup / p.head_groups;
+    w.head0 = kHeadsPerWarp * (hgroup - w.stream * p.head_groups);
+    w.table = p.table + static_cast<size_t>(w.stream) * p.table_stride;
+    if (lane == 0) {
 #pragma unroll
-    for (int s = 0; s < kStages; ++s) mbar_init(w.bar0 + 8 * s, 1);
-    fence_proxy_async();
+      for (int s = 0; s < kStages; ++s) mbar_init(w.bar0 + 8 * s, 1);
+      fence_proxy_async();
+    }
+    __syncwarp();
+    // The start of a launch is a chain of dependent look-ups (work list -> block table -> bytes): the first
+    // unit word is asked for here, its table entry right after the wait below.  unit_at() picks them up as its
+    // prefetched pair.
+    if constexpr (!SPARSE) {
+      if (first < w.item_end) w.pf_unit = w.units[first];
+    }
   }
-  __syncwarp();
-  // The start of a launch is a chain of dependent look-ups (work list -> block table -> bytes):
-  // the first unit word is asked for here, its table entry right after the wait below, so that both
-  // are on their way while the query is staged.  unit_at() picks them up as its prefetched pair.
-  if constexpr (!SPARSE) {
-    if (first < w.item_end) w.pf_unit = w.units[first];
-  }
-  // Launched with programmatic stream serialisation: what is above (descriptor fetch, barrier
-  // set-up, the first word of the host-written work list) may overlap the tail of the previous
-  // kernel in the stream.  Nothing that a previous kernel may have written (the block table, the
-  // query, appended rows, partial rows, tickets) is touched before this wait, which returns once
-  // that kernel has completed and its writes are visible.
+  // Launched with programmatic stream serialisation: what is above touches nothing that a previous kernel may
+  // have written (only descriptors and the first word of the host-written work list).  The block table, the query,
+  // appended rows, partial rows and tickets are touched after this wait, which returns once that kernel has
+  // completed and its writes are visible.
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  if (hgroup >= 0) {
   if constexpr (!SPARSE) {
     if (first < w.item_end) {
       w.pf_entry = *reinterpret_cast<const uint4*>(w.table + min(static_cast<int>(w.pf_unit & kUnitItemMask), p.n_closed));
       w.pf_pos = first;
     }
   }
-
-  // Query fragments: B operand Q^T[16 channels x 8 columns]; lane (r, c4) holds column r = the hi
-  // (r even) or lo (r odd) column of head r / 2 of the head group, channels 16 s + 2 c4 (+1) and
-  // 16 s + 8 + 2 c4 (+1), in bf16 (exact rows) and fp16 (quantised tiers).  Both columns of a head
-  // hold its query; the parts of the scaled query are formed per key group.
-  const int r = lane >> 2, c4 = lane & 3;
-  {
-    const int b = w.stream / p.n_kv_heads, kvh = w.stream - b * p.n_kv_heads;
-    const int n_q_heads = p.n_kv_heads * p.group;
-    const int head = w.head0 + (r >> 1);
-    const uint16_t* qrow = p.q + (static_cast<size_t>(b) * n_q_heads + static_cast<size_t>(kvh) * p.group + head) * kD;
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      uint32_t v0 = 0, v1 = 0;
-      if (head < p.group) {
-        v0 = *reinterpret_cast<const uint32_t*>(qrow + 16 * s + 2 * c4);
-        v1 = *reinterpret_cast<const uint32_t*>(qrow + 16 * s + 8 + 2 * c4);
-      }
-      asm volatile("st.shared.v2.u32 [%0], {%1,%2};\n" ::"r"(w.qb_addr + s * 256), "r"(v0), "r"(v1) : "memory");
-      const uint32_t h0 = h2_as_u32(__floats2half2_rn(bf16lo_to_f32(v0), bf16hi_to_f32(v0)));
-      const uint32_t h1 = h2_as_u32(__floats2half2_rn(bf16lo_to_f32(v1), bf16hi_to_f32(v1)));
-      asm volatile("st.shared.v2.u32 [%0], {%1,%2};\n" ::"r"(w.qh_addr + s * 256), "r"(h0), "r"(h1) : "memory");
-    }
-  }
-  __syncwarp();
+  fetch_query(w);
 
   SoftmaxState st;
   st.m = kNegInf;
@@ -1035,7 +1046,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   uint32_t pf[4] = {0, 0, 0, 0};
 
   // Software pipeline over steps: while step k is computed, step k + 1 is in flight.  The loop
-  // starts on an empty pseudo-unit (level 0) so that the cursor and copy code exists once.
+  // starts on an empty pseudo-unit (level 0) so that the cursor and copy code exists once; while the
+  // first unit's bytes are on their way, that iteration stages the query.
   Cursor cur;
   cur.item = first - 1;
   cur.first = 0;
@@ -1047,8 +1059,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   cur.tmask = 0;
   cur.off256 = 0;
   cur.resmask = 0;
-  bool have = true;
   int sidx = 1;
+  bool have = true;
   uint32_t phase = 0;             // bit s = parity to wait for on stage s
   bool failed = false;
   float mass_l = 0.f, mass_m = kNegInf;     // (l, m) when the current block began
@@ -1087,6 +1099,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
         }
       }
       __syncwarp();
+    } else {
+      stage_query(w);
     }
     cur = nxt;
     have = more;
@@ -1099,6 +1113,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
     st.l = 0.f;
   }
 
+  const int r = lane >> 2, c4 = lane & 3;
   // lane-partial sum -> the head's sum (reduce over the 8 r lanes that share c4)
 #pragma unroll
   for (int d = 4; d <= 16; d <<= 1) st.l += __shfl_xor_sync(kFull, st.l, d);
@@ -1117,118 +1132,125 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   }
   }   // hgroup >= 0
 
-  // Merge the rows of the CTA's warps that share a stream (they are neighbours) into one global
-  // partial row per (CTA, stream), in warp order; every warp of the CTA arrives here exactly once.
+  // Merge the rows of the CTA's warps that share a head group (they are neighbours), in warp order; every
+  // warp of the CTA arrives here exactly once.  Warp v takes 32 channels of head v / 4: lane i holds row i's
+  // (m, l), the maximum and the weights are made once per warp with shuffles, and the sum over the rows is a
+  // chain of independent loads.
   __syncthreads();
   constexpr int kRowFloats = kStages * kStageBytes / 4;     // distance between two warps' rows
   const float* rows = reinterpret_cast<const float*>(smem);
+  const int head = warp >> 2, chan = 32 * (warp & 3) + lane;
+  const int group_of = s_group[lane & 15];
   int gb = 0;
 #pragma unroll 1
   while (gb < kDecodeWarps) {
-    const int sid = s_group[gb];
-    int ge = gb + 1;
-#pragma unroll 1
-    while (ge < kDecodeWarps && s_group[ge] == sid) ++ge;
+    const int sid = __shfl_sync(kFull, group_of, gb);
+    const int ge = 32 - __clz(__ballot_sync(kFull, group_of == sid) & 0xffffu);
     if (sid >= 0) {
       const int sid_stream = sid / p.head_groups, sid_head0 = kHeadsPerWarp * (sid - sid_stream * p.head_groups);
       const int n_heads = min(kHeadsPerWarp, p.group - sid_head0);
-      const int n_pair = n_heads * ((kD + 2) / 2);
-      float* dst = p.partial + static_cast<size_t>(s_group[kDecodeWarps + gb]) * kPartialFloats;
-      // the stream's range of partial rows, asked for now and needed when the ticket is taken
-      // (sparse mode: a stream's CTAs are neighbours, one partial row each, row = CTA index)
-      int row_begin = 0, row_end = 0;
-      if (threadIdx.x == 0) {
+      const size_t hq0 = static_cast<size_t>(sid_stream) * p.group + sid_head0;      // [batch][n_q_heads], KV heads in order
+      // the head group's range of partial rows (sparse mode: its CTAs are neighbours, one row each, row = CTA index)
+      int begin, end;
+      if constexpr (SPARSE) {
         const int per = p.warps_per_stream / kDecodeWarps;
-        row_begin = sid * per;
-        row_end = row_begin + per;
-        if (p.parts) {
-          const StreamParts sp = p.parts[sid];
-          row_begin = sp.begin;
-          row_end = sp.end;
-        }
+        begin = sid * per;
+        end = begin + per;
+      } else {
+        begin = s_group[2 * kDecodeWarps + gb];
+        end = s_group[3 * kDecodeWarps + gb];
       }
-      // an element is a pair of floats of the row: (m, l) of a head, or two of its channels
-#pragma unroll 1
-      for (int e = threadIdx.x; e < n_pair; e += kDecodeWarps * 32) {
-        const int h = e / ((kD + 2) / 2), j = e - h * ((kD + 2) / 2);
-        // one pass in warp order: running maximum M and the sums relative to it (the loads of the
-        // rows do not depend on one another; only the short rescaling chain is serial)
-        const float* col = rows + h * (kD + 2);
-        float M = kNegInf, acc0 = 0.f, acc1 = 0.f;
-#pragma unroll 2
-        for (int i = gb; i < ge; ++i) {
-          const float m = col[i * kRowFloats];
-          const float2 v = *reinterpret_cast<const float2*>(col + i * kRowFloats + 2 * j);
-          const float Mn = fmaxf(M, m);
-          const float a = (M == kNegInf) ? 0.f : fast_exp2(M - Mn), bwt = (m == kNegInf) ? 0.f : fast_exp2(m - Mn);
-          acc0 = fmaf(acc0, a, v.x * bwt);
-          acc1 = fmaf(acc1, a, v.y * bwt);
-          M = Mn;
-        }
-        *reinterpret_cast<float2*>(dst + h * (kD + 2) + 2 * j) = make_float2(j == 0 ? M : acc0, acc1);
-      }
-      // The CTA that delivers the stream's last row normalises and writes the output: rows are
-      // published with a fence before the ticket is taken, and read back through L2.  Nobody
-      // waits for anybody; the order of summation is the row order, whichever CTA does it.
-      __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        const int begin = row_begin, end = row_end;
-        const int n = end - begin;
-        bool is_last = true;
-        if (n > 1) {
-          is_last = atomicAdd(&p.tickets[sid], 1) == n - 1;
-          if (is_last) p.tickets[sid] = 0;        // ready for the next launch
-        }
-        s_group[2 * kDecodeWarps] = is_last ? begin : -1;
-        s_group[2 * kDecodeWarps + 1] = end;
-      }
-      __syncthreads();
-      const int begin = s_group[2 * kDecodeWarps], end = s_group[2 * kDecodeWarps + 1];
-      if (begin >= 0) {
-        __threadfence();
-        const int b = sid_stream / p.n_kv_heads, kvh = sid_stream - b * p.n_kv_heads;
-        // a thread takes two neighbouring channels of a head and one half of the rows; the second half's
-        // aggregate joins the first's through shared memory (warp 0's stage memory behind its row), so
-        // the order of summation stays fixed whichever CTA does it
-        float4* s_half = reinterpret_cast<float4*>(smem + 5120);
-        const int e = threadIdx.x & 255, part = threadIdx.x >> 8;
-        const int n = end - begin, n0 = (n + 1) >> 1;
-        const bool on = e < n_heads * (kD / 2);
-        const int h = e / (kD / 2), ch = 2 * (e - h * (kD / 2));
-        float M = kNegInf, L = 0.f, acc0 = 0.f, acc1 = 0.f;
-        if (on) {
-          const int i0 = part ? n0 : 0, i1 = part ? n : n0;
-          const float* col = p.partial + static_cast<size_t>(begin) * kPartialFloats + h * (kD + 2);
-          // one pass in row order (rounds of independent loads; only the short rescaling chain is serial)
+      float* dst = p.partial + static_cast<size_t>(s_group[kDecodeWarps + gb]) * kPartialFloats;
+      if (head < n_heads) {
+        const float* col = rows + head * (kD + 2);
+        const bool mine = lane >= gb && lane < ge;
+        const float m = mine ? col[lane * kRowFloats] : kNegInf, l = mine ? col[lane * kRowFloats + 1] : 0.f;
+        float M = m;
+#pragma unroll
+        for (int d = 8; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, d));      // rows sit in lanes 0 - 15
+        const float wt = (m == kNegInf) ? 0.f : fast_exp2(m - M);
+        float L = wt * l;
+#pragma unroll
+        for (int d = 8; d > 0; d >>= 1) L += __shfl_xor_sync(kFull, L, d);
+        float acc = 0.f;
 #pragma unroll 8
-          for (int i = i0; i < i1; ++i) {
-            const float* row = col + static_cast<size_t>(i) * kPartialFloats;
-            const float2 ml = __ldcg(reinterpret_cast<const float2*>(row));
-            const float2 v = __ldcg(reinterpret_cast<const float2*>(row + 2 + ch));
-            const float Mn = fmaxf(M, ml.x);
-            const float a = (M == kNegInf) ? 0.f : exp2f(M - Mn), bwt = (ml.x == kNegInf) ? 0.f : exp2f(ml.x - Mn);
-            L = fmaf(L, a, ml.y * bwt);
-            acc0 = fmaf(acc0, a, v.x * bwt);
-            acc1 = fmaf(acc1, a, v.y * bwt);
-            M = Mn;
+        for (int i = gb; i < ge; ++i) acc = fmaf(__shfl_sync(kFull, wt, i), col[i * kRowFloats + 2 + chan], acc);
+        M = __shfl_sync(kFull, M, 0);
+        L = __shfl_sync(kFull, L, 0);
+        if (end - begin == 1) {
+          // the head group has no other row: normalise and write the result
+          const size_t hq = hq0 + head;
+          p.out[hq * kD + chan] = (L > 0.f) ? acc / L : 0.f;
+          if (chan == 0) {
+            const float z = (L > 0.f) ? M + log2f(L) : kNegInf;
+            if (p.lse) p.lse[hq] = z * 0.6931471805599453f;
+            if constexpr (MASS) p.lse2[hq] = z;
           }
-          if (part) s_half[e] = make_float4(M, L, acc0, acc1);
+        } else {
+          dst[head * (kD + 2) + 2 + chan] = acc;
+          if (chan == 0) *reinterpret_cast<float2*>(dst + head * (kD + 2)) = make_float2(M, L);
+        }
+      }
+      if (end - begin > 1) {
+        // The CTA that delivers the head group's last row normalises and writes the output: the rows are
+        // published by the fence that thread 0 issues behind the barrier, and read back through L2.  Nobody
+        // waits for anybody; the order of summation is the row order, whichever CTA does it.
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          __threadfence();
+          const bool is_last = atomicAdd(&p.tickets[sid], 1) == end - begin - 1;
+          s_group[4 * kDecodeWarps] = is_last;
+          if (is_last) {
+            p.tickets[sid] = 0;                   // ready for the next launch
+            __threadfence();
+          }
         }
         __syncthreads();
-        if (on && part == 0) {
-          const float4 o2 = s_half[e];
-          const float Mn = fmaxf(M, o2.x);
-          const float a = (M == kNegInf) ? 0.f : exp2f(M - Mn), bwt = (o2.x == kNegInf) ? 0.f : exp2f(o2.x - Mn);
-          L = fmaf(L, a, o2.y * bwt);
-          acc0 = fmaf(acc0, a, o2.z * bwt);
-          acc1 = fmaf(acc1, a, o2.w * bwt);
-          M = Mn;
-          const size_t hq = static_cast<size_t>(b) * p.n_kv_heads * p.group + static_cast<size_t>(kvh) * p.group + sid_head0 + h;
-          *reinterpret_cast<float2*>(p.out + hq * kD + ch) = (L > 0.f) ? make_float2(acc0 / L, acc1 / L) : make_float2(0.f, 0.f);
-          if (p.lse && ch == 0) p.lse[hq] = (L > 0.f) ? (M + log2f(L)) * 0.6931471805599453f : kNegInf;
-          if constexpr (MASS) {
-            if (ch == 0) p.lse2[hq] = (L > 0.f) ? M + log2f(L) : kNegInf;
+        if (s_group[4 * kDecodeWarps]) {
+          // a thread takes four neighbouring channels of a head and a quarter of the rows; the quarters are joined
+          // in order through shared memory (the second stage of warps 1 - 3)
+          struct Part { float M, L, a[4]; };
+          const int part = threadIdx.x >> 7, e = threadIdx.x & 127, h = e >> 5, ch = 4 * (e & 31);
+          const int n = end - begin;
+          float M = kNegInf, L = 0.f, acc[4] = {0.f, 0.f, 0.f, 0.f};
+          auto join = [&](float m2, float l2, const float (&v)[4]) {
+            const float Mn = fmaxf(M, m2);
+            const float a = (M == kNegInf) ? 0.f : exp2f(M - Mn), bwt = (m2 == kNegInf) ? 0.f : exp2f(m2 - Mn);
+            L = fmaf(L, a, l2 * bwt);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[i] = fmaf(acc[i], a, v[i] * bwt);
+            M = Mn;
+          };
+          if (h < n_heads) {
+            const float* col = p.partial + static_cast<size_t>(begin) * kPartialFloats + h * (kD + 2);
+            // one pass in row order (rounds of independent loads; only the short rescaling chain is serial)
+            const int i1 = n * (part + 1) / 4;
+#pragma unroll 5
+            for (int i = n * part / 4; i < i1; ++i) {
+              const float* row = col + static_cast<size_t>(i) * kPartialFloats;
+              const float2 ml = __ldcg(reinterpret_cast<const float2*>(row));
+              const float2 v0 = __ldcg(reinterpret_cast<const float2*>(row + 2 + ch)), v1 = __ldcg(reinterpret_cast<const float2*>(row + 4 + ch));
+              const float v[4] = {v0.x, v0.y, v1.x, v1.y};
+              join(ml.x, ml.y, v);
+            }
+          }
+          auto slot = [&](int k) { return reinterpret_cast<Part*>(smem + k * (kStages * kStageBytes) + kStageBytes) + e; };
+          if (part) *slot(part) = Part{M, L, {acc[0], acc[1], acc[2], acc[3]}};
+          __syncthreads();
+          if (part == 0 && h < n_heads) {
+#pragma unroll
+            for (int k = 1; k < 4; ++k) {
+              const Part o = *slot(k);
+              join(o.M, o.L, o.a);
+            }
+            const size_t hq = hq0 + h;
+            *reinterpret_cast<float4*>(p.out + hq * kD + ch) =
+                (L > 0.f) ? make_float4(acc[0] / L, acc[1] / L, acc[2] / L, acc[3] / L) : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (ch == 0) {
+              const float z = (L > 0.f) ? M + log2f(L) : kNegInf;
+              if (p.lse) p.lse[hq] = z * 0.6931471805599453f;
+              if constexpr (MASS) p.lse2[hq] = z;
+            }
           }
         }
       }
@@ -1242,7 +1264,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
 
 size_t decode_smem_bytes() {
   // per warp: pipeline stages, their mbarriers, and the bf16 query fragments (2 KiB)
-  return static_cast<size_t>(kDecodeWarps) * (kStages * kStageBytes + kStages * sizeof(uint64_t) + 2 * 2048 + 2 * sizeof(int)) + 2 * sizeof(int);
+  return static_cast<size_t>(kDecodeWarps) * (kStages * kStageBytes + kStages * sizeof(uint64_t) + 2 * 2048 + 4 * sizeof(int)) + sizeof(int);
 }
 
 cudaError_t launch_decode(const DecodeParams& p, int n_ctas, cudaStream_t st) {
