@@ -507,7 +507,7 @@ void build_descs(gkv_cache* c, LayerState& L, bool allow_split) {
     split = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost / 2;          // exact blocks only
     split_all = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost;         // quantised blocks
   }
-  L.desc_split = allow_split;             // the tail's tiles at least
+  L.desc_split = split || split_all;
   for (int s = 0; s < ns; ++s) {
     const int8_t* lv = L.level.data() + static_cast<size_t>(s) * c->max_blocks;
     same_as[s] = s;
@@ -540,8 +540,8 @@ void build_descs(gkv_cache* c, LayerState& L, bool allow_split) {
       const uint32_t base = static_cast<uint32_t>(i) | (static_cast<uint32_t>(run) << 24);
       const int8_t lvl = (run == 1 && i < L.n_closed) ? lv[i] : int8_t{0};
       // the tail's four tiles are units of their own (a tile that holds no row yet is skipped by the kernel): as
-      // one unit of up to eight steps it kept its warp 2 - 4 us beyond the others on small contexts
-      if ((split && lvl == 16) || (allow_split && i == L.n_closed)) {
+      // one unit of up to eight steps it kept its warp 2 - 4 us beyond the others
+      if ((split && lvl == 16) || (split_all && i == L.n_closed)) {
         for (uint32_t t = 0; t < 4; ++t) u.push_back(Unit{base | ((1u << t) << 20), static_cast<uint32_t>(k / 4)});
       } else if (split_all && (lvl == 8 || lvl == 4 || lvl == 2)) {
         u.push_back(Unit{base | (3u << 20), static_cast<uint32_t>(k / 2)});
