@@ -1714,42 +1714,30 @@ int decode_impl(gkv_cache* c, int32_t layer, const void* q, const int32_t* page_
   }
   CK(c, launch_decode(p, n_ctas, st));
   if (observe) {
-    MassFinishParams m{};
-    m.mass_raw = c->mass_raw_d;
-    m.res_raw = c->res_raw_d;
-    m.lse2 = c->lse2_d;
-    m.res_idx = L.res_idx_d;
-    m.res_count = L.res_count_d;
-    m.ema = L.ema_d;
-    m.observed = block_mass;
-    m.n_streams = c->n_streams;
-    m.n_items = L.n_closed + (L.n_tail > 0 ? 1 : 0);
-    m.mass_stride = c->max_blocks + 1;
-    m.res_cap = c->res_cap;
-    m.group = c->group;
-    CK(c, launch_mass_finish(m, st));
-    if (certificate) {
-      CertificateParams cp{};
-      cp.arena = c->arena;
-      cp.table = L.table_d;
-      cp.mass_raw = c->mass_raw_d;
-      cp.res_raw = c->res_raw_d;
-      cp.lse2 = c->lse2_d;
-      cp.err = L.err_d;
-      cp.res_count = L.res_count_d;
-      cp.q = static_cast<const uint16_t*>(q);
-      cp.out = certificate;
-      cp.n_streams = c->n_streams;
-      cp.group = c->group;
-      cp.n_closed = L.n_closed;
-      cp.n_tail = L.n_tail;
-      cp.table_stride = c->table_stride;
-      cp.mass_stride = c->max_blocks + 1;
-      cp.res_cap = c->res_cap;
-      cp.err_stride = c->max_blocks;
-      cp.scale = c->scale;
-      CK(c, launch_certificate(cp, st));
-    }
+    ObserveParams o{};
+    o.arena = c->arena;
+    o.table = L.table_d;
+    o.mass_raw = c->mass_raw_d;
+    o.res_raw = c->res_raw_d;
+    o.lse2 = c->lse2_d;
+    o.res_idx = L.res_idx_d;
+    o.res_count = L.res_count_d;
+    o.ema = L.ema_d;
+    o.observed = block_mass;
+    o.err = L.err_d;
+    o.q = static_cast<const uint16_t*>(q);
+    o.certificate = certificate;
+    o.n_streams = c->n_streams;
+    o.n_items = L.n_closed + (L.n_tail > 0 ? 1 : 0);
+    o.group = c->group;
+    o.n_closed = L.n_closed;
+    o.n_tail = L.n_tail;
+    o.table_stride = c->table_stride;
+    o.mass_stride = c->max_blocks + 1;
+    o.res_cap = c->res_cap;
+    o.err_stride = c->max_blocks;
+    o.scale = c->scale;
+    CK(c, launch_observe_finish(o, st));
   }
   return GKV_OK;
 }

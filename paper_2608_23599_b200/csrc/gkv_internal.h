@@ -80,26 +80,12 @@ struct DecodeParams {
   int32_t mass_stride, res_cap;
 };
 
-// Attention error certificate of the observing decode launch that just ran (Sec. 3.6, Eq. 9).
-struct CertificateParams {
+// What follows an observing decode launch: the raw pairs become block masses a_b (mean over the KV head's query
+// heads of the block's softmax weight, residual rows added to the block they sit in), the running mass is updated,
+// m_b <- 0.9 m_b + 0.1 a_b, and, where asked for, the attention error certificate (Sec. 3.6, Eq. 9) is made.
+struct ObserveParams {
   const uint8_t* arena;
   const TableEntry* table;
-  const float2* mass_raw;
-  const float2* res_raw;
-  const float* lse2;
-  const float4* err;            // [n_streams][err_stride]
-  const int32_t* res_count;
-  const uint16_t* q;            // bf16 [batch][n_q_heads][128]
-  float* out;                   // [batch][n_q_heads]
-  int32_t n_streams, group, n_closed, n_tail;
-  int32_t table_stride, mass_stride, res_cap, err_stride;
-  float scale;                  // softmax scale (natural-log domain)
-};
-
-// Turns the raw pairs of a decode launch into block masses a_b (mean over the KV head's query heads
-// of the block's softmax weight, residual rows added to the block they sit in) and updates the running
-// mass m_b <- 0.9 m_b + 0.1 a_b.
-struct MassFinishParams {
   const float2* mass_raw;
   const float2* res_raw;
   const float* lse2;
@@ -107,8 +93,13 @@ struct MassFinishParams {
   const int32_t* res_count;     // [n_streams]
   float* ema;                   // [n_streams][mass_stride]
   float* observed;              // nullable [n_streams][n_items]
+  const float4* err;            // [n_streams][err_stride]
+  const uint16_t* q;            // bf16 [batch][n_q_heads][128]
+  float* certificate;           // nullable [batch][n_q_heads]
   int32_t n_streams, n_items;   // items = n_closed + (n_tail > 0)
-  int32_t mass_stride, res_cap, group;
+  int32_t group, n_closed, n_tail;
+  int32_t table_stride, mass_stride, res_cap, err_stride;
+  float scale;                  // softmax scale (natural-log domain)
 };
 
 // One block to encode: read 64 tokens from `src`, write level `dst_level` at dst.
@@ -168,8 +159,7 @@ constexpr uint32_t kStatusRange = 1u;      // a scale or zero saturated
 constexpr uint32_t kStatusInternal = 2u;   // an index check failed inside a kernel
 
 cudaError_t launch_decode(const DecodeParams& p, int n_ctas, cudaStream_t st);
-cudaError_t launch_mass_finish(const MassFinishParams& p, cudaStream_t st);
-cudaError_t launch_certificate(const CertificateParams& p, cudaStream_t st);
+cudaError_t launch_observe_finish(const ObserveParams& p, cudaStream_t st);
 cudaError_t launch_encode(const EncodeParams& p, cudaStream_t st);
 cudaError_t launch_ingest(const EncodeParams& p, cudaStream_t st);   // every job reads the bf16 input rows; 16-byte aligned inputs
 cudaError_t launch_stats(const StatsParams& p, cudaStream_t st);
