@@ -163,7 +163,8 @@ namespace {
 inline bool is_mla(const gkv_config& c) { return c.v_aliases_k != 0; }
 inline int geo_slot_bytes(const gkv_config& c, int level) { return is_mla(c) ? mla_slot_bytes(level) : slot_bytes(level); }
 inline uint64_t nval_per_token(const gkv_config& c) { return is_mla(c) ? c.d_k : c.d_k + c.d_v; }
-constexpr int kMlaTargetCtas = 148;          // one CTA per SM (212 KB of shared memory, all of tensor memory)
+constexpr int kMlaTargetCtas = kMlaMaxRows;  // one CTA per SM (212 KB of shared memory, all of tensor memory)
+constexpr size_t kMlaMinCtaCost = 1000;      // one block: two of a CTA's four quads have a half each
 
 struct ArenaPlan {
   size_t status, debug, partial, range, mass, levels, scores, kper, tickets, jobs, mass_raw, res_raw, lse2, per_layer, heap_begin, total_meta;
@@ -213,6 +214,7 @@ Derived derive(const gkv_config& c) {
   d.table_stride = d.max_blocks + 2;
   d.max_warps = static_cast<int>(align_up(kTargetWarps + 2 * d.n_hgroups, kDecodeWarps));
   d.max_warps = std::max(d.max_warps, d.n_hgroups * sparse_ctas_per_stream(d.n_hgroups) * kDecodeWarps);
+  if (is_mla(c)) d.max_warps = std::max(d.max_warps, kMlaQuads * (kMlaTargetCtas + d.n_streams));      // quad descriptors
   d.res_cap = c.residual_fraction > 0.f
                   ? static_cast<int>(align_up(static_cast<size_t>(std::floor(static_cast<double>(c.residual_fraction) * c.max_ctx)) + 16, 16))
                   : 0;
@@ -1021,71 +1023,76 @@ int append_one(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* v
 // ---- latent-attention (MLA) host paths -----------------------------------------------------------
 // One stream per sequence; staircase or external plans only.  The block table, slot heap and
 // staging are shared with the GQA path; the kernels are those of gkv_mla.cu.
-size_t mla_item_cost(const gkv_cache* c, const LayerState& L, int stream, int item) {
-  // Cost of a block for the split of a stream over the CTAs and their quads, in units where a 4-bit
-  // block is 1000.  Exact, 8-bit and 4-bit blocks: measured on B200 as the time of a call over a cache that
-  // holds one rung only (262,144 tokens), less the call's fixed part.  A centroid block is one row of a
-  // 16-row unit: swept on the 1M-token staircase (a call over centroid blocks only is all fixed cost).
+//
+// Cost of an item for the split of a stream over the CTAs and their quads, in units where a 4-bit
+// block is 1000.  Exact, 8-bit and 4-bit blocks: measured on B200 as the time of a call over a cache that
+// holds one rung only (262,144 tokens), less the call's fixed part.  A centroid block is one row of a
+// 16-row unit: swept on the 1M-token staircase (a call over centroid blocks only is all fixed cost).
+// A quad's range is cut at quarter blocks: an exact block's four tiles, a quantised block's halves (quarters 0
+// and 2); `parts` = pieces of the item, `step` = quarters per piece.
+struct MlaItem { size_t cost; int parts, step; };
+MlaItem mla_item(const gkv_cache* c, const LayerState& L, int stream, int item) {
   if (item < L.n_closed) {
     switch (L.level[static_cast<size_t>(stream) * c->max_blocks + item]) {
-      case 16: return 1100;
-      case 8: return 1005;
-      case 4: return 1000;
-      default: return 24;
+      case 16: return {1100, 4, 1};
+      case 8: return {1004, 2, 2};
+      case 4: return {1000, 2, 2};
+      default: return {24, 1, 4};
     }
   }
-  return 900;                     // tail
+  return {900, 4, 1};             // tail
 }
 
 void mla_build_descs(gkv_cache* c, LayerState& L) {
   const int ns = c->n_streams;
+  const int n_items = L.n_closed + 1;
   std::vector<size_t> cost(ns, 0);
   size_t total = 0;
-  const int n_items = L.n_closed + 1;
   for (int s = 0; s < ns; ++s) {
-    for (int i = 0; i < n_items; ++i) cost[s] += mla_item_cost(c, L, s, i);
+    for (int i = 0; i < n_items; ++i) cost[s] += mla_item(c, L, s, i).cost;
     total += cost[s];
   }
-  const size_t target = std::max<size_t>(800, (total + kMlaTargetCtas - 1) / kMlaTargetCtas);
-  std::vector<WarpDesc> cta(static_cast<size_t>(kMlaTargetCtas) + 2 * ns);
+  // CTAs of every stream: one wave of the GPU shared out by cost, at least one each and, below that, no more than
+  // one per kMlaMinCtaCost.  A CTA beyond the wave runs after all others and doubles the call: eight sequences of
+  // 8191 tokens rounded up to 152 CTAs took 60.7 us a call.
+  std::vector<int> nw(ns);
+  std::vector<std::pair<size_t, int>> rest;           // what a stream's share lost to rounding down
+  int used = 0;
+  for (int s = 0; s < ns; ++s) {
+    const size_t share = total ? cost[s] * kMlaTargetCtas / total : 0;
+    const size_t most = std::max<size_t>(1, std::min<size_t>((cost[s] + kMlaMinCtaCost - 1) / kMlaMinCtaCost, kMlaMaxRows));
+    nw[s] = static_cast<int>(std::max<size_t>(1, std::min(share, most)));
+    used += nw[s];
+    if (static_cast<size_t>(nw[s]) < most) rest.emplace_back(cost[s] / static_cast<size_t>(nw[s]), s);
+  }
+  std::stable_sort(rest.begin(), rest.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+  for (size_t i = 0; i < rest.size() && used < kMlaTargetCtas; ++i, ++used) ++nw[rest[i].second];
   int w = 0;
   for (int s = 0; s < ns; ++s) {
-    int nw = static_cast<int>((cost[s] + target / 2) / target);
-    nw = std::max(1, std::min(nw, n_items));
-    nw = std::min(nw, kMlaTargetCtas + 2 * ns - w - (ns - 1 - s));
+    // the stream's quads in order: quad k takes the pieces up to (k + 1) / n of the stream's cost
+    const int n = nw[s] * kMlaQuads;
     L.parts_h[s].begin = w;
+    L.parts_h[s].end = w + nw[s];
+    int quad = 0, begin = 0, pos = 0;
     size_t acc = 0;
-    int item = 0;
-    for (int k = 0; k < nw; ++k) {
-      const size_t limit = cost[s] * (k + 1) / nw;
-      const int begin = item;
-      const int max_end = n_items - (nw - 1 - k);
-      do {
-        acc += mla_item_cost(c, L, s, item);
-        ++item;
-      } while (item < max_end && acc < limit);
-      cta[w] = WarpDesc{s, begin, item, w};
-      ++w;
-    }
-    cta[w - 1].item_end = n_items;
-    L.parts_h[s].end = w;
-  }
-  // a CTA's range is cut once more, by cost, into the contiguous ranges of its quads (descriptor
-  // kMlaQuads * cta + quad; all of them name the CTA's partial row)
-  for (int i = 0; i < w; ++i) {
-    size_t tot = 0;
-    for (int it = cta[i].item_begin; it < cta[i].item_end; ++it) tot += mla_item_cost(c, L, cta[i].stream, it);
-    size_t acc = 0;
-    int item = cta[i].item_begin;
-    for (int qd = 0; qd < kMlaQuads; ++qd) {
-      const size_t limit = tot * (qd + 1) / kMlaQuads;
-      const int begin = item;
-      while (item < cta[i].item_end && (qd == kMlaQuads - 1 || acc + mla_item_cost(c, L, cta[i].stream, item) / 2 < limit)) {
-        acc += mla_item_cost(c, L, cta[i].stream, item);
-        ++item;
+    auto close = [&](int end) {
+      L.warps_h[kMlaQuads * w + quad] = WarpDesc{s, begin, end, w + quad / kMlaQuads};
+      begin = end;
+      ++quad;
+    };
+    for (int i = 0; i < n_items; ++i) {
+      const MlaItem it = mla_item(c, L, s, i);
+      for (int k = 0; k < it.parts; ++k) {
+        const size_t piece = it.cost / it.parts;
+        // the piece belongs to the next quad when more than half of it lies beyond this quad's share
+        while (quad < n - 1 && (acc + piece / 2) * n >= cost[s] * (quad + 1)) close(pos);
+        acc += piece;
+        pos = 4 * i + (k + 1) * it.step;
       }
-      L.warps_h[kMlaQuads * i + qd] = WarpDesc{cta[i].stream, begin, item, cta[i].partial};
+      pos = 4 * (i + 1);
     }
+    while (quad < n) close(pos);
+    w += nw[s];
   }
   L.n_warps = w;                  // here: number of CTAs
   L.desc_dirty = false;

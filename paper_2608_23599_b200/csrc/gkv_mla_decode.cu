@@ -72,6 +72,7 @@ constexpr float kMSlack = 8.f;                         // keep a stale running m
 constexpr uint32_t kMFull = 0xffffffffu;
 static_assert(kMStageBytes >= 16 * kMRowPitch, "a stage holds 16 staged rows");
 static_assert(kMStages * kMStageBytes >= kMlaHeads * kMOutPitch * 4 + 128, "a quad's result fits its stages");
+static_assert(kMlaQuads == 4 && kMQuadBytes % 16 == 0, "the merge takes four quads' weights as one float4");
 
 // ---- PTX helpers -------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t m_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
@@ -135,6 +136,9 @@ __device__ __forceinline__ void m_stsf4(uint32_t a, float x, float y, float z, f
 __device__ __forceinline__ void m_stsf(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(a), "f"(v) : "memory"); }
 __device__ __forceinline__ void m_stsf2(uint32_t a, float x, float y) {
   asm volatile("st.shared.v2.f32 [%0], {%1,%2};\n" ::"r"(a), "f"(x), "f"(y) : "memory");
+}
+__device__ __forceinline__ void m_sts64(uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("st.shared.v2.u32 [%0], {%1,%2};\n" ::"r"(a), "r"(x), "r"(y) : "memory");
 }
 __device__ __forceinline__ void m_sts128(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
   asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};\n" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
@@ -200,12 +204,6 @@ __device__ __forceinline__ void m_tst8(uint32_t taddr, const float (&v)[2][4]) {
                : "memory");
 }
 __device__ __forceinline__ void m_twait_st() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ uint32_t m_ldg32(const void* p) {
-  uint32_t v;
-  asm volatile("ld.global.nc.u32 %0, [%1];\n" : "=r"(v) : "l"(p));
-  return v;
-}
-
 // q * s as an fp16 pair: hi = the rounded product, lo = the exact remainder
 __device__ __forceinline__ void m_split(uint32_t q, uint32_t s, uint32_t& hi, uint32_t& lo) {
   const __half2 h = __hmul2(m_h2(q), m_h2(s));
@@ -228,76 +226,106 @@ __device__ __forceinline__ float m_h2f(uint32_t pair, int hi) {
 // ---- units -------------------------------------------------------------------------------------
 // A quad's range of blocks is walked in units: one half block of a quantised block (kind 0), 16 rows
 // of an exact block or of the tail (kind 1), or a run of up to 16 neighbouring centroid blocks, one
-// row each (kind 2).  (m_load is called by whole, converged warps: the run is found with a ballot.)
+// row each (kind 2).  The walk runs two units ahead of the computation, which needs a unit's meta word only.
+// Block table entries come from a window of 32 that a warp holds in its lanes (whole, converged warps call
+// these functions): a look-up is a shuffle, not a load on the way to the next copy.
 struct MWalk {
   int it;                // item (block index; n_closed = the tail)
   uint32_t meta;         // sub | nsub << 4 | kind << 8 | level << 12 | run << 20 | nrows << 25
-  uint32_t off256;
-  __device__ __forceinline__ int sub() const { return static_cast<int>(meta & 15u); }        // unit inside the item
-  __device__ __forceinline__ int nsub() const { return static_cast<int>((meta >> 4) & 15u); }
-  __device__ __forceinline__ int kind() const { return static_cast<int>((meta >> 8) & 15u); }
-  __device__ __forceinline__ int level() const { return static_cast<int>((meta >> 12) & 255u); }
-  __device__ __forceinline__ int run() const { return static_cast<int>((meta >> 20) & 31u); }   // blocks the item covers
-  __device__ __forceinline__ int nrows() const { return static_cast<int>(meta >> 25); }         // rows of the item (kind 1) or run (kind 2)
+  int base;              // first item of the window
+  uint32_t off, lvl;     // this lane's entry: offset and level of item base + lane
 };
+constexpr uint32_t kMNoUnit = 0xffffffffu;
+__device__ __forceinline__ int m_sub(uint32_t meta) { return static_cast<int>(meta & 15u); }          // unit inside the item
+__device__ __forceinline__ int m_nsub(uint32_t meta) { return static_cast<int>((meta >> 4) & 15u); }
+__device__ __forceinline__ int m_kind(uint32_t meta) { return static_cast<int>((meta >> 8) & 15u); }
+__device__ __forceinline__ int m_level(uint32_t meta) { return static_cast<int>((meta >> 12) & 255u); }
+__device__ __forceinline__ int m_run(uint32_t meta) { return static_cast<int>((meta >> 20) & 31u); }  // blocks the item covers
+__device__ __forceinline__ int m_nrows(uint32_t meta) { return static_cast<int>(meta >> 25); }        // rows of the item (kind 1) or run (kind 2)
 __device__ __forceinline__ uint32_t m_meta(int nsub, int kind, int level, int run, int nrows) {
   return static_cast<uint32_t>(nsub) << 4 | static_cast<uint32_t>(kind) << 8 | static_cast<uint32_t>(level) << 12 |
          static_cast<uint32_t>(run) << 20 | static_cast<uint32_t>(nrows) << 25;
 }
+__device__ __forceinline__ void m_window(const MlaDecodeParams& p, const TableEntry* table, int lane, MWalk& w) {
+  const uint2 e = *reinterpret_cast<const uint2*>(table + min(w.it + lane, p.n_closed));
+  w.base = w.it;
+  w.off = e.x;
+  w.lvl = e.y;
+}
 
-__device__ __forceinline__ bool m_load(const MlaDecodeParams& p, const TableEntry* table, int item_end, MWalk& w) {
-  if (w.it >= item_end) return false;
-  const TableEntry e = table[min(w.it, p.n_closed)];
-  w.off256 = e.off256;
-  const int level = static_cast<int>(e.level);
+// Sets up the item w.it; kMNoUnit past the end.  `end4` = the end of the quad's range in quarter blocks (an exact
+// block's tiles; a quantised block's halves begin at 0 and 2; a centroid block is 0 only): a range may begin and
+// end inside a block.
+__device__ __forceinline__ void m_load(const MlaDecodeParams& p, const TableEntry* table, int end4, int lane, MWalk& w) {
+  const int left = end4 - 4 * w.it;                // quarters of the range from this item's start on
+  w.meta = kMNoUnit;
+  if (left <= 0) return;
   if (w.it == p.n_closed) {                        // the tail: exact rows, the last item of the stream
-    if (p.n_tail == 0) return false;
-    w.meta = m_meta((p.n_tail + 15) >> 4, 1, 16, 1, p.n_tail);
-    return true;
+    if (p.n_tail == 0) return;
+    w.meta = m_meta(min((p.n_tail + 15) >> 4, left), 1, 16, 1, p.n_tail);
+    if (w.it >= w.base + 32) m_window(p, table, lane, w);
+    return;
   }
+  if (w.it + 16 > w.base + 32) m_window(p, table, lane, w);
+  const int level = static_cast<int>(__shfl_sync(kMFull, w.lvl, w.it - w.base));
   if (level == 16) {
-    w.meta = m_meta(4, 1, 16, 1, kBlock);
+    w.meta = m_meta(min(4, left), 1, 16, 1, kBlock);
   } else if (level == 1) {
-    const int lim = min(min(item_end, p.n_closed) - w.it, 16);
-    const int ln = static_cast<int>(threadIdx.x & 31);
-    const bool c = ln < lim && table[w.it + ln].level == 1u;
-    const uint32_t b = __ballot_sync(kMFull, c);
-    const int run = __ffs(~b) - 1;                 // first lane that is not a centroid block (lanes >= 16 never are)
+    const int lim = min(min((end4 + 3) >> 2, p.n_closed) - w.it, 16);
+    const uint32_t b = __ballot_sync(kMFull, w.lvl == 1u) >> (w.it - w.base);
+    const int run = min(__clz(__brev(~b)), lim);   // neighbouring centroid blocks from here on
     w.meta = m_meta(1, 2, 1, run, run);
   } else {
-    w.meta = m_meta(2, 0, level, 1, kBlock);
+    w.meta = m_meta(left > 2 ? 2 : 1, 0, level, 1, kBlock);
   }
-  return true;
 }
-__device__ __forceinline__ bool m_advance(const MlaDecodeParams& p, const TableEntry* table, int item_end, MWalk& w) {
+// the first unit of a range
+__device__ __forceinline__ void m_begin(const MlaDecodeParams& p, const TableEntry* table, int begin4, int end4, int lane, MWalk& w) {
+  w.it = begin4 >> 2;
+  w.meta = kMNoUnit;
+  w.base = 0;
+  w.off = w.lvl = 0;
+  if (begin4 >= end4) return;
+  m_window(p, table, lane, w);
+  m_load(p, table, end4, lane, w);
+  if (w.meta == kMNoUnit) return;
+  const int quarter = begin4 & 3;                  // the range may begin inside the item
+  w.meta += static_cast<uint32_t>(m_kind(w.meta) == 0 ? quarter >> 1 : quarter);
+  if (m_sub(w.meta) >= m_nsub(w.meta)) {           // (a tail that has no rows there yet)
+    w.it += m_run(w.meta);
+    m_load(p, table, end4, lane, w);
+  }
+}
+__device__ __forceinline__ void m_advance(const MlaDecodeParams& p, const TableEntry* table, int end4, int lane, MWalk& w) {
   ++w.meta;                                        // sub + 1 (never carries: nsub <= 4)
-  if (w.sub() < w.nsub()) return true;
-  w.it += w.run();
-  return m_load(p, table, item_end, w);
+  if (m_sub(w.meta) < m_nsub(w.meta)) return;
+  w.it += m_run(w.meta);
+  m_load(p, table, end4, lane, w);
 }
-// valid rows of the current unit of a walk of kind 1 or 2
-__device__ __forceinline__ int m_unit_rows(const MWalk& w) { return min(16, w.nrows() - 16 * w.sub()); }
+// valid rows of a unit of kind 1 or 2
+__device__ __forceinline__ int m_unit_rows(uint32_t meta) { return min(16, m_nrows(meta) - 16 * m_sub(meta)); }
 
 // Start the copies of a unit into a stage (one warp, converged).  Rows past the end of a row unit
 // are written as zeros so that 0 * garbage never produces a NaN.
-__device__ __forceinline__ void m_issue(const MlaDecodeParams& p, const TableEntry* table, const MWalk& w, uint32_t st, uint32_t bar,
-                                        int lane) {
-  if (w.kind() == 0) {
+__device__ __forceinline__ void m_issue(const MlaDecodeParams& p, const MWalk& w, uint32_t st, uint32_t bar, int lane) {
+  const int kind = m_kind(w.meta), at = w.it - w.base;
+  // the slot of the unit's block, or of the lane's own block of a centroid run
+  const uint32_t off = __shfl_sync(kMFull, w.off, kind == 2 ? at + lane : at);
+  const uint8_t* slot = p.arena + static_cast<size_t>(off) * 256;
+  if (kind == 0) {
     if (lane == 0) {
-      const uint32_t bytes = static_cast<uint32_t>(mla_half_bytes(w.level()));
+      const uint32_t bytes = static_cast<uint32_t>(mla_half_bytes(m_level(w.meta)));
       m_expect_tx(bar, bytes);
-      m_bulk_g2s(st, p.arena + static_cast<size_t>(w.off256) * 256 + static_cast<size_t>(w.sub()) * bytes, bytes, bar);
+      m_bulk_g2s(st, slot + static_cast<size_t>(m_sub(w.meta)) * bytes, bytes, bar);
     }
     return;
   }
-  const int n = m_unit_rows(w);
+  const int n = m_unit_rows(w.meta);
   if (lane == 0) m_expect_tx(bar, static_cast<uint32_t>(n) * kMlaRowBytes);
   __syncwarp();
-  if (lane < n) {
-    const uint8_t* src = (w.kind() == 2) ? p.arena + static_cast<size_t>(table[w.it + lane].off256) * 256
-                                       : p.arena + static_cast<size_t>(w.off256) * 256 + static_cast<size_t>(16 * w.sub() + lane) * kMlaRowBytes;
-    m_bulk_g2s(st + lane * kMRowPitch, src, kMlaRowBytes, bar);
-  }
+  if (lane < n)
+    m_bulk_g2s(st + lane * kMRowPitch, slot + (kind == 2 ? size_t{0} : static_cast<size_t>(16 * m_sub(w.meta) + lane) * kMlaRowBytes),
+               kMlaRowBytes, bar);
   if (n < 16) {
     for (int idx = lane; idx < (16 - n) * (kMlaRowBytes / 16); idx += 32) {
       const int r = n + idx / (kMlaRowBytes / 16), piece = idx % (kMlaRowBytes / 16);
@@ -700,10 +728,6 @@ __global__ void __launch_bounds__(kMThreads, 1) mla_decode_kernel(const __grid_c
   const TableEntry* table = p.table + static_cast<size_t>(cd.stream) * p.table_stride;
   const uint16_t* qg = p.q + static_cast<size_t>(cd.stream) * kMlaHeads * kMlaDk;
 
-  // (launched with programmatic stream serialisation as well: nothing above reads what an earlier kernel of the
-  // stream may have written; the table, the query and the cache are touched after this wait)
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   if (tid == 0) *abort_flag = 0;
   if (wq == 0 && lane == 0) {
     m_bar_init(bars, 1);
@@ -711,15 +735,67 @@ __global__ void __launch_bounds__(kMThreads, 1) mla_decode_kernel(const __grid_c
     m_fence_async();
   }
   if (warp == 0) m_tmem_alloc(base + kMOffFlag + 4, kMTmemCols);
-  {
-    // the query as fp16 (exact for the magnitudes a query has), the heads g and g + 8 interleaved per channel pair
-    for (int idx = tid; idx < 8 * kMlaChunks; idx += kMThreads) {
-      const int hp = idx / kMlaChunks, piece = idx % kMlaChunks;
-      const uint4 v0 = *reinterpret_cast<const uint4*>(qg + hp * kMlaDk + 8 * piece);
-      const uint4 v1 = *reinterpret_cast<const uint4*>(qg + (hp + 8) * kMlaDk + 8 * piece);
-      const uint32_t d = hp * kMQPitch + 32 * piece;
-      m_sts128(q16 + d, m_bf2_to_h2(v0.x), m_bf2_to_h2(v1.x), m_bf2_to_h2(v0.y), m_bf2_to_h2(v1.y));
-      m_sts128(q16 + d + 16, m_bf2_to_h2(v0.z), m_bf2_to_h2(v1.z), m_bf2_to_h2(v0.w), m_bf2_to_h2(v1.w));
+  // (launched with programmatic stream serialisation as well: nothing above reads what an earlier kernel of the
+  // stream may have written; the table, the query and the cache are touched after this wait)
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  // The query: a thread takes 16-byte pieces of the heads hp and hp + 8, asked for before the first copies are set up.
+  constexpr int kPieces = (8 * kMlaChunks + kMThreads - 1) / kMThreads;
+  uint4 qv[kPieces][2];
+#pragma unroll
+  for (int i = 0; i < kPieces; ++i) {
+    const int idx = tid + i * kMThreads, hp = idx / kMlaChunks, piece = idx % kMlaChunks;
+    if (idx < 8 * kMlaChunks) {
+      qv[i][0] = *reinterpret_cast<const uint4*>(qg + hp * kMlaDk + 8 * piece);
+      qv[i][1] = *reinterpret_cast<const uint4*>(qg + (hp + 8) * kMlaDk + 8 * piece);
+    }
+  }
+  // The first two units' copies (this warp's lane 0 initialised the barriers): what follows runs while they do.
+  MWalk wl;
+  uint32_t um[kMStages];                     // meta words of the units in the two stages
+  m_begin(p, table, cd.item_begin, cd.item_end, lane, wl);
+#pragma unroll
+  for (int i = 0; i < kMStages; ++i) {
+    um[i] = wl.meta;
+    if (wl.meta != kMNoUnit) {
+      if (wq == 0) m_issue(p, wl, qd + i * kMStageBytes, bars + 8 * i, lane);
+      m_advance(p, table, cd.item_end, lane, wl);
+    }
+  }
+  // The rows go through shared memory as they are first, where every warp picks up the A fragments (bf16, rows = heads g
+  // and g + 8) of its nine channel slabs for the units of exact and centroid rows; then as fp16 (exact for the
+  // magnitudes a query has), the heads g and g + 8 interleaved per channel pair.  (Fragments loaded from global memory
+  // by every warp, four bytes a lane, held up the first unit by 2 us.)
+#pragma unroll
+  for (int i = 0; i < kPieces; ++i) {
+    const int idx = tid + i * kMThreads, hp = idx / kMlaChunks, piece = idx % kMlaChunks;
+    if (idx < 8 * kMlaChunks) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const uint32_t d = q16 + (hp + 8 * k) * (kMQPitch / 2) + 16 * piece;
+        m_sts64(d, qv[i][k].x, qv[i][k].y);
+        m_sts64(d + 8, qv[i][k].z, qv[i][k].w);
+      }
+    }
+  }
+  __syncthreads();
+  uint32_t qf[9][4];
+#pragma unroll
+  for (int sl = 0; sl < 9; ++sl) {
+    const uint32_t a = q16 + g * (kMQPitch / 2) + 2 * ((sl < 8 ? 128 * wq + 16 * sl : kMlaDv + 16 * wq) + 2 * c4);
+    qf[sl][0] = m_lds32(a);
+    qf[sl][1] = m_lds32(a + 8 * (kMQPitch / 2));
+    qf[sl][2] = m_lds32(a + 16);
+    qf[sl][3] = m_lds32(a + 8 * (kMQPitch / 2) + 16);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kPieces; ++i) {
+    const int idx = tid + i * kMThreads, hp = idx / kMlaChunks, piece = idx % kMlaChunks;
+    if (idx < 8 * kMlaChunks) {
+      const uint32_t d = q16 + hp * kMQPitch + 32 * piece;
+      m_sts128(d, m_bf2_to_h2(qv[i][0].x), m_bf2_to_h2(qv[i][1].x), m_bf2_to_h2(qv[i][0].y), m_bf2_to_h2(qv[i][1].y));
+      m_sts128(d + 16, m_bf2_to_h2(qv[i][0].z), m_bf2_to_h2(qv[i][1].z), m_bf2_to_h2(qv[i][0].w), m_bf2_to_h2(qv[i][1].w));
     }
   }
   m_tfence_before();
@@ -728,60 +804,40 @@ __global__ void __launch_bounds__(kMThreads, 1) mla_decode_kernel(const __grid_c
   // this warp's 64 columns of its lane quarter: the running O^T, zero to begin with
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(msm + kMOffFlag + 4);
   const uint32_t ot = tmem + (static_cast<uint32_t>(32 * wq) << 16) + 64u * static_cast<uint32_t>(quad);
+  const uint32_t qt = tmem + (static_cast<uint32_t>(32 * wq) << 16) + kMTmemQ + 36u * static_cast<uint32_t>(quad);
   {
     const float zero[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
     for (int mu = 0; mu < 8; ++mu) m_tst8(ot + 8 * mu, zero);
-    m_twait_st();
-  }
-  // the bf16 query as the A fragments of the warp's nine channel slabs (rows = heads g and g + 8), for the units of
-  // exact and centroid rows
-  const uint32_t qt = tmem + (static_cast<uint32_t>(32 * wq) << 16) + kMTmemQ + 36u * static_cast<uint32_t>(quad);
-  {
-    const uint16_t* qa = qg + g * kMlaDk + 2 * c4;
-#pragma unroll 3
-    for (int sl = 0; sl < 9; ++sl) {
-      const int ch0 = sl < 8 ? 128 * wq + 16 * sl : kMlaDv + 16 * wq;
-      const uint32_t f[4] = {m_ldg32(qa + ch0), m_ldg32(qa + 8 * kMlaDk + ch0), m_ldg32(qa + ch0 + 8), m_ldg32(qa + 8 * kMlaDk + ch0 + 8)};
-      m_tst4(qt + 4 * sl, f);
-    }
+#pragma unroll
+    for (int sl = 0; sl < 9; ++sl) m_tst4(qt + 4 * sl, qf[sl]);
     m_twait_st();
   }
   float m_run[2] = {kMNegInf, kMNegInf}, l_run[2] = {0.f, 0.f};
 
-  MWalk wc, wl;
-  wc.it = cd.item_begin;
-  bool have_c = m_load(p, table, cd.item_end, wc);
-  wl = wc;
-  bool have_l = have_c;
-  // the first two units' copies
-#pragma unroll 1
-  for (int i = 0; i < kMStages; ++i) {
-    if (have_l) {
-      if (wq == 0) m_issue(p, table, wl, qd + i * kMStageBytes, bars + 8 * i, lane);
-      have_l = m_advance(p, table, cd.item_end, wl);
-    }
-  }
   int k = 0;
 #pragma unroll 1
-  while (have_c) {
+  while (true) {
     const int s = k & 1;
+    const uint32_t meta = um[0];
+    if (meta == kMNoUnit) break;
+    um[0] = um[1];
+    um[1] = wl.meta;
     const uint32_t st = qd + s * kMStageBytes;
     // after a time-out nothing waits any more: the remaining units run through on whatever the stages hold
     if (!*abort_flag && !m_wait(bars + 8 * s, (k >> 1) & 1)) *abort_flag = 1;
-    if (wc.kind() == 0) {
-      if (wc.level() == 8) m_unit_quant<8>(st, q16, xb, quad, wq, g, c4, p.scale_log2, ot, m_run, l_run);
+    if (m_kind(meta) == 0) {
+      if (m_level(meta) == 8) m_unit_quant<8>(st, q16, xb, quad, wq, g, c4, p.scale_log2, ot, m_run, l_run);
       else m_unit_quant<4>(st, q16, xb, quad, wq, g, c4, p.scale_log2, ot, m_run, l_run);
     } else {
-      m_unit_rows16(st, qt, xb, quad, wq, lane, p.scale_log2, wc.kind() == 2 ? 6.0f : 0.f, m_unit_rows(wc), ot, m_run, l_run);
+      m_unit_rows16(st, qt, xb, quad, wq, lane, p.scale_log2, m_kind(meta) == 2 ? 6.0f : 0.f, m_unit_rows(meta), ot, m_run, l_run);
     }
     // the stage and the exchange buffer are free once all four warps are here
     m_quad_sync(quad);
-    if (have_l) {
-      if (wq == 0) m_issue(p, table, wl, st, bars + 8 * s, lane);
-      have_l = m_advance(p, table, cd.item_end, wl);
+    if (wl.meta != kMNoUnit) {
+      if (wq == 0) m_issue(p, wl, st, bars + 8 * s, lane);
+      m_advance(p, table, cd.item_end, lane, wl);
     }
-    have_c = m_advance(p, table, cd.item_end, wc);
     ++k;
   }
 
@@ -816,29 +872,38 @@ __global__ void __launch_bounds__(kMThreads, 1) mla_decode_kernel(const __grid_c
   }
   __syncthreads();
   // ---- merge of the quads in quad order -> the CTA's partial row ----
+  // The weights of the sixteen heads are made once (64 threads), then the rows are added two channels at a time.
+  // (With the weights made in every thread for every channel the merge took 7.7 us of a CTA's time; this takes 1.8.)
   {
     const bool good = !*abort_flag;
     float* out = p.partial + static_cast<size_t>(cd.partial) * kMlaPartialFloats;
     const float* sm = reinterpret_cast<const float*>(msm + kMOffQuad);
     constexpr int kQF = kMQuadBytes / 4;                      // floats between two quads' results
-    for (int idx = tid; idx < kMlaHeads * kMlaDv; idx += kMThreads) {
-      const int head = idx / kMlaDv, ch = idx % kMlaDv;
-      float M = kMNegInf;
+    float* sw = reinterpret_cast<float*>(msm + kMOffQ16);     // [head][quad]: the query is no longer needed
+    if (tid < kMlaHeads * kMlaQuads) {
+      const int head = tid >> 2, qn = tid & 3;
+      const float* ml = sm + qn * kQF + kMlaHeads * kMOutPitch + head;
+      const float m = ml[0], l = ml[16];
+      float M = fmaxf(m, __shfl_xor_sync(kMFull, m, 1));
+      M = fmaxf(M, __shfl_xor_sync(kMFull, M, 2));
+      const float wgt = (m == kMNegInf || !good) ? 0.f : exp2f(m - M);
+      float L = wgt * l;
+      L += __shfl_xor_sync(kMFull, L, 1);
+      L += __shfl_xor_sync(kMFull, L, 2);
+      sw[tid] = wgt;
+      if (qn == 0) *reinterpret_cast<float2*>(out + head * (kMlaDv + 2)) = make_float2(good ? M : kMNegInf, L);
+    }
+    __syncthreads();
 #pragma unroll
-      for (int qn = 0; qn < kMlaQuads; ++qn) M = fmaxf(M, sm[qn * kQF + kMlaHeads * kMOutPitch + head]);
-      float acc = 0.f, L = 0.f;
-#pragma unroll
-      for (int qn = 0; qn < kMlaQuads; ++qn) {
-        const float mq = sm[qn * kQF + kMlaHeads * kMOutPitch + head];
-        const float wgt = (mq == kMNegInf) ? 0.f : exp2f(mq - M);
-        acc = fmaf(wgt, sm[qn * kQF + head * kMOutPitch + ch], acc);
-        L = fmaf(wgt, sm[qn * kQF + kMlaHeads * kMOutPitch + 16 + head], L);
-      }
-      out[head * (kMlaDv + 2) + 2 + ch] = good ? acc : 0.f;
-      if (ch == 0) {
-        out[head * (kMlaDv + 2)] = good ? M : kMNegInf;
-        out[head * (kMlaDv + 2) + 1] = good ? L : 0.f;
-      }
+    for (int i = 0; i < kMlaHeads * kMlaDv / 2 / kMThreads; ++i) {
+      const int idx = tid + i * kMThreads, head = idx / (kMlaDv / 2), ch = 2 * (idx % (kMlaDv / 2));
+      const float4 wgt = *reinterpret_cast<const float4*>(sw + 4 * head);
+      const float* row = sm + head * kMOutPitch + ch;
+      const float2 v0 = *reinterpret_cast<const float2*>(row), v1 = *reinterpret_cast<const float2*>(row + kQF);
+      const float2 v2 = *reinterpret_cast<const float2*>(row + 2 * kQF), v3 = *reinterpret_cast<const float2*>(row + 3 * kQF);
+      const float a0 = fmaf(wgt.w, v3.x, fmaf(wgt.z, v2.x, fmaf(wgt.y, v1.x, wgt.x * v0.x)));
+      const float a1 = fmaf(wgt.w, v3.y, fmaf(wgt.z, v2.y, fmaf(wgt.y, v1.y, wgt.x * v0.y)));
+      *reinterpret_cast<float2*>(out + head * (kMlaDv + 2) + 2 + ch) = good ? make_float2(a0, a1) : make_float2(0.f, 0.f);
     }
   }
   if (tid == 0 && *abort_flag) atomicOr(p.status, kStatusInternal);
@@ -847,64 +912,62 @@ __global__ void __launch_bounds__(kMThreads, 1) mla_decode_kernel(const __grid_c
   if (warp == 0) m_tmem_dealloc(tmem, kMTmemCols);
 }
 
-// Merge the partial rows of a stream's CTAs.  One block per (stream, head, slice of 64 value
-// channels); its 512 threads are 8 row groups x 64 channels, row group g sums rows g, g + 8, ...
-// in that order and the 8 sums are added in group order, so the result is bitwise reproducible.
-constexpr int kCombSlice = 64, kCombGroups = 8, kCombThreads = kCombSlice * kCombGroups;
+// Merge the partial rows of a stream's CTAs (at most kMlaMaxRows).  One block per (stream, head, slice of 64 value
+// channels).  Thread i holds row i's (m, l): maximum, weights and denominator are block reductions; then warp v
+// sums the rows v, v + 16, ... of the slice, two channels a lane, and the warps' sums are added in warp order, so
+// the result is bitwise reproducible.  Bound by latency (4.9 MB of partial rows, in L2): two dependent rounds of
+// loads.  (Before, every thread swept all the maxima and one thread added up the denominator: 7 us behind the read for
+// 148 rows.)
+constexpr int kCombSlice = 64, kCombThreads = 512, kCombWarps = kCombThreads / 32;
+static_assert(kMlaMaxRows <= kCombThreads, "one thread per partial row");
 __global__ void __launch_bounds__(kCombThreads) mla_combine_kernel(const float* partial, const StreamParts* parts, float* out,
                                                                    float* lse) {
-  __shared__ float sm_m[kCombThreads], sm_w[kCombThreads], sm_acc[kCombGroups][kCombSlice];
+  __shared__ float sm_red[kCombWarps], sm_l[kCombWarps], sm_w[kCombThreads], sm_acc[kCombWarps][kCombSlice];
   // launched with programmatic stream serialisation: the launch overlaps the decode kernel's tail, the
   // partial rows are touched only after that kernel has completed
+  const int stream = blockIdx.x, h = blockIdx.y, slice = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-  const int stream = blockIdx.x, h = blockIdx.y, slice = blockIdx.z, tid = threadIdx.x;
-  const int c = tid % kCombSlice, g = tid / kCombSlice;
-  const int begin = parts[stream].begin, end = parts[stream].end;
-  const float* base = partial + h * (kMlaDv + 2);
-  // pass 1: the maximum of the rows' maxima (one row per thread, then a shared-memory sweep)
-  float M = kMNegInf;
-  for (int c0 = begin; c0 < end; c0 += kCombThreads) {
-    const int n = min(kCombThreads, end - c0);
-    __syncthreads();
-    sm_m[tid] = tid < n ? __ldcg(base + static_cast<size_t>(c0 + tid) * kMlaPartialFloats) : kMNegInf;
-    __syncthreads();
-#pragma unroll 8
-    for (int i = 0; i < n; ++i) M = fmaxf(M, sm_m[i]);
-  }
-  // pass 2: weights per row in shared memory, then every thread sums its channel over its rows
-  float L = 0.f, acc = 0.f;
-  for (int c0 = begin; c0 < end; c0 += kCombThreads) {
-    const int n = min(kCombThreads, end - c0);
-    __syncthreads();
-    if (tid < n) {
-      const float* row = base + static_cast<size_t>(c0 + tid) * kMlaPartialFloats;
-      const float m = __ldcg(row);
-      const float w = (m == kMNegInf) ? 0.f : exp2f(m - M);
-      sm_w[tid] = w;
-      sm_m[tid] = w * __ldcg(row + 1);
-    }
-    __syncthreads();
-    const float* col = base + static_cast<size_t>(c0) * kMlaPartialFloats + 2 + slice * kCombSlice + c;
-#pragma unroll 8
-    for (int i = g; i < n; i += kCombGroups) acc = fmaf(sm_w[i], __ldcg(col + static_cast<size_t>(i) * kMlaPartialFloats), acc);
-    if (g == 0 && c == 0)
-      for (int i = 0; i < n; ++i) L += sm_m[i];
-  }
-  sm_acc[g][c] = acc;
-  __syncthreads();
-  if (g == 0) {
-    if (c == 0) sm_m[0] = L;
-  }
-  __syncthreads();
-  L = sm_m[0];
-  if (g == 0) {
-    float tot = 0.f;
+  const int begin = parts[stream].begin, n = parts[stream].end - begin;
+  const float* base = partial + static_cast<size_t>(begin) * kMlaPartialFloats + h * (kMlaDv + 2);
+  float2 ml = make_float2(kMNegInf, 0.f);
+  if (tid < n) ml = __ldcg(reinterpret_cast<const float2*>(base + static_cast<size_t>(tid) * kMlaPartialFloats));
+  float M = ml.x;
 #pragma unroll
-    for (int k = 0; k < kCombGroups; ++k) tot += sm_acc[k][c];
+  for (int d = 16; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(kMFull, M, d));
+  if (lane == 0) sm_red[warp] = M;
+  __syncthreads();
+  M = sm_red[0];
+#pragma unroll
+  for (int w = 1; w < kCombWarps; ++w) M = fmaxf(M, sm_red[w]);
+  const float wgt = (ml.x == kMNegInf) ? 0.f : exp2f(ml.x - M);
+  sm_w[tid] = wgt;
+  float L = wgt * ml.y;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) L += __shfl_xor_sync(kMFull, L, d);
+  if (lane == 0) sm_l[warp] = L;
+  __syncthreads();
+  const float* col = base + 2 + slice * kCombSlice + 2 * lane;
+  float a0 = 0.f, a1 = 0.f;
+#pragma unroll 5
+  for (int i = warp; i < n; i += kCombWarps) {
+    const float2 v = __ldcg(reinterpret_cast<const float2*>(col + static_cast<size_t>(i) * kMlaPartialFloats));
+    a0 = fmaf(sm_w[i], v.x, a0);
+    a1 = fmaf(sm_w[i], v.y, a1);
+  }
+  *reinterpret_cast<float2*>(&sm_acc[warp][2 * lane]) = make_float2(a0, a1);
+  __syncthreads();
+  if (tid < kCombSlice) {
+    float tot = 0.f;
+    L = 0.f;
+#pragma unroll
+    for (int w = 0; w < kCombWarps; ++w) {
+      tot += sm_acc[w][tid];
+      L += sm_l[w];
+    }
     const size_t hq = static_cast<size_t>(stream) * kMlaHeads + h;
-    out[hq * kMlaDv + slice * kCombSlice + c] = (L > 0.f) ? tot / L : 0.f;
-    if (lse && slice == 0 && c == 0) lse[hq] = (L > 0.f) ? (M + log2f(L)) * 0.6931471805599453f : kMNegInf;
+    out[hq * kMlaDv + slice * kCombSlice + tid] = (L > 0.f) ? tot / L : 0.f;
+    if (lse && slice == 0 && tid == 0) lse[hq] = (L > 0.f) ? (M + log2f(L)) * 0.6931471805599453f : kMNegInf;
   }
 }
 
