@@ -8,6 +8,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <mutex>
 #include <numeric>
 #include <thread>
@@ -78,13 +79,78 @@ struct SlotHeap {
   void release(int level, uint32_t off) { free_list[level_index(level)].push_back(off); }
 };
 
+// Page-locked host memory for a cache's mirrors and staging.  Locking and unlocking pages is the slowest thing a
+// cache's creation and release do (1 - 3 ms per MB here, against 0.2 ms for the rest), and a serving process
+// makes a cache per request, so a released cache leaves its block to the next one.  What is kept is bounded (four
+// blocks, 64 MiB), and a block that eight creations in a row had no use for is given back.  A block goes
+// back only when its cache's copies are done (gkv_destroy waits for them), so the next owner may be another
+// thread's or stream's cache, on any device.
+class PinnedPool {
+ public:
+  cudaError_t take(size_t bytes, uint8_t** ptr, size_t* size) {
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      ++clock_;
+      size_t best = kept_.size();
+      for (size_t i = 0; i < kept_.size(); ++i)      // the smallest that is large enough, unless most of it would lie idle
+        if (kept_[i].size >= bytes && kept_[i].size <= 4 * bytes + kGranule && (best == kept_.size() || kept_[i].size < kept_[best].size)) best = i;
+      if (best < kept_.size()) {
+        const Block b = kept_[best];
+        kept_.erase(kept_.begin() + static_cast<std::ptrdiff_t>(best));
+        drop_stale();
+        cudaPointerAttributes attr{};
+        if (cudaPointerGetAttributes(&attr, b.ptr) == cudaSuccess && attr.type == cudaMemoryTypeHost) {
+          *ptr = b.ptr;
+          *size = b.size;
+          return cudaSuccess;
+        }
+        cudaGetLastError();                          // the device was reset meanwhile and took the block with it
+      } else {
+        drop_stale();
+      }
+    }
+    *size = align_up(bytes, kGranule);
+    return cudaHostAlloc(reinterpret_cast<void**>(ptr), *size, cudaHostAllocPortable);
+  }
+  void give(uint8_t* ptr, size_t size) {
+    std::lock_guard<std::mutex> lock(mutex_);
+    size_t held = size;
+    for (const Block& b : kept_) held += b.size;
+    while (!kept_.empty() && (held > kMaxBytes || kept_.size() >= kMaxBlocks)) held -= drop(0);       // oldest first
+    if (size > kMaxBytes) cudaFreeHost(ptr);
+    else kept_.push_back(Block{ptr, size, clock_});
+  }
+
+ private:
+  static constexpr size_t kGranule = 64 << 10, kMaxBytes = 64 << 20, kMaxBlocks = 4, kMaxAge = 8;
+  struct Block { uint8_t* ptr; size_t size, since; };
+  size_t drop(size_t i) {
+    const size_t n = kept_[i].size;
+    cudaFreeHost(kept_[i].ptr);
+    kept_.erase(kept_.begin() + static_cast<std::ptrdiff_t>(i));
+    return n;
+  }
+  void drop_stale() {
+    for (size_t i = kept_.size(); i-- > 0;)
+      if (clock_ - kept_[i].since > kMaxAge) drop(i);
+  }
+  std::mutex mutex_;
+  std::vector<Block> kept_;             // in the order in which they came
+  size_t clock_ = 0;                    // creations so far
+};
+// (never destroyed: at process exit the CUDA runtime may be gone before static objects are)
+PinnedPool& pinned_pool() {
+  static PinnedPool* pool = new PinnedPool();
+  return *pool;
+}
+
 struct LayerState {
   int n_closed = 0, n_tail = 0;
   bool has_tail_slot = false;
   std::vector<int8_t> level;            // [n_streams][max_blocks]
   TableEntry* table_h = nullptr;        // pinned [n_streams][table_stride]
   WarpDesc* warps_h = nullptr;          // pinned [max_warps]
-  uint32_t* units_h = nullptr;          // pinned [n_streams][unit_stride]
+  uint32_t* units_h = nullptr;          // pinned [units_cap]
   int n_units = 0;
   StreamParts* parts_h = nullptr;       // pinned [n_streams * head_groups]
   uint32_t* res_off_h = nullptr;        // pinned [n_streams]
@@ -153,7 +219,9 @@ struct gkv_cache {
   cudaEvent_t ev_demote[kDemoteSlots] = {};
   // shared pinned staging (jobs | levels | k-per-stream), guarded by ev_stage
   uint8_t* stage_h = nullptr;
-  size_t stage_bytes = 0;
+  // the page-locked block that all pinned members of the cache and of its layers lie in
+  uint8_t* pinned = nullptr;
+  size_t pinned_bytes = 0;
   cudaEvent_t ev_stage = nullptr;
   int last_cuda = 0;
 };
@@ -172,7 +240,8 @@ struct ArenaPlan {
 };
 
 struct Derived {
-  int n_streams, group, head_groups, n_hgroups, max_blocks, table_stride, max_warps, res_cap, box_stride, unit_stride;
+  int n_streams, group, head_groups, n_hgroups, max_blocks, table_stride, max_warps, res_cap, box_stride;
+  size_t units_cap;
 };
 
 int validate_config(const gkv_config* c) {
@@ -218,7 +287,9 @@ Derived derive(const gkv_config& c) {
   d.res_cap = c.residual_fraction > 0.f
                   ? static_cast<int>(align_up(static_cast<size_t>(std::floor(static_cast<double>(c.residual_fraction) * c.max_ctx)) + 16, 16))
                   : 0;
-  d.unit_stride = d.max_blocks + 1 + d.res_cap / 16 + 3 * (kTargetWarps / 2);      // small workloads list sub-block units
+  // units of a layer: every item, and up to three more for the items that small workloads cut (fewer than
+  // kTargetWarps items in all; a single stream's exact blocks only below half of that)
+  d.units_cap = static_cast<size_t>(d.n_streams) * (d.max_blocks + 1 + d.res_cap / 16) + static_cast<size_t>(std::min(d.n_streams, 2)) * 3 * (kTargetWarps / 2);
   d.box_stride = c.page_tokens > 0 ? static_cast<int>(align_up((c.max_ctx + c.page_tokens - 1) / c.page_tokens, 8)) : 0;
   return d;
 }
@@ -249,7 +320,7 @@ ArenaPlan plan_arena(const gkv_config& c, const Derived& d) {
   auto ltake = [&](size_t bytes) { size_t o = lo; lo = align_up(lo + bytes, 256); return o; };
   a.l_table = ltake(static_cast<size_t>(d.n_streams) * d.table_stride * sizeof(TableEntry));
   a.l_warps = ltake(static_cast<size_t>(d.max_warps) * sizeof(WarpDesc));
-  a.l_units = ltake(static_cast<size_t>(d.n_streams) * d.unit_stride * sizeof(uint32_t));
+  a.l_units = ltake(d.units_cap * sizeof(uint32_t));
   a.l_parts = ltake(static_cast<size_t>(d.n_hgroups) * sizeof(StreamParts));
   a.l_resoff = ltake(static_cast<size_t>(d.n_streams) * sizeof(uint32_t));
   a.l_rescount = ltake(static_cast<size_t>(d.n_streams) * sizeof(int32_t));
@@ -1404,16 +1475,38 @@ int gkv_create(const gkv_config* cfg, void* arena, size_t arena_bytes, gkv_cache
   };
   cudaError_t e = cudaMemset(c->arena, 0, a.heap_begin);
   if (e != cudaSuccess) return fail(e);
-  c->stage_bytes = align_up(c->jobs_cap * sizeof(EncodeJob), 256) + align_up(static_cast<size_t>(d.n_streams) * d.max_blocks, 256) +
-                   align_up(d.n_streams * sizeof(int32_t), 256) + 1024;
-  if ((e = cudaHostAlloc(reinterpret_cast<void**>(&c->stage_h), c->stage_bytes, cudaHostAllocDefault)) != cudaSuccess) return fail(e);
-  if ((e = cudaEventCreateWithFlags(&c->ev_stage, cudaEventDisableTiming)) != cudaSuccess) return fail(e);
   c->demote_cap = static_cast<size_t>(d.n_streams) * 8;
-  if ((e = cudaHostAlloc(reinterpret_cast<void**>(&c->demote_h), gkv_cache::kDemoteSlots * c->demote_cap * sizeof(EncodeJob),
-                         cudaHostAllocDefault)) != cudaSuccess) return fail(e);
+  const size_t stage_bytes = align_up(c->jobs_cap * sizeof(EncodeJob), 256) + align_up(static_cast<size_t>(d.n_streams) * d.max_blocks, 256) +
+                             align_up(d.n_streams * sizeof(int32_t), 256) + 1024;
+  const size_t table_bytes = static_cast<size_t>(d.n_streams) * d.table_stride * sizeof(TableEntry);
+  // lays the pinned members out from `base`; the distance to the end is the block's size
+  auto lay_out = [&](uint8_t* base) {
+    size_t off = 0;
+    auto take = [&](auto*& ptr, size_t bytes) {
+      if (base) ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(base + off);
+      off = align_up(off + bytes, 256);
+    };
+    take(c->stage_h, stage_bytes);
+    take(c->demote_h, gkv_cache::kDemoteSlots * c->demote_cap * sizeof(EncodeJob));
+    for (LayerState& L : c->layers) {
+      take(L.table_h, table_bytes);
+      take(L.warps_h, d.max_warps * sizeof(WarpDesc));
+      take(L.units_h, d.units_cap * sizeof(uint32_t));
+      take(L.parts_h, d.n_hgroups * sizeof(StreamParts));
+      take(L.res_off_h, d.n_streams * sizeof(uint32_t));
+      take(L.res_count_h, d.n_streams * sizeof(int32_t));
+    }
+    return off;
+  };
+  c->layers.resize(cfg->n_layers);
+  if ((e = pinned_pool().take(lay_out(nullptr), &c->pinned, &c->pinned_bytes)) != cudaSuccess) {
+    c->pinned = nullptr;
+    return fail(e);
+  }
+  lay_out(c->pinned);
+  if ((e = cudaEventCreateWithFlags(&c->ev_stage, cudaEventDisableTiming)) != cudaSuccess) return fail(e);
   for (int i = 0; i < gkv_cache::kDemoteSlots; ++i)
     if ((e = cudaEventCreateWithFlags(&c->ev_demote[i], cudaEventDisableTiming)) != cudaSuccess) return fail(e);
-  c->layers.resize(cfg->n_layers);
   for (int l = 0; l < cfg->n_layers; ++l) {
     LayerState& L = c->layers[l];
     uint8_t* lb = c->arena + a.per_layer + static_cast<size_t>(l) * a.layer_bytes;
@@ -1430,15 +1523,7 @@ int gkv_create(const gkv_config* cfg, void* arena, size_t arena_bytes, gkv_cache
     L.err_d = reinterpret_cast<float4*>(lb + a.l_err);
     L.level.assign(static_cast<size_t>(d.n_streams) * d.max_blocks, 0);
     L.res_idx.resize(d.n_streams);
-    const size_t tb = static_cast<size_t>(d.n_streams) * d.table_stride * sizeof(TableEntry);
-    if ((e = cudaHostAlloc(reinterpret_cast<void**>(&L.table_h), tb, cudaHostAllocDefault)) != cudaSuccess) return fail(e);
-    std::memset(L.table_h, 0, tb);
-    if ((e = cudaHostAlloc(reinterpret_cast<void**>(&L.warps_h), d.max_warps * sizeof(WarpDesc), cudaHostAllocDefault)) != cudaSuccess) return fail(e);
-    if ((e = cudaHostAlloc(reinterpret_cast<void**>(&L.units_h), static_cast<size_t>(d.n_streams) * d.unit_stride * sizeof(uint32_t),
-                           cudaHostAllocDefault)) != cudaSuccess) return fail(e);
-    if ((e = cudaHostAlloc(reinterpret_cast<void**>(&L.parts_h), d.n_hgroups * sizeof(StreamParts), cudaHostAllocDefault)) != cudaSuccess) return fail(e);
-    if ((e = cudaHostAlloc(reinterpret_cast<void**>(&L.res_off_h), d.n_streams * sizeof(uint32_t), cudaHostAllocDefault)) != cudaSuccess) return fail(e);
-    if ((e = cudaHostAlloc(reinterpret_cast<void**>(&L.res_count_h), d.n_streams * sizeof(int32_t), cudaHostAllocDefault)) != cudaSuccess) return fail(e);
+    std::memset(L.table_h, 0, table_bytes);
     for (int s = 0; s < d.n_streams; ++s) {
       L.res_count_h[s] = 0;
       L.res_off_h[s] = static_cast<uint32_t>((a.per_layer + static_cast<size_t>(l) * a.layer_bytes + a.l_respool +
@@ -1446,7 +1531,7 @@ int gkv_create(const gkv_config* cfg, void* arena, size_t arena_bytes, gkv_cache
     }
     if ((e = cudaEventCreateWithFlags(&L.ev, cudaEventDisableTiming)) != cudaSuccess) return fail(e);
     if ((e = cudaEventCreateWithFlags(&L.ev_desc, cudaEventDisableTiming)) != cudaSuccess) return fail(e);
-    if ((e = cudaMemcpy(L.res_off_d, L.res_off_h, d.n_streams * sizeof(uint32_t), cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e);
+    if ((e = cudaMemcpyAsync(L.res_off_d, L.res_off_h, d.n_streams * sizeof(uint32_t), cudaMemcpyHostToDevice, nullptr)) != cudaSuccess) return fail(e);
   }
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return fail(e);
   *out = c;
@@ -1583,22 +1668,22 @@ int gkv_debug_device_plan(gkv_cache* c, int32_t layer, int8_t* levels_out, float
 
 int gkv_destroy(gkv_cache* c) {
   if (!c) return GKV_ERR_INVALID_ARG;
+  // every copy from the pinned block has to be done before the block finds a new owner
+  int cur = -1;
+  const bool other = cudaGetDevice(&cur) == cudaSuccess && c->device >= 0 && cur != c->device;
   cudaDeviceSynchronize();
+  if (other && cudaSetDevice(c->device) == cudaSuccess) {
+    cudaDeviceSynchronize();
+    cudaSetDevice(cur);
+  }
   for (LayerState& L : c->layers) {
-    if (L.table_h) cudaFreeHost(L.table_h);
-    if (L.warps_h) cudaFreeHost(L.warps_h);
-    if (L.units_h) cudaFreeHost(L.units_h);
-    if (L.parts_h) cudaFreeHost(L.parts_h);
-    if (L.res_off_h) cudaFreeHost(L.res_off_h);
-    if (L.res_count_h) cudaFreeHost(L.res_count_h);
     if (L.ev) cudaEventDestroy(L.ev);
     if (L.ev_desc) cudaEventDestroy(L.ev_desc);
   }
-  if (c->stage_h) cudaFreeHost(c->stage_h);
-  if (c->demote_h) cudaFreeHost(c->demote_h);
   for (cudaEvent_t ev : c->ev_demote)
     if (ev) cudaEventDestroy(ev);
   if (c->ev_stage) cudaEventDestroy(c->ev_stage);
+  if (c->pinned) pinned_pool().give(c->pinned, c->pinned_bytes);
   delete c;
   return GKV_OK;
 }
