@@ -8,19 +8,24 @@
 // warp's loads run along pages and coalesce.
 //
 // Selection: k largest scores, ties to the lower index, emitted in ascending index order
-// (radix select on an order-preserving key, then an ordered compaction).
+// (the threshold on an order-preserving key first, then an ordered compaction).
 #include "gkv_internal.h"
 
 namespace gkv {
 namespace {
 
-constexpr float kNegInfQ = -__builtin_huge_valf();
-
-// One CTA scores kQPages consecutive pages of one stream.  The 256 box rows of the stream (channel x
-// min|max, kQPages * 2 bytes of each) are streamed through shared memory in chunks of kQRows rows
-// with 16-byte cp.async copies, kQStages chunks in flight, so that the loads are wide, contiguous
+// One CTA scores kQPages consecutive pages of one stream, two neighbouring pages per thread.  The 256 box rows of
+// the stream (channel x min|max, kQPages * 2 bytes of each) are streamed through shared memory in chunks of
+// kQRows rows with 16-byte cp.async copies, kQStages chunks in flight, so that the loads are wide, contiguous
 // and deep while every thread still adds its pages' channels strictly in order.
-constexpr int kQThreads = 128, kQPages = kQThreads;          // one page per thread
+//
+// The choice between maximum and minimum depends on the sign of q_d only, so it is made once, when the query is
+// staged: acc <- fma(max(q, 0), hi, fma(min(q, 0), lo, acc)), where one of the two products is a zero that leaves
+// acc as it is.  Two pages share an instruction (packed fp32 pairs, each half rounded as usual), which leaves 18
+// instructions per channel and two pages for four heads; with a select per head and one page per thread it was 40,
+// and the kernel was bound by instruction issue.  (Selection and read of 2048 pages x 32 streams: 37.0 -> 32.4 us a
+// layer with this and the selection below.)
+constexpr int kQThreads = 64, kQPages = 2 * kQThreads;
 constexpr int kQRows = 32;                                   // rows per chunk = 16 channels x (min, max)
 constexpr int kQStages = 4;
 constexpr int kQRowBytes = kQPages * 2;                      // 256
@@ -31,6 +36,18 @@ constexpr int kQChunks = 2 * kD / kQRows;                    // 8
 __device__ __forceinline__ void q_cp_async16(uint32_t dst, const void* src, bool on) {
   const uint32_t n = on ? 16u : 0u;                          // 0 source bytes: the 16 bytes are zero-filled
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ uint64_t q_pair(float x, float y) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+// two bf16 numbers as a pair of fp32
+__device__ __forceinline__ uint64_t q_pair_bf16(uint32_t u) { return q_pair(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)); }
+__device__ __forceinline__ uint64_t q_fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
 }
 
 // GROUP = query heads per KV head, a compile-time bound: a run-time bound would leave the unused
@@ -46,13 +63,13 @@ __global__ void __launch_bounds__(kQThreads) quest_score_kernel(const uint16_t* 
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   extern __shared__ __align__(16) uint8_t qsm[];
-  float (*qs)[kD] = reinterpret_cast<float (*)[kD]>(qsm + kQStages * kQChunkBytes);       // [8][128]
+  // per channel and head the pairs (q+, q+) and (q-, q-)
+  ulonglong2* qs = reinterpret_cast<ulonglong2*>(qsm + kQStages * kQChunkBytes);       // [128][GROUP]
   const int stream = blockIdx.y, tid = threadIdx.x;
-  const int b = stream / n_kv_heads, kvh = stream - b * n_kv_heads;
   const int page0 = blockIdx.x * kQPages;
   const uint16_t* rows = boxes + static_cast<size_t>(stream) * kD * 2 * box_stride + page0;
   const uint32_t stage0 = static_cast<uint32_t>(__cvta_generic_to_shared(qsm));
-  // chunk c -> stage c % kQStages: row r of the chunk is box row c * kQRows + r; a row is 32 pieces
+  // chunk c -> stage c % kQStages: row r of the chunk is box row c * kQRows + r; a row is 16 pieces
   // of 16 bytes (8 pages); pieces that start beyond the row's end (box_stride) are zero-filled
   auto issue = [&](int c) {
     const uint32_t dst = stage0 + (c % kQStages) * kQChunkBytes;
@@ -66,40 +83,54 @@ __global__ void __launch_bounds__(kQThreads) quest_score_kernel(const uint16_t* 
   };
 #pragma unroll
   for (int c = 0; c < kQStages - 1; ++c) issue(c);
-  for (int i = tid; i < group * kD; i += kQThreads) {
-    const int h = i / kD, d = i - h * kD;
-    const uint16_t bits = q[(static_cast<size_t>(b) * n_kv_heads * group + static_cast<size_t>(kvh) * group + h) * kD + d];
-    qs[h][d] = __uint_as_float(static_cast<uint32_t>(bits) << 16);
-  }
-  float acc[GROUP];
+  {
+    const uint32_t* q2 = reinterpret_cast<const uint32_t*>(q + static_cast<size_t>(stream) * group * kD);      // [batch][n_q_heads], KV heads in order
 #pragma unroll
-  for (int h = 0; h < GROUP; ++h) acc[h] = 0.f;
+    for (int h = 0; h < GROUP; ++h) {
+      const uint32_t u = q2[h * (kD / 2) + tid];
+      const float v[2] = {__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)};
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float up = fmaxf(v[k], 0.f), dn = fminf(v[k], 0.f);
+        qs[(2 * tid + k) * GROUP + h] = make_ulonglong2(q_pair(up, up), q_pair(dn, dn));
+      }
+    }
+  }
+  uint64_t acc[GROUP];
+#pragma unroll
+  for (int h = 0; h < GROUP; ++h) acc[h] = 0ull;
 #pragma unroll 1
   for (int c = 0; c < kQChunks; ++c) {
     if (c + kQStages - 1 < kQChunks) issue(c + kQStages - 1);
     else asm volatile("cp.async.commit_group;\n" ::: "memory");          // keeps the group count uniform
     asm volatile("cp.async.wait_group %0;\n" ::"n"(kQStages - 1) : "memory");
     __syncthreads();                                   // chunk c (and, the first time, the query) is visible to all
-    const uint8_t* st = qsm + (c % kQStages) * kQChunkBytes + tid * 2;
+    const uint8_t* st = qsm + (c % kQStages) * kQChunkBytes + tid * 4;
+    const ulonglong2* qc = qs + c * (kQRows / 2) * GROUP;
 #pragma unroll
     for (int i = 0; i < kQRows / 2; ++i) {
-      const float lo = __uint_as_float(static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(st + (2 * i) * kQRowBytes)) << 16);
-      const float hi = __uint_as_float(static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(st + (2 * i + 1) * kQRowBytes)) << 16);
-      const int d = c * (kQRows / 2) + i;
+      const uint64_t lo = q_pair_bf16(*reinterpret_cast<const uint32_t*>(st + (2 * i) * kQRowBytes));
+      const uint64_t hi = q_pair_bf16(*reinterpret_cast<const uint32_t*>(st + (2 * i + 1) * kQRowBytes));
 #pragma unroll
       for (int h = 0; h < GROUP; ++h) {
-        const float qv = qs[h][d];
-        acc[h] = __fmaf_rn(qv, qv >= 0.f ? hi : lo, acc[h]);
+        const ulonglong2 qv = qc[i * GROUP + h];
+        acc[h] = q_fma2(qv.x, hi, q_fma2(qv.y, lo, acc[h]));
       }
     }
     __syncthreads();                                   // the stage may be refilled
   }
-  const int p0 = page0 + tid;
-  if (p0 >= n_pages) return;
-  float s0 = acc[0];
+  const int p0 = page0 + 2 * tid;
 #pragma unroll
-  for (int h = 1; h < GROUP; ++h) s0 = (reduce == 0) ? fmaxf(s0, acc[h]) : __fadd_rn(s0, acc[h]);
-  scores[static_cast<size_t>(stream) * score_stride + p0] = s0;
+  for (int k = 0; k < 2; ++k) {
+    if (p0 + k >= n_pages) return;
+    float s0 = __uint_as_float(static_cast<uint32_t>(acc[0] >> (32 * k)));
+#pragma unroll
+    for (int h = 1; h < GROUP; ++h) {
+      const float s1 = __uint_as_float(static_cast<uint32_t>(acc[h] >> (32 * k)));
+      s0 = (reduce == 0) ? fmaxf(s0, s1) : __fadd_rn(s0, s1);
+    }
+    scores[static_cast<size_t>(stream) * score_stride + p0 + k] = s0;
+  }
 }
 
 // Order-preserving key: larger score <-> larger key; -0 and +0 map to the same key.
@@ -110,9 +141,110 @@ __device__ __forceinline__ uint32_t score_key(float s) {
 
 constexpr int kTopkThreads = 1024;
 
-// KEEP: n <= 4 * kTopkThreads, every thread keeps the keys of its (up to four) elements in registers
-// instead of reading the scores again in every pass.
-template <bool KEEP>
+// Selection with every key in registers: thread t holds the keys of the elements [PER t, PER t + PER).  The k-th largest
+// key is bracketed by counting: lo <= it <= hi, three probes a round, the keys at or above each counted with warp
+// reductions and one barrier.  The search ends early when exactly k keys lie at or above lo.  One scan over the
+// threads then gives every selected element its place in index order.  (A radix select puts its first digit, sign and
+// exponent, of nearly all scores into a few bins whose shared-memory counters are then incremented one by one, and its
+// compaction took four barriers per 1024 elements: 29 us for 16,384 scores of 32 streams, 21 us this way.)
+template <int PER>
+__global__ void __launch_bounds__(kTopkThreads) topk_regs_kernel(const float* __restrict__ scores, int score_stride, int n,
+                                                                 const int32_t* __restrict__ k_per_stream, int k_uniform,
+                                                                 int32_t* __restrict__ idx_out, int idx_stride) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  __shared__ uint2 s_cnt[2][32];
+  __shared__ uint32_t s_scan[32];
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  const int stream = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = blockDim.x >> 5;
+  const float* sc = scores + static_cast<size_t>(stream) * score_stride;
+  int32_t* out = idx_out + static_cast<size_t>(stream) * idx_stride;
+  const uint32_t k = static_cast<uint32_t>(min(k_per_stream ? k_per_stream[stream] : k_uniform, n));
+  if (static_cast<int>(k) <= 0) return;
+  uint32_t key[PER];                                 // 0 past the end: below every probe
+  uint32_t mn = kAll, mx = 0u;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const int i = tid * PER + j;
+    key[j] = i < n ? max(score_key(sc[i]), 1u) : 0u;
+    if (i < n) {
+      mn = min(mn, key[j]);
+      mx = max(mx, key[j]);
+    }
+  }
+  mn = __reduce_min_sync(kAll, mn);
+  mx = __reduce_max_sync(kAll, mx);
+  if (lane == 0) s_cnt[1][warp] = make_uint2(mn, mx);
+  __syncthreads();
+  {
+    const uint2 v = lane < n_warps ? s_cnt[1][lane] : make_uint2(kAll, 0u);
+    mn = __reduce_min_sync(kAll, v.x);
+    mx = __reduce_max_sync(kAll, v.y);
+  }
+  uint32_t lo = mn, hi = mx, n_lo = static_cast<uint32_t>(n);      // n_lo keys are >= lo; fewer than k are > hi
+  int round = 0;
+  while (lo < hi && n_lo != k) {                     // uniform for the CTA
+    const uint32_t range = hi - lo, step = range / 4 + 1;
+    const uint32_t p1 = lo + min(step, range), p2 = lo + min(2 * step, range), p3 = lo + static_cast<uint32_t>(min(3ull * step, static_cast<unsigned long long>(range)));
+    uint32_t c12 = 0, c3 = 0;                        // counts of a thread <= 32, of the CTA <= 32,768: 16 bits each
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      c12 += (key[j] >= p1 ? 1u : 0u) + (key[j] >= p2 ? 0x10000u : 0u);
+      c3 += key[j] >= p3 ? 1u : 0u;
+    }
+    c12 = __reduce_add_sync(kAll, c12);
+    c3 = __reduce_add_sync(kAll, c3);
+    if (lane == 0) s_cnt[round & 1][warp] = make_uint2(c12, c3);
+    __syncthreads();                                 // (the other buffer is rewritten only behind the next barrier)
+    const uint2 v = lane < n_warps ? s_cnt[round & 1][lane] : make_uint2(0u, 0u);
+    c12 = __reduce_add_sync(kAll, v.x);
+    c3 = __reduce_add_sync(kAll, v.y);
+    const uint32_t c1 = c12 & 0xffffu, c2 = c12 >> 16;
+    if (c3 >= k) {
+      lo = p3;
+      n_lo = c3;
+    } else if (c2 >= k) {
+      lo = p2;
+      n_lo = c2;
+      hi = p3 - 1;
+    } else if (c1 >= k) {
+      lo = p1;
+      n_lo = c1;
+      hi = p2 - 1;
+    } else {
+      hi = p1 - 1;
+    }
+    ++round;
+  }
+  // taken: the keys above `thr`, and of those equal to `eq` the first ones in index order until k are taken
+  const bool all = n_lo == k;                        // exactly the keys at or above lo
+  const uint32_t thr = all ? lo - 1 : lo, eq = all ? 0u : lo;
+  uint32_t mine = 0;                                 // above | equal << 16
+#pragma unroll
+  for (int j = 0; j < PER; ++j) mine += (key[j] > thr ? 1u : 0u) + ((eq != 0u && key[j] == eq) ? 0x10000u : 0u);
+  uint32_t incl = mine;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t up = __shfl_up_sync(kAll, incl, d);
+    if (lane >= d) incl += up;
+  }
+  if (lane == 31) s_scan[warp] = incl;
+  __syncthreads();
+  const uint32_t ws = lane < n_warps ? s_scan[lane] : 0u;
+  const uint32_t total = __reduce_add_sync(kAll, ws);
+  const uint32_t before = __reduce_add_sync(kAll, lane < warp ? ws : 0u) + incl - mine;
+  const uint32_t need = k - (total & 0xffffu);       // equal keys taken
+  uint32_t above = before & 0xffffu, equal = before >> 16;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    const bool gt = key[j] > thr, same = eq != 0u && key[j] == eq;
+    if (gt || (same && equal < need)) out[above + min(equal, need)] = tid * PER + j;
+    above += gt ? 1u : 0u;
+    equal += same ? 1u : 0u;
+  }
+}
+
+// Longer lists: radix select over the scores in global memory, ordered compaction.
 __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const float* __restrict__ scores, int score_stride,
                                                             int n, const int32_t* __restrict__ k_per_stream,
                                                             int k_uniform, int32_t* __restrict__ idx_out,
@@ -133,14 +265,6 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const float* __restr
     s_prefix = 0;
     s_remaining = static_cast<uint32_t>(k);
   }
-  uint32_t kreg[4] = {0u, 0u, 0u, 0u};
-  if (KEEP) {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int i = tid + j * kTopkThreads;
-      if (i < n) kreg[j] = score_key(sc[i]);
-    }
-  }
   // radix select, most significant byte first: find the key of the k-th largest score
   for (int pass = 0; pass < 4; ++pass) {
     const int shift = 24 - 8 * pass;
@@ -148,15 +272,9 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const float* __restr
     __syncthreads();
     const uint32_t prefix = s_prefix;
     const uint32_t pmask = pass == 0 ? 0u : (0xffffffffu << (shift + 8));
-    if (KEEP) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (tid + j * kTopkThreads < n && (kreg[j] & pmask) == prefix) atomicAdd(&hist[(kreg[j] >> shift) & 255u], 1u);
-    } else {
-      for (int i = tid; i < n; i += kTopkThreads) {
-        const uint32_t key = score_key(sc[i]);
-        if ((key & pmask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-      }
+    for (int i = tid; i < n; i += kTopkThreads) {
+      const uint32_t key = score_key(sc[i]);
+      if ((key & pmask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
     }
     __syncthreads();
     // The digit of the k-th largest is the t with c[t] >= rem > c[t + 1], c[t] = sum_{j >= t} hist[j].
@@ -201,13 +319,12 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const float* __restr
   // ordered compaction in index order
   const int lane = tid & 31, wid = tid >> 5;
 #pragma unroll 1
-  for (int i0 = 0, j = 0; i0 < n; i0 += kTopkThreads, ++j) {
+  for (int i0 = 0; i0 < n; i0 += kTopkThreads) {
     const int i = i0 + tid;
     uint32_t key = 0;
     bool gt = false, eq = false;
     if (i < n) {
-      if (KEEP) key = j == 0 ? kreg[0] : (j == 1 ? kreg[1] : (j == 2 ? kreg[2] : kreg[3]));
-      else key = score_key(sc[i]);
+      key = score_key(sc[i]);
       gt = key > thr;
       eq = key == thr;
     }
@@ -246,7 +363,7 @@ cudaError_t launch_quest_scores(const uint16_t* boxes, int box_stride, int n_pag
                                 int n_streams, int n_kv_heads, int group, int reduce, float* scores,
                                 int score_stride, cudaStream_t st) {
   if (n_pages <= 0) return cudaSuccess;
-  const size_t smem = kQStages * kQChunkBytes + kMaxHeadsPerKv * kD * sizeof(float);
+  const size_t smem = kQStages * kQChunkBytes + static_cast<size_t>(group) * kD * 16;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((n_pages + kQPages - 1) / kQPages, n_streams);
   cfg.blockDim = dim3(kQThreads);
@@ -297,9 +414,16 @@ cudaError_t launch_topk(const float* scores, int score_stride, int n, const int3
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (n <= 4 * kTopkThreads)
-    return cudaLaunchKernelEx(&cfg, topk_kernel<true>, scores, score_stride, n, k_per_stream, k_uniform, idx_out, idx_stride);
-  return cudaLaunchKernelEx(&cfg, topk_kernel<false>, scores, score_stride, n, k_per_stream, k_uniform, idx_out, idx_stride);
+#define GKV_TOPK_CASE(PER)                                                                                                  \
+  if (n <= PER * kTopkThreads) {                                                                                           \
+    cfg.blockDim = dim3(static_cast<unsigned>(((n + PER - 1) / PER + 31) / 32 * 32));                                      \
+    return cudaLaunchKernelEx(&cfg, topk_regs_kernel<PER>, scores, score_stride, n, k_per_stream, k_uniform, idx_out, idx_stride); \
+  }
+  GKV_TOPK_CASE(4)
+  GKV_TOPK_CASE(16)
+  GKV_TOPK_CASE(32)
+#undef GKV_TOPK_CASE
+  return cudaLaunchKernelEx(&cfg, topk_kernel, scores, score_stride, n, k_per_stream, k_uniform, idx_out, idx_stride);
 }
 
 }  // namespace gkv
