@@ -155,7 +155,8 @@ struct LayerState {
   StreamParts* parts_h = nullptr;       // pinned [n_streams * head_groups]
   uint32_t* res_off_h = nullptr;        // pinned [n_streams]
   int32_t* res_count_h = nullptr;       // pinned [n_streams]
-  std::vector<std::vector<int32_t>> res_idx;
+  std::vector<std::vector<int32_t>> res_idx;      // host copy of the residual rows' tokens, fetched when first asked for
+  bool res_idx_valid = true;
   bool desc_dirty = true;
   bool desc_split = false;              // the work lists hold sub-block units (never for observing calls)
   bool desc_allow_split = false;        // what the lists were built with
@@ -199,11 +200,9 @@ struct gkv_cache {
   uint32_t* status_d = nullptr;
   uint8_t* debug_d = nullptr;
   float* partial_d = nullptr;
-  float* range_d = nullptr;
-  float* mass_d = nullptr;
+  uint32_t* plan_flag_d = nullptr;      // set by the device allocator when a stream cannot meet the budget
   int8_t* levels_d = nullptr;
   float* scores_d = nullptr;            // residual scores [n_streams][max_ctx] or page scores
-  int32_t* kper_d = nullptr;
   int32_t* tickets_d = nullptr;         // per-head-group arrival counters of the decode kernel's final merge
   float2* mass_raw_d = nullptr;         // scratch of an observing decode call: [n_streams][max_blocks + 1][8]
   float2* res_raw_d = nullptr;          // [n_streams][res_cap][8]
@@ -235,7 +234,7 @@ constexpr int kMlaTargetCtas = kMlaMaxRows;  // one CTA per SM (212 KB of shared
 constexpr size_t kMlaMinCtaCost = 1000;      // one block: two of a CTA's four quads have a half each
 
 struct ArenaPlan {
-  size_t status, debug, partial, range, mass, levels, scores, kper, tickets, jobs, mass_raw, res_raw, lse2, per_layer, heap_begin, total_meta;
+  size_t status, debug, partial, plan_flag, levels, scores, tickets, jobs, mass_raw, res_raw, lse2, per_layer, heap_begin, total_meta;
   size_t l_table, l_warps, l_units, l_parts, l_resoff, l_rescount, l_residx, l_respool, l_boxes, l_ema, l_range, l_err, layer_bytes;
 };
 
@@ -302,12 +301,10 @@ ArenaPlan plan_arena(const gkv_config& c, const Derived& d) {
   a.debug = take(kBlock * kMlaDk + 2 * 4096 + kBlock * kMlaDk * 2);
   a.partial = take(is_mla(c) ? static_cast<size_t>(kMlaTargetCtas + 2 * d.n_streams) * kMlaPartialFloats * sizeof(float)
                              : static_cast<size_t>(d.max_warps) * kPartialFloats * sizeof(float));
-  a.range = take(static_cast<size_t>(d.n_streams) * d.max_blocks * sizeof(float));
-  a.mass = take(static_cast<size_t>(d.n_streams) * d.max_blocks * sizeof(float));
+  a.plan_flag = take(sizeof(uint32_t));
   a.levels = take(static_cast<size_t>(d.n_streams) * d.max_blocks);
   const size_t score_elems = std::max<size_t>(c.residual_fraction > 0.f ? c.max_ctx : 0, d.box_stride);
   a.scores = take(static_cast<size_t>(d.n_streams) * score_elems * sizeof(float));
-  a.kper = take(static_cast<size_t>(d.n_streams) * sizeof(int32_t));
   a.tickets = take(static_cast<size_t>(d.n_hgroups) * sizeof(int32_t));
   a.jobs = take(static_cast<size_t>(d.n_streams) * d.max_blocks * sizeof(EncodeJob));
   // block-mass observation (grouped-query layout only)
@@ -730,6 +727,76 @@ int wait_event(gkv_cache* c, cudaEvent_t ev) {
   return GKV_OK;
 }
 
+// Largest number of closed blocks whose breakpoints the device allocator sorts in shared memory.
+constexpr int kRdPlanMaxBlocks = 4095;
+
+// Queues the device allocator for every stream of a layer (running masses L.ema_d, range proxies L.range_d): levels into
+// c->levels_d, a flag into c->plan_flag_d when some stream cannot meet the budget.  n <= kRdPlanMaxBlocks.
+int rd_plan_launch(gkv_cache* c, LayerState& L, int n, int n_tail, bool use_prev, int n_res, int32_t* res_count, cudaStream_t st) {
+  const gkv_config& cfg = c->cfg;
+  const long long nval_tok = cfg.d_k + cfg.d_v;
+  const long long T = static_cast<long long>(n) * kBlock + n_tail;
+  RdPlanParams p{};
+  p.mass = L.ema_d;
+  p.range = L.range_d;
+  p.table = L.table_d;
+  p.levels_out = c->levels_d;
+  p.miss_flag = c->plan_flag_d;
+  p.n = n;
+  p.mass_stride = c->max_blocks + 1;
+  p.range_stride = c->max_blocks;
+  p.table_stride = c->table_stride;
+  p.out_stride = c->max_blocks;
+  rd_plan_smem_bytes(n, &p.m_pad);
+  p.n_sink_blocks = cfg.n_sink_blocks;
+  p.retire_after = cfg.retire_after;
+  p.monotone = cfg.monotone_in_age != 0;
+  p.use_prev = use_prev;
+  p.nval_tok = static_cast<unsigned long long>(nval_tok);
+  p.budget_bits = static_cast<unsigned long long>(std::floor(static_cast<double>(cfg.rd_budget_bpv) * static_cast<double>(T * nval_tok)));
+  p.tail_bits = static_cast<unsigned long long>(n_tail) * 16ull * static_cast<unsigned long long>(nval_tok);
+  p.res_count = res_count;
+  p.n_res = n_res;
+  p.res_cap = c->res_cap;
+  CK(c, cudaMemsetAsync(p.miss_flag, 0, sizeof(uint32_t), st));
+  CK(c, launch_rd_plan(p, c->n_streams, st));
+  return GKV_OK;
+}
+
+// Level plan of every stream of a layer on the host, from masses and ranges that are read back: more blocks than the
+// device allocator takes.  prev: nullable present levels [n_streams][max_blocks].  Synchronises.
+int rd_plan_host(gkv_cache* c, LayerState& L, int n, int n_tail, const int8_t* prev, int8_t* target, size_t stride, bool* missed, cudaStream_t st) {
+  const int ns = c->n_streams;
+  std::vector<float> mass(static_cast<size_t>(ns) * n), range(static_cast<size_t>(ns) * n);
+  CK(c, cudaMemcpy2DAsync(mass.data(), static_cast<size_t>(n) * sizeof(float), L.ema_d,
+                          static_cast<size_t>(c->max_blocks + 1) * sizeof(float), static_cast<size_t>(n) * sizeof(float), ns,
+                          cudaMemcpyDeviceToHost, st));
+  CK(c, cudaMemcpy2DAsync(range.data(), static_cast<size_t>(n) * sizeof(float), L.range_d,
+                          static_cast<size_t>(c->max_blocks) * sizeof(float), static_cast<size_t>(n) * sizeof(float), ns,
+                          cudaMemcpyDeviceToHost, st));
+  CK(c, cudaStreamSynchronize(st));
+  *missed = rd_allocate_streams(c->cfg, mass.data(), range.data(), n, n_tail, ns, prev, c->max_blocks, target, stride);
+  return GKV_OK;
+}
+
+// Level plan of a re-allocation: on the device where it takes the layer (one small launch and n bytes per stream back
+// instead of 8 n and the host's sort), else on the host.  target: [n_streams][n].  *missed: some stream cannot meet the
+// budget.  Synchronises `st` to read the plan back.
+int rd_plan_layer(gkv_cache* c, LayerState& L, int8_t* target, bool* missed, cudaStream_t st) {
+  const int n = L.n_closed;
+  *missed = false;
+  if (n > kRdPlanMaxBlocks) return rd_plan_host(c, L, n, L.n_tail, L.level.data(), target, n, missed, st);
+  int rc = rd_plan_launch(c, L, n, L.n_tail, true, 0, nullptr, st);
+  if (rc != GKV_OK) return rc;
+  uint32_t flag = 0;
+  CK(c, cudaMemcpy2DAsync(target, static_cast<size_t>(n), c->levels_d, static_cast<size_t>(c->max_blocks), static_cast<size_t>(n), c->n_streams,
+                          cudaMemcpyDeviceToHost, st));
+  CK(c, cudaMemcpyAsync(&flag, c->plan_flag_d, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+  CK(c, cudaStreamSynchronize(st));
+  *missed = flag != 0;
+  return GKV_OK;
+}
+
 int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* v_new, int n_new,
                 const float* token_mass, const int8_t* level_plan, cudaStream_t st) {
   const gkv_config& cfg = c->cfg;
@@ -755,13 +822,36 @@ int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* 
     sp.page_tokens = cfg.page_tokens;
     sp.boxes = L.boxes_d;
     sp.box_stride = c->box_stride;
-    sp.block_range = need_rd ? c->range_d : nullptr;
-    sp.block_mass = need_rd ? c->mass_d : nullptr;
+    // (the prefill observer's block masses start the running mass of the decode phase, Sec. 3.1)
+    sp.block_range = need_rd ? L.range_d : nullptr;
+    sp.block_mass = need_rd ? L.ema_d : nullptr;
+    sp.range_stride = c->max_blocks;
+    sp.mass_stride = c->max_blocks + 1;
     CK(c, launch_stats(sp, st));
   }
 
-  // 2. level plan
+  // 2. level plan, and the choice of the exact residual rows (Sec. 3.4: score every token, top fraction per stream).
+  // Under the rate-distortion policy the plan is made on the device and read back, one byte per block; the residual's
+  // score and selection follow it there, so that they run while the host, which waits for the plan only, allocates the
+  // slots.  (With masses and ranges read back, the allocator on host threads, and the selected rows read back for
+  // the masks, a request over 4 layers x 32 streams x 16,405 tokens took 5.8 ms, 3.9 now.)
+  const bool has_res = cfg.residual_fraction > 0.f && token_mass && n_closed > 0;
+  const int n_res_nom = static_cast<int>(std::floor(static_cast<double>(cfg.residual_fraction) * static_cast<double>(n_new)));
+  uint8_t* stage = c->stage_h;
+  size_t stage_off = 0;
+  auto stage_take = [&](size_t bytes) {
+    uint8_t* at = stage + stage_off;
+    stage_off = align_up(stage_off + bytes, 256);
+    return at;
+  };
+  auto residual_select = [&]() -> int {                // levels in c->levels_d, rows per stream in L.res_count_d
+    CK(c, launch_residual_scores(v_new, token_mass, c->levels_d, c->max_blocks, cfg.n_sink_blocks, ns,
+                                 cfg.n_kv_heads, n_new, n_closed, c->scores_d, st));
+    CK(c, launch_topk(c->scores_d, n_new, n_closed * kBlock, L.res_count_d, 0, L.res_idx_d, c->res_cap, ns, st));
+    return GKV_OK;
+  };
   std::fill(L.level.begin(), L.level.end(), 0);
+  bool selected = false;
   if (cfg.policy == GKV_POLICY_STAIRCASE) {
     std::vector<int8_t> lv(std::max(n_closed, 1));
     staircase_levels(cfg, n_closed, lv.data());
@@ -774,18 +864,25 @@ int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* 
         L.level[static_cast<size_t>(s) * c->max_blocks + b] = v;
       }
   } else if (n_closed > 0) {
-    std::vector<float> range(static_cast<size_t>(ns) * n_closed), mass(static_cast<size_t>(ns) * n_closed);
-    CK(c, cudaMemcpyAsync(range.data(), c->range_d, range.size() * sizeof(float), cudaMemcpyDeviceToHost, st));
-    CK(c, cudaMemcpyAsync(mass.data(), c->mass_d, mass.size() * sizeof(float), cudaMemcpyDeviceToHost, st));
-    CK(c, cudaStreamSynchronize(st));
-    // the prefill observer's block masses start the running mass of the decode phase (Sec. 3.1)
-    CK(c, cudaMemcpy2DAsync(L.ema_d, static_cast<size_t>(c->max_blocks + 1) * sizeof(float), c->mass_d,
-                            static_cast<size_t>(n_closed) * sizeof(float), static_cast<size_t>(n_closed) * sizeof(float), ns,
-                            cudaMemcpyDeviceToDevice, st));
-    CK(c, cudaMemcpy2DAsync(L.range_d, static_cast<size_t>(c->max_blocks) * sizeof(float), c->range_d,
-                            static_cast<size_t>(n_closed) * sizeof(float), static_cast<size_t>(n_closed) * sizeof(float), ns,
-                            cudaMemcpyDeviceToDevice, st));
-    if (rd_allocate_streams(cfg, mass.data(), range.data(), n_closed, n_tail, ns, nullptr, 0, L.level.data(), c->max_blocks)) {
+    bool missed = false;
+    if (n_closed <= kRdPlanMaxBlocks) {
+      if ((rc = rd_plan_launch(c, L, n_closed, n_tail, false, n_res_nom, has_res ? L.res_count_d : nullptr, st)) != GKV_OK) return rc;
+      uint8_t* lv = stage_take(static_cast<size_t>(ns) * n_closed);
+      uint32_t* flag = reinterpret_cast<uint32_t*>(stage_take(sizeof(uint32_t)));
+      CK(c, cudaMemcpy2DAsync(lv, n_closed, c->levels_d, c->max_blocks, n_closed, ns, cudaMemcpyDeviceToHost, st));
+      CK(c, cudaMemcpyAsync(flag, c->plan_flag_d, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+      CK(c, cudaEventRecord(c->ev_stage, st));
+      if (has_res) {
+        if ((rc = residual_select()) != GKV_OK) return rc;
+        selected = true;
+      }
+      if ((rc = wait_event(c, c->ev_stage)) != GKV_OK) return rc;
+      for (int s = 0; s < ns; ++s) std::memcpy(&L.level[static_cast<size_t>(s) * c->max_blocks], lv + static_cast<size_t>(s) * n_closed, n_closed);
+      missed = *flag != 0;
+    } else if ((rc = rd_plan_host(c, L, n_closed, n_tail, nullptr, L.level.data(), c->max_blocks, &missed, st)) != GKV_OK) {
+      return rc;
+    }
+    if (missed) {
       L.budget_flag = true;
       warn = GKV_ERR_BUDGET;
     }
@@ -794,7 +891,6 @@ int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* 
   // 3. slots + table mirror.  The fast encoder takes its work from the table itself, so on its path
   // the sequences go up in groups: slots of a group, its table rows, its encode launch, and the
   // host allocates the next group's slots while the GPU encodes this one.
-  const bool has_res = cfg.residual_fraction > 0.f && token_mass && n_closed > 0;
   const bool fast = n_closed > 0 && v_new &&
                     ((reinterpret_cast<uintptr_t>(k_new) | reinterpret_cast<uintptr_t>(v_new)) & 15u) == 0;
   auto alloc_streams = [&](int s0, int s1) -> int {
@@ -849,17 +945,11 @@ int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* 
   }
   L.has_tail_slot = true;
 
-  // 4. exact residual (Sec. 3.4): score, top fraction per stream, gather rows, mask the blocks
-  uint8_t* stage = c->stage_h;
-  size_t stage_off = 0;
-  if (cfg.residual_fraction > 0.f && token_mass && n_closed > 0) {
-    const int n_res_nom = static_cast<int>(std::floor(static_cast<double>(cfg.residual_fraction) * static_cast<double>(n_new)));
-    int8_t* lv_stage = reinterpret_cast<int8_t*>(stage + stage_off);
-    std::memcpy(lv_stage, L.level.data(), L.level.size());
-    stage_off = align_up(stage_off + L.level.size(), 256);
-    int32_t* k_stage = reinterpret_cast<int32_t*>(stage + stage_off);
-    stage_off = align_up(stage_off + ns * sizeof(int32_t), 256);
-    int max_k = 0;
+  // 4. exact residual rows per stream (the device allocator counts them itself), and their selection where the levels
+  // were made on the host
+  int max_k = 0;
+  if (has_res) {
+    int32_t* k_stage = reinterpret_cast<int32_t*>(stage_take(ns * sizeof(int32_t)));
     for (int s = 0; s < ns; ++s) {
       int eligible = 0;
       for (int b = 0; b < n_closed; ++b)
@@ -868,43 +958,28 @@ int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* 
       max_k = std::max(max_k, k_stage[s]);
       L.res_count_h[s] = k_stage[s];
     }
-    CK(c, cudaMemcpyAsync(c->levels_d, lv_stage, L.level.size(), cudaMemcpyHostToDevice, st));
-    CK(c, cudaMemcpyAsync(c->kper_d, k_stage, ns * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-    CK(c, launch_residual_scores(v_new, token_mass, c->levels_d, c->max_blocks, cfg.n_sink_blocks, ns,
-                                 cfg.n_kv_heads, n_new, n_closed, c->scores_d, st));
-    CK(c, launch_topk(c->scores_d, n_new, n_closed * kBlock, c->kper_d, 0, L.res_idx_d, c->res_cap, ns, st));
-    if (max_k > 0) {
-      std::vector<int32_t> idx(static_cast<size_t>(ns) * c->res_cap);
-      CK(c, cudaMemcpyAsync(idx.data(), L.res_idx_d, idx.size() * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-      CK(c, cudaStreamSynchronize(st));
-      for (int s = 0; s < ns; ++s) {
-        L.res_idx[s].assign(idx.begin() + static_cast<size_t>(s) * c->res_cap,
-                            idx.begin() + static_cast<size_t>(s) * c->res_cap + L.res_count_h[s]);
-        for (int32_t tok : L.res_idx[s]) {
-          if (tok < 0 || tok >= n_closed * kBlock) return GKV_ERR_BAD_STATE;
-          L.table_h[static_cast<size_t>(s) * c->table_stride + tok / kBlock].resmask |= 1ull << (tok % kBlock);
-        }
-      }
+    if (!selected) {
+      int8_t* lv_stage = reinterpret_cast<int8_t*>(stage_take(L.level.size()));
+      std::memcpy(lv_stage, L.level.data(), L.level.size());
+      CK(c, cudaMemcpyAsync(c->levels_d, lv_stage, L.level.size(), cudaMemcpyHostToDevice, st));
+      CK(c, cudaMemcpyAsync(L.res_count_d, k_stage, ns * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+      if ((rc = residual_select()) != GKV_OK) return rc;
     }
+    L.res_idx_valid = max_k == 0;
   }
 
-  // 5. uploads, then encode every closed block once at its planned level (unless done above), copy the tail rows
+  // 5. uploads, then encode every closed block once at its planned level (unless done above), copy the residual and tail
+  // rows.  The residual masks go into the table on the device, behind the table's upload.
   if (!encoded && !fast &&
       (rc = upload(c, L.table_d, L.table_h, static_cast<size_t>(ns) * c->table_stride * sizeof(TableEntry), st, L.ev)) != GKV_OK)
     return rc;
-  if ((rc = upload(c, L.res_count_d, L.res_count_h, ns * sizeof(int32_t), st, L.ev)) != GKV_OK) return rc;
-  if (L.res_count_d && cfg.residual_fraction > 0.f) {
-    int max_k = 0;
-    for (int s = 0; s < ns; ++s) max_k = std::max(max_k, L.res_count_h[s]);
-    CK(c, launch_residual_gather(c->arena, k_new, v_new, n_new, cfg.n_kv_heads, L.res_idx_d, c->res_cap,
-                                 L.res_count_d, L.res_off_d, max_k, ns, st));
-  }
+  if (!has_res && (rc = upload(c, L.res_count_d, L.res_count_h, ns * sizeof(int32_t), st, L.ev)) != GKV_OK) return rc;
   const size_t n_jobs = static_cast<size_t>(ns) * n_closed;
   if (!encoded && fast) {
     if ((rc = encode_streams(0, ns)) != GKV_OK) return rc;
   } else if (!encoded && n_jobs > 0) {
     // inputs that the fast encoder does not take (unaligned rows): the general block encoder, one job per block
-    EncodeJob* jobs = reinterpret_cast<EncodeJob*>(stage + stage_off);
+    EncodeJob* jobs = reinterpret_cast<EncodeJob*>(stage_take(n_jobs * sizeof(EncodeJob)));
     size_t j = 0;
     for (int s = 0; s < ns; ++s)
       for (int b = 0; b < n_closed; ++b) {
@@ -932,6 +1007,9 @@ int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* 
     CK(c, launch_encode(ep, st));
   }
   CK(c, cudaEventRecord(c->ev_stage, st));
+  if (max_k > 0)
+    CK(c, launch_residual_gather(c->arena, k_new, v_new, n_new, cfg.n_kv_heads, n_closed, L.res_idx_d, c->res_cap,
+                                 L.res_count_d, L.res_off_d, max_k, ns, L.table_d, c->table_stride, c->status_d, st));
   CK(c, launch_append_rows(c->arena, L.table_d, c->table_stride, n_closed, ns, cfg.n_kv_heads, k_new, v_new, n_new,
                            n_closed * kBlock, n_tail, 0, st));
   L.n_closed = n_closed;
@@ -1074,8 +1152,7 @@ int append_one(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* v
     sp.err_stride = c->max_blocks;
     if (cfg.policy == GKV_POLICY_RD) {       // range proxy of the closing block, kept for later re-allocation
       sp.block_range = L.range_d;
-      sp.stat_stride = c->max_blocks;
-      sp.stat_base = closed_block;
+      sp.range_stride = c->max_blocks;
     }
     CK(c, launch_stats(sp, st));
   }
@@ -1347,6 +1424,18 @@ int mla_decode(gkv_cache* c, LayerState& L, const void* q, float* out, float* ls
   return GKV_OK;
 }
 
+// The residual rows' tokens as the host's accounting and the parity helpers want them (synchronises the device).
+int fetch_residual(gkv_cache* c, LayerState& L) {
+  if (L.res_idx_valid) return GKV_OK;
+  const size_t ns = c->n_streams, cap = c->res_cap;
+  std::vector<int32_t> idx(ns * cap);
+  CK(c, cudaDeviceSynchronize());
+  CK(c, cudaMemcpy(idx.data(), L.res_idx_d, idx.size() * sizeof(int32_t), cudaMemcpyDeviceToHost));
+  for (size_t s = 0; s < ns; ++s) L.res_idx[s].assign(idx.begin() + s * cap, idx.begin() + s * cap + L.res_count_h[s]);
+  L.res_idx_valid = true;
+  return GKV_OK;
+}
+
 uint64_t full_read_bits(const gkv_cache* c, const LayerState& L) {
   const uint64_t nval_tok = nval_per_token(c->cfg);
   uint64_t bits = 0;
@@ -1456,11 +1545,9 @@ int gkv_create(const gkv_config* cfg, void* arena, size_t arena_bytes, gkv_cache
   c->status_d = reinterpret_cast<uint32_t*>(c->arena + a.status);
   c->debug_d = c->arena + a.debug;
   c->partial_d = reinterpret_cast<float*>(c->arena + a.partial);
-  c->range_d = reinterpret_cast<float*>(c->arena + a.range);
-  c->mass_d = reinterpret_cast<float*>(c->arena + a.mass);
+  c->plan_flag_d = reinterpret_cast<uint32_t*>(c->arena + a.plan_flag);
   c->levels_d = reinterpret_cast<int8_t*>(c->arena + a.levels);
   c->scores_d = reinterpret_cast<float*>(c->arena + a.scores);
-  c->kper_d = reinterpret_cast<int32_t*>(c->arena + a.kper);
   c->tickets_d = reinterpret_cast<int32_t*>(c->arena + a.tickets);
   c->mass_raw_d = reinterpret_cast<float2*>(c->arena + a.mass_raw);
   c->res_raw_d = reinterpret_cast<float2*>(c->arena + a.res_raw);
@@ -1568,62 +1655,6 @@ int gkv_debug_replan_levels(const gkv_config* cfg, int32_t n_closed, int32_t n_t
   if (budget_miss) *budget_miss = miss ? 1 : 0;
   return GKV_OK;
 }
-
-namespace {
-// Largest number of closed blocks whose breakpoints the device allocator sorts in shared memory.
-constexpr int kRdPlanMaxBlocks = 4095;
-
-// Level plan of every stream of a layer from its running masses and range proxies: on the device when
-// the breakpoints fit (one small launch and n bytes per stream back instead of 8 n and the host's
-// sort), else on the host.  target: [n_streams][n].  *missed: some stream cannot meet the budget.
-int rd_plan_layer(gkv_cache* c, LayerState& L, int8_t* target, bool* missed, cudaStream_t st) {
-  const gkv_config& cfg = c->cfg;
-  const int n = L.n_closed, ns = c->n_streams;
-  *missed = false;
-  if (n <= kRdPlanMaxBlocks) {
-    const long long nval_tok = cfg.d_k + cfg.d_v;
-    const long long T = static_cast<long long>(n) * kBlock + L.n_tail;
-    RdPlanParams p{};
-    p.mass = L.ema_d;
-    p.range = L.range_d;
-    p.table = L.table_d;
-    p.levels_out = c->levels_d;
-    p.miss_flag = reinterpret_cast<uint32_t*>(c->mass_d);        // ingest scratch, idle here
-    p.n = n;
-    p.mass_stride = c->max_blocks + 1;
-    p.range_stride = c->max_blocks;
-    p.table_stride = c->table_stride;
-    p.out_stride = c->max_blocks;
-    rd_plan_smem_bytes(n, &p.m_pad);
-    p.n_sink_blocks = cfg.n_sink_blocks;
-    p.retire_after = cfg.retire_after;
-    p.monotone = cfg.monotone_in_age != 0;
-    p.use_prev = 1;
-    p.nval_tok = static_cast<unsigned long long>(nval_tok);
-    p.budget_bits = static_cast<unsigned long long>(std::floor(static_cast<double>(cfg.rd_budget_bpv) * static_cast<double>(T * nval_tok)));
-    p.tail_bits = static_cast<unsigned long long>(L.n_tail) * 16ull * static_cast<unsigned long long>(nval_tok);
-    uint32_t flag = 0;
-    CK(c, cudaMemsetAsync(p.miss_flag, 0, sizeof(uint32_t), st));
-    CK(c, launch_rd_plan(p, ns, st));
-    CK(c, cudaMemcpy2DAsync(target, static_cast<size_t>(n), c->levels_d, static_cast<size_t>(c->max_blocks), static_cast<size_t>(n), ns,
-                            cudaMemcpyDeviceToHost, st));
-    CK(c, cudaMemcpyAsync(&flag, p.miss_flag, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-    CK(c, cudaStreamSynchronize(st));
-    *missed = flag != 0;
-    return GKV_OK;
-  }
-  std::vector<float> mass(static_cast<size_t>(ns) * n), range(static_cast<size_t>(ns) * n);
-  CK(c, cudaMemcpy2DAsync(mass.data(), static_cast<size_t>(n) * sizeof(float), L.ema_d,
-                          static_cast<size_t>(c->max_blocks + 1) * sizeof(float), static_cast<size_t>(n) * sizeof(float), ns,
-                          cudaMemcpyDeviceToHost, st));
-  CK(c, cudaMemcpy2DAsync(range.data(), static_cast<size_t>(n) * sizeof(float), L.range_d,
-                          static_cast<size_t>(c->max_blocks) * sizeof(float), static_cast<size_t>(n) * sizeof(float), ns,
-                          cudaMemcpyDeviceToHost, st));
-  CK(c, cudaStreamSynchronize(st));
-  *missed = rd_allocate_streams(cfg, mass.data(), range.data(), n, L.n_tail, ns, L.level.data(), c->max_blocks, target, n);
-  return GKV_OK;
-}
-}  // namespace
 
 int gkv_rd_reallocate(gkv_cache* c, int32_t layer, void* stream) {
   if (!c || layer < 0 || layer >= c->cfg.n_layers) return GKV_ERR_INVALID_ARG;
@@ -1990,6 +2021,8 @@ int gkv_bits_report(gkv_cache* c, int32_t layer, gkv_bits* out) {
     out->meta_bits += static_cast<uint64_t>(L.n_warps) * sizeof(WarpDesc) * 8 + static_cast<uint64_t>(L.n_units) * 32;
     if (L.last_mode == 1) out->last_read_bits += full_read_bits(c, L);
     if (L.last_mode == 2) {
+      const int rc = fetch_residual(c, L);
+      if (rc != GKV_OK) return rc;
       // fetch the page list that was used and count what it touched
       std::vector<int32_t> pages(static_cast<size_t>(c->n_streams) * std::max(L.last_n_sel, 1));
       if (L.last_n_sel > 0) {
@@ -2059,7 +2092,9 @@ int gkv_debug_export_residual(gkv_cache* c, int32_t layer, int32_t b, int32_t kv
   if (!c || layer < 0 || layer >= c->cfg.n_layers || b < 0 || b >= c->cfg.batch || kv_head < 0 ||
       kv_head >= c->cfg.n_kv_heads || !idx || !n)
     return GKV_ERR_INVALID_ARG;
-  const LayerState& L = c->layers[layer];
+  LayerState& L = c->layers[layer];
+  const int rc = fetch_residual(c, L);
+  if (rc != GKV_OK) return rc;
   const int s = b * c->cfg.n_kv_heads + kv_head;
   *n = static_cast<int32_t>(L.res_idx[s].size());
   for (int i = 0; i < std::min<int>(cap, *n); ++i) idx[i] = L.res_idx[s][i];

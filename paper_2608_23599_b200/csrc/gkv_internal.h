@@ -148,9 +148,9 @@ struct StatsParams {
   int32_t page_tokens;               // 0 = no boxes
   uint16_t* boxes;                   // [n_streams][128][2][box_stride] bf16
   int32_t box_stride;                // pages (padded)
-  float* block_range;                // [n_streams][n_blocks] or nullptr
-  float* block_mass;                 // [n_streams][n_blocks] or nullptr
-  int32_t stat_stride, stat_base;    // range / mass land at [stream * stat_stride + stat_base + i]; stride 0 = n_blocks
+  float* block_range;                // [n_streams][range_stride] by block, or nullptr
+  float* block_mass;                 // [n_streams][mass_stride] by block, or nullptr
+  int32_t range_stride, mass_stride;
   float4* err;                       // nullable; with k_in == nullptr: (0, 0, max_j |v_j|, 0) of the block's exact rows
   int32_t err_stride;
 };
@@ -176,6 +176,9 @@ struct RdPlanParams {
   int32_t m_pad;                // power of two >= 4 n + 1 (rd_plan_smem_bytes)
   int32_t n_sink_blocks, retire_after, monotone, use_prev;
   unsigned long long nval_tok, budget_bits, tail_bits;
+  // Bulk ingest with exact residual rows, nullable: rows of every stream = min(n_res, 64 x blocks planned below 16, res_cap)
+  int32_t* res_count;           // [n_streams]
+  int32_t n_res, res_cap;
 };
 size_t rd_plan_smem_bytes(int n, int* m_pad_out);
 cudaError_t launch_rd_plan(const RdPlanParams& p, int n_streams, cudaStream_t st);
@@ -188,8 +191,9 @@ cudaError_t launch_residual_scores(const uint16_t* v_in, const float* token_mass
 cudaError_t launch_topk(const float* scores, int score_stride, int n, const int32_t* k_per_stream, int k_uniform,
                         int32_t* idx_out, int idx_stride, int n_streams, cudaStream_t st);
 cudaError_t launch_residual_gather(uint8_t* arena, const uint16_t* k_in, const uint16_t* v_in, int n_tok,
-                                   int n_kv_heads, const int32_t* idx, int idx_stride, const int32_t* count,
-                                   const uint32_t* res_off256, int max_count, int n_streams, cudaStream_t st);
+                                   int n_kv_heads, int n_closed, const int32_t* idx, int idx_stride, const int32_t* count,
+                                   const uint32_t* res_off256, int max_count, int n_streams, TableEntry* table,
+                                   int table_stride, uint32_t* status, cudaStream_t st);
 cudaError_t launch_quest_scores(const uint16_t* boxes, int box_stride, int n_pages, const uint16_t* q,
                                 int n_streams, int n_kv_heads, int group, int reduce, float* scores,
                                 int score_stride, cudaStream_t st);

@@ -299,10 +299,24 @@ __global__ void __launch_bounds__(256) encode_kernel(const __grid_constant__ Enc
   }
 }
 
+__device__ __forceinline__ uint32_t bf16x2_min(uint32_t a, uint32_t b) {
+  const __nv_bfloat162 r = __hmin2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
+__device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
+  const __nv_bfloat162 r = __hmax2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
+
 // Per closed block: exact per-page key boxes (min/max of the unquantised bf16 keys), the block's
 // largest per-channel key range (allocator's range proxy) and its attention mass (sequential sum).
-__global__ void __launch_bounds__(kD) stats_kernel(const __grid_constant__ StatsParams p) {
-  const int bi = blockIdx.x, stream = blockIdx.y, c = threadIdx.x;
+// One CTA of two warps per block, two neighbouring channels per thread.  Should be bound by the reads of the rows; one
+// channel per thread with a compare and two selects per bound was bound by the integer pipe (80 % busy) instead.
+// 134 MB of keys (32 streams of 16,405 tokens): 42.5 us then, 29.0 with packed minima and maxima.
+constexpr int kStatThreads = kD / 2;
+__global__ void __launch_bounds__(kStatThreads) stats_kernel(const __grid_constant__ StatsParams p) {
+  __shared__ float s_mass[kBlock], s_red[kStatThreads / 32];
+  const int bi = blockIdx.x, stream = blockIdx.y, c = 2 * threadIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int block = p.first_block + bi;
   const int b = stream / p.n_kv_heads, kvh = stream - b * p.n_kv_heads;
   const uint16_t* rows;
@@ -315,77 +329,92 @@ __global__ void __launch_bounds__(kD) stats_kernel(const __grid_constant__ Stats
     rows = reinterpret_cast<const uint16_t*>(p.arena + static_cast<size_t>(e.off256) * 256);
     row_stride = kD;
   }
-  float bmn = 0.f, bmx = 0.f;
+  if (p.block_mass) s_mass[threadIdx.x] = p.token_mass[static_cast<size_t>(stream) * p.n_tok + static_cast<size_t>(block) * kBlock + threadIdx.x];
+  float bmn[2] = {0.f, 0.f}, bmx[2] = {0.f, 0.f};
   const int page = p.page_tokens > 0 ? p.page_tokens : kBlock;
-  // The block's 64 values of this channel are fetched 16 at a time (independent loads, issued
-  // together) and folded into the running page minimum / maximum; a page is 16, 32 or 64 tokens.
-  uint16_t lo_b = 0, hi_b = 0;
-  float lo = 0.f, hi = 0.f;
+  // The block's 64 values of a channel are fetched 16 at a time (independent loads, issued
+  // together) and folded into the running page minimum / maximum, two channels an instruction; a page is 16, 32
+  // or 64 tokens.
+  const uint16_t* col = rows + c;
+  auto pair_at = [&](int t) { return *reinterpret_cast<const uint32_t*>(col + static_cast<size_t>(t) * row_stride); };
+  uint32_t lo2 = 0, hi2 = 0;
 #pragma unroll 1
   for (int t0 = 0; t0 < kBlock; t0 += 16) {
-    uint16_t xb[16];
+    uint32_t xb[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) xb[i] = rows[static_cast<size_t>(t0 + i) * row_stride + c];
-    if (t0 % page == 0) {
-      lo_b = hi_b = xb[0];
-      lo = hi = bf16_bits_to_f32(xb[0]);
-    }
+    for (int i = 0; i < 16; ++i) xb[i] = pair_at(t0 + i);
+    if (t0 % page == 0) lo2 = hi2 = xb[0];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      const float x = bf16_bits_to_f32(xb[i]);
-      if (x < lo) { lo = x; lo_b = xb[i]; }
-      if (x > hi) { hi = x; hi_b = xb[i]; }
+      lo2 = bf16x2_min(lo2, xb[i]);
+      hi2 = bf16x2_max(hi2, xb[i]);
     }
     if ((t0 + 16) % page == 0) {                       // the page is complete
       const int p0 = t0 + 16 - page;
+      uint16_t lo[2] = {static_cast<uint16_t>(lo2 & 0xffffu), static_cast<uint16_t>(lo2 >> 16)};
+      uint16_t hi[2] = {static_cast<uint16_t>(hi2 & 0xffffu), static_cast<uint16_t>(hi2 >> 16)};
       if (p.page_tokens > 0) {
+        // an extreme that is a zero has the sign of the page's first zero (the instructions order -0 below +0)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if ((lo[k] & 0x7fffu) == 0u || (hi[k] & 0x7fffu) == 0u) {
+            uint16_t first = 0;
+            for (int t = p0 + page - 1; t >= p0; --t) {
+              const uint16_t x = static_cast<uint16_t>(pair_at(t) >> (16 * k));
+              if ((x & 0x7fffu) == 0u) first = x;
+            }
+            if ((lo[k] & 0x7fffu) == 0u) lo[k] = first;
+            if ((hi[k] & 0x7fffu) == 0u) hi[k] = first;
+          }
+        }
         const int pg = block * (kBlock / page) + p0 / page;
-        uint16_t* bx = p.boxes + (static_cast<size_t>(stream) * kD + c) * 2 * p.box_stride;
-        bx[pg] = lo_b;
-        bx[p.box_stride + pg] = hi_b;
+        uint16_t* bx = p.boxes + (static_cast<size_t>(stream) * kD + c) * 2 * p.box_stride + pg;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          bx[2 * k * p.box_stride] = lo[k];
+          bx[(2 * k + 1) * p.box_stride] = hi[k];
+        }
       }
-      if (p0 == 0) { bmn = lo; bmx = hi; }
-      else { bmn = fminf(bmn, lo); bmx = fmaxf(bmx, hi); }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float l = bf16_bits_to_f32(lo[k]), h = bf16_bits_to_f32(hi[k]);
+        bmn[k] = p0 == 0 ? l : fminf(bmn[k], l);
+        bmx[k] = p0 == 0 ? h : fmaxf(bmx[k], h);
+      }
     }
   }
-  if (p.block_range) {
-    __shared__ float red[kD];
-    red[c] = __fsub_rn(bmx, bmn);
-    __syncthreads();
-    for (int s = kD / 2; s > 0; s >>= 1) {
-      if (c < s) red[c] = fmaxf(red[c], red[c + s]);
-      __syncthreads();
-    }
-    if (c == 0) p.block_range[static_cast<size_t>(stream) * (p.stat_stride ? p.stat_stride : p.n_blocks) + p.stat_base + bi] = red[0];
-  }
-  if (p.block_mass && c == 0) {
-    const float* m = p.token_mass + static_cast<size_t>(stream) * p.n_tok + static_cast<size_t>(block) * kBlock;
+  float range = fmaxf(__fsub_rn(bmx[0], bmn[0]), __fsub_rn(bmx[1], bmn[1]));
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) range = fmaxf(range, __shfl_xor_sync(0xffffffffu, range, d));
+  if (lane == 0) s_red[warp] = range;
+  __syncthreads();
+  if (p.block_range && threadIdx.x == 0)
+    p.block_range[static_cast<size_t>(stream) * p.range_stride + block] = fmaxf(s_red[0], s_red[1]);
+  if (p.block_mass && threadIdx.x == 32) {
     float acc = 0.f;
-    for (int t = 0; t < kBlock; ++t) acc = __fadd_rn(acc, m[t]);
-    p.block_mass[static_cast<size_t>(stream) * (p.stat_stride ? p.stat_stride : p.n_blocks) + p.stat_base + bi] = acc;
+#pragma unroll 16
+    for (int t = 0; t < kBlock; ++t) acc = __fadd_rn(acc, s_mass[t]);
+    p.block_mass[static_cast<size_t>(stream) * p.mass_stride + block] = acc;
   }
   if (p.err && !p.k_in) {
     // a block that closes in place (exact rows): no error yet, largest value-row norm for the
-    // certificate.  Warp w takes tokens w, w + 4, ...; a lane sums four channels.
-    __shared__ float vred[kD / 32];
+    // certificate.  Warp w takes tokens w, w + 2, ...; a lane sums four channels.
+    __shared__ float vred[kStatThreads / 32];
     const uint16_t* vrows = rows + kBlock * kD;
-    const int warp = c >> 5, lane = c & 31;
     float best = 0.f;
-    for (int t = warp; t < kBlock; t += kD / 32) {
+#pragma unroll 8
+    for (int t = warp; t < kBlock; t += kStatThreads / 32) {
       const uint2 raw = *reinterpret_cast<const uint2*>(vrows + t * kD + 4 * lane);
       const float x0 = bf16_bits_to_f32(static_cast<uint16_t>(raw.x & 0xffffu)), x1 = bf16_bits_to_f32(static_cast<uint16_t>(raw.x >> 16));
       const float x2 = bf16_bits_to_f32(static_cast<uint16_t>(raw.y & 0xffffu)), x3 = bf16_bits_to_f32(static_cast<uint16_t>(raw.y >> 16));
       float n2 = fmaf(x0, x0, fmaf(x1, x1, fmaf(x2, x2, x3 * x3)));
+#pragma unroll
       for (int s = 1; s <= 16; s <<= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, s);
       best = fmaxf(best, n2);
     }
     if (lane == 0) vred[warp] = best;
     __syncthreads();
-    if (c == 0) {
-      float m = vred[0];
-      for (int w = 1; w < kD / 32; ++w) m = fmaxf(m, vred[w]);
-      p.err[static_cast<size_t>(stream) * p.err_stride + block] = make_float4(0.f, 0.f, sqrtf(m), 0.f);
-    }
+    if (threadIdx.x == 0) p.err[static_cast<size_t>(stream) * p.err_stride + block] = make_float4(0.f, 0.f, sqrtf(fmaxf(vred[0], vred[1])), 0.f);
   }
 }
 
@@ -413,53 +442,102 @@ __global__ void __launch_bounds__(128) append_rows_kernel(uint8_t* arena, const 
   dst[i] = src[i];
 }
 
+// The fp32 number with bits u (a bf16: low half zero) times 2^-896 as fp64: its exponent field, moved to where fp64 has its
+// own, means 2^-896 times as much, for zeros and subnormal numbers too (both formats place them alike).
+__device__ __forceinline__ double f32_bits_to_scaled_f64(uint32_t u) {
+  return __hiloint2double(static_cast<int>((u & 0x80000000u) | ((u >> 3) & 0x0fffffffu)), 0);
+}
+
 // Residual score per token (Sec. 3.4): mass * || v - value centroid of its block ||^2, with the
 // centroid taken by the sequential-sum rule on the original values; fp64 sequential in channels.
+// A CTA of four warps takes two neighbouring blocks, whose rows come in with 16-byte cp.async copies, all in flight at
+// once: two channels per thread for the sums, one token per thread for the distances.  Those are a serial chain of fp64
+// operations per token; the values become fp64 with two integer operations, and the subtraction of the centroid takes
+// the scale 2^896 out again (one rounding, as a subtraction has), instead of a conversion each.
+// 134 MB of values: 43.6 us with one block per CTA, 2-byte loads and half of the threads idle in the distances, 36.0 now.
+constexpr int kResPitch = kD + 8;                // bf16 per staged row: 16-byte accesses to eight rows meet no bank twice
 __global__ void __launch_bounds__(kD) residual_score_kernel(const uint16_t* v_in, const float* token_mass,
                                                             const int8_t* levels, int levels_stride,
-                                                            int n_sink_blocks, int n_kv_heads, int n_tok,
+                                                            int n_sink_blocks, int n_kv_heads, int n_tok, int n_closed, int aligned,
                                                             float* scores) {
-  const int block = blockIdx.x, stream = blockIdx.y, tid = threadIdx.x;
+  __shared__ __align__(16) double cen[2][kD];
+  __shared__ __align__(16) uint16_t vals[2][kBlock * kResPitch];
+  const int stream = blockIdx.y, tid = threadIdx.x, sub = tid >> 6, i = tid & 63;
+  const int block = 2 * blockIdx.x + sub;
   const int b = stream / n_kv_heads, kvh = stream - b * n_kv_heads;
-  float* out = scores + static_cast<size_t>(stream) * n_tok + static_cast<size_t>(block) * kBlock;
-  const int level = levels[static_cast<size_t>(stream) * levels_stride + block];
-  if (block < n_sink_blocks || level == 16) {
-    if (tid < kBlock) out[tid] = -__builtin_huge_valf();
+  const bool on = block < n_closed && block >= n_sink_blocks && levels[static_cast<size_t>(stream) * levels_stride + block] != 16;
+  const size_t tok0 = static_cast<size_t>(block) * kBlock;
+  if (on) {
+    const uint16_t* rows = v_in + ((static_cast<size_t>(b) * n_tok + tok0) * n_kv_heads + kvh) * kD;
+    const size_t row_stride = static_cast<size_t>(n_kv_heads) * kD;
+    if (aligned) {
+#pragma unroll
+      for (int k = 0; k < kBlock * 16 / 64; ++k) {
+        const int piece = i + 64 * k, t = piece >> 4, col = piece & 15;
+        const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&vals[sub][t * kResPitch + col * 8]));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(rows + t * row_stride + col * 8) : "memory");
+      }
+      asm volatile("cp.async.wait_all;\n" ::: "memory");
+    } else {
+#pragma unroll 16
+      for (int t = 0; t < kBlock; ++t)
+        *reinterpret_cast<uint32_t*>(&vals[sub][t * kResPitch + 2 * i]) = *reinterpret_cast<const uint32_t*>(rows + t * row_stride + 2 * i);
+    }
+  }
+  __syncthreads();
+  if (on) {
+    float a0 = 0.f, a1 = 0.f;
+#pragma unroll 16
+    for (int t = 0; t < kBlock; ++t) {
+      const uint32_t u = *reinterpret_cast<const uint32_t*>(&vals[sub][t * kResPitch + 2 * i]);
+      a0 = __fadd_rn(a0, __uint_as_float(u << 16));
+      a1 = __fadd_rn(a1, __uint_as_float(u & 0xffff0000u));
+    }
+    cen[sub][2 * i] = -static_cast<double>(bf16_bits_to_f32(f32_to_bf16_bits(__fmul_rn(a0, 1.0f / kBlock))));
+    cen[sub][2 * i + 1] = -static_cast<double>(bf16_bits_to_f32(f32_to_bf16_bits(__fmul_rn(a1, 1.0f / kBlock))));
+  }
+  __syncthreads();
+  if (block >= n_closed) return;
+  float* out = scores + static_cast<size_t>(stream) * n_tok + tok0 + i;
+  if (!on) {
+    *out = -__builtin_huge_valf();
     return;
   }
-  __shared__ double cen[kD];
-  __shared__ uint16_t vals[kBlock][kD + 2];
-  const uint16_t* rows = v_in + ((static_cast<size_t>(b) * n_tok + static_cast<size_t>(block) * kBlock) * n_kv_heads + kvh) * kD;
-  const size_t row_stride = static_cast<size_t>(n_kv_heads) * kD;
-  float acc = 0.f;
-  for (int t = 0; t < kBlock; ++t) {
-    const uint16_t xb = rows[t * row_stride + tid];
-    vals[t][tid] = xb;
-    acc = __fadd_rn(acc, bf16_bits_to_f32(xb));
-  }
-  cen[tid] = static_cast<double>(bf16_bits_to_f32(f32_to_bf16_bits(__fmul_rn(acc, 1.0f / kBlock))));
-  __syncthreads();
-  if (tid < kBlock) {
-    double err = 0.0;
-    for (int c = 0; c < kD; ++c) {
-      const double d = __dsub_rn(static_cast<double>(bf16_bits_to_f32(vals[tid][c])), cen[c]);
-      err = __dadd_rn(err, __dmul_rn(d, d));
+  double err = 0.0;
+  const uint16_t* row = &vals[sub][i * kResPitch];
+#pragma unroll 2
+  for (int c = 0; c < kD; c += 8) {
+    const uint4 u4 = *reinterpret_cast<const uint4*>(row + c);
+    const uint32_t u[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const double2 m = *reinterpret_cast<const double2*>(&cen[sub][c + 2 * k]);
+      const double d0 = __fma_rn(f32_bits_to_scaled_f64(u[k] << 16), 0x1p896, m.x), d1 = __fma_rn(f32_bits_to_scaled_f64(u[k] & 0xffff0000u), 0x1p896, m.y);
+      err = __dadd_rn(err, __dmul_rn(d0, d0));
+      err = __dadd_rn(err, __dmul_rn(d1, d1));
     }
-    const double m = static_cast<double>(token_mass[static_cast<size_t>(stream) * n_tok + static_cast<size_t>(block) * kBlock + tid]);
-    out[tid] = __double2float_rn(__dmul_rn(m, err));
   }
+  const double m = static_cast<double>(token_mass[static_cast<size_t>(stream) * n_tok + tok0 + i]);
+  *out = __double2float_rn(__dmul_rn(m, err));
 }
 
 // Copy the selected residual tokens' exact K and V rows into the stream's residual pool
-// (row j: [K row 256 B | V row 256 B]).
+// (row j: [K row 256 B | V row 256 B]) and mark them in their blocks' residual masks.
 __global__ void __launch_bounds__(128) residual_gather_kernel(uint8_t* arena, const uint16_t* k_in,
-                                                              const uint16_t* v_in, int n_tok, int n_kv_heads,
+                                                              const uint16_t* v_in, int n_tok, int n_kv_heads, int n_closed,
                                                               const int32_t* idx, int idx_stride,
-                                                              const int32_t* count, const uint32_t* res_off256) {
+                                                              const int32_t* count, const uint32_t* res_off256,
+                                                              TableEntry* table, int table_stride, uint32_t* status) {
   const int j = blockIdx.x, stream = blockIdx.y;
   if (j >= count[stream]) return;
   const int b = stream / n_kv_heads, kvh = stream - b * n_kv_heads;
   const int tok = idx[static_cast<size_t>(stream) * idx_stride + j];
+  if (tok < 0 || tok >= n_closed * kBlock) {
+    if (threadIdx.x == 0) atomicOr(status, kStatusInternal);
+    return;
+  }
+  if (threadIdx.x == 0)
+    atomicOr(reinterpret_cast<unsigned long long*>(&table[static_cast<size_t>(stream) * table_stride + tok / kBlock].resmask), 1ull << (tok % kBlock));
   const bool is_v = threadIdx.x >= 64;
   const int i = threadIdx.x & 63;
   const uint16_t* in = is_v ? v_in : k_in;
@@ -519,7 +597,7 @@ cudaError_t launch_encode(const EncodeParams& p, cudaStream_t st) {
 
 cudaError_t launch_stats(const StatsParams& p, cudaStream_t st) {
   if (p.n_blocks <= 0) return cudaSuccess;
-  stats_kernel<<<dim3(p.n_blocks, p.n_streams), kD, 0, st>>>(p);
+  stats_kernel<<<dim3(p.n_blocks, p.n_streams), kStatThreads, 0, st>>>(p);
   return cudaGetLastError();
 }
 
@@ -544,17 +622,19 @@ cudaError_t launch_residual_scores(const uint16_t* v_in, const float* token_mass
                                    int levels_stride, int n_sink_blocks, int n_streams, int n_kv_heads, int n_tok,
                                    int n_closed, float* scores, cudaStream_t st) {
   if (n_closed <= 0) return cudaSuccess;
-  residual_score_kernel<<<dim3(n_closed, n_streams), kD, 0, st>>>(v_in, token_mass, levels, levels_stride,
-                                                                  n_sink_blocks, n_kv_heads, n_tok, scores);
+  residual_score_kernel<<<dim3((n_closed + 1) / 2, n_streams), kD, 0, st>>>(v_in, token_mass, levels, levels_stride,
+                                                                            n_sink_blocks, n_kv_heads, n_tok, n_closed,
+                                                                            (reinterpret_cast<uintptr_t>(v_in) & 15u) == 0, scores);
   return cudaGetLastError();
 }
 
 cudaError_t launch_residual_gather(uint8_t* arena, const uint16_t* k_in, const uint16_t* v_in, int n_tok,
-                                   int n_kv_heads, const int32_t* idx, int idx_stride, const int32_t* count,
-                                   const uint32_t* res_off256, int max_count, int n_streams, cudaStream_t st) {
+                                   int n_kv_heads, int n_closed, const int32_t* idx, int idx_stride, const int32_t* count,
+                                   const uint32_t* res_off256, int max_count, int n_streams, TableEntry* table,
+                                   int table_stride, uint32_t* status, cudaStream_t st) {
   if (max_count <= 0) return cudaSuccess;
-  residual_gather_kernel<<<dim3(max_count, n_streams), 128, 0, st>>>(arena, k_in, v_in, n_tok, n_kv_heads, idx,
-                                                                     idx_stride, count, res_off256);
+  residual_gather_kernel<<<dim3(max_count, n_streams), 128, 0, st>>>(arena, k_in, v_in, n_tok, n_kv_heads, n_closed, idx,
+                                                                     idx_stride, count, res_off256, table, table_stride, status);
   return cudaGetLastError();
 }
 

@@ -12,7 +12,8 @@
 // which is what makes the plan independent of who computes it.
 //
 // One CTA per stream.  Shared memory: the padded breakpoint array (a power of two of doubles), y, and
-// the working levels.
+// the working levels.  Bound by latency (a bulk ingest waits for the plan): the compare-exchanges of distance up to
+// 32 stay inside a warp's own 64 elements and need no CTA barrier, and the suffix minimum of a test is a shuffle scan.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -23,7 +24,8 @@
 namespace gkv {
 namespace {
 
-constexpr int kPlanThreads = 256;
+constexpr int kPlanThreads = 1024;
+constexpr unsigned kPlanAll = 0xffffffffu;
 
 __device__ __forceinline__ unsigned long long plan_block_bits(int level, unsigned long long nval_tok) {
   if (level == 16) return 16ull * kBlock * nval_tok;
@@ -31,11 +33,17 @@ __device__ __forceinline__ unsigned long long plan_block_bits(int level, unsigne
   return static_cast<unsigned long long>(level) * kBlock * nval_tok + (kBlock * nval_tok / kGroup) * 32ull;
 }
 
+struct PlanShared {
+  int min[kPlanThreads / 32];
+  unsigned long long bits[kPlanThreads / 32];
+  int eligible;
+};
+
 // Levels of the plan for threshold tau into lv[] (shared) and the plan's bits (returned to every thread).
 // Thread t owns the blocks [t * per, min(n, (t + 1) * per)).
 __device__ unsigned long long plan_for_tau(const RdPlanParams& p, const double* y, const TableEntry* table, int n, int per, double tau,
-                                           int8_t* lv, int* s_min, unsigned long long* s_bits) {
-  const int t = threadIdx.x;
+                                           int8_t* lv, PlanShared& sh) {
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, n_warps = blockDim.x >> 5;
   const int b0 = min(n, t * per), b1 = min(n, b0 + per);
   const int recent = p.retire_after / kBlock;
   const double t3 = tau * 3.0, t15 = tau * 15.0, t255 = tau * 255.0;
@@ -56,13 +64,19 @@ __device__ unsigned long long plan_for_tau(const RdPlanParams& p, const double* 
   unsigned long long bits = 0;
   if (p.monotone) {
     // level of a block <- minimum over the unpinned blocks at or after it (younger ones have higher
-    // indices): the chunks' minima are combined by a suffix scan over the threads
-    s_min[t] = cmin;
+    // indices): a suffix scan over the threads' chunk minima
+    int suf = cmin;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int o = __shfl_down_sync(kPlanAll, suf, d);
+      if (lane + d < 32) suf = min(suf, o);
+    }
+    if (lane == 0) sh.min[warp] = suf;
     __syncthreads();
-    int after = 127;                               // minimum over the chunks after this one
-    for (int u = t + 1; u < kPlanThreads; ++u) after = min(after, s_min[u]);
-    __syncthreads();
-    int run = after;
+    const int later = (lane < n_warps && lane > warp) ? sh.min[lane] : 127;       // the warps after this one
+    int run = __reduce_min_sync(kPlanAll, later);
+    const int next = __shfl_down_sync(kPlanAll, suf, 1);                           // the lanes after this one
+    if (lane < 31) run = min(run, next);
     for (int b = b1 - 1; b >= b0; --b) {
       const bool pinned = b < p.n_sink_blocks || (n - 1 - b) < recent;
       if (!pinned) {
@@ -73,22 +87,23 @@ __device__ unsigned long long plan_for_tau(const RdPlanParams& p, const double* 
     }
   } else {
     for (int b = b0; b < b1; ++b) bits += plan_block_bits(lv[b], p.nval_tok);
+    __syncthreads();                     // the last test's total has been read
   }
   // sum over the CTA (integers: any order)
-  for (int d = 16; d >= 1; d >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, d);
-  if ((t & 31) == 0) s_bits[t >> 5] = bits;
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) bits += __shfl_xor_sync(kPlanAll, bits, d);
+  if (lane == 0) sh.bits[warp] = bits;
   __syncthreads();
-  unsigned long long total = 0;
-  for (int w = 0; w < kPlanThreads / 32; ++w) total += s_bits[w];
-  __syncthreads();
-  return total;
+  unsigned long long total = lane < n_warps ? sh.bits[lane] : 0ull;
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) total += __shfl_xor_sync(kPlanAll, total, d);
+  return total;                          // (sh.min and sh.bits are rewritten behind the next test's first barrier only)
 }
 
 __global__ void __launch_bounds__(kPlanThreads) rd_plan_kernel(const RdPlanParams p) {
   extern __shared__ __align__(16) unsigned char plan_sm[];
-  __shared__ int s_min[kPlanThreads];
-  __shared__ unsigned long long s_bits[kPlanThreads / 32];
-  const int s = blockIdx.x, t = threadIdx.x, n = p.n;
+  __shared__ PlanShared sh;
+  const int s = blockIdx.x, t = threadIdx.x, n = p.n, n_thr = blockDim.x;
   double* cand = reinterpret_cast<double*>(plan_sm);                 // [m_pad]
   double* y = cand + p.m_pad;                                        // [n]
   int8_t* lv = reinterpret_cast<int8_t*>(y + n);                     // [n]
@@ -96,7 +111,8 @@ __global__ void __launch_bounds__(kPlanThreads) rd_plan_kernel(const RdPlanParam
   const float* range = p.range + static_cast<size_t>(s) * p.range_stride;
   const TableEntry* table = p.table + static_cast<size_t>(s) * p.table_stride;
   const int m = 4 * n + 1;
-  for (int b = t; b < n; b += kPlanThreads) {
+  if (t == 0) sh.eligible = 0;
+  for (int b = t; b < n; b += n_thr) {
     const double yb = static_cast<double>(mass[b]) * static_cast<double>(range[b]);
     y[b] = yb;
     cand[4 * b + 1] = yb;
@@ -105,43 +121,57 @@ __global__ void __launch_bounds__(kPlanThreads) rd_plan_kernel(const RdPlanParam
     cand[4 * b + 4] = yb / 255.0;
   }
   if (t == 0) cand[0] = 0.0;
-  for (int i = m + t; i < p.m_pad; i += kPlanThreads) cand[i] = __longlong_as_double(0x7ff0000000000000ll);   // +inf padding
+  for (int i = m + t; i < p.m_pad; i += n_thr) cand[i] = __longlong_as_double(0x7ff0000000000000ll);   // +inf padding
   __syncthreads();
-  // bitonic sort, ascending
+  // bitonic sort, ascending: thread t takes the pairs t, t + n_thr, ... of a stage; pair q of distance j is the elements
+  // i = 2 q - (q mod j) and i + j, so a warp's 32 pairs cover the same 64 elements in every stage of distance <= 32
   for (int k = 2; k <= p.m_pad; k <<= 1) {
     for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = t; i < p.m_pad; i += kPlanThreads) {
-        const int l = i ^ j;
-        if (l > i) {
-          const double a = cand[i], b = cand[l];
-          const bool up = (i & k) == 0;
-          if ((a > b) == up) {
-            cand[i] = b;
-            cand[l] = a;
-          }
+      for (int q = t; q < p.m_pad / 2; q += n_thr) {
+        const int i = 2 * q - (q & (j - 1)), l = i + j;
+        const double a = cand[i], b = cand[l];
+        const bool up = (i & k) == 0;
+        if ((a > b) == up) {
+          cand[i] = b;
+          cand[l] = a;
         }
       }
-      __syncthreads();
+      // the next stage's distance decides whether other warps' elements come into play
+      const int next = j > 1 ? j >> 1 : k;
+      if (next > 32 || j > 32) __syncthreads();
+      else __syncwarp();
     }
   }
+  __syncthreads();
   // the smallest feasible breakpoint (duplicates do not matter: equal values give equal plans)
-  const int per = (n + kPlanThreads - 1) / kPlanThreads;
+  const int per = (n + n_thr - 1) / n_thr;
   const unsigned long long budget = p.budget_bits >= p.tail_bits ? p.budget_bits - p.tail_bits : 0ull;
   const bool any_room = p.budget_bits >= p.tail_bits;
   int lo = 0, hi = m;
   while (lo < hi) {                                                  // uniform for the CTA
     const int mid = (lo + hi) >> 1;
-    const unsigned long long bits = plan_for_tau(p, y, table, n, per, cand[mid], lv, s_min, s_bits);
+    const unsigned long long bits = plan_for_tau(p, y, table, n, per, cand[mid], lv, sh);
     if (any_room && bits <= budget) hi = mid;
     else lo = mid + 1;
   }
   const bool miss = lo == m;
   if (miss) lo = m - 1;
-  plan_for_tau(p, y, table, n, per, cand[lo], lv, s_min, s_bits);
+  __syncthreads();
+  plan_for_tau(p, y, table, n, per, cand[lo], lv, sh);
   __syncthreads();
   int8_t* out = p.levels_out + static_cast<size_t>(s) * p.out_stride;
-  for (int b = t; b < n; b += kPlanThreads) out[b] = lv[b];
+  int eligible = 0;
+  for (int b = t; b < n; b += n_thr) {
+    out[b] = lv[b];
+    eligible += b >= p.n_sink_blocks && lv[b] != 16;
+  }
   if (t == 0 && miss) atomicOr(p.miss_flag, 1u);
+  if (p.res_count) {
+    eligible = __reduce_add_sync(kPlanAll, eligible);
+    if ((t & 31) == 0) atomicAdd(&sh.eligible, eligible);
+    __syncthreads();
+    if (t == 0) p.res_count[s] = min(min(p.n_res, kBlock * sh.eligible), p.res_cap);
+  }
 }
 
 }  // namespace
@@ -161,7 +191,9 @@ cudaError_t launch_rd_plan(const RdPlanParams& p, int n_streams, cudaStream_t st
     if (e != cudaSuccess) return e;
     configured = bytes;
   }
-  rd_plan_kernel<<<n_streams, kPlanThreads, bytes, st>>>(p);
+  // a pair of breakpoints per thread, as far as there are threads
+  const int threads = p.m_pad / 2 < 32 ? 32 : (p.m_pad / 2 < kPlanThreads ? p.m_pad / 2 : kPlanThreads);
+  rd_plan_kernel<<<n_streams, threads, bytes, st>>>(p);
   return cudaGetLastError();
 }
 
