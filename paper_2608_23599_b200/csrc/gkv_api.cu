@@ -149,8 +149,8 @@ struct LayerState {
   bool has_tail_slot = false;
   std::vector<int8_t> level;            // [n_streams][max_blocks]
   TableEntry* table_h = nullptr;        // pinned [n_streams][table_stride]
-  WarpDesc* warps_h = nullptr;          // pinned [max_warps]
-  uint32_t* units_h = nullptr;          // pinned [units_cap]
+  WarpDesc* warps_h = nullptr;          // pinned [max_warps] (latent streams: the quads' ranges)
+  StreamPlan* plans_h = nullptr;        // pinned [n_streams]
   int n_units = 0;
   StreamParts* parts_h = nullptr;       // pinned [n_streams * head_groups]
   uint32_t* res_off_h = nullptr;        // pinned [n_streams]
@@ -158,7 +158,7 @@ struct LayerState {
   std::vector<std::vector<int32_t>> res_idx;      // host copy of the residual rows' tokens, fetched when first asked for
   bool res_idx_valid = true;
   bool desc_dirty = true;
-  bool desc_split = false;              // the work lists hold sub-block units (never for observing calls)
+  bool split = false, split_all = false;      // the work lists hold parts of exact blocks / of others (never for observing calls)
   bool desc_allow_split = false;        // what the lists were built with
   int n_warps = 0;
   cudaEvent_t ev = nullptr;             // last upload from this layer's pinned table / residual mirrors
@@ -167,6 +167,7 @@ struct LayerState {
   TableEntry* table_d = nullptr;
   WarpDesc* warps_d = nullptr;
   uint32_t* units_d = nullptr;
+  StreamPlan* plans_d = nullptr;
   StreamParts* parts_d = nullptr;
   uint32_t* res_off_d = nullptr;
   int32_t* res_count_d = nullptr;
@@ -235,7 +236,7 @@ constexpr size_t kMlaMinCtaCost = 1000;      // one block: two of a CTA's four q
 
 struct ArenaPlan {
   size_t status, debug, partial, plan_flag, levels, scores, tickets, jobs, mass_raw, res_raw, lse2, per_layer, heap_begin, total_meta;
-  size_t l_table, l_warps, l_units, l_parts, l_resoff, l_rescount, l_residx, l_respool, l_boxes, l_ema, l_range, l_err, layer_bytes;
+  size_t l_table, l_warps, l_units, l_plans, l_parts, l_resoff, l_rescount, l_residx, l_respool, l_boxes, l_ema, l_range, l_err, layer_bytes;
 };
 
 struct Derived {
@@ -286,9 +287,10 @@ Derived derive(const gkv_config& c) {
   d.res_cap = c.residual_fraction > 0.f
                   ? static_cast<int>(align_up(static_cast<size_t>(std::floor(static_cast<double>(c.residual_fraction) * c.max_ctx)) + 16, 16))
                   : 0;
-  // units of a layer: every item, and up to three more for the items that small workloads cut (fewer than
-  // kTargetWarps items in all; a single stream's exact blocks only below half of that)
-  d.units_cap = static_cast<size_t>(d.n_streams) * (d.max_blocks + 1 + d.res_cap / 16) + static_cast<size_t>(std::min(d.n_streams, 2)) * 3 * (kTargetWarps / 2);
+  // units of a layer: every item, up to three more for the items that small workloads cut (fewer than
+  // kTargetWarps items in all; a single stream's exact blocks only below half of that), and a list's unused place
+  // per warp
+  d.units_cap = static_cast<size_t>(d.n_streams) * (d.max_blocks + 1 + d.res_cap / 16) + static_cast<size_t>(std::min(d.n_streams, 2)) * 3 * (kTargetWarps / 2) + d.max_warps;
   d.box_stride = c.page_tokens > 0 ? static_cast<int>(align_up((c.max_ctx + c.page_tokens - 1) / c.page_tokens, 8)) : 0;
   return d;
 }
@@ -318,6 +320,7 @@ ArenaPlan plan_arena(const gkv_config& c, const Derived& d) {
   a.l_table = ltake(static_cast<size_t>(d.n_streams) * d.table_stride * sizeof(TableEntry));
   a.l_warps = ltake(static_cast<size_t>(d.max_warps) * sizeof(WarpDesc));
   a.l_units = ltake(d.units_cap * sizeof(uint32_t));
+  a.l_plans = ltake(static_cast<size_t>(d.n_streams) * sizeof(StreamPlan));
   a.l_parts = ltake(static_cast<size_t>(d.n_hgroups) * sizeof(StreamParts));
   a.l_resoff = ltake(static_cast<size_t>(d.n_streams) * sizeof(uint32_t));
   a.l_rescount = ltake(static_cast<size_t>(d.n_streams) * sizeof(int32_t));
@@ -509,29 +512,17 @@ bool rd_allocate_streams(const gkv_config& c, const float* mass, const float* ra
 // (in units where a 4-bit block is 1000): an exact block 1590, 8-bit 1070, 4-bit 1000, 2-bit 1015, a
 // centroid block 47 (a run of 16 costs 745).  Bytes are the wrong weight: below 8 bits the kernel
 // is bound by instruction issue and a block costs the same whatever its code width.
-size_t item_cost(const gkv_cache* c, const LayerState& L, int stream, int item) {
-  if (item < L.n_closed) {
-    switch (L.level[static_cast<size_t>(stream) * c->max_blocks + item]) {
-      case 16: return 1590;
-      case 8: return 1070;
-      case 4: return 1000;
-      case 2: return 1015;
-      default: return 47;
-    }
-  }
-  if (item == L.n_closed) return 800;      // tail: mid-fill estimate (its size changes every step)
-  return 550;                              // residual group of 16 exact rows
-}
+constexpr size_t kCost16 = 1590, kCost8 = 1070, kCost4 = 1000, kCost2 = 1015, kCost1 = 47;
+constexpr size_t kCostTail = 800;            // mid-fill estimate (its size changes every step)
+constexpr size_t kCostRes = 550;             // residual group of 16 exact rows
 
-// Units of a stream (a block, a run of up to 16 neighbouring centroid blocks, the tail, a residual
-// group) are dealt to the stream's warps longest-first onto the least loaded warp, so that every
-// warp ends up with the same cost whatever the order of levels along the context; each warp then
-// walks its units in a mixed order (see below).
-void build_descs(gkv_cache* c, LayerState& L, bool allow_split) {
-  const int ns = c->n_streams;
-  // The lists depend only on the streams' levels and residual counts.  Layers usually close a block
+// The host's part of a layer's work lists: every stream's cost and units, the warps that it gets, and where its lists,
+// warps and partial rows lie (L.plans_h, L.parts_h).  The lists themselves are made on the device (gkv_units.cu).
+void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
+  const int ns = c->n_streams, hg = c->head_groups;
+  // The plan depends only on the streams' levels and residual counts.  Layers usually close a block
   // in the same step and, under the staircase, with the same plan: a layer whose levels equal those
-  // of the layer built last takes a copy of that layer's lists instead of building its own.
+  // of the layer planned last takes a copy.
   const int self = static_cast<int>(&L - c->layers.data());
   if (c->desc_src >= 0 && c->desc_src != self) {
     const LayerState& S = c->layers[c->desc_src];
@@ -541,12 +532,12 @@ void build_descs(gkv_cache* c, LayerState& L, bool allow_split) {
       same = std::memcmp(S.level.data() + static_cast<size_t>(s) * c->max_blocks, L.level.data() + static_cast<size_t>(s) * c->max_blocks,
                          static_cast<size_t>(L.n_closed)) == 0;
     if (same) {
-      std::memcpy(L.warps_h, S.warps_h, static_cast<size_t>(S.n_warps) * sizeof(WarpDesc));
-      std::memcpy(L.units_h, S.units_h, static_cast<size_t>(S.n_units) * sizeof(uint32_t));
+      std::memcpy(L.plans_h, S.plans_h, static_cast<size_t>(ns) * sizeof(StreamPlan));
       std::memcpy(L.parts_h, S.parts_h, static_cast<size_t>(c->n_hgroups) * sizeof(StreamParts));
       L.n_warps = S.n_warps;
       L.n_units = S.n_units;
-      L.desc_split = S.desc_split;
+      L.split = S.split;
+      L.split_all = S.split_all;
       L.desc_allow_split = allow_split;
       L.desc_dirty = false;
       return;
@@ -554,166 +545,114 @@ void build_descs(gkv_cache* c, LayerState& L, bool allow_split) {
   }
   c->desc_src = self;
   L.desc_allow_split = allow_split;
-  struct Unit { uint32_t word; uint32_t cost; };
-  // Pass 1: the units of every stream and their total cost.  Streams with the same levels and the
-  // same number of residual rows (all streams under the staircase policy) have the same units:
-  // stream s then refers to the first stream it equals (same_as[s]) and nothing is built twice.
-  std::vector<int> same_as(ns);
-  std::vector<std::vector<Unit>> units(ns);
-  std::vector<size_t> cost(ns, 0);
-  size_t total = 0;
   // A small workload leaves most warps of the GPU without work, and its launch then lasts as long
   // as its longest unit (an exact block: eight steps).  Such lists are cut finer: an exact block
-  // into its four tiles and a quantised block into its two halves, a warp holding as little as one of
+  // into its four tiles, a quantised block into its two halves and the tail into its four tiles (as one unit of
+  // up to eight steps it kept its warp 2 - 4 us beyond the others), a warp holding as little as one of
   // them.  More, finer units also mean more partial rows to merge at the end, so it stops where the whole
   // blocks fill the GPU's warps: half blocks take a call over 4001 tokens of 8 streams from 13.6 to 11.1 us,
   // over 8000 tokens from 14.9 to 13.3, over 16000 tokens of 2 streams from 14.2 to 13.0 and, near the line,
   // over 2000 tokens of 64 streams from 16.2 to 15.8.  (Exact blocks stop at half of that: the lists have room for
   // three extra units of as many blocks.)
-  bool split = false, split_all = false;
+  L.split = L.split_all = false;
   if (allow_split) {
     size_t rough = 0;
     for (int s = 0; s < ns; ++s) rough += static_cast<size_t>(L.n_closed + 1) * 1000 + static_cast<size_t>(L.res_count_h[s] / 16) * 550;
-    split = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost / 2;          // exact blocks only
-    split_all = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost;         // quantised blocks
+    L.split = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost / 2;          // exact blocks
+    L.split_all = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost;          // quantised blocks, the tail
   }
-  L.desc_split = split || split_all;
+  // Cost and units of every stream.  Streams with the same levels and the same number of residual rows (all streams
+  // under the staircase policy) have the same.
+  struct Sum { size_t cost; int units; };
+  std::vector<Sum> sum(ns);
+  size_t total = 0;
   for (int s = 0; s < ns; ++s) {
     const int8_t* lv = L.level.data() + static_cast<size_t>(s) * c->max_blocks;
-    same_as[s] = s;
-    if (s > 0) {
-      const int r = same_as[s - 1];
-      if (L.res_count_h[s] == L.res_count_h[r] &&
-          std::memcmp(lv, L.level.data() + static_cast<size_t>(r) * c->max_blocks, static_cast<size_t>(L.n_closed)) == 0)
-        same_as[s] = r;
-    }
-    if (same_as[s] != s) {
-      cost[s] = cost[same_as[s]];
-      total += cost[s];
-      continue;
-    }
-    const int groups = (L.res_count_h[s] + 15) / 16;
-    const int n_items = L.n_closed + 1 + groups;
-    std::vector<Unit>& u = units[s];
-    u.reserve(n_items);
-    for (int i = 0; i < n_items;) {
-      int run = 1;
-      if (i < L.n_closed && lv[i] != 16 && lv[i] != 8 && lv[i] != 4 && lv[i] != 2) {
-        while (run < 16 && i + run < L.n_closed) {
-          const int8_t l2 = lv[i + run];
-          if (l2 == 16 || l2 == 8 || l2 == 4 || l2 == 2) break;
-          ++run;
-        }
+    if (s > 0 && L.res_count_h[s] == L.res_count_h[s - 1] && std::memcmp(lv, lv - c->max_blocks, static_cast<size_t>(L.n_closed)) == 0) {
+      sum[s] = sum[s - 1];
+    } else {
+      int n16 = 0, n8 = 0, n4 = 0, n2 = 0, n1 = 0, runs = 0;
+      for (int b = 0; b < L.n_closed; ++b) {
+        const int v = lv[b];
+        n16 += v == 16;
+        n8 += v == 8;
+        n4 += v == 4;
+        n2 += v == 2;
+        n1 += v == 1;
+        runs += v == 1 && ((b & 15) == 0 || lv[b - 1] != 1);
       }
-      size_t k = 0;
-      for (int j = 0; j < run; ++j) k += item_cost(c, L, s, i + j);
-      const uint32_t base = static_cast<uint32_t>(i) | (static_cast<uint32_t>(run) << 24);
-      const int8_t lvl = (run == 1 && i < L.n_closed) ? lv[i] : int8_t{0};
-      // the tail's four tiles are units of their own (a tile that holds no row yet is skipped by the kernel): as
-      // one unit of up to eight steps it kept its warp 2 - 4 us beyond the others
-      if ((split && lvl == 16) || (split_all && i == L.n_closed)) {
-        for (uint32_t t = 0; t < 4; ++t) u.push_back(Unit{base | ((1u << t) << 20), static_cast<uint32_t>(k / 4)});
-      } else if (split_all && (lvl == 8 || lvl == 4 || lvl == 2)) {
-        u.push_back(Unit{base | (3u << 20), static_cast<uint32_t>(k / 2)});
-        u.push_back(Unit{base | (12u << 20), static_cast<uint32_t>(k - k / 2)});
-      } else {
-        u.push_back(Unit{base | (15u << 20), static_cast<uint32_t>(k)});
-      }
-      cost[s] += k;
-      i += run;
+      const int groups = (L.res_count_h[s] + 15) / 16;
+      sum[s].cost = static_cast<size_t>(n16) * kCost16 + static_cast<size_t>(n8) * kCost8 + static_cast<size_t>(n4) * kCost4 +
+                    static_cast<size_t>(n2) * kCost2 + static_cast<size_t>(n1) * kCost1 + kCostTail + static_cast<size_t>(groups) * kCostRes;
+      sum[s].units = n16 * (L.split ? 4 : 1) + (n8 + n4 + n2) * (L.split_all ? 2 : 1) + runs + (L.split_all ? 4 : 1) + groups;
     }
-    total += cost[s];
+    total += sum[s].cost;
   }
   // every head group of a stream (up to four query heads each) walks the stream's units with warps of its own
-  const int hg = c->head_groups;
   total *= static_cast<size_t>(hg);
-  const size_t target = std::max(split_all ? kMinWarpCost / 4 : kMinWarpCost, (total + kTargetWarps - 1) / kTargetWarps);
-  // Pass 2: deal each distinct stream's units to its warps, then lay the warps out.
-  int w = 0, pos = 0, row = 0;
-  int dealt_for = -1, dealt_nw = 0;                 // the stream and warp count `lists` was dealt for
-  std::vector<std::vector<uint32_t>> lists;         // per warp (in layout order): its units, ascending
-  std::vector<std::pair<size_t, int>> heap;         // (load, warp): least loaded first, then lowest index
+  const size_t target = std::max(L.split_all ? kMinWarpCost / 4 : kMinWarpCost, (total + kTargetWarps - 1) / kTargetWarps);
+  int w = 0, pos = 0, row = 0, last_nw = 0, stride = 1, stride_inv = 1;
+  L.n_units = 0;
   for (int s = 0; s < ns; ++s) {
-    const int src = same_as[s];
-    const std::vector<Unit>& u0 = units[src];
-    int nw = static_cast<int>((cost[s] + target / 2) / target);
-    nw = std::max(1, std::min(nw, static_cast<int>(u0.size())));
+    int nw = static_cast<int>((sum[s].cost + target / 2) / target);
+    nw = std::max(1, std::min(nw, sum[s].units));
     nw = std::min(nw, (c->max_warps - w) / hg - (ns - 1 - s));
-    if (dealt_for != src || dealt_nw != nw) {
-      std::vector<Unit> u(u0);
-      std::stable_sort(u.begin(), u.end(), [](const Unit& a, const Unit& b) { return a.cost > b.cost; });
-      std::vector<std::vector<uint32_t>> mine(nw);
-      heap.clear();
-      for (int k = 0; k < nw; ++k) heap.emplace_back(0, k);
-      auto later = [](const std::pair<size_t, int>& a, const std::pair<size_t, int>& b) { return a > b; };
-      std::make_heap(heap.begin(), heap.end(), later);
-      for (const Unit& x : u) {                      // longest first onto the least loaded warp
-        std::pop_heap(heap.begin(), heap.end(), later);
-        std::pair<size_t, int>& best = heap.back();
-        best.first += x.cost;
-        mine[best.second].push_back(x.word);
-        std::push_heap(heap.begin(), heap.end(), later);
-      }
-      // Longest-first dealing hands the costliest units (exact blocks, then 8-bit ones) to the first
-      // warps, and a CTA is a window of consecutive warps: walk the warps with a golden-ratio stride
-      // so that every window holds the same mixture of levels.  Warps of one SM share its issue
-      // slots, and a CTA whose warps all run the issue-heavy levels would finish last.
-      int stride = std::max(1, static_cast<int>(nw * 0.6180339887 + 0.5));
+    if (nw != last_nw) {
+      stride = std::max(1, static_cast<int>(nw * 0.6180339887 + 0.5));
       while (std::gcd(stride, nw) != 1) ++stride;
-      lists.assign(nw, {});
-      for (int k = 0; k < nw; ++k) {
-        std::vector<uint32_t>& m = mine[static_cast<size_t>((static_cast<long long>(k) * stride) % nw)];
-        std::sort(m.begin(), m.end(), [](uint32_t a, uint32_t b) {       // by block, then by tile mask
-          return (((a & kUnitItemMask) << 4) | ((a >> 20) & 15u)) < (((b & kUnitItemMask) << 4) | ((b >> 20) & 15u));
-        });
-        // Ascending token order runs from the oldest, narrowest blocks to the newest, widest ones, and
-        // the warps of an SM would walk it in step: all of them unpacking 2- and 4-bit codes (bound
-        // by instruction issue, memory idle), later all of them waiting for 8-bit and exact tiles
-        // (issue slots idle).  Taking the units alternately from both ends makes every warp follow a
-        // byte-heavy unit with an issue-heavy one, so its two-stage pipeline always has a long
-        // compute to hide a long copy behind; starting every warp at a different place of its list
-        // (below) also keeps both kinds of step in every SM at all times.  (Shifting whole CTAs
-        // against one another instead - every SM uniform, the GPU mixed - gains nothing.)
-        std::vector<uint32_t>& out = lists[k];
-        out.clear();
-        for (size_t lo = 0, hi = m.size(); lo < hi;) {
-          out.push_back(m[lo++]);
-          if (lo < hi) out.push_back(m[--hi]);
-        }
-        if (out.size() > 1) std::rotate(out.begin(), out.begin() + (static_cast<size_t>(k) * 5) % out.size(), out.end());
-      }
-      dealt_for = src;
-      dealt_nw = nw;
+      stride_inv = 1;
+      while (static_cast<long long>(stride) * stride_inv % nw != 1 % nw) ++stride_inv;
+      last_nw = nw;
     }
-    // One partial row per (CTA, head group): the kernel merges the warps of a CTA that share a head
-    // group.  The head groups of a stream get the same lists (stored once) and neighbouring warps, so
-    // that the second reader of a block finds it in L2.
-    const int pos0 = pos;
-    for (int g = 0; g < hg; ++g) {
+    const int pitch = (sum[s].units + nw - 1) / nw;
+    L.plans_h[s] = StreamPlan{pos, pitch, sum[s].units, nw, w, stride, stride_inv, L.res_count_h[s]};
+    pos += nw * pitch;
+    L.n_units += sum[s].units;
+    for (int g = 0; g < hg; ++g) {            // one partial row per (CTA, head group)
       const int hgi = s * hg + g;
       L.parts_h[hgi].begin = row;
-      pos = pos0;
-      for (int k = 0; k < nw; ++k) {
-        const std::vector<uint32_t>& m = lists[k];
-        WarpDesc& d = L.warps_h[w];
-        d.stream = hgi;
-        d.item_begin = pos;
-        if (g == 0) std::memcpy(L.units_h + pos, m.data(), m.size() * sizeof(uint32_t));
-        pos += static_cast<int>(m.size());
-        d.item_end = pos;
-        if (k > 0 && w % kDecodeWarps == 0) ++row;
-        d.partial = row;
-        ++w;
-      }
-      ++row;
+      row += (w + nw - 1) / kDecodeWarps - w / kDecodeWarps + 1;
+      w += nw;
       L.parts_h[hgi].end = row;
     }
   }
-  const int padded = static_cast<int>(align_up(w, kDecodeWarps));
-  for (int i = w; i < padded; ++i) L.warps_h[i] = WarpDesc{-1, 0, 0, 0};
-  L.n_warps = padded;
-  L.n_units = pos;
+  L.n_warps = static_cast<int>(align_up(w, kDecodeWarps));
   L.desc_dirty = false;
+}
+
+// Work lists of a layer on their way: the host's plan up, the lists behind it.
+int make_units(gkv_cache* c, LayerState& L, bool allow_split, cudaStream_t st) {
+  // the plans have their own event: waiting for the table's would wait for copies that
+  // the append of this very step has just queued, i.e. drain the stream
+  CK(c, cudaEventSynchronize(L.ev_desc));
+  plan_units(c, L, allow_split);
+  int rc;
+  if ((rc = upload(c, L.plans_d, L.plans_h, static_cast<size_t>(c->n_streams) * sizeof(StreamPlan), st, L.ev_desc)) != GKV_OK) return rc;
+  if ((rc = upload(c, L.parts_d, L.parts_h, static_cast<size_t>(c->n_hgroups) * sizeof(StreamParts), st, L.ev_desc)) != GKV_OK) return rc;
+  UnitsParams p{};
+  p.table = L.table_d;
+  p.plans = L.plans_d;
+  p.parts = L.parts_d;
+  p.units = L.units_d;
+  p.warps = L.warps_d;
+  p.table_stride = c->table_stride;
+  p.n_closed = L.n_closed;
+  p.head_groups = c->head_groups;
+  p.n_warps = L.n_warps;
+  p.split = L.split;
+  p.split_all = L.split_all;
+  const size_t head[6] = {kCost16 / (L.split ? 4 : 1), kCost8 / (L.split_all ? 2 : 1), kCost2 / (L.split_all ? 2 : 1),
+                          kCost4 / (L.split_all ? 2 : 1), kCostTail / (L.split_all ? 4 : 1), kCostRes};
+  for (int i = 0; i < kUnitClasses; ++i) p.cost[i] = static_cast<int32_t>(i < 6 ? head[i] : kCost1 * (22 - i));
+  int max_units = 0, max_nw = 1;
+  for (int s = 0; s < c->n_streams; ++s) {
+    max_units = std::max(max_units, L.plans_h[s].n_units);
+    max_nw = std::max(max_nw, L.plans_h[s].n_warps);
+  }
+  p.pad = 128;
+  while (p.pad < max_nw) p.pad <<= 1;
+  CK(c, launch_units(p, c->n_streams, max_units, st));
+  return GKV_OK;
 }
 
 void set_entry(gkv_cache* c, LayerState& L, int stream, int block, uint32_t off, int level) {
@@ -1577,8 +1516,8 @@ int gkv_create(const gkv_config* cfg, void* arena, size_t arena_bytes, gkv_cache
     take(c->demote_h, gkv_cache::kDemoteSlots * c->demote_cap * sizeof(EncodeJob));
     for (LayerState& L : c->layers) {
       take(L.table_h, table_bytes);
-      take(L.warps_h, d.max_warps * sizeof(WarpDesc));
-      take(L.units_h, d.units_cap * sizeof(uint32_t));
+      if (is_mla(c->cfg)) take(L.warps_h, d.max_warps * sizeof(WarpDesc));
+      take(L.plans_h, d.n_streams * sizeof(StreamPlan));
       take(L.parts_h, d.n_hgroups * sizeof(StreamParts));
       take(L.res_off_h, d.n_streams * sizeof(uint32_t));
       take(L.res_count_h, d.n_streams * sizeof(int32_t));
@@ -1600,6 +1539,7 @@ int gkv_create(const gkv_config* cfg, void* arena, size_t arena_bytes, gkv_cache
     L.table_d = reinterpret_cast<TableEntry*>(lb + a.l_table);
     L.warps_d = reinterpret_cast<WarpDesc*>(lb + a.l_warps);
     L.units_d = reinterpret_cast<uint32_t*>(lb + a.l_units);
+    L.plans_d = reinterpret_cast<StreamPlan*>(lb + a.l_plans);
     L.parts_d = reinterpret_cast<StreamParts*>(lb + a.l_parts);
     L.res_off_d = reinterpret_cast<uint32_t*>(lb + a.l_resoff);
     L.res_count_d = reinterpret_cast<int32_t*>(lb + a.l_rescount);
@@ -1798,6 +1738,7 @@ int decode_impl(gkv_cache* c, int32_t layer, const void* q, const int32_t* page_
   p.out = out;
   p.lse = lse;
   int n_ctas;
+  bool overlap = true;
   if (page_idx) {
     if (cfg.page_tokens <= 0) return GKV_ERR_BAD_STATE;
     if (n_sel < 0 || n_sel > L.n_closed * (kBlock / cfg.page_tokens)) return GKV_ERR_INVALID_ARG;
@@ -1817,15 +1758,10 @@ int decode_impl(gkv_cache* c, int32_t layer, const void* q, const int32_t* page_
     L.last_read_scored = L.quest_ran;     // a later read with a list of the caller's own does not inherit it
     L.quest_ran = false;
   } else {
-    if (L.desc_dirty || (observe && L.desc_split)) {      // an observing call needs whole-block units
-      // the work lists have their own event: waiting for the table's would wait for copies that
-      // the append of this very step has just queued, i.e. drain the stream
-      int rc = wait_event(c, L.ev_desc);
+    if (L.desc_dirty || (observe && (L.split || L.split_all))) {      // an observing call needs whole-block units
+      const int rc = make_units(c, L, !observe, st);
       if (rc != GKV_OK) return rc;
-      build_descs(c, L, !observe);
-      if ((rc = upload(c, L.warps_d, L.warps_h, static_cast<size_t>(L.n_warps) * sizeof(WarpDesc), st, L.ev_desc)) != GKV_OK) return rc;
-      if ((rc = upload(c, L.units_d, L.units_h, static_cast<size_t>(L.n_units) * sizeof(uint32_t), st, L.ev_desc)) != GKV_OK) return rc;
-      if ((rc = upload(c, L.parts_d, L.parts_h, static_cast<size_t>(c->n_hgroups) * sizeof(StreamParts), st, L.ev_desc)) != GKV_OK) return rc;
+      overlap = false;
     }
     p.warps = L.warps_d;
     p.units = L.units_d;
@@ -1835,7 +1771,7 @@ int decode_impl(gkv_cache* c, int32_t layer, const void* q, const int32_t* page_
     L.last_mode = 1;
     L.quest_ran = false;
   }
-  CK(c, launch_decode(p, n_ctas, st));
+  CK(c, launch_decode(p, n_ctas, overlap, st));
   if (observe) {
     ObserveParams o{};
     o.arena = c->arena;

@@ -1,9 +1,9 @@
 // Graded single-query decode attention (paper Sec. 3.7: dequantisation inside the online-softmax
 // loop, all KV heads of a layer in one launch, split-context partials merged in the same launch).
 //
-// Work split: the host cuts every stream into units (a block, half of a quantised block, a run of
-// centroid blocks, the tail, a group of exact residual rows) and deals them longest-first to the
-// stream's warps; a warp walks its unit list and keeps its own online-softmax state for the g <= 8
+// Work split: every stream is cut into units (a block, half of a quantised block, a run of
+// centroid blocks, the tail, a group of exact residual rows), which are dealt to the stream's warps by falling cost
+// (gkv_units.cu); a warp walks its unit list and keeps its own online-softmax state for the g <= 8
 // query heads of the KV head (one read of the KV bytes serves the whole GQA group, Sec. 3.1).
 // Warps never wait on each other: each one runs a private double-buffered pipeline of TMA bulk
 // copies (cp.async.bulk global -> shared, completion on a per-warp mbarrier) and consumes only what
@@ -1023,7 +1023,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
     }
   }
   // Launched with programmatic stream serialisation: what is above touches nothing that a previous kernel may
-  // have written (only descriptors and the first word of the host-written work list).  The block table, the query,
+  // have written (only descriptors and the first word of the work list, made by a launch that this one is not overlapped with).  The block table, the query,
   // appended rows, partial rows and tickets are touched after this wait, which returns once that kernel has
   // completed and its writes are visible.
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
@@ -1267,7 +1267,7 @@ size_t decode_smem_bytes() {
   return static_cast<size_t>(kDecodeWarps) * (kStages * kStageBytes + kStages * sizeof(uint64_t) + 2 * 2048 + 4 * sizeof(int)) + sizeof(int);
 }
 
-cudaError_t launch_decode(const DecodeParams& p, int n_ctas, cudaStream_t st) {
+cudaError_t launch_decode(const DecodeParams& p, int n_ctas, bool overlap, cudaStream_t st) {
   static bool configured = false;
   if (!configured) {
     const int bytes = static_cast<int>(decode_smem_bytes());
@@ -1289,7 +1289,7 @@ cudaError_t launch_decode(const DecodeParams& p, int n_ctas, cudaStream_t st) {
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = overlap ? 1 : 0;
   if (p.page_idx) return cudaLaunchKernelEx(&cfg, decode_kernel<true, false>, p);
   if (p.mass_raw) return cudaLaunchKernelEx(&cfg, decode_kernel<false, true>, p);
   return cudaLaunchKernelEx(&cfg, decode_kernel<false, false>, p);

@@ -17,7 +17,7 @@ struct alignas(16) TableEntry {
 };
 
 // Work of one warp of the decode kernel: positions [item_begin, item_end) of the layer's unit
-// list, all of one stream; `stream` is the index of the warp's head group (up to four query heads of
+// lists, all of one stream; `stream` is the index of the warp's head group (up to four query heads of
 // one KV head): stream * head_groups + group number.  A unit is one item or a run of consecutive centroid blocks:
 // `first item | run << 24`.  Items: [0, n_closed) closed blocks, n_closed = tail block,
 // n_closed + 1 + j = residual group j (16 residual rows each).  (The MLA kernel uses the same
@@ -36,6 +36,33 @@ constexpr uint32_t kUnitItemMask = 0xfffffu;
 
 struct alignas(8) StreamParts {
   int32_t begin, end;  // partial rows [begin, end) belong to this head group (GQA) / stream (MLA)
+};
+
+// What the host decides about a stream's work lists (gkv_units.cu makes the lists).
+struct alignas(16) StreamPlan {
+  int32_t unit_base;      // first unit word of the stream's lists
+  int32_t pitch;          // room per list: ceil(n_units / n_warps)
+  int32_t n_units;        // units of the stream
+  int32_t n_warps;        // warps per head group, at most n_units
+  int32_t warp_base;      // first warp of the stream's first head group
+  int32_t stride;         // the warp at place k takes the k * stride mod n_warps-th hand of the deal
+  int32_t stride_inv;     // stride * stride_inv = 1 mod n_warps
+  int32_t n_res;          // exact residual rows
+};
+
+constexpr int kUnitClasses = 22;            // exact, 8, 2, 4 bits, tail, residual group, centroid runs of 16 .. 1
+
+struct UnitsParams {
+  const TableEntry* table;      // [n_streams][table_stride]
+  const StreamPlan* plans;      // [n_streams]
+  const StreamParts* parts;     // [head groups]
+  uint32_t* units;
+  WarpDesc* warps;              // [n_warps]
+  int32_t table_stride, n_closed, head_groups, n_warps;
+  int32_t split, split_all;     // exact blocks as four tiles; quantised blocks as two halves, the tail as four tiles
+  int32_t cost[kUnitClasses];   // of a unit, by class
+  int32_t pad;                  // a power of two, at least 128 and the warps of any stream
+  int32_t dealt;                // set by the launch
 };
 
 constexpr int kDecodeWarps = 16;            // warps per CTA of the decode kernel
@@ -158,7 +185,10 @@ struct StatsParams {
 constexpr uint32_t kStatusRange = 1u;      // a scale or zero saturated
 constexpr uint32_t kStatusInternal = 2u;   // an index check failed inside a kernel
 
-cudaError_t launch_decode(const DecodeParams& p, int n_ctas, cudaStream_t st);
+// overlap: launched under programmatic stream serialisation; not behind a kernel that writes the work lists, which the read
+// looks at before it waits for its predecessor
+cudaError_t launch_decode(const DecodeParams& p, int n_ctas, bool overlap, cudaStream_t st);
+cudaError_t launch_units(UnitsParams p, int n_streams, int max_units, cudaStream_t st);
 cudaError_t launch_observe_finish(const ObserveParams& p, cudaStream_t st);
 cudaError_t launch_encode(const EncodeParams& p, cudaStream_t st);
 cudaError_t launch_ingest(const EncodeParams& p, cudaStream_t st);   // every job reads the bf16 input rows; 16-byte aligned inputs
