@@ -872,11 +872,15 @@ int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* 
   bool encoded = false;
   if (fast && !has_res) {
     const int per_seq = n_closed * cfg.n_kv_heads;
-    const int seqs = std::max(1, (8192 + per_seq - 1) / per_seq);       // at least ~8192 blocks per launch
-    for (int q0 = 0; q0 < cfg.batch; q0 += seqs) {
-      const int s0 = q0 * cfg.n_kv_heads, s1 = std::min(cfg.batch, q0 + seqs) * cfg.n_kv_heads;
+    // about 8192 blocks in the first launch, three times as many in each that follows: the host takes a quarter of the
+    // GPU's time per block, and every launch costs a copy of table rows that the GPU waits for (20 us)
+    int seqs = std::max(1, (8192 + per_seq - 1) / per_seq);
+    for (int q0 = 0; q0 < cfg.batch;) {
+      const int q1 = std::min(cfg.batch, q0 + seqs), s0 = q0 * cfg.n_kv_heads, s1 = q1 * cfg.n_kv_heads;
       if ((rc = alloc_streams(s0, s1)) != GKV_OK) return rc;
       if ((rc = encode_streams(s0, s1)) != GKV_OK) return rc;
+      q0 = q1;
+      seqs = std::min(3 * seqs, cfg.batch);
     }
     encoded = true;
   } else if ((rc = alloc_streams(0, ns)) != GKV_OK) {

@@ -16,8 +16,10 @@
 // the eight lanes that share a group; the division for scale and reciprocal is done once per
 // group by one lane and handed to the others.
 //
-// One CTA (8 warps: 4 for keys, 4 for values) per block; the next block's 32 KB of rows are in
-// flight (cp.async, second buffer) while the current one is encoded.
+// One CTA (8 warps: 4 for keys, 4 for values) per block, four CTAs per SM, which take turns loading and encoding; the next
+// block's rows are on their way to L2 while the current one is encoded.  Bound by instruction issue (17.7 instructions
+// per value and lane, 63 % of the issue slots; 22 and three double-buffered CTAs per SM before packed fp32 arithmetic):
+// 8192 blocks of the staircase mixture 109 us (117 before), 45 us at the measured copy bandwidth.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -31,7 +33,8 @@ constexpr int kInRow = kRowBytes + 16;            // padded shared-memory row: l
 constexpr int kInTensor = kBlock * kInRow;        // 17408
 constexpr int kInBuf = 2 * kInTensor;             // keys, values
 constexpr int kInThreads = 256;
-constexpr int kInSmem = 2 * kInBuf + (256 + 128 + 16) * static_cast<int>(sizeof(float)) + 8 * 32 * 16;   // + the warps' group parameters
+constexpr int kInCtas = 4;                         // CTAs per SM
+constexpr int kInSmem = kInBuf + (256 + 128 + 16) * static_cast<int>(sizeof(float)) + 8 * 32 * 16;   // + the warps' group parameters
 constexpr float kMagic = 12582912.f;              // 1.5 * 2^23: x + kMagic rounds x to an integer (ties to even)
 constexpr uint32_t kMagicBits = 0x4B400000u;
 constexpr uint32_t kFullI = 0xffffffffu;
@@ -120,6 +123,56 @@ __device__ __forceinline__ void i_quant2(uint32_t x, float s0, float z0, float i
   e1 = fmaf(d1, d1, e1);
 }
 
+// ---- the same on packed pairs of fp32 (each half rounded as an instruction of its own would) ----
+__device__ __forceinline__ uint64_t i_pair(float x, float y) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+__device__ __forceinline__ void i_halves(uint64_t v, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;\n" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ uint64_t i_add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t i_mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t i_fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+// The parameters of a register's two values as pairs, scale and zero point negated.
+struct PairParams {
+  uint64_t ns, nz, inv;
+  uint64_t one;          // (1, 1), unknown to the compiler
+};
+// Quantise the two values of a register (already as a pair X), add the codes to `word` at the bit positions b0 and
+// b0 + 16, and add the squared reconstruction errors to the pair e.  Needs every value within 2^15 steps of its zero
+// point, which parameters inside the fp16 range imply (the inputs are bf16: their spacing bounds the rounding of the zero
+// point by 16 steps, and a rounded scale is at least half of the unrounded one): the codes are clamped as 16-bit
+// integers, both at once, behind the rounding, and go into their word with one multiply-add.  14 instructions for two
+// values, where clamping each as fp32 and taking the magic constants off the word takes 22.
+// The magic constant is added by a multiply-add with a 1 that the compiler cannot see: it joins a packed multiplication and a
+// packed addition into one operation, which would round the scaled value once instead of twice and move codes.
+template <int BITS>
+__device__ __forceinline__ void i_quant_pair(uint64_t X, const PairParams& g, int b0, uint32_t& word, uint64_t& e) {
+  constexpr uint32_t qmax = (1u << BITS) - 1u;
+  const uint64_t magic = i_pair(kMagic, kMagic), unmagic = i_pair(-kMagic, -kMagic);
+  float r0, r1;
+  i_halves(i_fma2(i_mul2(i_add2(X, g.nz), g.inv), g.one, magic), r0, r1);
+  uint32_t c = __byte_perm(__float_as_uint(r0), __float_as_uint(r1), 0x5410);
+  c = __vimin_s16x2_relu(c, qmax | (qmax << 16));                     // max(min(c, qmax), 0)
+  word += c << b0;
+  const uint64_t code = i_add2(i_pair(__uint_as_float(__byte_perm(c, kMagicBits, 0x7610)), __uint_as_float(__byte_perm(c, kMagicBits, 0x7632))), unmagic);
+  const uint64_t d = i_add2(X, i_fma2(code, g.ns, g.nz));             // x - (code s + z)
+  e = i_fma2(d, d, e);
+}
+__device__ __forceinline__ uint64_t i_pair_bf16(uint32_t u) { return i_pair(i_lo(u), i_hi(u)); }
+
 // Parameters of a group as the warp keeps them in shared memory between its two passes:
 // {scale | zero << 16 (fp16 bits), reciprocal} of the low and of the high half of a register pair.
 __device__ __forceinline__ uint4 i_pack_params(const GroupParams& g0, const GroupParams& g1) {
@@ -128,6 +181,10 @@ __device__ __forceinline__ uint4 i_pack_params(const GroupParams& g0, const Grou
 }
 __device__ __forceinline__ float i_h_lo(uint32_t u) { return __half2float(__ushort_as_half(static_cast<unsigned short>(u & 0xffffu))); }
 __device__ __forceinline__ float i_h_hi(uint32_t u) { return __half2float(__ushort_as_half(static_cast<unsigned short>(u >> 16))); }
+__device__ __forceinline__ PairParams i_pair_params(const uint4& P, uint64_t one) {
+  const uint32_t a = P.x ^ 0x80008000u, b = P.z ^ 0x80008000u;
+  return PairParams{i_pair(i_h_lo(a), i_h_lo(b)), i_pair(i_h_hi(a), i_h_hi(b)), i_pair(__uint_as_float(P.y), __uint_as_float(P.w)), one};
+}
 
 // Keys of one half (32 tokens) x 64 channels.  ldmatrix hands a lane, per 16-token tile and slice of
 // 16 channels, registers a = 0..3: token 8 (a & 1) + r, channels 16 s + 8 (a >> 1) + 2 c4 + {0, 1}
@@ -137,8 +194,9 @@ __device__ __forceinline__ float i_h_hi(uint32_t u) { return __half2float(__usho
 // the rows again, quantises and stores whole words.  Both passes are rolled loops over the slices
 // (the code of all rungs together has to stay inside the instruction cache).
 // e[tile][a & 1]: squared error of token 16 tile + 8 (a & 1) + r summed over the lane's channels.
+// The general form: any parameters, one value at a time.  (Out of line: only blocks whose parameters saturate come here.)
 template <int BITS>
-__device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base, int half, int chh, int lane, uint4* prm, float (&e)[2][2]) {
+__device__ __noinline__ bool ingest_keys_wide(uint32_t tile_k, uint8_t* half_base, int half, int chh, int lane, uint4* prm, float (&e)[2][2]) {
   const int r = lane >> 2, c4 = lane & 3, mi = lane >> 3;
   const uint32_t ld = tile_k + (32 * half + (mi & 1) * 8 + (lane & 7)) * kInRow + (64 * chh + (mi >> 1) * 8) * 2;
   uint32_t my_mn = 0u, my_mx = 0u;
@@ -220,6 +278,90 @@ __device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base,
   return g0.range || g1.range;
 }
 
+template <int BITS>
+__device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base, int half, int chh, int lane, uint4* prm, uint64_t one, float (&e)[2][2]) {
+  const int r = lane >> 2, c4 = lane & 3, mi = lane >> 3;
+  const uint32_t ld = tile_k + (32 * half + (mi & 1) * 8 + (lane & 7)) * kInRow + (64 * chh + (mi >> 1) * 8) * 2;
+  uint32_t my_mn = 0u, my_mx = 0u;
+#pragma unroll 1
+  for (int sl = 0; sl < 4; ++sl) {
+    uint32_t x0[4], x1[4];
+    i_ldm4(ld + sl * 32, x0);
+    i_ldm4(ld + 16 * kInRow + sl * 32, x1);
+#pragma unroll
+    for (int ah = 0; ah < 2; ++ah) {
+      uint32_t mn = i_min2(i_min2(x0[2 * ah], x0[2 * ah + 1]), i_min2(x1[2 * ah], x1[2 * ah + 1]));
+      uint32_t mx = i_max2(i_max2(x0[2 * ah], x0[2 * ah + 1]), i_max2(x1[2 * ah], x1[2 * ah + 1]));
+#pragma unroll
+      for (int d = 4; d <= 16; d <<= 1) {
+        mn = i_min2(mn, __shfl_xor_sync(kFullI, mn, d));
+        mx = i_max2(mx, __shfl_xor_sync(kFullI, mx, d));
+      }
+      if (r == 2 * sl + ah) {
+        my_mn = mn;
+        my_mx = mx;
+      }
+    }
+  }
+  const GroupParams g0 = i_params<BITS>(i_lo(my_mn), i_lo(my_mx)), g1 = i_params<BITS>(i_hi(my_mn), i_hi(my_mx));
+  if (__any_sync(kFullI, g0.range || g1.range)) return ingest_keys_wide<BITS>(tile_k, half_base, half, chh, lane, prm, e);
+  {
+    // per (slab, c4) a record of zero points and one of scales, each {s0: c0 c1, s1: c0 c1, s0: c2 c3, s1: c2 c3}
+    // (gkv_layout.cuh); this lane holds the pair (c0, c1) or (c2, c3) (r & 1) of MMA index s_glob
+    const int s_glob = 4 * chh + (r >> 1);
+    uint32_t* rec = reinterpret_cast<uint32_t*>(half_base + off_kp() + ((s_glob >> 1) * 4 + c4) * 32) + (r & 1) * 2 + (s_glob & 1);
+    rec[0] = static_cast<uint32_t>(g0.z_bits) | (static_cast<uint32_t>(g1.z_bits) << 16);
+    rec[4] = static_cast<uint32_t>(g0.s_bits) | (static_cast<uint32_t>(g1.s_bits) << 16);
+  }
+  prm[r * 4 + c4] = i_pack_params(g0, g1);
+  __syncwarp();
+  constexpr int SL = BITS == 2 ? 2 : 1;             // slices that fill whole words
+  uint64_t err[2][2] = {{0ull, 0ull}, {0ull, 0ull}};      // [tile][a & 1], the lane's two channels side by side
+#pragma unroll 1
+  for (int u = 0; u < 4 / SL; ++u) {
+    uint32_t w[2][2] = {{0u, 0u}, {0u, 0u}};        // [tile][word]: 8 bits: one word per a >> 1; else one word
+#pragma unroll
+    for (int ss = 0; ss < SL; ++ss) {
+      const int sl = u * SL + ss;
+      uint32_t x[2][4];
+      i_ldm4(ld + sl * 32, x[0]);
+      i_ldm4(ld + 16 * kInRow + sl * 32, x[1]);
+#pragma unroll
+      for (int ah = 0; ah < 2; ++ah) {
+        const uint4 P = prm[(2 * sl + ah) * 4 + c4];
+        const PairParams g = i_pair_params(P, one);
+        const int wi = BITS == 8 ? ah : 0;
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+          for (int al = 0; al < 2; ++al)
+            i_quant_pair<BITS>(i_pair_bf16(x[t][2 * ah + al]), g, i_bit<BITS>(ss, 2 * ah + al, 0), w[t][wi], err[t][al]);
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      uint8_t* codes = half_base + off_kc(BITS, t);
+      if (BITS == 8) {          // words 8 chh + 2 u + {0, 1}
+        *reinterpret_cast<uint2*>(codes + ((2 * chh + (u >> 1)) * 32 + lane) * 16 + (u & 1) * 8) =
+            make_uint2(w[t][0], w[t][1]);
+      } else if (BITS == 4) {   // word 4 chh + u
+        *reinterpret_cast<uint32_t*>(codes + (chh * 32 + lane) * 16 + u * 4) = w[t][0];
+      } else {                  // word 2 chh + u
+        *reinterpret_cast<uint32_t*>(codes + lane * 16 + chh * 8 + u * 4) = w[t][0];
+      }
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < 2; ++t)
+#pragma unroll
+    for (int al = 0; al < 2; ++al) {
+      float x0, x1;
+      i_halves(err[t][al], x0, x1);
+      e[t][al] = x0 + x1;
+    }
+  return false;
+}
+
 // Values of one tile (16 tokens) x 128 channels.  ldmatrix.trans hands a lane, per slice of 16
 // channels, registers a = 0..3: channel 16 s + r + 8 (a & 1), tokens 8 (a >> 1) + 2 c4 + {0, 1}.  Groups
 // are 32 channels of one token: slices 2 g and 2 g + 1, a & 1 and the eight lanes r.  Pair
@@ -227,7 +369,7 @@ __device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base,
 // e[a >> 1][0 / 1], n[a >> 1][0 / 1]: squared error / squared norm of token 8 (a >> 1) + 2 c4 + {0, 1}
 // summed over the lane's channels.
 template <int BITS>
-__device__ __forceinline__ bool ingest_values(uint32_t ld, uint8_t* vp, uint8_t* codes, int lane, uint4* prm, float (&e)[2][2],
+__device__ __noinline__ bool ingest_values_wide(uint32_t ld, uint8_t* vp, uint8_t* codes, int lane, uint4* prm, float (&e)[2][2],
                                               float (&n)[2][2]) {
   const int r = lane >> 2, c4 = lane & 3;
   uint32_t my_mn = 0u, my_mx = 0u;
@@ -314,62 +456,158 @@ __device__ __forceinline__ bool ingest_values(uint32_t ld, uint8_t* vp, uint8_t*
   return g0.range || g1.range || g0.s > v_scale_limit(BITS) || g1.s > v_scale_limit(BITS);
 }
 
-__global__ void __launch_bounds__(kInThreads, 3) ingest_kernel(const __grid_constant__ EncodeParams p) {
+template <int BITS>
+__device__ __forceinline__ bool ingest_values(uint32_t ld, uint8_t* vp, uint8_t* codes, int lane, uint4* prm, uint64_t one, float (&e)[2][2],
+                                              float (&n)[2][2]) {
+  const int r = lane >> 2, c4 = lane & 3;
+  uint32_t my_mn = 0u, my_mx = 0u;
+#pragma unroll 1
+  for (int g = 0; g < 4; ++g) {
+    uint32_t x0[4], x1[4];
+    i_ldm4t(ld + g * 64, x0);
+    i_ldm4t(ld + g * 64 + 32, x1);
+#pragma unroll
+    for (int ah = 0; ah < 2; ++ah) {
+      uint32_t mn = i_min2(i_min2(x0[2 * ah], x0[2 * ah + 1]), i_min2(x1[2 * ah], x1[2 * ah + 1]));
+      uint32_t mx = i_max2(i_max2(x0[2 * ah], x0[2 * ah + 1]), i_max2(x1[2 * ah], x1[2 * ah + 1]));
+#pragma unroll
+      for (int d = 4; d <= 16; d <<= 1) {
+        mn = i_min2(mn, __shfl_xor_sync(kFullI, mn, d));
+        mx = i_max2(mx, __shfl_xor_sync(kFullI, mx, d));
+      }
+      if (r == 2 * g + ah) {
+        my_mn = mn;
+        my_mx = mx;
+      }
+    }
+  }
+  const GroupParams g0 = i_params<BITS>(i_lo(my_mn), i_lo(my_mx)), g1 = i_params<BITS>(i_hi(my_mn), i_hi(my_mx));
+  if (__any_sync(kFullI, g0.range || g1.range)) return ingest_values_wide<BITS>(ld, vp, codes, lane, prm, e, n);
+  {
+    // scales [c4][group] = {tA0, tA1, tB0, tB1}, zeros [group][c4] likewise from fp16 index 64; pair r = (group, a >> 1)
+    const int g = r >> 1, ah = r & 1;
+    uint16_t* p16 = reinterpret_cast<uint16_t*>(vp);
+    *reinterpret_cast<uint32_t*>(p16 + (c4 * 4 + g) * 4 + ah * 2) = static_cast<uint32_t>(g0.s_bits) | (static_cast<uint32_t>(g1.s_bits) << 16);
+    *reinterpret_cast<uint32_t*>(p16 + 64 + (g * 4 + c4) * 4 + ah * 2) = static_cast<uint32_t>(g0.z_bits) | (static_cast<uint32_t>(g1.z_bits) << 16);
+  }
+  prm[r * 4 + c4] = i_pack_params(g0, g1);
+  __syncwarp();
+  uint64_t err[2] = {0ull, 0ull}, nrm[2] = {0ull, 0ull};      // [a >> 1], the lane's two tokens side by side
+#pragma unroll 1
+  for (int g = 0; g < 4; ++g) {
+    uint32_t x[2][4];
+    i_ldm4t(ld + g * 64, x[0]);
+    i_ldm4t(ld + g * 64 + 32, x[1]);
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int ah = 0; ah < 2; ++ah) {
+      const uint4 P = prm[(2 * g + ah) * 4 + c4];
+      const PairParams pp = i_pair_params(P, one);
+#pragma unroll
+      for (int ss = 0; ss < 2; ++ss) {
+        // word of (slice 2 g + ss, a): 8 bits: 4 g + 2 ss + (a >> 1), 4 bits: 2 g + ss, 2 bits: g
+        const int wi = BITS == 8 ? 2 * ss + ah : (BITS == 4 ? ss : 0);
+#pragma unroll
+        for (int al = 0; al < 2; ++al) {
+          const uint64_t X = i_pair_bf16(x[ss][2 * ah + al]);
+          i_quant_pair<BITS>(X, pp, i_bit_v<BITS>(ss, 2 * ah + al, 0), w[wi], err[ah]);
+          nrm[ah] = i_fma2(X, X, nrm[ah]);
+        }
+      }
+    }
+    if (BITS == 8) {
+      *reinterpret_cast<uint4*>(codes + (g * 32 + lane) * 16) =
+          make_uint4(w[0], w[1], w[2], w[3]);
+    } else if (BITS == 4) {
+      *reinterpret_cast<uint2*>(codes + ((g >> 1) * 32 + lane) * 16 + (g & 1) * 8) = make_uint2(w[0], w[1]);
+    } else {
+      *reinterpret_cast<uint32_t*>(codes + lane * 16 + g * 4) = w[0];
+    }
+  }
+#pragma unroll
+  for (int ah = 0; ah < 2; ++ah) {
+    i_halves(err[ah], e[ah][0], e[ah][1]);
+    i_halves(nrm[ah], n[ah][0], n[ah][1]);
+  }
+  return g0.s > v_scale_limit(BITS) || g1.s > v_scale_limit(BITS);
+}
+
+// One work item: a closed block of a stream.
+struct alignas(16) IngestJob {
+  unsigned long long first;     // its first element in the input rows
+  uint32_t dst_off256;
+  int32_t level, stream, block;
+};
+
+__global__ void __launch_bounds__(kInThreads, kInCtas) ingest_kernel(const __grid_constant__ EncodeParams p) {
   extern __shared__ __align__(16) uint8_t ism[];
-  float* cen = reinterpret_cast<float*>(ism + 2 * kInBuf);      // [2][128] centroid of keys, of values
+  __shared__ IngestJob s_jobs[3];
+  float* cen = reinterpret_cast<float*>(ism + kInBuf);          // [2][128] centroid of keys, of values
   float* kd2 = cen + 256;                                       // [2 channel halves][64 tokens]
   float* red = kd2 + 128;                                       // [4 value warps][2]: max error, max norm (squared)
   uint4* prm_all = reinterpret_cast<uint4*>(red + 16);          // [8 warps][8 pairs][4 lanes c4]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int r = lane >> 2, c4 = lane & 3, mi = lane >> 3;
   uint4* prm = prm_all + warp * 32;
-  const uint32_t sbase = i_u32(ism);
+  const uint32_t tile_s = i_u32(ism);
   const size_t row_stride = static_cast<size_t>(p.n_kv_heads) * kD;      // elements between two tokens of a stream
+  const float one_f = __int_as_float(0x3f800000 + (p.n_jobs >> 31));     // n_jobs is not negative
+  const uint64_t one = i_pair(one_f, one_f);
 
-  // work item -> (stream, block, slot, level): from the job list, or counted off in the order
-  // (sequence, block, KV head) with slot and level taken from the block table
-  auto job_of = [&](int item) -> EncodeJob {
-    if (p.jobs) return p.jobs[item];
+  // Work items are counted off in the order (sequence, block, KV head), slot and level taken from the block table: by one
+  // thread, two items ahead.
+  auto make_job = [&](int item, int slot) {
+    if (item >= p.n_jobs) return;
     const int per_seq = p.n_blocks * p.n_kv_heads;
     const int sq = item / per_seq, rem = item - sq * per_seq;
-    EncodeJob job;
+    IngestJob job;
     job.block = rem / p.n_kv_heads;
-    job.stream = (p.first_seq + sq) * p.n_kv_heads + (rem - job.block * p.n_kv_heads);
+    const int kvh = rem - job.block * p.n_kv_heads, b = p.first_seq + sq;
+    job.stream = b * p.n_kv_heads + kvh;
     const TableEntry te = p.table[static_cast<size_t>(job.stream) * p.table_stride + job.block];
-    job.src_off256 = 0;
     job.dst_off256 = te.off256;
-    job.src_level = 0;
-    job.dst_level = static_cast<int16_t>(te.level);
-    job.pad = 0;
-    return job;
+    job.level = static_cast<int32_t>(te.level);
+    job.first = (static_cast<size_t>(b) * p.n_tok + static_cast<size_t>(job.block) * kBlock) * row_stride + static_cast<size_t>(kvh) * kD;
+    s_jobs[slot] = job;
   };
-  auto stage = [&](int item, int buf) {
-    const EncodeJob job = job_of(item);
-    const int b = job.stream / p.n_kv_heads, kvh = job.stream - b * p.n_kv_heads;
-    const size_t first = (static_cast<size_t>(b) * p.n_tok + static_cast<size_t>(job.block) * kBlock) * row_stride + static_cast<size_t>(kvh) * kD;
+  // the thread's eight 16-byte pieces of a block: rows row0 + 16 i of the keys, then of the values
+  const int row0 = tid >> 4, col = tid & 15;
+  auto stage = [&](const IngestJob& job) {
+    const uint32_t d = tile_s + row0 * kInRow + col * 16;
+    const size_t off = job.first + row0 * row_stride + col * 8;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int q = tid + kInThreads * i;
-      const int tensor = q >> 10, row = (q >> 4) & 63, col = q & 15;
-      const uint16_t* src = (tensor ? p.v_in : p.k_in) + first + static_cast<size_t>(row) * row_stride + col * 8;
-      i_cp16(sbase + buf * kInBuf + tensor * kInTensor + row * kInRow + col * 16, src);
+    for (int i = 0; i < 4; ++i) {
+      i_cp16(d + i * 16 * kInRow, p.k_in + off + i * 16 * row_stride);
+      i_cp16(d + kInTensor + i * 16 * kInRow, p.v_in + off + i * 16 * row_stride);
     }
+    i_commit();
+  };
+  // ... and its share of a later block on the way to L2: 128 rows of 256 bytes, one line per thread
+  auto prefetch = [&](const IngestJob& job) {
+    const int row = (tid >> 1) & 63;
+    const uint16_t* src = (tid < 128 ? p.k_in : p.v_in) + job.first + row * row_stride + (tid & 1) * 64;
+    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(src));
   };
 
-  int item = blockIdx.x, buf = 0;
-  if (item < p.n_jobs) stage(item, 0);
-  i_commit();
-  for (; item < p.n_jobs; item += gridDim.x, buf ^= 1) {
-    const EncodeJob job = job_of(item);
+  int item = blockIdx.x;
+  if (tid == 0) {
+    make_job(item, 0);
+    make_job(item + gridDim.x, 1);
+  }
+  __syncthreads();
+  if (item < p.n_jobs) stage(s_jobs[0]);
+  for (int k = 0; item < p.n_jobs; item += gridDim.x, k = k == 2 ? 0 : k + 1) {
+    const IngestJob job = s_jobs[k];
+    const int knext = k == 2 ? 0 : k + 1;
+    const bool more = item + static_cast<int>(gridDim.x) < p.n_jobs;
     i_wait_all();
-    __syncthreads();                       // the block's rows are there; nobody still reads the other buffer
-    if (item + static_cast<int>(gridDim.x) < p.n_jobs) stage(item + gridDim.x, buf ^ 1);
-    i_commit();
+    __syncthreads();                       // the block's rows are there
+    if (more) prefetch(s_jobs[knext]);
+    if (tid == 0) make_job(item + 2 * gridDim.x, knext == 2 ? 0 : knext + 1);      // (the slot of the item before this one)
 
     uint8_t* dst = p.arena + static_cast<size_t>(job.dst_off256) * 256;
-    const int L = job.dst_level;
-    const uint8_t* tile_g = ism + buf * kInBuf;
-    const uint32_t tile_s = sbase + buf * kInBuf;
+    const int L = job.level;
+    const uint8_t* tile_g = ism;
 
     if (L == 16) {
       // exact rows: keys, then values, row-major
@@ -399,9 +637,9 @@ __global__ void __launch_bounds__(kInThreads, 3) ingest_kernel(const __grid_cons
       const int half = warp >> 1, chh = warp & 1;
       float e[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
       uint8_t* half_base = dst + half * half_bytes(L);
-      if (L == 8) range = ingest_keys<8>(tile_s, half_base, half, chh, lane, prm, e);
-      else if (L == 4) range = ingest_keys<4>(tile_s, half_base, half, chh, lane, prm, e);
-      else if (L == 2) range = ingest_keys<2>(tile_s, half_base, half, chh, lane, prm, e);
+      if (L == 8) range = ingest_keys<8>(tile_s, half_base, half, chh, lane, prm, one, e);
+      else if (L == 4) range = ingest_keys<4>(tile_s, half_base, half, chh, lane, prm, one, e);
+      else if (L == 2) range = ingest_keys<2>(tile_s, half_base, half, chh, lane, prm, one, e);
       else if (L == 1) {
         // distance from the centroid
         const uint32_t ld = tile_s + (32 * half + (mi & 1) * 8 + (lane & 7)) * kInRow + (64 * chh + (mi >> 1) * 8) * 2;
@@ -443,9 +681,9 @@ __global__ void __launch_bounds__(kInThreads, 3) ingest_kernel(const __grid_cons
         uint8_t* hb = dst + (tile >> 1) * half_bytes(L);
         uint8_t* vp = hb + off_vp(L, tile & 1);
         uint8_t* codes = hb + off_vc(L, tile & 1);
-        if (L == 8) range = ingest_values<8>(ld, vp, codes, lane, prm, e, n);
-        else if (L == 4) range = ingest_values<4>(ld, vp, codes, lane, prm, e, n);
-        else range = ingest_values<2>(ld, vp, codes, lane, prm, e, n);
+        if (L == 8) range = ingest_values<8>(ld, vp, codes, lane, prm, one, e, n);
+        else if (L == 4) range = ingest_values<4>(ld, vp, codes, lane, prm, one, e, n);
+        else range = ingest_values<2>(ld, vp, codes, lane, prm, one, e, n);
       } else {
         // squared norms of the rows; for a centroid block also the distance from the centroid
 #pragma unroll 1
@@ -495,7 +733,8 @@ __global__ void __launch_bounds__(kInThreads, 3) ingest_kernel(const __grid_cons
       }
     }
     if (range) atomicOr(p.status, kStatusRange);
-    __syncthreads();
+    __syncthreads();                       // nobody reads the rows any more
+    if (more) stage(s_jobs[knext]);
     if (warp == 0 && p.err) {
       // bound on |k - k^| (largest token), on |v - v^|, and the largest |v| of the block
       float km = fmaxf(kd2[lane] + kd2[kBlock + lane], kd2[32 + lane] + kd2[kBlock + 32 + lane]);
@@ -631,7 +870,7 @@ cudaError_t launch_ingest(const EncodeParams& p, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  const int grid = p.n_jobs < 148 * 3 ? p.n_jobs : 148 * 3;
+  const int grid = p.n_jobs < 148 * kInCtas ? p.n_jobs : 148 * kInCtas;
   ingest_kernel<<<grid, kInThreads, kInSmem, st>>>(p);
   return cudaGetLastError();
 }
