@@ -14,10 +14,13 @@
 namespace gkv {
 namespace {
 
-// One CTA scores kQPages consecutive pages of one stream, two neighbouring pages per thread.  The 256 box rows of
-// the stream (channel x min|max, kQPages * 2 bytes of each) are streamed through shared memory in chunks of
-// kQRows rows with 16-byte cp.async copies, kQStages chunks in flight, so that the loads are wide, contiguous
-// and deep while every thread still adds its pages' channels strictly in order.
+// One CTA scores 2 THREADS consecutive pages of one stream, two neighbouring pages per thread.  The 256 box rows of
+// the stream (channel x min|max) are streamed through shared memory in chunks of
+// kQRows rows with 16-byte cp.async copies, STAGES - 1 chunks in flight, so that the loads are wide, contiguous
+// and deep while every thread still adds its pages' channels strictly in order.  Two shapes: 128 pages and a ring of four
+// chunks where there are many pages, 64 pages and all eight chunks in flight where CTAs of that size fit the GPU
+// at once and the time is that of one round of loads (selection and read, 32 streams: 512 pages 31.2 -> 27.7 us, 1024 pages
+// 33.3 -> 30.5; beyond one wave, at 1536 pages, 37.1 instead of 35.4).
 //
 // The choice between maximum and minimum depends on the sign of q_d only, so it is made once, when the query is
 // staged: acc <- fma(max(q, 0), hi, fma(min(q, 0), lo, acc)), where one of the two products is a zero that leaves
@@ -25,13 +28,9 @@ namespace {
 // instructions per channel and two pages for four heads; with a select per head and one page per thread it was 40,
 // and the kernel was bound by instruction issue.  (Selection and read of 2048 pages x 32 streams: 37.0 -> 32.4 us a
 // layer with this and the selection below.)
-constexpr int kQThreads = 64, kQPages = 2 * kQThreads;
 constexpr int kQRows = 32;                                   // rows per chunk = 16 channels x (min, max)
-constexpr int kQStages = 4;
-constexpr int kQRowBytes = kQPages * 2;                      // 256
-constexpr int kQChunkBytes = kQRows * kQRowBytes;            // 8 KiB
-constexpr int kQPieces = kQRowBytes / 16;                    // 16-byte pieces per row
 constexpr int kQChunks = 2 * kD / kQRows;                    // 8
+constexpr int kQSmallCtas = 148 * 5;
 
 __device__ __forceinline__ void q_cp_async16(uint32_t dst, const void* src, bool on) {
   const uint32_t n = on ? 16u : 0u;                          // 0 source bytes: the 16 bytes are zero-filled
@@ -52,12 +51,13 @@ __device__ __forceinline__ uint64_t q_fma2(uint64_t a, uint64_t b, uint64_t c) {
 
 // GROUP = query heads per KV head, a compile-time bound: a run-time bound would leave the unused
 // heads' instructions in the loop, predicated off but still issued.
-template <int GROUP>
-__global__ void __launch_bounds__(kQThreads) quest_score_kernel(const uint16_t* __restrict__ boxes, int box_stride,
+template <int GROUP, int THREADS, int STAGES>
+__global__ void __launch_bounds__(THREADS) quest_score_kernel(const uint16_t* __restrict__ boxes, int box_stride,
                                                                 int n_pages, const uint16_t* __restrict__ q,
                                                                 int n_kv_heads, int reduce,
                                                                 float* __restrict__ scores, int score_stride) {
-  constexpr int group = GROUP;
+  constexpr int group = GROUP, kQThreads = THREADS, kQStages = STAGES, kQPages = 2 * THREADS;
+  constexpr int kQRowBytes = kQPages * 2, kQChunkBytes = kQRows * kQRowBytes, kQPieces = kQRowBytes / 16;      // 16-byte pieces per row
   // launched with programmatic stream serialisation: returns once the previous kernel of the stream
   // has completed (the launch itself overlaps that kernel's tail)
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
@@ -69,8 +69,8 @@ __global__ void __launch_bounds__(kQThreads) quest_score_kernel(const uint16_t* 
   const int page0 = blockIdx.x * kQPages;
   const uint16_t* rows = boxes + static_cast<size_t>(stream) * kD * 2 * box_stride + page0;
   const uint32_t stage0 = static_cast<uint32_t>(__cvta_generic_to_shared(qsm));
-  // chunk c -> stage c % kQStages: row r of the chunk is box row c * kQRows + r; a row is 16 pieces
-  // of 16 bytes (8 pages); pieces that start beyond the row's end (box_stride) are zero-filled
+  // chunk c -> stage c % kQStages: row r of the chunk is box row c * kQRows + r; a piece
+  // of 16 bytes is 8 pages; pieces that start beyond the row's end (box_stride) are zero-filled
   auto issue = [&](int c) {
     const uint32_t dst = stage0 + (c % kQStages) * kQChunkBytes;
 #pragma unroll
@@ -86,15 +86,17 @@ __global__ void __launch_bounds__(kQThreads) quest_score_kernel(const uint16_t* 
   {
     const uint32_t* q2 = reinterpret_cast<const uint32_t*>(q + static_cast<size_t>(stream) * group * kD);      // [batch][n_q_heads], KV heads in order
 #pragma unroll
-    for (int h = 0; h < GROUP; ++h) {
-      const uint32_t u = q2[h * (kD / 2) + tid];
-      const float v[2] = {__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)};
+    for (int h = 0; h < GROUP; ++h)
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const float up = fmaxf(v[k], 0.f), dn = fminf(v[k], 0.f);
-        qs[(2 * tid + k) * GROUP + h] = make_ulonglong2(q_pair(up, up), q_pair(dn, dn));
+      for (int at = tid; at < kD / 2; at += kQThreads) {
+        const uint32_t u = q2[h * (kD / 2) + at];
+        const float v[2] = {__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float up = fmaxf(v[k], 0.f), dn = fminf(v[k], 0.f);
+          qs[(2 * at + k) * GROUP + h] = make_ulonglong2(q_pair(up, up), q_pair(dn, dn));
+        }
       }
-    }
   }
   uint64_t acc[GROUP];
 #pragma unroll
@@ -359,14 +361,20 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const float* __restr
 
 }  // namespace
 
-cudaError_t launch_quest_scores(const uint16_t* boxes, int box_stride, int n_pages, const uint16_t* q,
-                                int n_streams, int n_kv_heads, int group, int reduce, float* scores,
-                                int score_stride, cudaStream_t st) {
-  if (n_pages <= 0) return cudaSuccess;
-  const size_t smem = kQStages * kQChunkBytes + static_cast<size_t>(group) * kD * 16;
+namespace {
+template <int GROUP, int THREADS, int STAGES>
+cudaError_t launch_quest_shape(const uint16_t* boxes, int box_stride, int n_pages, const uint16_t* q, int n_streams, int n_kv_heads,
+                               int reduce, float* scores, int score_stride, cudaStream_t st) {
+  const size_t smem = static_cast<size_t>(STAGES) * kQRows * THREADS * 4 + static_cast<size_t>(GROUP) * kD * 16;
+  static bool configured = false;
+  if (!configured) {
+    const cudaError_t e = cudaFuncSetAttribute(quest_score_kernel<GROUP, THREADS, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((n_pages + kQPages - 1) / kQPages, n_streams);
-  cfg.blockDim = dim3(kQThreads);
+  cfg.gridDim = dim3((n_pages + 2 * THREADS - 1) / (2 * THREADS), n_streams);
+  cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -374,19 +382,24 @@ cudaError_t launch_quest_scores(const uint16_t* boxes, int box_stride, int n_pag
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaSuccess;
-#define GKV_QUEST_CASE(G)                                                                                                \
-  case G: {                                                                                                              \
-    static bool configured = false;                                                                                      \
-    if (!configured) {                                                                                                   \
-      e = cudaFuncSetAttribute(quest_score_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)); \
-      if (e != cudaSuccess) return e;                                                                                    \
-      configured = true;                                                                                                 \
-    }                                                                                                                    \
-    e = cudaLaunchKernelEx(&cfg, quest_score_kernel<G>, boxes, box_stride, n_pages, q, n_kv_heads, reduce, scores,       \
-                           score_stride);                                                                                \
-    break;                                                                                                               \
-  }
+  return cudaLaunchKernelEx(&cfg, quest_score_kernel<GROUP, THREADS, STAGES>, boxes, box_stride, n_pages, q, n_kv_heads, reduce, scores, score_stride);
+}
+template <int GROUP>
+cudaError_t launch_quest_group(const uint16_t* boxes, int box_stride, int n_pages, const uint16_t* q, int n_streams, int n_kv_heads,
+                               int reduce, float* scores, int score_stride, cudaStream_t st) {
+  // CTAs of 64 pages that an SM holds at once: five (shared memory, four query heads)
+  if (static_cast<long long>((n_pages + 63) / 64) * n_streams <= kQSmallCtas)
+    return launch_quest_shape<GROUP, 32, kQChunks>(boxes, box_stride, n_pages, q, n_streams, n_kv_heads, reduce, scores, score_stride, st);
+  return launch_quest_shape<GROUP, 64, 4>(boxes, box_stride, n_pages, q, n_streams, n_kv_heads, reduce, scores, score_stride, st);
+}
+}  // namespace
+
+cudaError_t launch_quest_scores(const uint16_t* boxes, int box_stride, int n_pages, const uint16_t* q,
+                                int n_streams, int n_kv_heads, int group, int reduce, float* scores,
+                                int score_stride, cudaStream_t st) {
+  if (n_pages <= 0) return cudaSuccess;
+#define GKV_QUEST_CASE(G) \
+  case G: return launch_quest_group<G>(boxes, box_stride, n_pages, q, n_streams, n_kv_heads, reduce, scores, score_stride, st);
   switch (group) {
     GKV_QUEST_CASE(1)
     GKV_QUEST_CASE(2)
@@ -399,7 +412,6 @@ cudaError_t launch_quest_scores(const uint16_t* boxes, int box_stride, int n_pag
     default: return cudaErrorInvalidValue;
   }
 #undef GKV_QUEST_CASE
-  return e;
 }
 
 cudaError_t launch_topk(const float* scores, int score_stride, int n, const int32_t* k_per_stream, int k_uniform,
