@@ -158,6 +158,7 @@ struct LayerState {
   std::vector<std::vector<int32_t>> res_idx;      // host copy of the residual rows' tokens, fetched when first asked for
   bool res_idx_valid = true;
   bool desc_dirty = true;
+  int cluster = 0;                      // CTAs per head group of the work lists, 0 = head groups share CTAs
   bool split = false, split_all = false;      // the work lists hold parts of exact blocks / of others (never for observing calls)
   bool desc_allow_split = false;        // what the lists were built with
   int n_warps = 0;
@@ -538,6 +539,7 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
       L.n_units = S.n_units;
       L.split = S.split;
       L.split_all = S.split_all;
+      L.cluster = S.cluster;
       L.desc_allow_split = allow_split;
       L.desc_dirty = false;
       return;
@@ -554,13 +556,11 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   // over 8000 tokens from 14.9 to 13.3, over 16000 tokens of 2 streams from 14.2 to 13.0 and, near the line,
   // over 2000 tokens of 64 streams from 16.2 to 15.8.  (Exact blocks stop at half of that: the lists have room for
   // three extra units of as many blocks.)
-  L.split = L.split_all = false;
-  if (allow_split) {
-    size_t rough = 0;
-    for (int s = 0; s < ns; ++s) rough += static_cast<size_t>(L.n_closed + 1) * 1000 + static_cast<size_t>(L.res_count_h[s] / 16) * 550;
-    L.split = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost / 2;          // exact blocks
-    L.split_all = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost;          // quantised blocks, the tail
-  }
+  size_t rough = 0;
+  for (int s = 0; s < ns; ++s) rough += static_cast<size_t>(L.n_closed + 1) * 1000 + static_cast<size_t>(L.res_count_h[s] / 16) * 550;
+  const bool small = rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost;
+  L.split = allow_split && rough < static_cast<size_t>(kTargetWarps) * kMinWarpCost / 2;          // exact blocks
+  L.split_all = allow_split && small;                                                             // quantised blocks, the tail
   // Cost and units of every stream.  Streams with the same levels and the same number of residual rows (all streams
   // under the staircase policy) have the same.
   struct Sum { size_t cost; int units; };
@@ -591,12 +591,25 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   // every head group of a stream (up to four query heads each) walks the stream's units with warps of its own
   total *= static_cast<size_t>(hg);
   const size_t target = std::max(L.split_all ? kMinWarpCost / 4 : kMinWarpCost, (total + kTargetWarps - 1) / kTargetWarps);
+  // Small workloads: CTAs of its own for every head group, launched as a cluster and merged through distributed shared
+  // memory, where all clusters fit the GPU at once and its warps get at most twice what they would get of the whole GPU.
+  // Against shared CTAs with rows in global memory and a ticket: 2 streams of 4001 tokens 10.2 -> 7.8 us a call, 64 of
+  // 2000 16.0 -> 12.9, 16 of 9000 17.2 -> 15.2; two streams of 12,000 tokens at three times the load 11.9 -> 12.4.
+  L.cluster = 0;
+  if (small) {
+    int most = 0;
+    for (int s = 0; s < ns; ++s) most = std::max(most, std::min(static_cast<int>((sum[s].cost + target / 2) / target), sum[s].units));
+    int ctas = std::max(1, std::min((most + kDecodeWarps - 1) / kDecodeWarps, kMaxCluster));
+    while (ctas > 1 && (c->n_hgroups * ctas > 148 || c->n_hgroups > decode_max_clusters(ctas))) --ctas;
+    if (most <= 2 * ctas * kDecodeWarps && c->n_hgroups <= decode_max_clusters(ctas)) L.cluster = ctas;
+  }
   int w = 0, pos = 0, row = 0, last_nw = 0, stride = 1, stride_inv = 1;
   L.n_units = 0;
   for (int s = 0; s < ns; ++s) {
     int nw = static_cast<int>((sum[s].cost + target / 2) / target);
     nw = std::max(1, std::min(nw, sum[s].units));
-    nw = std::min(nw, (c->max_warps - w) / hg - (ns - 1 - s));
+    if (L.cluster > 0) nw = std::min(std::max(nw, std::min(L.cluster, sum[s].units)), L.cluster * kDecodeWarps);
+    else nw = std::min(nw, (c->max_warps - w) / hg - (ns - 1 - s));
     if (nw != last_nw) {
       stride = std::max(1, static_cast<int>(nw * 0.6180339887 + 0.5));
       while (std::gcd(stride, nw) != 1) ++stride;
@@ -610,6 +623,11 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
     L.n_units += sum[s].units;
     for (int g = 0; g < hg; ++g) {            // one partial row per (CTA, head group)
       const int hgi = s * hg + g;
+      if (L.cluster > 0) {
+        L.parts_h[hgi] = StreamParts{0, 1};
+        w += L.cluster * kDecodeWarps;
+        continue;
+      }
       L.parts_h[hgi].begin = row;
       row += (w + nw - 1) / kDecodeWarps - w / kDecodeWarps + 1;
       w += nw;
@@ -641,6 +659,7 @@ int make_units(gkv_cache* c, LayerState& L, bool allow_split, cudaStream_t st) {
   p.n_warps = L.n_warps;
   p.split = L.split;
   p.split_all = L.split_all;
+  p.cluster = L.cluster;
   const size_t head[6] = {kCost16 / (L.split ? 4 : 1), kCost8 / (L.split_all ? 2 : 1), kCost2 / (L.split_all ? 2 : 1),
                           kCost4 / (L.split_all ? 2 : 1), kCostTail / (L.split_all ? 4 : 1), kCostRes};
   for (int i = 0; i < kUnitClasses; ++i) p.cost[i] = static_cast<int32_t>(i < 6 ? head[i] : kCost1 * (22 - i));
@@ -1755,6 +1774,8 @@ int decode_impl(gkv_cache* c, int32_t layer, const void* q, const int32_t* page_
     p.n_warps = c->n_hgroups * p.warps_per_stream;
     p.warps = nullptr;
     p.parts = nullptr;
+    const int ctas = p.warps_per_stream / kDecodeWarps;
+    p.cluster = c->n_hgroups <= decode_max_clusters(ctas) ? ctas : 0;      // (as for the work lists: all clusters at once)
     n_ctas = (p.n_warps + kDecodeWarps - 1) / kDecodeWarps;
     L.last_mode = 2;
     L.last_pages = page_idx;
@@ -1771,6 +1792,7 @@ int decode_impl(gkv_cache* c, int32_t layer, const void* q, const int32_t* page_
     p.units = L.units_d;
     p.n_warps = L.n_warps;
     p.parts = L.parts_d;
+    p.cluster = L.cluster;
     n_ctas = L.n_warps / kDecodeWarps;
     L.last_mode = 1;
     L.quest_ran = false;

@@ -26,7 +26,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
-#include <cstdio>
+#include <atomic>
 
 #include "gkv_internal.h"
 
@@ -1141,6 +1141,84 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   const float* rows = reinterpret_cast<const float*>(smem);
   const int head = warp >> 2, chan = 32 * (warp & 3) + lane;
   const int group_of = s_group[lane & 15];
+  // rows [gb, ge) for this warp's head and channels: maximum, sum and the channel's accumulator relative to the maximum
+  auto merge_rows = [&](int gb, int ge, float& M, float& L, float& acc) {
+    const float* col = rows + head * (kD + 2);
+    const bool mine = lane >= gb && lane < ge;
+    const float m = mine ? col[lane * kRowFloats] : kNegInf, l = mine ? col[lane * kRowFloats + 1] : 0.f;
+    M = m;
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, d));      // rows sit in lanes 0 - 15
+    const float wt = (m == kNegInf) ? 0.f : fast_exp2(m - M);
+    L = wt * l;
+#pragma unroll
+    for (int d = 8; d > 0; d >>= 1) L += __shfl_xor_sync(kFull, L, d);
+    acc = 0.f;
+#pragma unroll 8
+    for (int i = gb; i < ge; ++i) acc = fmaf(__shfl_sync(kFull, wt, i), col[i * kRowFloats + 2 + chan], acc);
+    M = __shfl_sync(kFull, M, 0);
+    L = __shfl_sync(kFull, L, 0);
+  };
+  auto write_out = [&](size_t hq, int ch, float M, float L, float acc) {
+    p.out[hq * kD + ch] = (L > 0.f) ? acc / L : 0.f;
+    if (ch == 0) {
+      const float z = (L > 0.f) ? M + log2f(L) : kNegInf;
+      if (p.lse) p.lse[hq] = z * 0.6931471805599453f;
+      if constexpr (MASS) p.lse2[hq] = z;
+    }
+  };
+  if (p.cluster > 0) {
+    // The head group's warps are those of this cluster's CTAs: the CTAs' rows are exchanged through distributed shared
+    // memory, each CTA finishes a share of the channels, and nothing goes through global memory.
+    // (A CTA may have no warp at work: its row is empty.)
+    const int sid = static_cast<int>(blockIdx.x) / p.cluster, ge = __popc(__ballot_sync(kFull, group_of == sid) & 0xffffu);
+    const int sid_stream = sid / p.head_groups, sid_head0 = kHeadsPerWarp * (sid - sid_stream * p.head_groups);
+    const int n_heads = min(kHeadsPerWarp, p.group - sid_head0);
+    const size_t hq0 = static_cast<size_t>(sid_stream) * p.group + sid_head0;
+    float M = kNegInf, L = 0.f, acc = 0.f;
+    if (head < n_heads) merge_rows(0, ge, M, L, acc);
+    if (p.cluster == 1) {
+      if (head < n_heads) write_out(hq0 + head, chan, M, L, acc);
+      return;
+    }
+    float* mine = reinterpret_cast<float*>(smem + kStageBytes);        // the second stage of warp 0: idle
+    mine[head * (kD + 2) + 2 + chan] = acc;
+    if (chan == 0) *reinterpret_cast<float2*>(mine + head * (kD + 2)) = make_float2(M, L);
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    uint32_t rank;
+    asm("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
+    const int share = (kHeadsPerWarp * kD + p.cluster - 1) / p.cluster, e = static_cast<int>(rank) * share + threadIdx.x;
+    if (static_cast<int>(threadIdx.x) < share && e < n_heads * kD) {
+      const int h = e / kD, ch = e - h * kD;
+      const uint32_t at = smem_u32(mine) + h * (kD + 2) * 4;
+      float cm[kMaxCluster], cl[kMaxCluster], ca[kMaxCluster];
+#pragma unroll
+      for (int c = 0; c < kMaxCluster; ++c) {
+        cm[c] = kNegInf;
+        cl[c] = ca[c] = 0.f;
+        if (c < p.cluster) {
+          uint32_t remote;
+          asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(remote) : "r"(at), "r"(c));
+          asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(cm[c]), "=f"(cl[c]) : "r"(remote));
+          asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(ca[c]) : "r"(remote + 8 + ch * 4));
+        }
+      }
+      M = kNegInf;
+#pragma unroll
+      for (int c = 0; c < kMaxCluster; ++c) M = fmaxf(M, cm[c]);
+      L = acc = 0.f;
+#pragma unroll
+      for (int c = 0; c < kMaxCluster; ++c) {            // in the CTAs' order
+        const float wt = (cm[c] == kNegInf) ? 0.f : fast_exp2(cm[c] - M);
+        L = fmaf(wt, cl[c], L);
+        acc = fmaf(wt, ca[c], acc);
+      }
+      write_out(hq0 + h, ch, M, L, acc);
+    }
+    // nobody leaves while a neighbour may still read its row
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\nbarrier.cluster.wait.aligned;\n" ::: "memory");
+    return;
+  }
   int gb = 0;
 #pragma unroll 1
   while (gb < kDecodeWarps) {
@@ -1162,30 +1240,10 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
       }
       float* dst = p.partial + static_cast<size_t>(s_group[kDecodeWarps + gb]) * kPartialFloats;
       if (head < n_heads) {
-        const float* col = rows + head * (kD + 2);
-        const bool mine = lane >= gb && lane < ge;
-        const float m = mine ? col[lane * kRowFloats] : kNegInf, l = mine ? col[lane * kRowFloats + 1] : 0.f;
-        float M = m;
-#pragma unroll
-        for (int d = 8; d > 0; d >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, d));      // rows sit in lanes 0 - 15
-        const float wt = (m == kNegInf) ? 0.f : fast_exp2(m - M);
-        float L = wt * l;
-#pragma unroll
-        for (int d = 8; d > 0; d >>= 1) L += __shfl_xor_sync(kFull, L, d);
-        float acc = 0.f;
-#pragma unroll 8
-        for (int i = gb; i < ge; ++i) acc = fmaf(__shfl_sync(kFull, wt, i), col[i * kRowFloats + 2 + chan], acc);
-        M = __shfl_sync(kFull, M, 0);
-        L = __shfl_sync(kFull, L, 0);
+        float M, L, acc;
+        merge_rows(gb, ge, M, L, acc);
         if (end - begin == 1) {
-          // the head group has no other row: normalise and write the result
-          const size_t hq = hq0 + head;
-          p.out[hq * kD + chan] = (L > 0.f) ? acc / L : 0.f;
-          if (chan == 0) {
-            const float z = (L > 0.f) ? M + log2f(L) : kNegInf;
-            if (p.lse) p.lse[hq] = z * 0.6931471805599453f;
-            if constexpr (MASS) p.lse2[hq] = z;
-          }
+          write_out(hq0 + head, chan, M, L, acc);      // the head group has no other row
         } else {
           dst[head * (kD + 2) + 2 + chan] = acc;
           if (chan == 0) *reinterpret_cast<float2*>(dst + head * (kD + 2)) = make_float2(M, L);
@@ -1267,29 +1325,65 @@ size_t decode_smem_bytes() {
   return static_cast<size_t>(kDecodeWarps) * (kStages * kStageBytes + kStages * sizeof(uint64_t) + 2 * 2048 + 4 * sizeof(int)) + sizeof(int);
 }
 
-cudaError_t launch_decode(const DecodeParams& p, int n_ctas, bool overlap, cudaStream_t st) {
+namespace {
+cudaError_t configure_decode() {
   static bool configured = false;
-  if (!configured) {
-    const int bytes = static_cast<int>(decode_smem_bytes());
-    cudaError_t e = cudaFuncSetAttribute(decode_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(decode_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(decode_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e != cudaSuccess) return e;
-    configured = true;
+  if (configured) return cudaSuccess;
+  const int bytes = static_cast<int>(decode_smem_bytes());
+  cudaError_t e = cudaFuncSetAttribute(decode_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  configured = e == cudaSuccess;
+  return e;
+}
+}  // namespace
+
+int decode_max_clusters(int ctas) {
+  // by cluster size; -1 = not asked yet.  A property of the chip's layout (which SMs share a cluster's region): the same for
+  // every caller, so two threads that ask at once write the same value.
+  static std::atomic<int> known[kMaxCluster + 1] = {-1, -1, -1, -1, -1, -1, -1, -1, -1};
+  if (ctas < 1 || ctas > kMaxCluster) return 0;
+  if (known[ctas] >= 0) return known[ctas];
+  if (configure_decode() != cudaSuccess) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(ctas));
+  cfg.blockDim = dim3(kDecodeWarps * 32);
+  cfg.dynamicSmemBytes = decode_smem_bytes();
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(ctas);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, decode_kernel<false, false>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
   }
+  known[ctas] = n;
+  return n;
+}
+
+cudaError_t launch_decode(const DecodeParams& p, int n_ctas, bool overlap, cudaStream_t st) {
+  const cudaError_t ce = configure_decode();
+  if (ce != cudaSuccess) return ce;
   if (n_ctas <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_ctas);
   cfg.blockDim = dim3(kDecodeWarps * 32);
   cfg.dynamicSmemBytes = decode_smem_bytes();
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = overlap ? 1 : 0;
+  if (p.cluster > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = static_cast<unsigned>(p.cluster);
+    attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
   if (p.page_idx) return cudaLaunchKernelEx(&cfg, decode_kernel<true, false>, p);
   if (p.mass_raw) return cudaLaunchKernelEx(&cfg, decode_kernel<false, true>, p);
   return cudaLaunchKernelEx(&cfg, decode_kernel<false, false>, p);

@@ -63,6 +63,7 @@ struct UnitsParams {
   int32_t cost[kUnitClasses];   // of a unit, by class
   int32_t pad;                  // a power of two, at least 128 and the warps of any stream
   int32_t dealt;                // set by the launch
+  int32_t cluster;              // CTAs per head group, 0 = head groups share CTAs
 };
 
 constexpr int kDecodeWarps = 16;            // warps per CTA of the decode kernel
@@ -70,6 +71,7 @@ constexpr int kStageBytes = 5120;           // per-warp pipeline stage
 constexpr int kStages = 2;
 constexpr int kDecodeCtasPerSm = 1;
 constexpr int kMaxHeadsPerKv = 8;           // query heads per KV head
+constexpr int kMaxCluster = 8;              // CTAs per cluster (portable size)
 constexpr int kHeadsPerWarp = 4;            // a warp's head group: the n = 8 tensor-core dimension holds (hi, lo) column pairs
 constexpr int kPartialFloats = kHeadsPerWarp * (kD + 2);    // per partial row: m, l, o[128] per head
 
@@ -87,6 +89,7 @@ struct DecodeParams {
   int32_t n_closed, n_tail;
   int32_t n_kv_heads, group;    // group = query heads per KV head
   int32_t head_groups;          // head groups per KV head: ceil(group / kHeadsPerWarp)
+  int32_t cluster;              // CTAs per head group where each head group has CTAs of its own, launched as one cluster; else 0
   float scale_log2;             // softmax scale * log2(e)
   // sparse (page list) mode
   const int32_t* page_idx;      // [n_streams][n_sel] or nullptr
@@ -188,6 +191,7 @@ constexpr uint32_t kStatusInternal = 2u;   // an index check failed inside a ker
 // overlap: launched under programmatic stream serialisation; not behind a kernel that writes the work lists, which the read
 // looks at before it waits for its predecessor
 cudaError_t launch_decode(const DecodeParams& p, int n_ctas, bool overlap, cudaStream_t st);
+int decode_max_clusters(int ctas);          // clusters of that many decode CTAs that the GPU holds at once
 cudaError_t launch_units(UnitsParams p, int n_streams, int max_units, cudaStream_t st);
 cudaError_t launch_observe_finish(const ObserveParams& p, cudaStream_t st);
 cudaError_t launch_encode(const EncodeParams& p, cudaStream_t st);

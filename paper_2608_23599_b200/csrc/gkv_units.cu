@@ -208,12 +208,24 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
 
   // the warps' descriptors: the head groups of a stream get the same lists and neighbouring warps, so that the second
   // reader of a block finds it in L2; one partial row per (CTA, head group)
-  for (int i = tid; i < nw * p.head_groups; i += kUnitThreads) {
-    const int g = i / nw, k = i - g * nw, hg = s * p.head_groups + g, w0 = plan.warp_base + g * nw, w = w0 + k;
+  auto describe = [&](int k, int hg, int partial) {
     const int d = static_cast<int>(static_cast<long long>(k) * plan.stride % nw);
     const int m = full + static_cast<int>(s_key[d]);
     const int begin = plan.unit_base + k * plan.pitch;
-    p.warps[w] = WarpDesc{hg, begin, begin + m, p.parts[hg].begin + w / kDecodeWarps - w0 / kDecodeWarps};
+    return WarpDesc{hg, begin, begin + m, partial};
+  };
+  if (p.cluster > 0) {
+    // CTAs of the head group's own, its warps dealt round by round to them
+    const int room = p.cluster * kDecodeWarps;
+    for (int i = tid; i < room * p.head_groups; i += kUnitThreads) {
+      const int g = i / room, at = i - g * room, k = (at % kDecodeWarps) * p.cluster + at / kDecodeWarps;
+      p.warps[plan.warp_base + i] = k < nw ? describe(k, s * p.head_groups + g, 0) : WarpDesc{-1, 0, 0, 0};
+    }
+    return;
+  }
+  for (int i = tid; i < nw * p.head_groups; i += kUnitThreads) {
+    const int g = i / nw, k = i - g * nw, hg = s * p.head_groups + g, w0 = plan.warp_base + g * nw, w = w0 + k;
+    p.warps[w] = describe(k, hg, p.parts[hg].begin + w / kDecodeWarps - w0 / kDecodeWarps);
   }
   if (s == static_cast<int>(gridDim.x) - 1)
     for (int w = plan.warp_base + nw * p.head_groups + tid; w < p.n_warps; w += kUnitThreads) p.warps[w] = WarpDesc{-1, 0, 0, 0};
