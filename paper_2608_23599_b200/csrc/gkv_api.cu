@@ -594,9 +594,11 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   // Small workloads: CTAs of its own for every head group, launched as a cluster and merged through distributed shared
   // memory, where all clusters fit the GPU at once and its warps get at most twice what they would get of the whole GPU.
   // Against shared CTAs with rows in global memory and a ticket: 2 streams of 4001 tokens 10.2 -> 7.8 us a call, 64 of
-  // 2000 16.0 -> 12.9, 16 of 9000 17.2 -> 15.2; two streams of 12,000 tokens at three times the load 11.9 -> 12.4.
+  // 2000 16.0 -> 12.9, 16 of 9000 17.2 -> 15.2, 64 of 4000 18.2 -> 16.1; two streams of 12,000 tokens at three times the
+  // load 11.9 -> 12.4.  Up to two blocks per warp of the GPU: at 3.5, 16 streams of 32,768 tokens take 30.0 us instead of
+  // 27.6, although 64 of 8000 would take 24.8 instead of 26.4.
   L.cluster = 0;
-  if (small) {
+  if (rough < 2 * static_cast<size_t>(kTargetWarps) * kMinWarpCost) {
     int most = 0;
     for (int s = 0; s < ns; ++s) most = std::max(most, std::min(static_cast<int>((sum[s].cost + target / 2) / target), sum[s].units));
     int ctas = std::max(1, std::min((most + kDecodeWarps - 1) / kDecodeWarps, kMaxCluster));
