@@ -707,7 +707,7 @@ int rd_plan_launch(gkv_cache* c, LayerState& L, int n, int n_tail, bool use_prev
   p.range_stride = c->max_blocks;
   p.table_stride = c->table_stride;
   p.out_stride = c->max_blocks;
-  rd_plan_smem_bytes(n, &p.m_pad);
+  rd_plan_smem_bytes(n, &p.pad);
   p.n_sink_blocks = cfg.n_sink_blocks;
   p.retire_after = cfg.retire_after;
   p.monotone = cfg.monotone_in_age != 0;

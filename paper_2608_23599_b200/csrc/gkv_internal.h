@@ -207,14 +207,14 @@ struct RdPlanParams {
   int8_t* levels_out;           // [n_streams][out_stride]
   uint32_t* miss_flag;          // set to 1 when a stream cannot meet the budget (its plan is still written)
   int32_t n, mass_stride, range_stride, table_stride, out_stride;
-  int32_t m_pad;                // power of two >= 4 n + 1 (rd_plan_smem_bytes)
+  int32_t pad;                  // power of two >= n (rd_plan_smem_bytes)
   int32_t n_sink_blocks, retire_after, monotone, use_prev;
   unsigned long long nval_tok, budget_bits, tail_bits;
   // Bulk ingest with exact residual rows, nullable: rows of every stream = min(n_res, 64 x blocks planned below 16, res_cap)
   int32_t* res_count;           // [n_streams]
   int32_t n_res, res_cap;
 };
-size_t rd_plan_smem_bytes(int n, int* m_pad_out);
+size_t rd_plan_smem_bytes(int n, int* pad_out);
 cudaError_t launch_rd_plan(const RdPlanParams& p, int n_streams, cudaStream_t st);
 cudaError_t launch_append_rows(uint8_t* arena, const TableEntry* table, int table_stride, int tail_index,
                                int n_streams, int n_kv_heads, const uint16_t* k_in, const uint16_t* v_in,
