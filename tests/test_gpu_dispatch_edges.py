@@ -1,0 +1,209 @@
+"""The sizes at which a kernel or a dispatch rule changes: selection lists around the number of keys a thread
+holds, page scorer shapes, work lists that become clusters of one to eight CTAs or share CTAs, device allocator sizes,
+parameters outside the fp16 range in the bulk encoder, signed zeros in page boxes, latent batches around one wave of
+CTAs, and caches that hand their page-locked block on between threads."""
+import dataclasses
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import gkv_oracle as O
+from paper_2608_23599_b200 import workloads as W
+import parity_util as U
+
+pytestmark = pytest.mark.gpu
+
+
+def _binding():
+    from paper_2608_23599_b200 import binding as B
+    return B
+
+
+def _gqa(ctx, batch=1, n_kv=1, group=1, **kw):
+    return W.Workload("edge", 60, 1, batch, n_kv * group, n_kv, 128, 128, ctx, ctx + 128, n_heavy=0, **kw)
+
+
+# ---- page scores and selection ----------------------------------------------------------------------
+@pytest.mark.parametrize("n_pages", [4, 64, 68, 4096, 4100, 16384, 16388, 32768, 32772])
+def test_selection_around_the_lengths_that_change_its_kernel(n_pages):
+    """One stream of n_pages 16-token pages whose keys are small integers, so that many scores are equal: scores against
+    the sequential fp32 rule, selected pages against a stable sort, for one page, an eighth and all of them."""
+    B = _binding()
+    T = 16 * n_pages + 3
+    w = _gqa(T, group=2, page_tokens=16, stair_tokens=(64, 0, 0, 0))
+    g = B.Cache(B.config_from_workload(w))
+    gen = torch.Generator(device=g.device)
+    gen.manual_seed(n_pages)
+    k = torch.randint(-2, 3, (1, T, 1, 128), generator=gen, device=g.device).to(torch.bfloat16)
+    q = torch.randint(-1, 2, (1, 2, 128), generator=gen, device=g.device).to(torch.bfloat16)
+    g.gkv_append_demote(0, k, k)
+    score = g.gkv_debug_export_scores(0, q)[0, 0]
+    pages = k[0, : 16 * n_pages, 0].float().reshape(n_pages, 16, 128)
+    lo, hi, qf = pages.amin(1), pages.amax(1), q[0].float()
+    acc = torch.zeros((2, n_pages), device=g.device)
+    for d in range(128):
+        acc = acc + qf[:, d: d + 1] * torch.where(qf[:, d: d + 1] >= 0, hi[:, d], lo[:, d])
+    assert np.array_equal(score, torch.maximum(acc[0], acc[1]).cpu().numpy())
+    order = np.argsort(-score, kind="stable")
+    for n_sel in sorted({1, max(1, n_pages // 8), n_pages}):
+        out = torch.full((1, 1, n_sel), -1, dtype=torch.int32, device=g.device)
+        assert g.gkv_quest_select(0, q, 16 * n_sel, out) == n_sel
+        torch.cuda.synchronize()
+        assert np.array_equal(out.cpu().numpy()[0, 0], np.sort(order[:n_sel])), n_sel
+
+
+def test_box_of_signed_zeros_takes_the_sign_of_the_first():
+    """Pages whose smallest or largest key is a zero of either sign: the box holds the page's first zero, bit for bit."""
+    B = _binding()
+    T = 640
+    w = _gqa(T, page_tokens=16, stair_tokens=(-1, 0, 0, 0))
+    g = B.Cache(B.config_from_workload(w))
+    rs = np.random.RandomState(3)
+    bits = np.where(rs.rand(T, 128) < 0.5, 0x0000, 0x8000).astype(np.uint16)
+    bits[:, 32:64] = np.where(rs.rand(T, 32) < 0.3, 0x3f80, bits[:, 32:64])      # zeros and ones: the minimum is a zero
+    bits[:, 64:96] = np.where(rs.rand(T, 32) < 0.3, 0xbf80, bits[:, 64:96])      # zeros and minus ones: the maximum is
+    k = torch.from_numpy(bits.view(np.int16)).to(g.device).view(torch.bfloat16).reshape(1, T, 1, 128)
+    g.gkv_append_demote(0, k, k)
+    lo, hi = g.gkv_debug_export_boxes(0, 0, 0)
+    val = (bits.astype(np.uint32) << 16).view(np.float32).reshape(T // 16, 16, 128)
+    raw = bits.reshape(T // 16, 16, 128)
+    first = lambda ext: np.take_along_axis(raw, np.argmax(val == ext[:, None], axis=1)[:, None], axis=1)[:, 0]   # noqa: E731
+    assert np.array_equal(lo, first(val.min(1))) and np.array_equal(hi, first(val.max(1)))
+
+
+# ---- work lists --------------------------------------------------------------------------------------
+@pytest.mark.parametrize("batch,n_kv,group,T", [
+    (1, 1, 1, 70), (1, 1, 8, 200), (1, 2, 4, 1000), (2, 1, 5, 2500), (2, 2, 4, 4100), (3, 6, 2, 1500), (5, 4, 6, 700),
+    (37, 4, 1, 130), (38, 4, 1, 130), (1, 1, 4, 9000)])
+def test_work_lists_from_one_cta_to_shared_ctas(batch, n_kv, group, T):
+    """Random plans with centroid runs of every length: one CTA per head group, clusters of two to eight, more head groups
+    than SMs, and streams that share CTAs; the read, and the observing read, which takes whole blocks only."""
+    B = _binding()
+    w = _gqa(T, batch, n_kv, group, policy=W.POLICY_EXTERNAL)
+    data = W.make_layer(w, 0, "cpu")
+    rs = np.random.RandomState(T + batch)
+    plan = np.empty((batch, n_kv, T // 64), dtype=np.int8)
+    for b in range(batch):
+        for h in range(n_kv):
+            i = 0
+            while i < T // 64:
+                n = int(rs.randint(1, 25))
+                plan[b, h, i:i + n] = rs.choice(np.array([16, 8, 4, 2, 1, 1], dtype=np.int8))
+                i += n
+    ocache, g = O.GradedCache(U.oracle_config(w)), B.Cache(B.config_from_workload(w))
+    U.ingest_both(w, 0, data, ocache, g, level_plan=plan)
+    out, lse, o_out, o_lse = U.decode_both(ocache, g, 0, data["q"])
+    U.assert_outputs_close(out, o_out, "read")
+    assert np.max(np.abs(lse.cpu().numpy() - o_lse)) < 5e-3
+    mass = torch.empty((batch, n_kv, -(-T // 64)), dtype=torch.float32, device=g.device)
+    out2 = torch.empty_like(out)
+    g.gkv_decode_attn_observe(0, data["q"].to(g.device), out2, None, mass)
+    torch.cuda.synchronize()
+    U.assert_outputs_close(out2, o_out, "observing read")
+    assert np.allclose(mass.cpu().numpy().sum(-1), 1.0, atol=2e-3)
+    again = torch.empty_like(out)
+    g.gkv_decode_attn(0, data["q"].to(g.device), again)
+    assert torch.equal(again, out2)              # the same lists until a block closes
+
+
+@pytest.mark.parametrize("batch,T", [(1, 65), (2, 333), (9, 300), (148, 70), (149, 70)])
+def test_latent_batches_around_one_wave_of_ctas(batch, T):
+    B = _binding()
+    w = W.Workload("edge_latent", 61, 1, batch, 16, 1, 576, 512, T, T + 128, v_aliases_k=1, stair_tokens=(64, 64, 128, 0),
+                   softmax_scale=1.0 / 192.0 ** 0.5, n_outlier=8, outlier_gain=6.0, n_heavy=0)
+    data = W.make_layer(w, 0, "cpu")
+    ocache, g = O.GradedCache(U.oracle_config(w)), B.Cache(B.config_from_workload(w))
+    U.ingest_both(w, 0, data, ocache, g)
+    for step in range(3):                        # the tail grows into new 16-row units
+        out, lse, o_out, o_lse = U.decode_both(ocache, g, 0, data["q"])
+        U.assert_outputs_close(out, o_out, f"latent batch {batch}, step {step}")
+        assert np.max(np.abs(lse.cpu().numpy() - o_lse)) < 5e-3
+        for i in range(11):
+            tok = W.make_decode_tokens(w, 0, 100 * step + i, "cpu")
+            ocache.append_demote(0, U.f32(tok["k"]), None)
+            g.gkv_append_demote(0, tok["k"].to(g.device), None)
+
+
+# ---- allocator and encoder ---------------------------------------------------------------------------
+@pytest.mark.parametrize("n_closed", [1, 2, 3, 31, 33, 1023, 1025, 4095, 4097])
+def test_ingest_plan_equals_host_allocator(n_closed):
+    """The plan of a bulk ingest (made on the device up to 4095 blocks) against the host-only entry point on the same
+    masses and ranges."""
+    B = _binding()
+    T = 64 * n_closed + 7
+    w = _gqa(T, n_kv=2, policy=W.POLICY_RD, rd_budget_bpv=5.0, retire_after=128)
+    g = B.Cache(B.config_from_workload(w))
+    gen = torch.Generator(device=g.device)
+    gen.manual_seed(n_closed)
+    k = torch.randn((1, T, 2, 128), generator=gen, device=g.device).to(torch.bfloat16)
+    mass = torch.softmax(3 * torch.randn((1, 2, T), generator=gen, device=g.device), -1)
+    g.gkv_append_demote(0, k, k, token_mass=mass)
+    _, ms, rg, _ = g.gkv_debug_device_plan(0)
+    for h in range(2):
+        want, _ = B.gkv_debug_plan_levels(g.cfg, n_closed, 7, ms[0, h], rg[0, h])
+        assert np.array_equal(g.gkv_debug_export_levels(0, 0, h), want), h
+
+
+@pytest.mark.parametrize("level", [8, 4, 2])
+def test_bulk_encoder_with_parameters_outside_the_fp16_range(level):
+    """Blocks whose scale or zero point saturates beside ordinary ones (the two go through different code): the stored
+    state against the oracle, bit for bit."""
+    B = _binding()
+    T = 256
+    w = _gqa(T, policy=W.POLICY_EXTERNAL)
+    data = W.make_layer(w, 0, "cpu")
+    for name, sign in (("k", 1.0), ("v", -1.0)):
+        x = data[name].float()
+        x[0, 3, 0, 5] = sign * 3e38              # a scale and, negative, a zero point beyond 65504
+        x[0, 70, 0, 60:64] = -1e6
+        x[0, 71, 0, 100] = 1e-30                 # a range that fp16 scales cannot express
+        x[0, 130:194] = sign * 7e4               # constant blocks beyond the range
+        data[name] = x.to(torch.bfloat16)
+    ocache, g = O.GradedCache(U.oracle_config(w)), B.Cache(B.config_from_workload(w))
+    with np.errstate(over="ignore", invalid="ignore"):
+        U.ingest_both(w, 0, data, ocache, g, level_plan=np.full((1, 1, T // 64), level, dtype=np.int8))
+    U.assert_state_equal(ocache, g, 0)
+
+
+# ---- caches one after another -------------------------------------------------------------------------
+def test_caches_of_two_threads_hand_on_their_host_blocks():
+    """Two threads, each with a stream of its own, make, use and release caches of changing size; every read equals the
+    one of the same cache made alone."""
+    B = _binding()
+    shapes = [(1, 200), (2, 1500), (1, 5000), (4, 300), (1, 200), (2, 1500)]
+
+    def request(i, side):
+        batch, T = shapes[i]
+        w = dataclasses.replace(_gqa(T, batch, 2, 4, stair_tokens=(64, 128, 256, 512)), config_id=60 + side)
+        data = W.make_layer(w, i, "cuda")
+        cache = B.Cache(B.config_from_workload(w))
+        out = torch.empty((batch, 8, 128), dtype=torch.float32, device=cache.device)
+        cache.gkv_append_demote(0, data["k"], data["v"])
+        for s in range(70):
+            cache.gkv_append_demote(0, data["k"][:, s: s + 1].contiguous(), data["v"][:, s: s + 1].contiguous())
+            cache.gkv_decode_attn(0, data["q"], out)
+        torch.cuda.current_stream().synchronize()
+        cache.close()
+        return out.cpu()
+
+    alone = {(i, side): request(i, side) for i in range(len(shapes)) for side in range(2)}
+    got, errors = {}, []
+
+    def work(side):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for i in range(len(shapes)):
+                    got[(i, side)] = request(i, side)
+        except Exception as e:      # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(side,)) for side in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for key, want in alone.items():
+        assert torch.equal(got[key], want), key
