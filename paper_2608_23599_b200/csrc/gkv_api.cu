@@ -1186,18 +1186,22 @@ void mla_build_descs(gkv_cache* c, LayerState& L) {
     L.parts_h[s].begin = w;
     L.parts_h[s].end = w + nw[s];
     int quad = 0, begin = 0, pos = 0;
-    size_t acc = 0;
+    size_t acc = 0, share = 0;                     // share: what the quads up to this one take
     auto close = [&](int end) {
-      L.warps_h[kMlaQuads * w + quad] = WarpDesc{s, begin, end, w + quad / kMlaQuads};
-      begin = end;
-      ++quad;
+      if (end >= 0) {
+        L.warps_h[kMlaQuads * w + quad] = WarpDesc{s, begin, end, w + quad / kMlaQuads};
+        begin = end;
+        ++quad;
+      }
+      share = quad < n - 1 ? (cost[s] * (quad + 1) + n - 1) / n : ~size_t{0};
     };
+    close(-1);
     for (int i = 0; i < n_items; ++i) {
       const MlaItem it = mla_item(c, L, s, i);
+      const size_t piece = it.cost / it.parts;
       for (int k = 0; k < it.parts; ++k) {
-        const size_t piece = it.cost / it.parts;
         // the piece belongs to the next quad when more than half of it lies beyond this quad's share
-        while (quad < n - 1 && (acc + piece / 2) * n >= cost[s] * (quad + 1)) close(pos);
+        while (acc + piece / 2 >= share) close(pos);
         acc += piece;
         pos = 4 * i + (k + 1) * it.step;
       }
