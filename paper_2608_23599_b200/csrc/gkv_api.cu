@@ -619,9 +619,8 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
       while (static_cast<long long>(stride) * stride_inv % nw != 1 % nw) ++stride_inv;
       last_nw = nw;
     }
-    const int pitch = (sum[s].units + nw - 1) / nw;
-    L.plans_h[s] = StreamPlan{pos, pitch, sum[s].units, nw, w, stride, stride_inv, L.res_count_h[s]};
-    pos += nw * pitch;
+    L.plans_h[s] = StreamPlan{pos, sum[s].units, nw, w, stride, stride_inv, L.res_count_h[s]};
+    pos += sum[s].units;
     L.n_units += sum[s].units;
     for (int g = 0; g < hg; ++g) {            // one partial row per (CTA, head group)
       const int hgi = s * hg + g;

@@ -41,7 +41,6 @@ struct alignas(8) StreamParts {
 // What the host decides about a stream's work lists (gkv_units.cu makes the lists).
 struct alignas(16) StreamPlan {
   int32_t unit_base;      // first unit word of the stream's lists
-  int32_t pitch;          // room per list: ceil(n_units / n_warps)
   int32_t n_units;        // units of the stream
   int32_t n_warps;        // warps per head group, at most n_units
   int32_t warp_base;      // first warp of the stream's first head group

@@ -2,11 +2,13 @@
 //
 // A stream's items (closed blocks, the tail, groups of 16 exact residual rows) become units: an item, a run of up to 16
 // neighbouring centroid blocks that does not cross a multiple of 16, or, in small workloads, a part of a block.  The
-// units are put in order of falling cost and dealt to the stream's warps in rounds of one unit each, the costliest unit of
-// a round to the warp that has least so far, so that every warp ends up with about the same cost whatever the order
-// of levels along the context, and with about the same share of every level.  (Dealing forth and back without a look at
+// units are put in order of falling cost and dealt to the stream's warps in rounds: the costliest unit of a round goes to
+// the warp that has least so far, the next one to the next warp, up to the first warp that already has more than the least
+// laden one will have with its unit.  So every warp ends up with about the same cost whatever the order of levels along
+// the context, and with about the same share of every level.  (Dealing forth and back without a look at
 // what a warp has balances the cost as well, but leaves the 8-bit blocks to the warps that have an exact one: 64 streams
-// of 32,757 tokens took 73.6 us a call instead of 72.3.)
+// of 32,757 tokens took 73.6 us a call instead of 72.3.  One unit to every warp in every round leaves a warp with an exact
+// block 12 % more than the others where the rest is cheap: 64 streams with exact residual rows 32.7 us a call.)
 //
 // The first round hands the costliest units (exact blocks, then 8-bit ones) to the first warps, and a CTA is a window of
 // consecutive warps: the warps are walked with a golden-ratio stride, so that every window holds the same mixture of
@@ -31,12 +33,12 @@ static_assert(148 * kDecodeCtasPerSm * kDecodeWarps + 1 < (1 << kUnitHandBits), 
 
 __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_constant__ UnitsParams p) {
   __shared__ int s_base[kUnitClasses], s_start[kUnitClasses + 1], s_at[kUnitWarps][kUnitClasses];
-  extern __shared__ __align__(16) uint32_t s_key[];                          // [pad] load / 16 << 12 | warp
+  extern __shared__ __align__(16) uint32_t s_key[];            // [pad] load / 16 << 12 | warp; later where a list begins
   const int s = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const StreamPlan plan = p.plans[s];
   const TableEntry* table = p.table + static_cast<size_t>(s) * p.table_stride;
   const int n_items = p.n_closed + 1 + (plan.n_res + 15) / 16;
-  const int nw = plan.n_warps, full = plan.n_units / nw, rem = plan.n_units - full * nw;
+  const int nw = plan.n_warps;
 
   // an item's class (-1: it is part of an earlier unit, or past the end), its unit word without the tile mask, its parts
   auto classify = [&](int it, uint32_t& word, int& parts) -> int {
@@ -94,29 +96,38 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
   clear();
   const int pad = p.pad;                               // a power of two, at least the warps of any stream
   uint32_t* s_mix = s_key + pad;                       // [pad] a warp's 2-bit units, and its 4-bit ones << 16
-  uint16_t* hand_of = reinterpret_cast<uint16_t*>(s_mix + pad);              // [n_units] the warp that a rank goes to
+  uint32_t* s_cnt = s_mix + pad;                       // [pad] units of a warp
+  uint32_t* hand_of = s_cnt + pad;                     // [n_units] a rank's place in its list << 12 | the warp that it goes to
   for (int i = tid; i < pad; i += kUnitThreads) {
     s_key[i] = i < nw ? static_cast<uint32_t>(i) : 0xffffffffu;
     s_mix[i] = 0u;
+    s_cnt[i] = 0u;
   }
   __syncthreads();
 
-  // the deal: per round the warps in order of what they have.  A thread's ranks only grow, so its class does, too.
-  int cls_at = 0;
+  // The deal: per round the warps in order of what they have, those left out that have more than the least laden one
+  // will have with its unit.  A thread's ranks only grow, so its class does, too.
+  const int n_units = plan.n_units;
+  int cls_at = 0, cls_base = 0, base = 0;
   auto deal = [&](int rank, uint32_t key) -> uint32_t {
-    if (rank >= plan.n_units) return key;
+    if (rank >= n_units) return key;
     const uint32_t hand = key & ((1u << kUnitHandBits) - 1u);
-    hand_of[rank] = static_cast<uint16_t>(hand);
+    hand_of[rank] = (s_cnt[hand]++ << kUnitHandBits) | hand;                         // (one unit per warp and round)
     while (cls_at < kUnitClasses - 1 && rank >= s_start[cls_at + 1]) ++cls_at;
-    if (cls_at == 2 || cls_at == 3) s_mix[hand] += cls_at == 2 ? 1u : 0x10000u;      // (one unit per warp and round)
+    if (cls_at == 2 || cls_at == 3) s_mix[hand] += cls_at == 2 ? 1u : 0x10000u;
     return key + (static_cast<uint32_t>(p.cost[cls_at]) / 16 << kUnitHandBits);
+  };
+  // keys below this take part in the round that begins with rank `base`; least is the smallest key
+  auto limit = [&](uint32_t least) -> uint32_t {
+    while (cls_base < kUnitClasses - 1 && base >= s_start[cls_base + 1]) ++cls_base;
+    return ((least >> kUnitHandBits) + static_cast<uint32_t>(p.cost[cls_base]) / 16) << kUnitHandBits;
   };
   if (p.dealt && nw <= 64) {
     // one warp, two keys a lane (places lane and lane + 32), sorted with shuffles
     if (warp == 0) {
       uint32_t k0 = lane < nw ? static_cast<uint32_t>(lane) : 0xffffffffu, k1 = lane + 32 < nw ? static_cast<uint32_t>(lane + 32) : 0xffffffffu;
-      for (int r = 0; r * nw < plan.n_units; ++r) {
-        if (r > 0) {
+      while (base < n_units) {
+        if (base > 0) {
 #pragma unroll
           for (int k = 2; k <= 64; k <<= 1) {
 #pragma unroll
@@ -134,15 +145,19 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
             }
           }
         }
-        if (lane < nw) k0 = deal(r * nw + lane, k0);
-        if (lane + 32 < nw) k1 = deal(r * nw + lane + 32, k1);
+        const uint32_t lim = limit(__shfl_sync(kUnitAll, k0, 0));
+        const bool in0 = k0 < lim || lane == 0, in1 = k1 < lim;      // the least laden warp always: every round ends with fewer units left
+        if (in0) k0 = deal(base + lane, k0);
+        if (in1) k1 = deal(base + lane + 32, k1);
+        base += __popc(__ballot_sync(kUnitAll, in0)) + __popc(__ballot_sync(kUnitAll, in1));
+        __syncwarp();
       }
     }
   } else if (p.dealt) {
     int small = 128;
     while (small < nw) small <<= 1;
-    for (int r = 0; r * nw < plan.n_units; ++r) {
-      if (r > 0) {
+    while (base < n_units) {
+      if (base > 0) {
         for (int k = 2; k <= small; k <<= 1) {
           for (int j = k >> 1; j > 0; j >>= 1) {
             for (int q = tid; q < small / 2; q += kUnitThreads) {
@@ -157,15 +172,38 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
           }
         }
       }
-      for (int i = tid; i < nw; i += kUnitThreads) s_key[i] = deal(r * nw + i, s_key[i]);
+      const uint32_t lim = limit(s_key[0]);
+      int m = 1, end = nw;                             // how many keys, in order, are below the limit (the first one is)
+      while (m < end) {
+        const int mid = (m + end) >> 1;
+        if (s_key[mid] < lim) m = mid + 1;
+        else end = mid;
+      }
+      __syncthreads();
+      for (int i = tid; i < m; i += kUnitThreads) s_key[i] = deal(base + i, s_key[i]);
+      base += m;
       __syncthreads();
     }
+  } else {
+    const int full = n_units / nw;
+    for (int i = tid; i < nw; i += kUnitThreads) s_cnt[i] = static_cast<uint32_t>(full + (i < n_units - full * nw));
   }
   __syncthreads();
-  // who has one more than the full rounds (the keys are done with)
-  for (int i = tid; i < nw; i += kUnitThreads) s_key[i] = 0u;
-  __syncthreads();
-  for (int i = tid; i < rem; i += kUnitThreads) s_key[p.dealt ? hand_of[full * nw + i] : i] = 1u;
+  // where the warps' lists begin (the keys are done with)
+  if (warp == 0) {
+    uint32_t at = static_cast<uint32_t>(plan.unit_base);
+    for (int i0 = 0; i0 < nw; i0 += 32) {
+      const uint32_t n = i0 + lane < nw ? s_cnt[i0 + lane] : 0u;
+      uint32_t incl = n;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t up = __shfl_up_sync(kUnitAll, incl, d);
+        if (lane >= d) incl += up;
+      }
+      if (i0 + lane < nw) s_key[i0 + lane] = at + incl - n;
+      at += __shfl_sync(kUnitAll, incl, 31);
+    }
+  }
   __syncthreads();
 
   // pass 2: every unit's rank, and from it its warp and its place in the warp's list
@@ -190,15 +228,17 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
     if (cls >= 0) {
       int rank = s_at[warp][cls] + __popc(peers & ((1u << lane) - 1u)) * parts;
       for (int t = 0; t < parts; ++t, ++rank) {
-        if (rank >= plan.n_units) break;               // (never: the host counts units by the same rule)
+        if (rank >= n_units) break;               // (never: the host counts units by the same rule)
         const uint32_t mask = parts == 4 ? (1u << t) : (parts == 2 ? (t ? 12u : 3u) : 15u);
-        const int r = rank / nw, d = p.dealt ? hand_of[rank] : rank - r * nw;
-        const int k = d * plan.stride_inv % nw;
-        const int m = full + static_cast<int>(s_key[d]);
+        const uint32_t to = p.dealt ? hand_of[rank] : 0u;
+        const int r = p.dealt ? static_cast<int>(to >> kUnitHandBits) : rank / nw;
+        const int d = p.dealt ? static_cast<int>(to & ((1u << kUnitHandBits) - 1u)) : rank - r * nw;
+        const int k = static_cast<int>(static_cast<long long>(d) * plan.stride_inv % nw);
+        const int m = static_cast<int>(s_cnt[d]);
         // the unit's number in its list from the narrowest level on (2-bit blocks are dealt before 4-bit ones)
         const int z = m - 1 - (cls == 2 ? r + static_cast<int>(s_mix[d] >> 16) : (cls == 3 ? r - static_cast<int>(s_mix[d] & 0xffffu) : r));
         const int place = z < (m + 1) / 2 ? 2 * z : 2 * (m - 1 - z) + 1;
-        p.units[plan.unit_base + k * plan.pitch + (place + m - (k * 5) % m) % m] = word | (mask << 20);
+        p.units[s_key[d] + (place + m - (k * 5) % m) % m] = word | (mask << 20);
       }
     }
     __syncthreads();
@@ -210,9 +250,8 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
   // reader of a block finds it in L2; one partial row per (CTA, head group)
   auto describe = [&](int k, int hg, int partial) {
     const int d = static_cast<int>(static_cast<long long>(k) * plan.stride % nw);
-    const int m = full + static_cast<int>(s_key[d]);
-    const int begin = plan.unit_base + k * plan.pitch;
-    return WarpDesc{hg, begin, begin + m, partial};
+    const int begin = static_cast<int>(s_key[d]);
+    return WarpDesc{hg, begin, begin + static_cast<int>(s_cnt[d]), partial};
   };
   if (p.cluster > 0) {
     // CTAs of the head group's own, its warps dealt round by round to them
@@ -234,16 +273,14 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
 }  // namespace
 
 cudaError_t launch_units(UnitsParams p, int n_streams, int max_units, cudaStream_t st) {
-  // the ranks' warps in shared memory; a context of more than kUnitsDealt units per stream (six million tokens) is dealt
+  // the ranks' warps in shared memory; a context of more than kUnitsDealt units per stream (2.8 million tokens) is dealt
   // round by round without a look at what a warp has
-  constexpr int kUnitsDealt = 98304;
+  constexpr int kUnitsDealt = 45056;
   p.dealt = max_units <= kUnitsDealt;
-  const size_t bytes = static_cast<size_t>(p.pad) * 2 * sizeof(uint32_t) + (p.dealt ? static_cast<size_t>(max_units) * sizeof(uint16_t) : 0);
-  static size_t configured = 0;
-  if (bytes > 40 * 1024 && bytes > configured) {
+  const size_t bytes = (static_cast<size_t>(p.pad) * 3 + (p.dealt ? static_cast<size_t>(max_units) : 0)) * sizeof(uint32_t);
+  if (bytes > 40 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(units_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
     if (e != cudaSuccess) return e;
-    configured = bytes;
   }
   units_kernel<<<n_streams, kUnitThreads, bytes, st>>>(p);
   return cudaGetLastError();
