@@ -991,12 +991,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   if (lane == 0) {
     s_group[warp] = hgroup;
     s_group[kDecodeWarps + warp] = partial_row;
-    if constexpr (!SPARSE) {
-      const StreamParts sp = hgroup >= 0 ? p.parts[hgroup] : StreamParts{0, 0};
-      s_group[2 * kDecodeWarps + warp] = sp.begin;
-      s_group[3 * kDecodeWarps + warp] = sp.end;
-    }
   }
+  StreamParts parts{0, 0};
   uint8_t* sbase = smem + warp * (kStages * kStageBytes);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kDecodeWarps * kStages * kStageBytes) + warp * kStages;
   uint8_t* qb_smem = smem + kDecodeWarps * (kStages * kStageBytes + kStages * 8) + warp * 2048;
@@ -1020,6 +1016,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
     // prefetched pair.
     if constexpr (!SPARSE) {
       if (first < w.item_end) w.pf_unit = w.units[first];
+      if (lane == 0) parts = p.parts[hgroup];          // (stored below: nothing waits for it before the wait)
     }
   }
   // Launched with programmatic stream serialisation: what is above touches nothing that a previous kernel may
@@ -1036,6 +1033,12 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
     }
   }
   fetch_query(w);
+  if constexpr (!SPARSE) {
+    if (lane == 0) {
+      s_group[2 * kDecodeWarps + warp] = parts.begin;
+      s_group[3 * kDecodeWarps + warp] = parts.end;
+    }
+  }
 
   SoftmaxState st;
   st.m = kNegInf;
