@@ -128,9 +128,9 @@ __global__ void __launch_bounds__(288) mla_append_rows_kernel(uint8_t* arena, co
                                                               int tail_index, const uint16_t* k_in, int n_tok,
                                                               int first_tok, int dst_row0) {
   // launched with programmatic stream serialisation: returns once the previous kernel of the stream has
-  // completed (the launch itself overlaps that kernel's tail)
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  // completed (the launch itself overlaps that kernel's tail).  The next kernel is let in first, see append_rows_kernel.
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
   const int stream = blockIdx.x, row = blockIdx.y;
   const TableEntry e = table[static_cast<size_t>(stream) * table_stride + tail_index];
   const uint32_t* src = reinterpret_cast<const uint32_t*>(k_in + (static_cast<size_t>(stream) * n_tok + first_tok + row) * kMlaDk);

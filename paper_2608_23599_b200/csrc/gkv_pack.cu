@@ -436,9 +436,12 @@ __global__ void __launch_bounds__(128) append_rows_kernel(uint8_t* arena, const 
   uint32_t* dst = reinterpret_cast<uint32_t*>(slot + (is_v ? kBlock * kRowBytes : 0) +
                                               static_cast<size_t>(dst_row0 + row) * kRowBytes);
   // launched with programmatic stream serialisation: the address set-up above overlaps the tail
-  // of the previous kernel; the new rows are read, and the slot written, only after it completed
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  // of the previous kernel; the new rows are read, and the slot written, only after it completed.  The next kernel is let
+  // in before that: the read of the layer takes its SMs as the previous layer's read leaves them, and what it does
+  // before its own wait (which ends when this kernel has, and so the one before) reads nothing that either writes.  (A step of
+  // 36 layers over one sequence of 16,379 tokens 0.576 -> 0.526 ms, of 4 layers over 64 streams 0.288 -> 0.286.)
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
   dst[i] = src[i];
 }
 
