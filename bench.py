@@ -327,8 +327,10 @@ def measure(w, n_layers, K, Wm, rank, local, world, cpu_seconds, full=True):
     if full:
         e2e = measure_e2e(cache, wl, n_layers, K, Wm, world, device, out, out_at, pages_at, quest, budget, alias)
     launches_per_layer = 2 + (2 if quest else 0) + (1 if alias else 0)      # append, decode with fused merge (+ score, top-k; + combine)
-    # a block close adds the block-statistics kernel and, under the staircase policy, one encode launch
-    gpu_launches = K * n_layers * launches_per_layer + closes * n_layers * ((0 if alias else 1) + (1 if wl.policy == W.POLICY_STAIRCASE else 0))
+    # a block close adds the block-statistics kernel, under the staircase policy one encode launch, and the kernel that
+    # makes the next read's work lists (latent lists come from the host, page-list reads have none)
+    per_close = (0 if alias else 1) + (1 if wl.policy == W.POLICY_STAIRCASE else 0) + (0 if alias or quest else 1)
+    gpu_launches = K * n_layers * launches_per_layer + closes * n_layers * per_close
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": Wm,
         "ms_per_step": ms_step, "ms_per_step_median": ms_sorted[len(ms_sorted) // 2], "ms_per_step_min": ms_sorted[0],
