@@ -42,7 +42,10 @@ struct PlanShared {
   uint32_t bits[kPlanThreads / 32];
   int lo[kPlanLists], hi[kPlanLists];        // candidates below lo are too small, from hi on they fit
   int pick;                                  // list that is bisected, -1 = done
-  double tau;
+  double tau;                                // value tried
+  // the result (fields of its own: a warp may still be on its way out of the search, reading `pick`, when they are written)
+  int found;
+  double best;
   int eligible;
 };
 
@@ -195,12 +198,12 @@ __global__ void __launch_bounds__(kPlanThreads) rd_plan_kernel(const RdPlanParam
         found = true;
         best = fmin(best, cand(l, sh.hi[l]));
       }
-    sh.pick = found ? 0 : -1;
-    sh.tau = found ? best : fmax(list0[n - 1], 0.0);                 // no plan fits: the largest candidate's
+    sh.found = found;
+    sh.best = found ? best : fmax(list0[n - 1], 0.0);                // no plan fits: the largest candidate's
   }
   __syncthreads();
-  const bool miss = sh.pick < 0;
-  plan_for_tau(p, y, table, n, per, sh.tau, lv, sh);
+  const bool miss = !sh.found;
+  plan_for_tau(p, y, table, n, per, sh.best, lv, sh);
   __syncthreads();
   int8_t* out = p.levels_out + static_cast<size_t>(s) * p.out_stride;
   int eligible = 0;
