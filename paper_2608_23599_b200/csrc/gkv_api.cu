@@ -686,9 +686,6 @@ int wait_event(gkv_cache* c, cudaEvent_t ev) {
   return GKV_OK;
 }
 
-// Largest number of closed blocks whose breakpoints the device allocator sorts in shared memory.
-constexpr int kRdPlanMaxBlocks = 4095;
-
 // Queues the device allocator for every stream of a layer (running masses L.ema_d, range proxies L.range_d): levels into
 // c->levels_d, a flag into c->plan_flag_d when some stream cannot meet the budget.  n <= kRdPlanMaxBlocks.
 int rd_plan_launch(gkv_cache* c, LayerState& L, int n, int n_tail, bool use_prev, int n_res, int32_t* res_count, cudaStream_t st) {

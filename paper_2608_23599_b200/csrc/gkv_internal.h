@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "gkv_layout.cuh"
 
 namespace gkv {
@@ -184,6 +186,21 @@ struct StatsParams {
   int32_t err_stride;
 };
 
+// Raises a kernel's limit of dynamic shared memory on the current device, once per device (`done`: a bit each).  The limit
+// belongs to the kernel and not to a launch: set to what one launch needs, it can fall below what another thread is about to
+// launch with, so `bytes` is the most that any launch of the kernel asks for.
+template <typename... Args>
+cudaError_t raise_smem_limit(void (*kernel)(Args...), size_t bytes, std::atomic<uint64_t>& done) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev < 64 ? uint64_t{1} << dev : 0;
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
+
 constexpr uint32_t kStatusRange = 1u;      // a scale or zero saturated
 constexpr uint32_t kStatusInternal = 2u;   // an index check failed inside a kernel
 
@@ -213,6 +230,7 @@ struct RdPlanParams {
   int32_t* res_count;           // [n_streams]
   int32_t n_res, res_cap;
 };
+constexpr int kRdPlanMaxBlocks = 4095;      // closed blocks per stream that the device allocator takes (it sorts them in shared memory)
 size_t rd_plan_smem_bytes(int n, int* pad_out);
 cudaError_t launch_rd_plan(const RdPlanParams& p, int n_streams, cudaStream_t st);
 cudaError_t launch_append_rows(uint8_t* arena, const TableEntry* table, int table_stride, int tail_index,

@@ -231,11 +231,10 @@ size_t rd_plan_smem_bytes(int n, int* pad_out) {
 
 cudaError_t launch_rd_plan(const RdPlanParams& p, int n_streams, cudaStream_t st) {
   const size_t bytes = rd_plan_smem_bytes(p.n, nullptr);
-  static size_t configured = 0;
-  if (bytes > 48 * 1024 && bytes > configured) {
-    cudaError_t e = cudaFuncSetAttribute(rd_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+  if (bytes > 48 * 1024) {
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = raise_smem_limit(rd_plan_kernel, rd_plan_smem_bytes(kRdPlanMaxBlocks, nullptr), done);
     if (e != cudaSuccess) return e;
-    configured = bytes;
   }
   // a block per thread, as far as there are threads
   const int threads = p.pad < 32 ? 32 : (p.pad < kPlanThreads ? p.pad : kPlanThreads);

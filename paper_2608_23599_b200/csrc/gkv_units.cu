@@ -276,10 +276,12 @@ cudaError_t launch_units(UnitsParams p, int n_streams, int max_units, cudaStream
   // the ranks' warps in shared memory; a context of more than kUnitsDealt units per stream (2.8 million tokens) is dealt
   // round by round without a look at what a warp has
   constexpr int kUnitsDealt = 45056;
+  constexpr size_t kMost = (static_cast<size_t>(3) << kUnitHandBits) * sizeof(uint32_t) + kUnitsDealt * sizeof(uint32_t);      // 224 KB
   p.dealt = max_units <= kUnitsDealt;
   const size_t bytes = (static_cast<size_t>(p.pad) * 3 + (p.dealt ? static_cast<size_t>(max_units) : 0)) * sizeof(uint32_t);
   if (bytes > 40 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(units_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = raise_smem_limit(units_kernel, kMost, done);
     if (e != cudaSuccess) return e;
   }
   units_kernel<<<n_streams, kUnitThreads, bytes, st>>>(p);

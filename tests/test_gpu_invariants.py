@@ -1,6 +1,8 @@
 """What has to hold whatever the timing, the order of the calls and the number of threads: plans that do not depend on when
 a warp arrives, caches that do not disturb one another, state that a refused call leaves as it was, and work lists that hold
 every item once and are balanced."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -44,3 +46,87 @@ def test_device_plans_do_not_depend_on_timing(n_closed, monotone):
         prev = g.gkv_debug_export_levels(0, b, h).astype(np.int8)
         want, _ = B.gkv_debug_replan_levels(g.cfg, 9, ms[b, h], rg[b, h], prev)
         assert np.array_equal(first[b, h], want), (b, h)
+
+
+# ---- threads ---------------------------------------------------------------------------------------------
+def _in_two_threads(work):
+    """work(side, meet) for side 0 and 1, each in a thread with a stream of its own; meet() lets the two go on together."""
+    errors, barrier = [], threading.Barrier(2, timeout=60)
+
+    def body(side):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                work(side, barrier.wait)
+                torch.cuda.current_stream().synchronize()
+        except Exception as e:      # noqa: BLE001
+            errors.append((side, e))
+            barrier.abort()
+
+    threads = [threading.Thread(target=body, args=(side,)) for side in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+
+
+def test_lists_of_two_long_contexts_made_by_two_threads():
+    """Contexts whose work lists need more shared memory than a kernel has without asking, a different amount each: the
+    lists are remade again and again (a block closes), and every read equals the one of a cache worked on alone."""
+    B = _binding()
+    sizes, rounds = (140_000, 300_000), 40
+
+    def decode(side, outs, meet=lambda: None):
+        w = _gqa(sizes[side], room=64 * (rounds + 1), stair_tokens=(64, 64, 64, -1))
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(side)
+        k = torch.randn((1, w.ctx, 1, 128), generator=gen, device="cuda").to(torch.bfloat16)
+        q = torch.randn((1, 1, 128), generator=gen, device="cuda").to(torch.bfloat16)
+        cache = B.Cache(B.config_from_workload(w))
+        cache.gkv_append_demote(0, k, k)
+        row = k[:, :1].contiguous()
+        for r in range(rounds):
+            for _ in range(64):
+                cache.gkv_append_demote(0, row, row)
+            out = torch.empty((1, 1, 128), dtype=torch.float32, device="cuda")
+            meet()
+            cache.gkv_decode_attn(0, q, out)
+            outs[side].append(out)
+        torch.cuda.current_stream().synchronize()
+        cache.close()
+
+    alone, both = ([], []), ([], [])
+    for side in range(2):
+        decode(side, alone)
+    _in_two_threads(lambda side, meet: decode(side, both, meet))
+    for side in range(2):
+        assert len(both[side]) == rounds
+        for r in range(rounds):
+            assert torch.equal(alone[side][r], both[side][r]), (side, r)
+
+
+def test_plans_of_two_sizes_made_by_two_threads():
+    """Allocations whose breakpoints need more shared memory than a kernel has without asking, a different amount each."""
+    B = _binding()
+    sizes = (1700, 4095)
+
+    def plans(side, out, meet=lambda: None):
+        w = _gqa(64 * sizes[side] + 5, policy=W.POLICY_RD, rd_budget_bpv=4.0, retire_after=64)
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(side)
+        k = torch.randn((1, w.ctx, 1, 128), generator=gen, device="cuda").to(torch.bfloat16)
+        mass = torch.softmax(3 * torch.randn((1, 1, w.ctx), generator=gen, device="cuda"), -1)
+        cache = B.Cache(B.config_from_workload(w))
+        cache.gkv_append_demote(0, k, k, token_mass=mass)
+        out[side] = []
+        for _ in range(40):
+            meet()
+            out[side].append(cache.gkv_debug_device_plan(0)[0])
+        cache.close()
+
+    alone, both = [None, None], [None, None]
+    for side in range(2):
+        plans(side, alone)
+    _in_two_threads(lambda side, meet: plans(side, both, meet))
+    for side in range(2):
+        assert all(np.array_equal(p, alone[side][0]) for p in both[side])
