@@ -121,7 +121,8 @@ GKV_API int gkv_destroy(gkv_cache* c);
  *   level_plan  HOST int8 [batch][n_kv_heads][n_new/64], values in {16,8,4,2,1};
  *          required for GKV_POLICY_EXTERNAL at bulk ingest, else NULL
  * Bulk ingest under GKV_POLICY_RD (and residual selection) synchronises the stream once, to
- * run the allocator (Sec. 3.3) on the host.  Decode-step appends never synchronise.
+ * read the level plan back.  Decode-step appends never synchronise.
+ * GKV_ERR_ARENA_TOO_SMALL leaves the layer as it was (a bulk ingest: empty), with no slot taken.
  * May return GKV_ERR_RANGE / GKV_ERR_BUDGET as warnings after completing the work. */
 GKV_API int gkv_append_demote(gkv_cache* c, int32_t layer, const void* k_new, const void* v_new, int32_t n_new,
                       const float* token_mass, const int8_t* level_plan, void* stream);

@@ -753,11 +753,26 @@ int rd_plan_layer(gkv_cache* c, LayerState& L, int8_t* target, bool* missed, cud
   return GKV_OK;
 }
 
+// A bulk ingest that finds no room leaves the layer as it was, empty: the slots taken so far go back, and what the device
+// already holds of it (numbers of residual rows, running masses) is cleared behind the launches under way, which write
+// nothing else that a later call would read.
+int refuse_ingest(gkv_cache* c, LayerState& L, SlotHeap& before, bool budget_flag, cudaStream_t st) {
+  const size_t ns = c->n_streams;
+  std::swap(c->heap, before);
+  L.budget_flag = budget_flag;
+  std::fill(L.level.begin(), L.level.end(), 0);
+  std::memset(L.res_count_h, 0, ns * sizeof(int32_t));
+  CK(c, cudaMemsetAsync(L.res_count_d, 0, ns * sizeof(int32_t), st));
+  if (!is_mla(c->cfg)) CK(c, cudaMemsetAsync(L.ema_d, 0, ns * (c->max_blocks + 1) * sizeof(float), st));
+  return GKV_ERR_ARENA_TOO_SMALL;
+}
+
 int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* v_new, int n_new,
                 const float* token_mass, const int8_t* level_plan, cudaStream_t st) {
   const gkv_config& cfg = c->cfg;
   LayerState& L = c->layers[layer];
   const int ns = c->n_streams, n_closed = n_new / kBlock, n_tail = n_new % kBlock;
+  const bool budget_before = L.budget_flag;
   int warn = GKV_OK;
   int rc;
   if ((rc = wait_event(c, L.ev)) != GKV_OK) return rc;
@@ -849,12 +864,13 @@ int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* 
   // host allocates the next group's slots while the GPU encodes this one.
   const bool fast = n_closed > 0 && v_new &&
                     ((reinterpret_cast<uintptr_t>(k_new) | reinterpret_cast<uintptr_t>(v_new)) & 15u) == 0;
+  SlotHeap heap_before = c->heap;
   auto alloc_streams = [&](int s0, int s1) -> int {
     for (int s = s0; s < s1; ++s) {
       for (int b = 0; b <= n_closed; ++b) {
         const int lvl = b < n_closed ? L.level[static_cast<size_t>(s) * c->max_blocks + b] : 16;
         uint32_t off;
-        if (!c->heap.alloc(lvl, &off)) return GKV_ERR_ARENA_TOO_SMALL;
+        if (!c->heap.alloc(lvl, &off)) return refuse_ingest(c, L, heap_before, budget_before, st);
         set_entry(c, L, s, b, off, lvl);
         L.table_h[static_cast<size_t>(s) * c->table_stride + b].resmask = 0;
       }
@@ -1230,11 +1246,12 @@ int mla_bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, int n_new, c
         L.level[static_cast<size_t>(s) * c->max_blocks + b] = v;
       }
   }
+  SlotHeap heap_before = c->heap;
   for (int s = 0; s < ns; ++s) {
     for (int b = 0; b <= n_closed; ++b) {
       const int lvl = b < n_closed ? L.level[static_cast<size_t>(s) * c->max_blocks + b] : 16;
       uint32_t off;
-      if (!c->heap.alloc(lvl, &off)) return GKV_ERR_ARENA_TOO_SMALL;
+      if (!c->heap.alloc(lvl, &off)) return refuse_ingest(c, L, heap_before, L.budget_flag, st);
       set_entry(c, L, s, b, off, lvl);
       L.table_h[static_cast<size_t>(s) * c->table_stride + b].resmask = 0;
     }

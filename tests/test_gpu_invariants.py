@@ -130,3 +130,74 @@ def test_plans_of_two_sizes_made_by_two_threads():
     _in_two_threads(lambda side, meet: plans(side, both, meet))
     for side in range(2):
         assert all(np.array_equal(p, alone[side][0]) for p in both[side])
+
+
+# ---- a refused ingest ---------------------------------------------------------------------------------------
+def _smallest_arena(B, cfg):
+    """Fewest bytes that a cache of this configuration is made in: its metadata and one exact block."""
+    lo, hi = 4096, B.gkv_query_arena_bytes(cfg)
+    while hi - lo > 256:
+        mid = (lo + hi) // 2
+        try:
+            B.Cache(cfg, arena_bytes=mid).close()
+            hi = mid
+        except B.GkvError:
+            lo = mid
+    return hi
+
+
+@pytest.mark.parametrize("policy", ["rd", "staircase", "latent"])
+def test_refused_ingest_leaves_the_layer_empty(policy):
+    """A prompt that the arena has no room for, first; then the same calls as on a cache that never saw it: single tokens
+    (an observing read and, where there are pages, a read by list: both look at residual rows), or a prompt that fits."""
+    B = _binding()
+    latent = policy == "latent"
+    if latent:
+        w = W.Workload("refused", 71, 1, 2, 16, 1, 576, 512, 2000, 2200, v_aliases_k=1, stair_tokens=(64, 64, -1, 0), n_heavy=0,
+                       softmax_scale=0.07)
+    else:
+        w = _gqa(2000, 2, 2, 4, room=200, page_tokens=64, residual_fraction=0.1,
+                 **(dict(policy=W.POLICY_RD, rd_budget_bpv=5.0, retire_after=64) if policy == "rd" else dict(stair_tokens=(64, 64, 64, -1))))
+    cfg = B.config_from_workload(w)
+    small = _smallest_arena(B, cfg) + (14 * 73728 if latent else 20 * 32768)
+    assert small < B.gkv_query_arena_bytes(cfg)
+    data = W.make_layer(w, 0, "cuda")
+    mass = None if latent else torch.softmax(3 * torch.randn((2, 2, 2000), device="cuda"), -1)
+
+    def ingest(cache, n):
+        return cache.gkv_append_demote(0, data["k"][:, :n].contiguous(), None if latent else data["v"][:, :n].contiguous(),
+                                       token_mass=None if latent else mass[:, :, :n].contiguous())
+
+    def reads(cache, first, n):
+        got = []
+        for t in range(first, first + n):
+            cache.gkv_append_demote(0, data["k"][:, t:t + 1].contiguous(), None if latent else data["v"][:, t:t + 1].contiguous())
+            out = torch.empty((2, w.n_q_heads, w.d_v), device="cuda")
+            cache.gkv_decode_attn(0, data["q"], out)
+            got.append(out)
+            if latent or t % 9:
+                continue
+            out, m = torch.empty_like(out), torch.empty((2, 2, -(-(t + 1) // 64)), device="cuda")
+            cache.gkv_decode_attn_observe(0, data["q"], out, None, m)
+            got += [out, m, torch.from_numpy(cache.gkv_debug_export_mass(0))]
+            n_pages = (t + 1) // 64
+            pages = torch.arange(n_pages, dtype=torch.int32, device="cuda").expand(2, 2, -1).contiguous()
+            out = torch.empty_like(out)
+            cache.gkv_decode_attn(0, data["q"], out, page_idx=pages, n_sel=n_pages)
+            got.append(out)
+        torch.cuda.synchronize()
+        bits = cache.gkv_bits_report(0)
+        return got, (bits.values, bits.resident_bits, bits.residual_bits, cache.last_report_status)
+
+    fits = 300
+    for calls in (lambda c: reads(c, 0, 150), lambda c: (ingest(c, fits), reads(c, fits, 40))[1]):
+        fresh, used = B.Cache(cfg), B.Cache(cfg, arena_bytes=small)
+        for _ in range(2):                         # (what the first refusal took has come back)
+            with pytest.raises(B.GkvError) as e:
+                ingest(used, 2000)
+            assert e.value.status == B.ERR_ARENA_TOO_SMALL
+        assert used.gkv_ctx_len(0) == 0
+        (a, bits_a), (b, bits_b) = calls(fresh), calls(used)
+        assert bits_a == bits_b
+        for i, (x, y) in enumerate(zip(a, b)):
+            assert torch.equal(x, y), i
