@@ -69,6 +69,11 @@ constexpr int kMOutPitch = kMlaDv + 2;                 // floats per head row of
 constexpr int kMWaitSpins = 1 << 22;
 constexpr float kMNegInf = -INFINITY;
 constexpr float kMSlack = 8.f;                         // keep a stale running max while logits stay within 2^8 of it
+// What the softmax reference lies above the maximum it is taken from (log2).  The value MMAs truncate their sums at a distance
+// below the exponent of the largest product, so a probability of exactly 1 costs all others of its unit a bit that 0.9986
+// does not: error against 64 bits of 16,384 tokens of 2 sequences 3.8e-5 -> 2.3e-5, of 4-bit blocks alone 5.3e-5 -> 3.5e-5.
+// (Ranges that are cut inside blocks have more first units, those with the 1: 3.6e-5 -> 3.8e-5 without this.)
+constexpr float kMAbove = 1.f / 512.f;
 constexpr uint32_t kMFull = 0xffffffffu;
 static_assert(kMStageBytes >= 16 * kMRowPitch, "a stage holds 16 staged rows");
 static_assert(kMStages * kMStageBytes >= kMlaHeads * kMOutPitch * 4 + 128, "a quad's result fits its stages");
@@ -338,8 +343,8 @@ __device__ __forceinline__ void m_issue(const MlaDecodeParams& p, const MWalk& w
 // ---- softmax -------------------------------------------------------------------------------------
 // The four warps' partial logits -> this lane's share of the unit's probabilities.  A lane holds, for
 // the heads g and g + 8, the tokens 16 ks + 8 j + 2 c4 + e: the B-fragment layout of the value MMAs.
-// The running maximum may stay stale by up to kMSlack (then nothing is rescaled); when it moves, the
-// running sums and O^T are rescaled.  Outputs: the probabilities as a pair hi + lo (fp16 or bf16) and
+// m_run, a little above a running maximum, may stay stale by up to kMSlack (then nothing is rescaled); when it
+// moves, the running sums and O^T are rescaled.  Outputs: the probabilities as a pair hi + lo (fp16 or bf16) and
 // the unit's probability sums of the heads 2 c4 + e (+ 8 hg), the columns of the lane's O^T registers.
 template <int NKS, bool BF16>
 __device__ __forceinline__ void m_softmax(uint32_t xb, int lane, float scale_log2, float bias, int nvalid, uint32_t ot,
@@ -381,7 +386,7 @@ __device__ __forceinline__ void m_softmax(uint32_t xb, int lane, float scale_log
     float al[2];
 #pragma unroll
     for (int hg = 0; hg < 2; ++hg) {
-      const float mn = fmaxf(m_run[hg], mloc[hg]);
+      const float mn = mloc[hg] > m_run[hg] ? mloc[hg] + kMAbove : m_run[hg];
       al[hg] = (m_run[hg] == kMNegInf) ? 0.f : m_ex2(m_run[hg] - mn);
       m_run[hg] = mn;
       l_run[hg] *= al[hg];
