@@ -122,7 +122,8 @@ GKV_API int gkv_destroy(gkv_cache* c);
  *          required for GKV_POLICY_EXTERNAL at bulk ingest, else NULL
  * Bulk ingest under GKV_POLICY_RD (and residual selection) synchronises the stream once, to
  * read the level plan back.  Decode-step appends never synchronise.
- * GKV_ERR_ARENA_TOO_SMALL leaves the layer as it was (a bulk ingest: empty), with no slot taken.
+ * GKV_ERR_ARENA_TOO_SMALL: a bulk ingest leaves the layer empty; an append leaves it as it was or, when the room is missing
+ * for the demotions of a block that has just closed, with the token taken and every level as before.
  * May return GKV_ERR_RANGE / GKV_ERR_BUDGET as warnings after completing the work. */
 GKV_API int gkv_append_demote(gkv_cache* c, int32_t layer, const void* k_new, const void* v_new, int32_t n_new,
                       const float* token_mass, const int8_t* level_plan, void* stream);
@@ -266,6 +267,12 @@ GKV_API int gkv_debug_export_residual(gkv_cache* c, int32_t layer, int32_t b, in
 /* Levels of all closed blocks of one stream.  levels: host int8 [cap]; n: host. */
 GKV_API int gkv_debug_export_levels(gkv_cache* c, int32_t layer, int32_t b, int32_t kv_head, int8_t* levels,
                             int32_t cap, int32_t* n);
+/* Work lists of the last full read of `layer` (grouped-query layout; GKV_ERR_BAD_STATE when levels have changed since and the
+ * next read makes new ones).  units: host int32 [cap][6], one row per unit of every warp: the warp's place in the launch, its head group
+ * (stream * groups of up to four query heads + group), the unit's first item (closed blocks in order, then the partial block, then
+ * the groups of 16 residual rows), its mask of 16-token tiles (15 = the whole block), the number of centroid blocks in its
+ * run (1 for other units) and the cost that it is balanced by.  n: rows there are (GKV_ERR_INVALID_ARG above cap). */
+GKV_API int gkv_debug_export_units(gkv_cache* c, int32_t layer, int32_t* units, int32_t cap, int32_t* n);
 /* The host-side level plan on its own, without a cache or a device (all pointers host): what
  * gkv_append_demote decides for one stream whose n_closed blocks are closed and whose tail holds
  * n_tail tokens.  Staircase policy (Sec. 3.2, Fig. 1): from cfg->stair_tokens / n_sink_blocks;

@@ -28,7 +28,7 @@ EXPORTS = [
     "gkv_decode_attn_observe", "gkv_debug_export_mass", "gkv_debug_export_bounds", "gkv_rd_reallocate", "gkv_debug_device_plan",
     "gkv_debug_replan_levels",
     "gkv_quest_select", "gkv_quest_select_static", "gkv_debug_export_boxes", "gkv_debug_export_scores", "gkv_bits_report",
-    "gkv_debug_export_block", "gkv_debug_export_residual",
+    "gkv_debug_export_block", "gkv_debug_export_residual", "gkv_debug_export_units",
     "gkv_debug_export_levels", "gkv_debug_plan_levels", "gkv_ctx_len", "gkv_strerror", "gkv_last_cuda_error",
 ]
 
@@ -97,6 +97,7 @@ def load():
     lib.gkv_bits_report.argtypes = [vp, i32, C.POINTER(GkvBits)]
     lib.gkv_debug_export_block.argtypes = [vp, i32, i32, i32, i32, i32, C.POINTER(i32), vp, vp, vp, vp, C.POINTER(i32)]
     lib.gkv_debug_export_residual.argtypes = [vp, i32, i32, i32, vp, i32, C.POINTER(i32)]
+    lib.gkv_debug_export_units.argtypes = [vp, i32, vp, i32, C.POINTER(i32)]
     lib.gkv_debug_export_levels.argtypes = [vp, i32, i32, i32, vp, i32, C.POINTER(i32)]
     lib.gkv_debug_plan_levels.argtypes = [C.POINTER(GkvConfig), i32, i32, C.POINTER(C.c_float), C.POINTER(C.c_float),
                                           C.POINTER(C.c_int8), C.POINTER(i32)]
@@ -344,6 +345,14 @@ class Cache:
         _check(load().gkv_debug_export_residual(self.handle, layer, b, kv_head, idx.ctypes.data, cap, C.byref(n)),
                "gkv_debug_export_residual")
         return idx[: n.value]
+
+    def gkv_debug_export_units(self, layer):
+        """Work lists of the last full read: int32 [n][6] of (warp, head group, first item, tile mask, run, cost)."""
+        n = C.c_int32(0)
+        _check(load().gkv_debug_export_units(self.handle, layer, None, 0, C.byref(n)), "gkv_debug_export_units", allow=(ERR_INVALID_ARG,))
+        out = np.zeros((n.value, 6), dtype=np.int32)
+        _check(load().gkv_debug_export_units(self.handle, layer, out.ctypes.data, n.value, C.byref(n)), "gkv_debug_export_units")
+        return out
 
     def gkv_debug_export_block(self, layer, b, kv_head, block, which):
         """Returns dict(level, codes u8 [64][d], scale/zero uint16 fp16 bits, rows uint16 bf16 bits, n_rows)."""

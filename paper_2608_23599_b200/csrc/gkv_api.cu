@@ -288,9 +288,9 @@ Derived derive(const gkv_config& c) {
   d.res_cap = c.residual_fraction > 0.f
                   ? static_cast<int>(align_up(static_cast<size_t>(std::floor(static_cast<double>(c.residual_fraction) * c.max_ctx)) + 16, 16))
                   : 0;
-  // units of a layer: every item, up to three more for the items that small workloads cut (fewer than
-  // kTargetWarps items in all; a single stream's exact blocks only below half of that), and a list's unused place
-  // per warp
+  // units of a layer: every item, and in small workloads the parts of those that are cut: three more per exact block
+  // (fewer than kTargetWarps / 2 items in all), else one more per quantised block and three per partial block (fewer than
+  // kTargetWarps items; a single stream has one partial block, several have at most that many)
   d.units_cap = static_cast<size_t>(d.n_streams) * (d.max_blocks + 1 + d.res_cap / 16) + static_cast<size_t>(std::min(d.n_streams, 2)) * 3 * (kTargetWarps / 2) + d.max_warps;
   d.box_stride = c.page_tokens > 0 ? static_cast<int>(align_up((c.max_ctx + c.page_tokens - 1) / c.page_tokens, 8)) : 0;
   return d;
@@ -639,6 +639,16 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   L.desc_dirty = false;
 }
 
+// Cost of a unit of the layer's lists, by class.
+void unit_costs(const LayerState& L, size_t (&cost)[kUnitClasses]) {
+  const size_t parts = L.split_all ? 2 : 1;
+  const size_t head[6] = {kCost16 / (L.split ? 4 : 1), kCost8 / parts, kCost2 / parts, kCost4 / parts, kCostTail / (L.split_all ? 4 : 1), kCostRes};
+  for (size_t i = 0; i < kUnitClasses; ++i) cost[i] = i < 6 ? head[i] : kCost1 * (22 - i);
+}
+// (no cost lies between a 2-bit block's and a 4-bit one's, whole or half, so the two classes are neighbours in any order)
+static_assert(kCost2 > kCost4 && kCost2 - kCost4 < kCost1 && kCost4 / kCost1 == kCost2 / kCost1 && kCost4 / 2 / kCost1 == kCost2 / 2 / kCost1,
+              "a run of centroid blocks would come between the 2-bit and the 4-bit blocks");
+
 // Work lists of a layer on their way: the host's plan up, the lists behind it.
 int make_units(gkv_cache* c, LayerState& L, bool allow_split, cudaStream_t st) {
   // the plans have their own event: waiting for the table's would wait for copies that
@@ -661,9 +671,18 @@ int make_units(gkv_cache* c, LayerState& L, bool allow_split, cudaStream_t st) {
   p.split = L.split;
   p.split_all = L.split_all;
   p.cluster = L.cluster;
-  const size_t head[6] = {kCost16 / (L.split ? 4 : 1), kCost8 / (L.split_all ? 2 : 1), kCost2 / (L.split_all ? 2 : 1),
-                          kCost4 / (L.split_all ? 2 : 1), kCostTail / (L.split_all ? 4 : 1), kCostRes};
-  for (int i = 0; i < kUnitClasses; ++i) p.cost[i] = static_cast<int32_t>(i < 6 ? head[i] : kCost1 * (22 - i));
+  // Splitting changes which class is the costliest (a quarter of an exact block 397, half an 8-bit one 535, a residual group 550,
+  // a run of 16 centroid blocks 752), so the order is made here.  In a fixed order (whole blocks first) the fullest warp of a list had up
+  // to 1.58 times what it has with the units dealt one by one, longest first, to the least laden warp; now at most 1.01 times.
+  size_t cost[kUnitClasses];
+  int order[kUnitClasses];
+  unit_costs(L, cost);
+  std::iota(order, order + kUnitClasses, 0);
+  std::stable_sort(order, order + kUnitClasses, [&](int a, int b) { return cost[a] > cost[b]; });
+  for (int i = 0; i < kUnitClasses; ++i) {
+    p.place[order[i]] = i;
+    p.cost[i] = static_cast<int32_t>(cost[order[i]]);
+  }
   int max_units = 0, max_nw = 1;
   for (int s = 0; s < c->n_streams; ++s) {
     max_units = std::max(max_units, L.plans_h[s].n_units);
@@ -2066,6 +2085,38 @@ int gkv_debug_export_levels(gkv_cache* c, int32_t layer, int32_t b, int32_t kv_h
   *n = L.n_closed;
   for (int i = 0; i < std::min(cap, L.n_closed); ++i) levels[i] = L.level[static_cast<size_t>(s) * c->max_blocks + i];
   return GKV_OK;
+}
+
+int gkv_debug_export_units(gkv_cache* c, int32_t layer, int32_t* units, int32_t cap, int32_t* n) {
+  if (!c || layer < 0 || layer >= c->cfg.n_layers || !n || cap < 0 || (cap > 0 && !units)) return GKV_ERR_INVALID_ARG;
+  if (is_mla(c->cfg)) return GKV_ERR_UNSUPPORTED;
+  const LayerState& L = c->layers[layer];
+  if (L.desc_dirty) return GKV_ERR_BAD_STATE;
+  CK(c, cudaDeviceSynchronize());
+  std::vector<WarpDesc> warps(static_cast<size_t>(L.n_warps));
+  std::vector<uint32_t> words(static_cast<size_t>(L.n_units));
+  CK(c, cudaMemcpy(warps.data(), L.warps_d, warps.size() * sizeof(WarpDesc), cudaMemcpyDeviceToHost));
+  CK(c, cudaMemcpy(words.data(), L.units_d, words.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost));
+  size_t cost[kUnitClasses];
+  unit_costs(L, cost);
+  *n = 0;
+  for (int w = 0; w < L.n_warps; ++w) {
+    const WarpDesc& d = warps[w];
+    if (d.stream < 0) continue;
+    if (d.stream >= c->n_hgroups || d.item_begin < 0 || d.item_end > L.n_units) return GKV_ERR_BAD_STATE;
+    for (int i = d.item_begin; i < d.item_end; ++i, ++*n) {
+      if (*n >= cap) continue;                       // (counted all the same)
+      const int item = static_cast<int>(words[i] & kUnitItemMask), run = static_cast<int>(words[i] >> 24);
+      int cls = item > L.n_closed ? 5 : 4;
+      if (item < L.n_closed) {
+        const int lv = L.level[static_cast<size_t>(d.stream / c->head_groups) * c->max_blocks + item];
+        cls = lv == 16 ? 0 : lv == 8 ? 1 : lv == 2 ? kClass2Bits : lv == 4 ? kClass4Bits : 22 - std::min(std::max(run, 1), 16);
+      }
+      const int32_t row[6] = {w, d.stream, item, static_cast<int32_t>((words[i] >> 20) & 15u), run, static_cast<int32_t>(cost[cls])};
+      std::memcpy(units + static_cast<size_t>(*n) * 6, row, sizeof(row));
+    }
+  }
+  return *n > cap ? GKV_ERR_INVALID_ARG : GKV_OK;
 }
 
 int gkv_debug_export_residual(gkv_cache* c, int32_t layer, int32_t b, int32_t kv_head, int32_t* idx, int32_t cap,

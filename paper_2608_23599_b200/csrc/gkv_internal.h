@@ -51,7 +51,8 @@ struct alignas(16) StreamPlan {
   int32_t n_res;          // exact residual rows
 };
 
-constexpr int kUnitClasses = 22;            // exact, 8, 2, 4 bits, tail, residual group, centroid runs of 16 .. 1
+constexpr int kUnitClasses = 22;            // exact, 8, 2, 4 bits, tail, residual group, centroid runs of 16 .. 1 (in this order)
+constexpr int kClass2Bits = 2, kClass4Bits = 3;
 
 struct UnitsParams {
   const TableEntry* table;      // [n_streams][table_stride]
@@ -61,7 +62,8 @@ struct UnitsParams {
   WarpDesc* warps;              // [n_warps]
   int32_t table_stride, n_closed, head_groups, n_warps;
   int32_t split, split_all;     // exact blocks as four tiles; quantised blocks as two halves, the tail as four tiles
-  int32_t cost[kUnitClasses];   // of a unit, by class
+  int32_t place[kUnitClasses];  // a class's place in the order of falling cost; the 4-bit class follows the 2-bit one
+  int32_t cost[kUnitClasses];   // of a unit, by place
   int32_t pad;                  // a power of two, at least 128 and the warps of any stream
   int32_t dealt;                // set by the launch
   int32_t cluster;              // CTAs per head group, 0 = head groups share CTAs

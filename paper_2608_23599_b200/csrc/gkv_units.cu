@@ -8,9 +8,11 @@
 // the context, and with about the same share of every level.  (Dealing forth and back without a look at
 // what a warp has balances the cost as well, but leaves the 8-bit blocks to the warps that have an exact one: 64 streams
 // of 32,757 tokens took 73.6 us a call instead of 72.3.  One unit to every warp in every round leaves a warp with an exact
-// block 12 % more than the others where the rest is cheap: 64 streams with exact residual rows 32.7 us a call.)
+// block 12 % more than the others where the rest is cheap: 64 streams with exact residual rows 32.7 us a call.  Classes in a
+// fixed order, exact blocks first and centroid runs last, 256 exact tokens, centroids and 10 % exact rows: 32.2 us a call for 64
+// streams of 32,747 tokens, 21.6 for 32, 21.1 for 64 of 16,384; by falling cost 31.75, 19.8 and 20.3.)
 //
-// The first round hands the costliest units (exact blocks, then 8-bit ones) to the first warps, and a CTA is a window of
+// The first round hands the costliest units (of whole blocks the exact ones, then 8-bit ones) to the first warps, and a CTA is a window of
 // consecutive warps: the warps are walked with a golden-ratio stride, so that every window holds the same mixture of
 // levels.  Warps of one SM share its issue slots, and a CTA whose warps all run the issue-heavy levels would finish
 // last.  Within its list a warp takes the units alternately from both ends (a byte-heavy unit after an issue-heavy one: its
@@ -40,7 +42,9 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
   const int n_items = p.n_closed + 1 + (plan.n_res + 15) / 16;
   const int nw = plan.n_warps;
 
-  // an item's class (-1: it is part of an earlier unit, or past the end), its unit word without the tile mask, its parts
+  // the place of an item's class in the order of falling cost (-1: the item is part of an earlier unit, or past the end), its
+  // unit word without the tile mask, its parts
+  const int at2 = p.place[kClass2Bits], at4 = p.place[kClass4Bits];
   auto classify = [&](int it, uint32_t& word, int& parts) -> int {
     const int level = it < p.n_closed ? static_cast<int>(table[it].level) : 0;
     const bool cent = it < p.n_closed && level != 16 && level != 8 && level != 4 && level != 2;
@@ -53,19 +57,19 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
       if (pos > 0 && ((group >> (pos - 1)) & 1u)) return -1;
       const int run = __ffs(static_cast<int>(~(group >> pos))) - 1;
       word = static_cast<uint32_t>(it) | (static_cast<uint32_t>(run) << 24);
-      return 22 - run;
+      return p.place[22 - run];
     }
-    if (it > p.n_closed) return 5;
+    if (it > p.n_closed) return p.place[5];
     if (it == p.n_closed) {
       parts = p.split_all ? 4 : 1;
-      return 4;
+      return p.place[4];
     }
     if (level == 16) {
       parts = p.split ? 4 : 1;
-      return 0;
+      return p.place[0];
     }
     parts = p.split_all ? 2 : 1;
-    return level == 8 ? 1 : (level == 2 ? 2 : 3);
+    return level == 8 ? p.place[1] : (level == 2 ? at2 : at4);
   };
   auto clear = [&]() {
     for (int i = tid; i < kUnitWarps * kUnitClasses; i += kUnitThreads) s_at[i / kUnitClasses][i % kUnitClasses] = 0;
@@ -114,7 +118,7 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
     const uint32_t hand = key & ((1u << kUnitHandBits) - 1u);
     hand_of[rank] = (s_cnt[hand]++ << kUnitHandBits) | hand;                         // (one unit per warp and round)
     while (cls_at < kUnitClasses - 1 && rank >= s_start[cls_at + 1]) ++cls_at;
-    if (cls_at == 2 || cls_at == 3) s_mix[hand] += cls_at == 2 ? 1u : 0x10000u;
+    if (cls_at == at2 || cls_at == at4) s_mix[hand] += cls_at == at2 ? 1u : 0x10000u;
     return key + (static_cast<uint32_t>(p.cost[cls_at]) / 16 << kUnitHandBits);
   };
   // keys below this take part in the round that begins with rank `base`; least is the smallest key
@@ -236,7 +240,7 @@ __global__ void __launch_bounds__(kUnitThreads) units_kernel(const __grid_consta
         const int k = static_cast<int>(static_cast<long long>(d) * plan.stride_inv % nw);
         const int m = static_cast<int>(s_cnt[d]);
         // the unit's number in its list from the narrowest level on (2-bit blocks are dealt before 4-bit ones)
-        const int z = m - 1 - (cls == 2 ? r + static_cast<int>(s_mix[d] >> 16) : (cls == 3 ? r - static_cast<int>(s_mix[d] & 0xffffu) : r));
+        const int z = m - 1 - (cls == at2 ? r + static_cast<int>(s_mix[d] >> 16) : (cls == at4 ? r - static_cast<int>(s_mix[d] & 0xffffu) : r));
         const int place = z < (m + 1) / 2 ? 2 * z : 2 * (m - 1 - z) + 1;
         p.units[s_key[d] + (place + m - (k * 5) % m) % m] = word | (mask << 20);
       }

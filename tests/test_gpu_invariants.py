@@ -1,6 +1,7 @@
 """What has to hold whatever the timing, the order of the calls and the number of threads: plans that do not depend on when
 a warp arrives, caches that do not disturb one another, state that a refused call leaves as it was, and work lists that hold
 every item once and are balanced."""
+import heapq
 import threading
 
 import numpy as np
@@ -223,3 +224,104 @@ def test_latent_read_loses_no_bit_to_the_largest_probability(stair, bound, seed)
     out, _, want, _ = U.decode_both(ocache, g, 0, data["q"])
     rel = np.linalg.norm(out.double().cpu().numpy() - want) / np.linalg.norm(want)
     assert rel <= bound, rel
+
+
+# ---- work lists -------------------------------------------------------------------------------------------------
+def _mixed_plan(rs, shape, n, levels=(16, 8, 4, 2, 1, 1)):
+    """Runs of 1 to 24 blocks of one rung, rungs at random."""
+    plan = np.empty(shape + (n,), dtype=np.int8)
+    for at in np.ndindex(shape):
+        i = 0
+        while i < n:
+            m = int(rs.randint(1, 25))
+            plan[at][i:i + m] = rs.choice(np.array(levels, dtype=np.int8))
+            i += m
+    return plan
+
+
+def _check_lists(rows, levels, n_res, head_groups):
+    """Every tile of every closed block, the partial block and every residual group once per head group; whole runs of
+    centroid blocks; and no warp with more than 1.02 times what the fullest one has when the units are dealt one by one,
+    longest first, to the least laden warp."""
+    n = levels.shape[1]
+    for hg in range(levels.shape[0] * head_groups):
+        mine = rows[rows[:, 1] == hg]
+        lv = levels[hg // head_groups]
+        groups = -(-int(n_res[hg // head_groups]) // 16)
+        tiles = np.zeros(n + 1 + groups, dtype=np.int64)
+        for t in range(4):
+            one = mine[(mine[:, 3] >> t & 1 == 1) & (mine[:, 4] == 1)]
+            np.add.at(tiles, one[:, 2], 1 << (4 * t))
+        for _, _, item, mask, run, _ in mine[mine[:, 4] > 1]:
+            assert mask == 15 and np.all(lv[item:item + run] == 1) and item // 16 == (item + run - 1) // 16
+            tiles[item:item + run] += 0x1111
+        assert np.all(tiles == 0x1111), (hg, np.nonzero(tiles != 0x1111)[0][:8])
+        warps = np.unique(mine[:, 0])
+        load = np.zeros(int(mine[:, 0].max()) + 1, dtype=np.int64)
+        np.add.at(load, mine[:, 0], mine[:, 5])
+        heap = [0] * len(warps)
+        for cost in np.sort(mine[:, 5])[::-1]:
+            heapq.heapreplace(heap, heap[0] + int(cost))
+        assert load.max() <= 1.02 * max(heap), (hg, int(load.max()), max(heap))
+
+
+@pytest.mark.parametrize("batch,n_kv,group,T,residual,fixed", [
+    (1, 1, 1, 70, 0.0, None), (2, 2, 8, 13_100, 0.0, None), (2, 1, 8, 27_300, 0.0, None), (4, 1, 8, 16_750, 0.0, None),
+    (1, 2, 8, 16_384, 0.01, None), (4, 8, 4, 32_763, 0.10, "newest"), (8, 8, 4, 16_384, 0.10, "newest"), (2, 1, 4, 6000, 0.05, "newest"),
+    (1, 1, 4, 140_000, 0.02, None)])
+def test_work_lists_are_complete_and_balanced(batch, n_kv, group, T, residual, fixed):
+    B = _binding()
+    w = _gqa(T, batch, n_kv, group, policy=W.POLICY_EXTERNAL, residual_fraction=residual)
+    rs = np.random.RandomState(T)
+    plan = _mixed_plan(rs, (batch, n_kv), T // 64)
+    if fixed:                                       # 256 exact tokens, centroids, exact residual rows
+        plan[:] = 1
+        plan[..., -4:] = 16
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(T)
+    k = torch.randn((batch, T, n_kv, 128), generator=gen, device="cuda").to(torch.bfloat16)
+    mass = torch.softmax(torch.randn((batch, n_kv, T), generator=gen, device="cuda"), -1) if residual else None
+    g = B.Cache(B.config_from_workload(w))
+    g.gkv_append_demote(0, k, k, token_mass=mass, level_plan=plan)
+    q = torch.randn((batch, n_kv * group, 128), generator=gen, device="cuda").to(torch.bfloat16)
+    out = torch.empty((batch, n_kv * group, 128), device="cuda")
+    with pytest.raises(B.GkvError):
+        g.gkv_debug_export_units(0)                  # none made yet
+    n_res = [len(g.gkv_debug_export_residual(0, b, h)) for b in range(batch) for h in range(n_kv)]
+    levels = plan.reshape(batch * n_kv, -1).astype(np.int64)
+    for observe in (False, True):                    # parts of blocks in small workloads; whole blocks
+        if observe:
+            g.gkv_decode_attn_observe(0, q, out)
+        else:
+            g.gkv_decode_attn(0, q, out)
+        _check_lists(g.gkv_debug_export_units(0), levels, n_res, -(-group // 4))
+
+
+@pytest.mark.parametrize("levels", [(16,), (16, 8, 4, 2)])
+@pytest.mark.parametrize("n_closed", [3125, 45_200])
+def test_long_context_lists(n_closed, levels):
+    """One stream whose work list needs more shared memory than a kernel has without asking, and one that is longer than the
+    units whose warps are kept in shared memory (it is dealt without a look at what a warp has): every block once, and, of
+    exact blocks, the read against the one by page list, which has no work lists.  Both sum exact products in fp32: 1e-4 of
+    the output is ten times what they differ by, and a block left out or read twice changes it by 1 / sqrt(blocks) = 5e-3."""
+    B = _binding()
+    T = 64 * n_closed + 33
+    w = _gqa(T, room=64, page_tokens=64, policy=W.POLICY_EXTERNAL)
+    plan = _mixed_plan(np.random.RandomState(n_closed), (1, 1), n_closed, levels)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n_closed)
+    k = torch.randn((1, T, 1, 128), generator=gen, device="cuda", dtype=torch.bfloat16)
+    q = (0.25 * torch.randn((1, 1, 128), generator=gen, device="cuda")).to(torch.bfloat16)
+    g = B.Cache(B.config_from_workload(w))
+    g.gkv_append_demote(0, k, k, level_plan=plan)
+    del k
+    out, listed = torch.empty((1, 1, 128), device="cuda"), torch.empty((1, 1, 128), device="cuda")
+    g.gkv_decode_attn(0, q, out)
+    rows = g.gkv_debug_export_units(0)
+    assert np.array_equal(np.sort(rows[:, 2]), np.arange(n_closed + 1)) and np.all(rows[:, 3] == 15)
+    assert 147 * 16 < len(np.unique(rows[:, 0])) <= 148 * 16      # about one wave of warps
+    if levels == (16,):
+        pages = torch.arange(n_closed, dtype=torch.int32, device="cuda").reshape(1, 1, -1)
+        g.gkv_decode_attn(0, q, listed, page_idx=pages, n_sel=n_closed)
+        torch.cuda.synchronize()
+        assert float((out - listed).norm() / listed.norm()) < 1e-4
