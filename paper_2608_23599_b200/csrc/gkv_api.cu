@@ -240,6 +240,9 @@ struct ArenaPlan {
   size_t l_table, l_warps, l_units, l_plans, l_parts, l_resoff, l_rescount, l_residx, l_respool, l_boxes, l_ema, l_range, l_err, layer_bytes;
 };
 
+// Room of a layer's stream plans; the ranges of partial rows (StreamParts) follow directly, on the device and in the mirror.
+size_t plans_bytes(int n_streams) { return align_up(static_cast<size_t>(n_streams) * sizeof(StreamPlan), 256); }
+
 struct Derived {
   int n_streams, group, head_groups, n_hgroups, max_blocks, table_stride, max_warps, res_cap, box_stride;
   size_t units_cap;
@@ -321,7 +324,7 @@ ArenaPlan plan_arena(const gkv_config& c, const Derived& d) {
   a.l_table = ltake(static_cast<size_t>(d.n_streams) * d.table_stride * sizeof(TableEntry));
   a.l_warps = ltake(static_cast<size_t>(d.max_warps) * sizeof(WarpDesc));
   a.l_units = ltake(d.units_cap * sizeof(uint32_t));
-  a.l_plans = ltake(static_cast<size_t>(d.n_streams) * sizeof(StreamPlan));
+  a.l_plans = ltake(plans_bytes(d.n_streams));
   a.l_parts = ltake(static_cast<size_t>(d.n_hgroups) * sizeof(StreamParts));
   a.l_resoff = ltake(static_cast<size_t>(d.n_streams) * sizeof(uint32_t));
   a.l_rescount = ltake(static_cast<size_t>(d.n_streams) * sizeof(int32_t));
@@ -656,8 +659,9 @@ int make_units(gkv_cache* c, LayerState& L, bool allow_split, cudaStream_t st) {
   CK(c, cudaEventSynchronize(L.ev_desc));
   plan_units(c, L, allow_split);
   int rc;
-  if ((rc = upload(c, L.plans_d, L.plans_h, static_cast<size_t>(c->n_streams) * sizeof(StreamPlan), st, L.ev_desc)) != GKV_OK) return rc;
-  if ((rc = upload(c, L.parts_d, L.parts_h, static_cast<size_t>(c->n_hgroups) * sizeof(StreamParts), st, L.ev_desc)) != GKV_OK) return rc;
+  // plans and parts lie behind one another in the arena as in the mirror: one copy (a second one kept the GPU waiting 5 us)
+  const size_t bytes = plans_bytes(c->n_streams) + static_cast<size_t>(c->n_hgroups) * sizeof(StreamParts);
+  if ((rc = upload(c, L.plans_d, L.plans_h, bytes, st, L.ev_desc)) != GKV_OK) return rc;
   UnitsParams p{};
   p.table = L.table_d;
   p.plans = L.plans_d;
@@ -1578,7 +1582,7 @@ int gkv_create(const gkv_config* cfg, void* arena, size_t arena_bytes, gkv_cache
     for (LayerState& L : c->layers) {
       take(L.table_h, table_bytes);
       if (is_mla(c->cfg)) take(L.warps_h, d.max_warps * sizeof(WarpDesc));
-      take(L.plans_h, d.n_streams * sizeof(StreamPlan));
+      take(L.plans_h, plans_bytes(d.n_streams));
       take(L.parts_h, d.n_hgroups * sizeof(StreamParts));
       take(L.res_off_h, d.n_streams * sizeof(uint32_t));
       take(L.res_count_h, d.n_streams * sizeof(int32_t));
