@@ -105,8 +105,14 @@ GKV_API int gkv_query_arena_bytes(const gkv_config* cfg, size_t* bytes);
  * the default ordering of `stream`-less cudaMemset, so the call synchronises.  out: host. */
 GKV_API int gkv_create(const gkv_config* cfg, void* arena, size_t arena_bytes, gkv_cache** out);
 
-/* Free the host object (synchronises the device first).  The arena is not touched. */
+/* Free the host object (synchronises the device first).  The arena is not touched.  The cache's page-locked host memory (16
+ * bytes per block that max_ctx has room for, in every layer, and staging) is kept for the next cache of about its size: up to four
+ * such pieces and 320 MiB in all stay locked in the process, and one that eight creations in a row had no use for is freed. */
 GKV_API int gkv_destroy(gkv_cache* c);
+
+/* Free the page-locked host memory that destroyed caches have left (caches in use keep theirs).  bytes: host, receives how
+ * much that was, or NULL.  May be called from any thread at any time. */
+GKV_API int gkv_release_host_memory(size_t* bytes);
 
 /* Append n_new tokens to every sequence of `layer`, then move full blocks down the ladder
  * (Sec. 3.2: monotone demotion, never upward, requantised from the block's current

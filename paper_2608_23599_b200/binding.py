@@ -24,7 +24,7 @@ ERR_INVALID_ARG, ERR_ARENA_TOO_SMALL, ERR_CTX_FULL, ERR_BAD_STATE, ERR_UNSUPPORT
 ERR_RANGE, ERR_BUDGET, ERR_CUDA = -6, -7, -8
 
 EXPORTS = [
-    "gkv_query_arena_bytes", "gkv_create", "gkv_destroy", "gkv_append_demote", "gkv_decode_attn",
+    "gkv_query_arena_bytes", "gkv_create", "gkv_destroy", "gkv_release_host_memory", "gkv_append_demote", "gkv_decode_attn",
     "gkv_decode_attn_observe", "gkv_debug_export_mass", "gkv_debug_export_bounds", "gkv_rd_reallocate", "gkv_debug_device_plan",
     "gkv_debug_replan_levels",
     "gkv_quest_select", "gkv_quest_select_static", "gkv_debug_export_boxes", "gkv_debug_export_scores", "gkv_bits_report",
@@ -81,6 +81,7 @@ def load():
     lib.gkv_query_arena_bytes.argtypes = [C.POINTER(GkvConfig), C.POINTER(sz)]
     lib.gkv_create.argtypes = [C.POINTER(GkvConfig), vp, sz, C.POINTER(vp)]
     lib.gkv_destroy.argtypes = [vp]
+    lib.gkv_release_host_memory.argtypes = [C.POINTER(sz)]
     lib.gkv_append_demote.argtypes = [vp, i32, vp, vp, i32, vp, vp, vp]
     lib.gkv_decode_attn.argtypes = [vp, i32, vp, vp, i32, vp, vp, vp]
     lib.gkv_decode_attn_observe.argtypes = [vp, i32, vp, vp, vp, vp, vp, vp]
@@ -161,6 +162,13 @@ def _check(rc: int, what: str, allow=()):
 def gkv_query_arena_bytes(cfg: GkvConfig) -> int:
     out = C.c_size_t(0)
     _check(load().gkv_query_arena_bytes(C.byref(cfg), C.byref(out)), "gkv_query_arena_bytes")
+    return out.value
+
+
+def gkv_release_host_memory() -> int:
+    """Frees the page-locked host memory that closed caches have left for later ones; returns the bytes."""
+    out = C.c_size_t(0)
+    _check(load().gkv_release_host_memory(C.byref(out)), "gkv_release_host_memory")
     return out.value
 
 

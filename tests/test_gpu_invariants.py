@@ -325,3 +325,57 @@ def test_long_context_lists(n_closed, levels):
         g.gkv_decode_attn(0, q, listed, page_idx=pages, n_sel=n_closed)
         torch.cuda.synchronize()
         assert float((out - listed).norm() / listed.norm()) < 1e-4
+
+
+# ---- page-locked host memory -----------------------------------------------------------------------------------
+def _centroid_cache(B, layers, batch, ctx):
+    return B.Cache(B.make_config(layers, batch, 32, 8, 128, 128, ctx, stair_tokens=(0, 0, 0, 0)))
+
+
+def test_host_memory_of_a_large_cache_is_kept_and_given_back():
+    """The block tables of 32 layers x 64 streams x 131,072 tokens (67 MB): kept after the cache is gone, given back on
+    request or when eight caches of another size have come and gone; a cache in use keeps its own."""
+    B = _binding()
+    table = 32 * 64 * (131_072 // 64) * 16
+    B.gkv_release_host_memory()
+    _centroid_cache(B, 32, 8, 131_072).close()
+    assert table <= B.gkv_release_host_memory() < 1.25 * table
+    assert B.gkv_release_host_memory() == 0
+    live = _centroid_cache(B, 2, 1, 1024)
+    assert B.gkv_release_host_memory() == 0
+    k = torch.randn((1, 130, 8, 128), device="cuda").to(torch.bfloat16)
+    out = torch.empty((1, 32, 128), device="cuda")
+    live.gkv_append_demote(0, k, k)
+    live.gkv_decode_attn(0, torch.zeros((1, 32, 128), dtype=torch.bfloat16, device="cuda"), out)
+    torch.cuda.synchronize()
+    want = k.float().mean(1).repeat_interleave(4, 1)      # equal weights; two centroids of 64 tokens (bf16) and two tokens
+    assert torch.allclose(out, want, atol=2.0 ** -9)
+    live.close()
+    _centroid_cache(B, 32, 8, 131_072).close()
+    for _ in range(9):
+        _centroid_cache(B, 2, 1, 1024).close()
+    assert B.gkv_release_host_memory() < table
+
+
+def test_host_memory_that_is_kept_is_bounded():
+    B = _binding()
+    B.gkv_release_host_memory()
+    caches = [_centroid_cache(B, 32, b, 131_072) for b in (2, 3, 5, 8, 12, 16)]      # 18 to 140 MB each
+    for c in caches:
+        c.close()
+    assert B.gkv_release_host_memory() <= 320 << 20
+
+
+def test_host_memory_is_given_back_while_other_threads_make_caches():
+    B = _binding()
+
+    def work(side, meet):
+        meet()
+        for i in range(40):
+            _centroid_cache(B, 2, 1 + (i + side) % 3, 2048).close()
+            if i % 4 == side:
+                B.gkv_release_host_memory()
+
+    _in_two_threads(work)
+    assert B.gkv_release_host_memory() <= 4 << 20
+    assert B.gkv_release_host_memory() == 0
