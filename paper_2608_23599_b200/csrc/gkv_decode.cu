@@ -1330,13 +1330,10 @@ size_t decode_smem_bytes() {
 
 namespace {
 cudaError_t configure_decode() {
-  static bool configured = false;
-  if (configured) return cudaSuccess;
-  const int bytes = static_cast<int>(decode_smem_bytes());
-  cudaError_t e = cudaFuncSetAttribute(decode_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(decode_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  configured = e == cudaSuccess;
+  static std::atomic<uint64_t> done[3];
+  cudaError_t e = raise_smem_limit(decode_kernel<false, false>, decode_smem_bytes(), done[0]);
+  if (e == cudaSuccess) e = raise_smem_limit(decode_kernel<true, false>, decode_smem_bytes(), done[1]);
+  if (e == cudaSuccess) e = raise_smem_limit(decode_kernel<false, true>, decode_smem_bytes(), done[2]);
   return e;
 }
 }  // namespace

@@ -861,15 +861,12 @@ __global__ void __launch_bounds__(kMlaInThreads, 3) mla_ingest_kernel(const __gr
 
 }  // namespace
 
-// All jobs read the bf16 input rows (src_level == 0); without a job list the work is counted off the block table.
+// Every block is read from the bf16 input rows; the work is counted off the block table.
 cudaError_t launch_ingest(const EncodeParams& p, cudaStream_t st) {
   if (p.n_jobs <= 0) return cudaSuccess;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(ingest_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kInSmem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = raise_smem_limit(ingest_kernel, kInSmem, done);
+  if (e != cudaSuccess) return e;
   const int grid = p.n_jobs < 148 * kInCtas ? p.n_jobs : 148 * kInCtas;
   ingest_kernel<<<grid, kInThreads, kInSmem, st>>>(p);
   return cudaGetLastError();
@@ -881,12 +878,9 @@ namespace gkv {
 // Bulk ingest of latent-attention rows: every job reads the bf16 input (src_level == 0), rows 16-byte aligned.
 cudaError_t launch_mla_ingest(const MlaEncodeParams& p, cudaStream_t st) {
   if (p.n_jobs <= 0) return cudaSuccess;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(mla_ingest_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlaInTile);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = raise_smem_limit(mla_ingest_kernel, kMlaInTile, done);
+  if (e != cudaSuccess) return e;
   const int grid = p.n_jobs < 148 * 3 ? p.n_jobs : 148 * 3;
   mla_ingest_kernel<<<grid, kMlaInThreads, kMlaInTile, st>>>(p);
   return cudaGetLastError();

@@ -165,7 +165,8 @@ __global__ void __launch_bounds__(256) mla_export_kernel(const uint8_t* arena, u
 cudaError_t launch_mla_encode(const MlaEncodeParams& p, cudaStream_t st) {
   if (p.n_jobs <= 0) return cudaSuccess;
   const size_t smem = kBlock * kMTileLd * sizeof(float) + kBlock * kMlaDk;
-  cudaError_t e = cudaFuncSetAttribute(mla_encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = raise_smem_limit(mla_encode_kernel, smem, done);
   if (e != cudaSuccess) return e;
   const int grid = p.n_jobs < 148 * 8 ? p.n_jobs : 148 * 8;
   mla_encode_kernel<<<grid, 256, smem, st>>>(p);

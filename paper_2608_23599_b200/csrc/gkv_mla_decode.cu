@@ -981,12 +981,9 @@ __global__ void __launch_bounds__(kCombThreads) mla_combine_kernel(const float* 
 cudaError_t launch_mla_decode(const MlaDecodeParams& p, int n_ctas, const StreamParts* parts, int n_streams, float* out,
                               float* lse, cudaStream_t st) {
   if (n_ctas <= 0) return cudaSuccess;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(mla_decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMSmem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t limit = raise_smem_limit(mla_decode_kernel, kMSmem, done);
+  if (limit != cudaSuccess) return limit;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;

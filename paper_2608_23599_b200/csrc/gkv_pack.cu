@@ -587,12 +587,9 @@ __global__ void __launch_bounds__(256) export_kernel(const uint8_t* arena, uint3
 cudaError_t launch_encode(const EncodeParams& p, cudaStream_t st) {
   if (p.n_jobs <= 0) return cudaSuccess;
   const size_t smem = kBlock * kTileLd * sizeof(float) + kBlock * kD + (256 + 256 + 16) * sizeof(float);
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = raise_smem_limit(encode_kernel, smem, done);
+  if (e != cudaSuccess) return e;
   const int grid = 2 * p.n_jobs < 148 * 16 ? 2 * p.n_jobs : 148 * 16;
   encode_kernel<<<grid, 256, smem, st>>>(p);
   return cudaGetLastError();

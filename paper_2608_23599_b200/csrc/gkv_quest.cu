@@ -365,12 +365,9 @@ template <int GROUP, int THREADS, int STAGES>
 cudaError_t launch_quest_shape(const uint16_t* boxes, int box_stride, int n_pages, const uint16_t* q, int n_streams, int n_kv_heads,
                                int reduce, float* scores, int score_stride, cudaStream_t st) {
   const size_t smem = static_cast<size_t>(STAGES) * kQRows * THREADS * 4 + static_cast<size_t>(GROUP) * kD * 16;
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(quest_score_kernel<GROUP, THREADS, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = raise_smem_limit(quest_score_kernel<GROUP, THREADS, STAGES>, smem, done);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((n_pages + 2 * THREADS - 1) / (2 * THREADS), n_streams);
   cfg.blockDim = dim3(THREADS);

@@ -1,7 +1,7 @@
-"""The shared-memory limit of a kernel is the kernel's, not a launch's.  Two host threads that make work lists (level plans)
-of different sizes at once must both be able to launch: here with the two launch functions linked against a small fake of
-the CUDA runtime that applies the threads' limits in the worst order, larger one first, and refuses a launch above the
-limit as the runtime does."""
+"""The shared-memory limit of a kernel is the kernel's on a device, not a launch's and not the process's.  Two host threads that make work lists (level plans)
+of different sizes at once must both be able to launch, and every kernel on every device: here with the launch functions
+linked against a small fake of the CUDA runtime that applies the threads' limits in the worst order, larger one first, and
+refuses a launch above the limit as the runtime does."""
 import os
 import shutil
 import subprocess
@@ -19,6 +19,7 @@ FAKE = r"""
 #include <thread>
 #include <vector>
 #include "gkv_internal.h"
+#include "gkv_mla.h"
 
 static std::mutex mu;
 static std::condition_variable cv;
@@ -53,6 +54,13 @@ cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void**, size_t bytes, cu
   last = bytes > limit_of(f) ? cudaErrorInvalidValue : cudaSuccess;
   return last;
 }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+  return cudaLaunchKernel(f, c->gridDim, c->blockDim, nullptr, c->dynamicSmemBytes, c->stream);
+}
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaunchConfig_t* c) {
+  *n = 18;
+  return c->dynamicSmemBytes > limit_of(f) ? cudaErrorInvalidValue : cudaSuccess;
+}
 static thread_local struct { dim3 g, b; size_t s; cudaStream_t st; } pushed;
 unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t s, cudaStream_t st) { pushed = {g, b, s, st}; return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* s, void* st) {
@@ -77,7 +85,43 @@ static cudaError_t plans(int blocks) {
   return gkv::launch_rd_plan(p, 1, nullptr);
 }
 
+// every other kernel with a limit of its own, on two devices in turn
+static int every_kernel() {
+  using namespace gkv;
+  int bad = 0, at = 0;
+  auto check = [&](cudaError_t e) {
+    bad += e != cudaSuccess;
+    std::printf("device %d, kernel %d: %d\n", device, at++, e);
+  };
+  static int32_t some;
+  for (int d = 0; d < 4; ++d) {
+    device = d & 1;
+    at = 0;
+    DecodeParams read{};
+    check(launch_decode(read, 1, true, nullptr));
+    read.mass_raw = reinterpret_cast<float2*>(&some);
+    check(launch_decode(read, 1, false, nullptr));
+    read.mass_raw = nullptr;
+    read.page_idx = &some;
+    check(launch_decode(read, 1, true, nullptr));
+    check(decode_max_clusters(2) == 18 ? cudaSuccess : cudaErrorInvalidValue);
+    EncodeParams enc{};
+    enc.n_jobs = 1;
+    check(launch_encode(enc, nullptr));
+    check(launch_ingest(enc, nullptr));
+    MlaEncodeParams lat{};
+    lat.n_jobs = 1;
+    check(launch_mla_encode(lat, nullptr));
+    check(launch_mla_ingest(lat, nullptr));
+    check(launch_mla_decode(MlaDecodeParams{}, 1, nullptr, 1, nullptr, nullptr, nullptr));
+    for (int group = 1; group <= kMaxHeadsPerKv; ++group)
+      for (int streams : {1, 1024}) check(launch_quest_scores(nullptr, 4096, 4096, nullptr, streams, 1, group, 0, nullptr, 4096, nullptr));
+  }
+  return bad != 0;
+}
+
 int main(int argc, char** argv) {
+  if (argc > 1 && !std::strcmp(argv[1], "kernels")) return every_kernel();
   cudaError_t (*launch)(int) = argc > 1 && !std::strcmp(argv[1], "plans") ? plans : lists;
   const bool is_plans = launch == plans;
   const int small = is_plans ? 1700 : 2300, large = is_plans ? 4095 : 45056;
@@ -114,11 +158,11 @@ def harness(tmp_path_factory):
     d = tmp_path_factory.mktemp("limits")
     src, exe = d / "fake.cpp", d / "fake"
     src.write_text(FAKE)
-    objs = []
-    for name in ("gkv_units", "gkv_rdplan"):
-        objs.append(str(d / f"{name}.o"))
-        subprocess.run([os.path.join(cuda, "bin", "nvcc"), *_build.NVCC_FLAGS, "-c", os.path.join(_build.CSRC, f"{name}.cu"), "-o", objs[-1]],
-                       check=True, capture_output=True)
+    names = [s[:-3] for s in _build.SOURCES if s != "gkv_api.cu"]
+    objs = [str(d / f"{name}.o") for name in names]
+    made = [subprocess.Popen([os.path.join(cuda, "bin", "nvcc"), *_build.NVCC_FLAGS, "-c", os.path.join(_build.CSRC, f"{name}.cu"), "-o", obj],
+                             stdout=subprocess.DEVNULL, stderr=subprocess.DEVNULL) for name, obj in zip(names, objs)]
+    assert [p.wait(600) for p in made] == [0] * len(made)
     subprocess.run(["g++", "-std=c++17", "-I", _build.CSRC, "-I", os.path.join(cuda, "include"), str(src), *objs, "-o", str(exe), "-lpthread"],
                    check=True)
     return str(exe)
@@ -127,4 +171,9 @@ def harness(tmp_path_factory):
 @pytest.mark.parametrize("what", ["lists", "plans"])
 def test_a_launch_is_not_refused_for_another_threads_smaller_one(harness, what):
     r = subprocess.run([harness, what], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_every_kernel_launches_on_every_device(harness):
+    r = subprocess.run([harness, "kernels"], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
