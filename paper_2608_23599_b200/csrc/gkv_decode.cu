@@ -1357,8 +1357,8 @@ int decode_max_clusters(int ctas) {
   cfg.numAttrs = 1;
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, decode_kernel<false, false>, &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    n = 0;
+    cudaGetLastError();                  // (asked again by the next call: a failure is not an answer)
+    return 0;
   }
   known[ctas] = n;
   return n;

@@ -28,6 +28,7 @@ static thread_local int device = 0;
 static thread_local cudaError_t last = cudaSuccess;
 static int expected = 0;                                         // threads that meet in cudaFuncSetAttribute
 static std::vector<int> asked;
+static bool refuse_query = false;
 
 static size_t& limit_of(const void* f) {
   auto it = limit.find({device, f});
@@ -59,6 +60,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
 }
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaunchConfig_t* c) {
   *n = 18;
+  if (refuse_query) return last = cudaErrorMemoryAllocation;
   return c->dynamicSmemBytes > limit_of(f) ? cudaErrorInvalidValue : cudaSuccess;
 }
 static thread_local struct { dim3 g, b; size_t s; cudaStream_t st; } pushed;
@@ -122,6 +124,15 @@ static int every_kernel() {
 
 int main(int argc, char** argv) {
   if (argc > 1 && !std::strcmp(argv[1], "kernels")) return every_kernel();
+  if (argc > 1 && !std::strcmp(argv[1], "clusters")) {
+    refuse_query = true;
+    const int none = gkv::decode_max_clusters(4);
+    const bool clean = cudaGetLastError() == cudaSuccess;      // the caller does not find the query's error
+    refuse_query = false;
+    const int some = gkv::decode_max_clusters(4);
+    std::printf("%d %d %d\n", none, clean, some);
+    return none == 0 && clean && some == 18 ? 0 : 1;
+  }
   cudaError_t (*launch)(int) = argc > 1 && !std::strcmp(argv[1], "plans") ? plans : lists;
   const bool is_plans = launch == plans;
   const int small = is_plans ? 1700 : 2300, large = is_plans ? 4095 : 45056;
@@ -176,4 +187,9 @@ def test_a_launch_is_not_refused_for_another_threads_smaller_one(harness, what):
 
 def test_every_kernel_launches_on_every_device(harness):
     r = subprocess.run([harness, "kernels"], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_a_refused_query_of_cluster_room_is_asked_again(harness):
+    r = subprocess.run([harness, "clusters"], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
