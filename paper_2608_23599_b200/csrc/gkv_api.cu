@@ -182,6 +182,7 @@ struct LayerState {
   int32_t* res_count_h = nullptr;       // pinned [n_streams]
   std::vector<std::vector<int32_t>> res_idx;      // host copy of the residual rows' tokens, fetched when first asked for
   bool res_idx_valid = true;
+  bool has_residual = false;            // some stream has exact residual rows
   bool desc_dirty = true;
   int cluster = 0;                      // CTAs per head group of the work lists, 0 = head groups share CTAs
   bool split = false, split_all = false;      // the work lists hold parts of exact blocks / of others (never for observing calls)
@@ -990,6 +991,7 @@ int bulk_ingest(gkv_cache* c, int layer, const uint16_t* k_new, const uint16_t* 
       if ((rc = residual_select()) != GKV_OK) return rc;
     }
     L.res_idx_valid = max_k == 0;
+    L.has_residual = max_k > 0;
   }
 
   // 5. uploads, then encode every closed block once at its planned level (unless done above), copy the residual and tail
@@ -1895,7 +1897,7 @@ int decode_impl(gkv_cache* c, int32_t layer, const void* q, const int32_t* page_
     o.res_cap = c->res_cap;
     o.err_stride = c->max_blocks;
     o.scale = c->scale;
-    CK(c, launch_observe_finish(o, st));
+    CK(c, launch_observe_finish(o, !L.has_residual, st));
   }
   return GKV_OK;
 }

@@ -1397,13 +1397,20 @@ constexpr int kObsThreads = 256;
 __device__ __forceinline__ void finish_mass(const ObserveParams& p, int idx) {
   if (idx >= p.n_streams * p.n_items) return;
   const int s = idx / p.n_items, b = idx - s * p.n_items;
-  const float* lse2 = p.lse2 + static_cast<size_t>(s) * p.group;
-  const float2* raw = p.mass_raw + (static_cast<size_t>(s) * p.mass_stride + b) * kMaxHeadsPerKv;
+  float lse2[kMaxHeadsPerKv];
+#pragma unroll
+  for (int h = 0; h < kMaxHeadsPerKv; ++h) lse2[h] = h < p.group ? p.lse2[static_cast<size_t>(s) * p.group + h] : -INFINITY;
   float a = 0.f;
-  for (int h = 0; h < p.group; ++h) {
-    const float2 v = raw[h];
-    if (v.y > 0.f && lse2[h] != -INFINITY) a += v.y * exp2f(v.x - lse2[h]);
-  }
+  auto add = [&](const float2* pairs) {             // the heads' pairs of a block or residual row, 16 bytes at a time, in order
+#pragma unroll
+    for (int h = 0; h < kMaxHeadsPerKv; h += 2) {
+      if (h >= p.group) break;
+      const float4 v = *reinterpret_cast<const float4*>(pairs + h);
+      if (v.y > 0.f && lse2[h] != -INFINITY) a += v.y * exp2f(v.x - lse2[h]);
+      if (v.w > 0.f && lse2[h + 1] != -INFINITY) a += v.w * exp2f(v.z - lse2[h + 1]);
+    }
+  };
+  add(p.mass_raw + (static_cast<size_t>(s) * p.mass_stride + b) * kMaxHeadsPerKv);
   const int n_res = p.res_count ? p.res_count[s] : 0;
   if (n_res > 0) {
     const int32_t* ri = p.res_idx + static_cast<size_t>(s) * p.res_cap;
@@ -1413,13 +1420,7 @@ __device__ __forceinline__ void finish_mass(const ObserveParams& p, int idx) {
       if (ri[mid] < b * kBlock) lo = mid + 1;
       else hi = mid;
     }
-    for (int i = lo; i < n_res && ri[i] < (b + 1) * kBlock; ++i) {
-      const float2* rr = p.res_raw + (static_cast<size_t>(s) * p.res_cap + i) * kMaxHeadsPerKv;
-      for (int h = 0; h < p.group; ++h) {
-        const float2 v = rr[h];
-        if (v.y > 0.f && lse2[h] != -INFINITY) a += v.y * exp2f(v.x - lse2[h]);
-      }
-    }
+    for (int i = lo; i < n_res && ri[i] < (b + 1) * kBlock; ++i) add(p.res_raw + (static_cast<size_t>(s) * p.res_cap + i) * kMaxHeadsPerKv);
   }
   a /= static_cast<float>(p.group);
   float* e = p.ema + static_cast<size_t>(s) * p.mass_stride + b;
@@ -1505,7 +1506,10 @@ __device__ __forceinline__ void finish_certificate(const ObserveParams& p, int h
 // What an observing read leaves to do: CTAs [0, n_cert) make one query head's certificate each, the others
 // finish the block masses.  Bound by latency: both parts read what the decode launch has just written, so they
 // share one launch, which overlaps that launch's tail (with two launches one after the other and no
-// overlap an observing call over 8200 tokens of 16 streams took 28.9 us, with this one 21.2).
+// overlap an observing call over 8200 tokens of 16 streams took 28.9 us, with this one 21.2).  Not where there are residual
+// rows: an overlapped launch's CTAs crowd the first SMs that the decode kernel leaves, whose L1 is what its 225 KB of shared
+// memory left over, and the rows' pairs, looked up block by block, live off L1: 12,000 rows in blocks of 64 streams of 8200
+// tokens 99 us a call overlapped, 30 not; 105,000 rows of 32 streams of 32,700 tokens 113 and 38.
 __global__ void __launch_bounds__(kObsThreads) observe_finish_kernel(const __grid_constant__ ObserveParams p) {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
@@ -1516,7 +1520,7 @@ __global__ void __launch_bounds__(kObsThreads) observe_finish_kernel(const __gri
 }
 }  // namespace
 
-cudaError_t launch_observe_finish(const ObserveParams& p, cudaStream_t st) {
+cudaError_t launch_observe_finish(const ObserveParams& p, bool overlap, cudaStream_t st) {
   const int n_cert = p.certificate ? p.n_streams * p.group : 0;
   const int n_mass = (p.n_streams * p.n_items + kObsThreads - 1) / kObsThreads;
   if (n_cert + n_mass <= 0) return cudaSuccess;
@@ -1528,7 +1532,7 @@ cudaError_t launch_observe_finish(const ObserveParams& p, cudaStream_t st) {
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = overlap ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, observe_finish_kernel, p);
 }
 

@@ -268,7 +268,7 @@ def _check_lists(rows, levels, n_res, head_groups):
 @pytest.mark.parametrize("batch,n_kv,group,T,residual,fixed", [
     (1, 1, 1, 70, 0.0, None), (2, 2, 8, 13_100, 0.0, None), (2, 1, 8, 27_300, 0.0, None), (4, 1, 8, 16_750, 0.0, None),
     (1, 2, 8, 16_384, 0.01, None), (4, 8, 4, 32_763, 0.10, "newest"), (8, 8, 4, 16_384, 0.10, "newest"), (2, 1, 4, 6000, 0.05, "newest"),
-    (1, 1, 4, 140_000, 0.02, None)])
+    (2, 1, 5, 3000, 0.05, "newest"), (3, 2, 3, 2500, 0.03, None), (1, 1, 4, 140_000, 0.02, None)])
 def test_work_lists_are_complete_and_balanced(batch, n_kv, group, T, residual, fixed):
     B = _binding()
     w = _gqa(T, batch, n_kv, group, policy=W.POLICY_EXTERNAL, residual_fraction=residual)
@@ -291,7 +291,9 @@ def test_work_lists_are_complete_and_balanced(batch, n_kv, group, T, residual, f
     levels = plan.reshape(batch * n_kv, -1).astype(np.int64)
     for observe in (False, True):                    # parts of blocks in small workloads; whole blocks
         if observe:
-            g.gkv_decode_attn_observe(0, q, out)
+            m = torch.empty((batch, n_kv, -(-T // 64)), device="cuda")
+            g.gkv_decode_attn_observe(0, q, out, None, m)
+            assert torch.allclose(m.sum(-1), torch.ones((), device="cuda"), atol=2e-3)      # residual rows in their blocks
         else:
             g.gkv_decode_attn(0, q, out)
         _check_lists(g.gkv_debug_export_units(0), levels, n_res, -(-group // 4))
