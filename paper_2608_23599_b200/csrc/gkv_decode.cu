@@ -916,30 +916,26 @@ __device__ __forceinline__ void compute_step(const WarpCtx& w, const Cursor& c, 
   }
 }
 
-// The four query rows of the warp's head group into its second stage (idle until the first unit is under
-// way), zeros for heads that the group does not have.
-__device__ __forceinline__ void fetch_query(const WarpCtx& w) {
+// The words of the query rows that the lane puts into fragments (below), zeros for heads that the group does not have.  Plain
+// loads, asked for before the first step's copies and needed behind them: they go through L1, which the CTA's warps share.
+// (As cp.async.cg copies into the stage every warp of the GPU asked L2 for them: where all warps work for one or two head groups,
+// thousands of requests for the same sectors, the start of a launch took 2 - 7 us instead of 2, and a first step of exact
+// rows was waited for together with them.  One stream of 65,000 4-bit tokens 21.4 -> 14.3 us a call, exact 25.9 -> 17.1.)
+__device__ __forceinline__ void fetch_query(const WarpCtx& w, uint32_t (&qv)[16]) {
   const DecodeParams& p = *w.p;
-  const uint16_t* q0 = p.q + (static_cast<size_t>(w.stream) * p.group + w.head0) * kD;      // [batch][n_q_heads], KV heads in order
+  const int head = w.head0 + (w.lane >> 3);
+  const uint16_t* q0 = p.q + (static_cast<size_t>(w.stream) * p.group + head) * kD + 2 * (w.lane & 3);
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int piece = w.lane + 32 * i, j = piece >> 4, col = piece & 15;
-    const bool on = w.head0 + j < p.group;
-    cp_async16(w.stage0 + kStageBytes + j * kRowPitch + col * 16, q0 + (on ? j * kD + col * 8 : 0), on ? 16u : 0u);
-  }
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  for (int s = 0; s < 16; ++s) qv[s] = head < p.group ? *reinterpret_cast<const uint32_t*>(q0 + 8 * s) : 0u;
 }
 // Query fragments: B operand Q^T[16 channels x 8 columns]; lane (r, c4) holds column r = the hi (r even)
 // or lo (r odd) column of head r / 2 of the head group, channels 16 s + 2 c4 (+1) and 16 s + 8 + 2 c4 (+1), in
 // bf16 (exact rows) and fp16 (quantised tiers).  Both columns of a head hold its query; the parts of the
 // scaled query are formed per key group.
-__device__ __forceinline__ void stage_query(const WarpCtx& w) {
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-  __syncwarp();
-  const uint32_t row = w.stage0 + kStageBytes + (w.lane >> 3) * kRowPitch + (w.lane & 3) * 4;
+__device__ __forceinline__ void stage_query(const WarpCtx& w, const uint32_t (&qv)[16]) {
 #pragma unroll
   for (int s = 0; s < 8; ++s) {
-    const uint32_t v0 = lds32(row + 32 * s), v1 = lds32(row + 32 * s + 16);
+    const uint32_t v0 = qv[2 * s], v1 = qv[2 * s + 1];
     asm volatile("st.shared.v2.u32 [%0], {%1,%2};\n" ::"r"(w.qb_addr + s * 256), "r"(v0), "r"(v1) : "memory");
     const uint32_t h0 = h2_as_u32(__floats2half2_rn(bf16lo_to_f32(v0), bf16hi_to_f32(v0)));
     const uint32_t h1 = h2_as_u32(__floats2half2_rn(bf16lo_to_f32(v1), bf16hi_to_f32(v1)));
@@ -1032,7 +1028,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
       w.pf_pos = first;
     }
   }
-  fetch_query(w);
+  uint32_t qv[16];
+  fetch_query(w, qv);
   if constexpr (!SPARSE) {
     if (lane == 0) {
       s_group[2 * kDecodeWarps + warp] = parts.begin;
@@ -1048,9 +1045,11 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   st.zc = 0.f;
   uint32_t pf[4] = {0, 0, 0, 0};
 
-  // Software pipeline over steps: while step k is computed, step k + 1 is in flight.  The loop
-  // starts on an empty pseudo-unit (level 0) so that the cursor and copy code exists once; while the
-  // first unit's bytes are on their way, that iteration stages the query.
+  // Software pipeline over steps: while step k is computed, step k + 1 is in flight.  The query is staged while the first
+  // step's bytes are on their way: for full reads in front of the loop, at the price of a second copy of the cursor and
+  // copy code, because the staging inside the loop, in a first round on an empty pseudo-unit (level 0), slows every other round
+  // (64 streams of 32,700 tokens 71.1 -> 66.9 us a call, of 100,000 193 -> 183); page-list reads, which walk a few steps per
+  // warp and are short of registers, keep the pseudo-unit.
   Cursor cur;
   cur.item = first - 1;
   cur.first = 0;
@@ -1064,6 +1063,14 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   cur.resmask = 0;
   int sidx = 1;
   bool have = true;
+  if constexpr (!SPARSE) {
+    have = advance<SPARSE>(w, cur);
+    sidx = 0;
+    if (have) issue_step<SPARSE>(w, cur, 0);
+    stage_query(w, qv);
+  } else {
+    stage_query(w, qv);
+  }
   uint32_t phase = 0;             // bit s = parity to wait for on stage s
   bool failed = false;
   float mass_l = 0.f, mass_m = kNegInf;     // (l, m) when the current block began
@@ -1071,7 +1078,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
     Cursor nxt = cur;
     const bool more = advance<SPARSE>(w, nxt);
     if (more) issue_step<SPARSE>(w, nxt, sidx ^ 1);
-    if (cur.level != 0) {
+    if (!SPARSE || cur.level != 0) {
       // bounded wait for this step's bytes
       int spins = 0;
       while (!mbar_try_wait(w.bar0 + 8 * sidx, (phase >> sidx) & 1u)) {
@@ -1102,8 +1109,6 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
         }
       }
       __syncwarp();
-    } else {
-      stage_query(w);
     }
     cur = nxt;
     have = more;
