@@ -619,7 +619,17 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   }
   // every head group of a stream (up to four query heads each) walks the stream's units with warps of its own
   total *= static_cast<size_t>(hg);
-  const size_t target = std::max(L.split_all ? kMinWarpCost / 4 : kMinWarpCost, (total + kTargetWarps - 1) / kTargetWarps);
+  const size_t even = (total + kTargetWarps - 1) / kTargetWarps;
+  size_t target = std::max(L.split_all ? kMinWarpCost / 4 : kMinWarpCost, even);
+  // Rounded to whole warps the streams may come to more than one wave, and a CTA beyond it doubles the call (24 streams of 16,400
+  // tokens at 99 warps each, 149 CTAs, 30.4 us; at 98 21.4): a little more to every warp until they fit.
+  auto warps_of = [&](const Sum& x) { return std::max(1, std::min(static_cast<int>((x.cost + target / 2) / target), x.units)); };
+  for (int i = 0; i < 64 && ns * hg < kTargetWarps; ++i) {
+    int all = 0;
+    for (const Sum& x : sum) all += warps_of(x) * hg;
+    if (all <= kTargetWarps) break;
+    target += target / 64 + 1;
+  }
   // Small workloads: CTAs of its own for every head group, launched as a cluster and merged through distributed shared
   // memory, where all clusters fit the GPU at once and its warps get at most twice what they would get of the whole GPU.
   // Against shared CTAs with rows in global memory and a ticket: 2 streams of 4001 tokens 10.2 -> 7.8 us a call, 64 of
@@ -629,7 +639,7 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   L.cluster = 0;
   if (rough < 2 * static_cast<size_t>(kTargetWarps) * kMinWarpCost) {
     int most = 0;
-    for (int s = 0; s < ns; ++s) most = std::max(most, std::min(static_cast<int>((sum[s].cost + target / 2) / target), sum[s].units));
+    for (const Sum& x : sum) most = std::max(most, warps_of(x));
     int ctas = std::max(1, std::min((most + kDecodeWarps - 1) / kDecodeWarps, kMaxCluster));
     while (ctas > 1 && (c->n_hgroups * ctas > 148 || c->n_hgroups > decode_max_clusters(ctas))) --ctas;
     if (most <= 2 * ctas * kDecodeWarps && c->n_hgroups <= decode_max_clusters(ctas)) L.cluster = ctas;
@@ -637,8 +647,7 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   int w = 0, pos = 0, row = 0, last_nw = 0, stride = 1, stride_inv = 1;
   L.n_units = 0;
   for (int s = 0; s < ns; ++s) {
-    int nw = static_cast<int>((sum[s].cost + target / 2) / target);
-    nw = std::max(1, std::min(nw, sum[s].units));
+    int nw = warps_of(sum[s]);
     if (L.cluster > 0) nw = std::min(std::max(nw, std::min(L.cluster, sum[s].units)), L.cluster * kDecodeWarps);
     else nw = std::min(nw, (c->max_warps - w) / hg - (ns - 1 - s));
     if (nw != last_nw) {

@@ -268,13 +268,16 @@ def _check_lists(rows, levels, n_res, head_groups):
 @pytest.mark.parametrize("batch,n_kv,group,T,residual,fixed", [
     (1, 1, 1, 70, 0.0, None), (2, 2, 8, 13_100, 0.0, None), (2, 1, 8, 27_300, 0.0, None), (4, 1, 8, 16_750, 0.0, None),
     (1, 2, 8, 16_384, 0.01, None), (4, 8, 4, 32_763, 0.10, "newest"), (8, 8, 4, 16_384, 0.10, "newest"), (2, 1, 4, 6000, 0.05, "newest"),
-    (2, 1, 5, 3000, 0.05, "newest"), (3, 2, 3, 2500, 0.03, None), (1, 1, 4, 140_000, 0.02, None)])
+    (2, 1, 5, 3000, 0.05, "newest"), (3, 2, 3, 2500, 0.03, None), (3, 8, 4, 16_400, 0.0, "4 bits"),
+    (12, 8, 4, 4000, 0.0, "4 bits"), (6, 4, 8, 16_400, 0.0, "4 bits"), (1, 1, 4, 140_000, 0.02, None)])
 def test_work_lists_are_complete_and_balanced(batch, n_kv, group, T, residual, fixed):
     B = _binding()
     w = _gqa(T, batch, n_kv, group, policy=W.POLICY_EXTERNAL, residual_fraction=residual)
     rs = np.random.RandomState(T)
     plan = _mixed_plan(rs, (batch, n_kv), T // 64)
-    if fixed:                                       # 256 exact tokens, centroids, exact residual rows
+    if fixed == "4 bits":                           # equal streams, whose warps round up to more than a wave of CTAs
+        plan[:] = 4
+    elif fixed:                                     # 256 exact tokens, centroids, exact residual rows
         plan[:] = 1
         plan[..., -4:] = 16
     gen = torch.Generator(device="cuda")
@@ -296,7 +299,9 @@ def test_work_lists_are_complete_and_balanced(batch, n_kv, group, T, residual, f
             assert torch.allclose(m.sum(-1), torch.ones((), device="cuda"), atol=2e-3)      # residual rows in their blocks
         else:
             g.gkv_decode_attn(0, q, out)
-        _check_lists(g.gkv_debug_export_units(0), levels, n_res, -(-group // 4))
+        rows = g.gkv_debug_export_units(0)
+        _check_lists(rows, levels, n_res, -(-group // 4))
+        assert rows[:, 0].max() < 148 * 16           # one wave of CTAs
 
 
 @pytest.mark.parametrize("levels", [(16,), (16, 8, 4, 2)])
