@@ -26,6 +26,7 @@ constexpr int kTargetWarps = 148 * kDecodeCtasPerSm * kDecodeWarps;   // one res
 // Page-list reads: a stream's pages are split over whole CTAs, as many as fill the GPU once (at most 8)
 int sparse_ctas_per_stream(int n_streams) { return std::max(1, std::min(8, 148 / std::max(n_streams, 1))); }
 constexpr size_t kMinWarpCost = 1000;     // do not split below about one block per warp
+constexpr size_t kFineRows = 48;          // rows of partial results per head group up to which warps get less than a block
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 inline int level_index(int level) { return level == 16 ? 0 : level == 8 ? 1 : level == 4 ? 2 : level == 2 ? 3 : 4; }
@@ -619,8 +620,18 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   }
   // every head group of a stream (up to four query heads each) walks the stream's units with warps of its own
   total *= static_cast<size_t>(hg);
+  // (Where blocks are cut a warp gets as little as a quarter of one, unless that would leave more than kFineRows rows of
+  // partial results to the CTA that merges a head group: then whole blocks' worth.  One stream, 4 bits: 32 rows of 16,400 tokens
+  // 10.3 us a call, 11.4 with half as many; 64 rows of 32,700 tokens 14.7 and 13.5; 127 of 65,000 21.4 and 16.8.)
   const size_t even = (total + kTargetWarps - 1) / kTargetWarps;
-  size_t target = std::max(L.split_all ? kMinWarpCost / 4 : kMinWarpCost, even);
+  size_t least = kMinWarpCost;
+  if (L.split_all) {
+    const size_t fine = std::max(kMinWarpCost / 4, even);
+    size_t rows = 0;
+    for (const Sum& x : sum) rows = std::max(rows, std::min(x.cost / fine, static_cast<size_t>(x.units)) / kDecodeWarps);
+    if (rows <= kFineRows) least = kMinWarpCost / 4;
+  }
+  size_t target = std::max(least, even);
   // Rounded to whole warps the streams may come to more than one wave, and a CTA beyond it doubles the call (24 streams of 16,400
   // tokens at 99 warps each, 149 CTAs, 30.4 us; at 98 21.4): a little more to every warp until they fit.
   auto warps_of = [&](const Sum& x) { return std::max(1, std::min(static_cast<int>((x.cost + target / 2) / target), x.units)); };
