@@ -26,6 +26,8 @@ constexpr int kTargetWarps = 148 * kDecodeCtasPerSm * kDecodeWarps;   // one res
 // Page-list reads: a stream's pages are split over whole CTAs, as many as fill the GPU once (at most 8)
 int sparse_ctas_per_stream(int n_streams) { return std::max(1, std::min(8, 148 / std::max(n_streams, 1))); }
 constexpr size_t kMinWarpCost = 1000;     // do not split below about one block per warp
+constexpr size_t kClusterMore = 850;      // what a cluster's warps may get beyond what they would of the whole GPU
+constexpr size_t kClusterMoreAlone = 400; // the same where there is one head group only
 constexpr size_t kFineRows = 48;          // rows of partial results per head group up to which warps get less than a block
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -641,19 +643,27 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
     if (all <= kTargetWarps) break;
     target += target / 64 + 1;
   }
-  // Small workloads: CTAs of its own for every head group, launched as a cluster and merged through distributed shared
-  // memory, where all clusters fit the GPU at once and its warps get at most twice what they would get of the whole GPU.
-  // Against shared CTAs with rows in global memory and a ticket: 2 streams of 4001 tokens 10.2 -> 7.8 us a call, 64 of
-  // 2000 16.0 -> 12.9, 16 of 9000 17.2 -> 15.2, 64 of 4000 18.2 -> 16.1; two streams of 12,000 tokens at three times the
-  // load 11.9 -> 12.4.  Up to two blocks per warp of the GPU: at 3.5, 16 streams of 32,768 tokens take 30.0 us instead of
-  // 27.6, although 64 of 8000 would take 24.8 instead of 26.4.
+  // CTAs of its own for every head group, launched as a cluster and merged through distributed shared memory, where all
+  // clusters fit the GPU at once and the most laden one's warps get little more than they would of the whole GPU: up to 0.85 of a
+  // block, which takes about as long as the rows in global memory and the ticket that the cluster saves.  A single head group's rows
+  // are merged by a GPU that is otherwise done: 0.4 of a block.  Clusters and shared CTAs, us a call (more, in blocks): 4 streams of
+  // 8200 tokens 9.9 and 10.6 (0.5), 16 of 8200 11.9 and 14.1 (0.5), 24 of 16,400 19.8 and 20.8 (0.6), 64 of 8200 23.1 and 25.0 (0.6),
+  // 12 of 16,400 15.8 and 14.8 (0.7), 16 of 16,400 17.5 and 16.5 (0.9), 8 of 32,700 with eight query heads each 29.9 and 24.7
+  // (1.9); one stream of 8200 10.3 and 9.1 (0.5).
   L.cluster = 0;
-  if (rough < 2 * static_cast<size_t>(kTargetWarps) * kMinWarpCost) {
-    int most = 0;
-    for (const Sum& x : sum) most = std::max(most, warps_of(x));
+  if (c->n_hgroups <= 148) {
+    int most = 0;                              // warps of the most laden stream
+    size_t largest = 0;
+    for (const Sum& x : sum)
+      if (x.cost > largest) {
+        largest = x.cost;
+        most = warps_of(x);
+      }
     int ctas = std::max(1, std::min((most + kDecodeWarps - 1) / kDecodeWarps, kMaxCluster));
     while (ctas > 1 && (c->n_hgroups * ctas > 148 || c->n_hgroups > decode_max_clusters(ctas))) --ctas;
-    if (most <= 2 * ctas * kDecodeWarps && c->n_hgroups <= decode_max_clusters(ctas)) L.cluster = ctas;
+    if (c->n_hgroups <= decode_max_clusters(ctas) && largest / std::min(most, ctas * kDecodeWarps) <=
+                                                             largest / most + (c->n_hgroups > 1 ? kClusterMore : kClusterMoreAlone))
+      L.cluster = ctas;
   }
   int w = 0, pos = 0, row = 0, last_nw = 0, stride = 1, stride_inv = 1;
   L.n_units = 0;
