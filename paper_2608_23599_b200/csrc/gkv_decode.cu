@@ -407,6 +407,7 @@ __device__ __forceinline__ bool load_item_sparse(WarpCtx& w, int pos, Cursor& c)
   const int pages_per_block = kBlock / p.page_tokens;
   const int n_pages = p.n_closed * pages_per_block;
   const int32_t* list = p.page_idx + static_cast<size_t>(w.stream) * p.n_sel;
+  const TableEntry* table = p.table + static_cast<size_t>(w.stream) * p.table_stride;
   while (pos < w.item_end) {
     const int page = list[pos];
     if (page < 0 || page >= n_pages) {
@@ -423,9 +424,9 @@ __device__ __forceinline__ bool load_item_sparse(WarpCtx& w, int pos, Cursor& c)
       mask |= ((1 << tiles_per_page) - 1) << (tiles_per_page * (pg % pages_per_block));
       ++adv;
     }
-    const TableEntry e = w.table[blk];
+    const TableEntry e = table[blk];
     c.item = pos;
-    c.first = page;              // the visit's first page (the centroid gather looks its block up again)
+    c.first = page;              // the visit's first page
     c.sub = 0;
     c.adv = adv;
     c.off256 = e.off256;
@@ -444,8 +445,8 @@ __device__ __forceinline__ bool load_item_sparse(WarpCtx& w, int pos, Cursor& c)
   }
   // pos == item_end (also after skipped entries): the tail, one 16-token tile each for the head group's last four warps
   const int tail_tile = p.warps_per_stream - 1 - w.sparse_rank;
-  if (pos == w.item_end && tail_tile < 4 && 16 * tail_tile < p.n_tail) {
-    const TableEntry e = w.table[p.n_closed];
+  if (pos == w.item_end && static_cast<unsigned>(tail_tile) < static_cast<unsigned>((p.n_tail + 15) >> 4)) {
+    const TableEntry e = table[p.n_closed];
     c.item = pos;
     c.sub = 0;
     c.adv = 1;
@@ -478,8 +479,10 @@ __device__ __forceinline__ bool load_item_sparse(WarpCtx& w, int pos, Cursor& c)
   return true;
 }
 
-// Page-list reads: is the page of token `tok` in the stream's ascending list?
-__device__ __forceinline__ bool page_listed(const DecodeParams& p, int stream, int tok) {
+// Page-list reads: is the page of token `tok` in the stream's ascending list?  (Out of line, and pointers and tests of the page walk
+// made where they are used: the kernel is short of registers, and what it spilled in its step loop cost lists of many small pages
+// 10 %: 64 streams of 100,000 tokens, 6250 pages each of 16 tokens, 262 -> 237 us a call.)
+__device__ __noinline__ bool page_listed(const DecodeParams& p, int stream, int tok) {
   const int32_t* list = p.page_idx + static_cast<size_t>(stream) * p.n_sel;
   const int page = tok / p.page_tokens;
   int lo = 0, hi = p.n_sel;
@@ -559,10 +562,9 @@ __device__ __forceinline__ void issue_step(const WarpCtx& w, const Cursor& c, in
     const uint8_t* src = nullptr;
     const int nrows = c.ntok;
     if (lane < nrows) {
-      int blk;
-      if constexpr (SPARSE) blk = c.first / (kBlock / p.page_tokens);      // c.first = the visit's (range-checked) first page
-      else blk = c.first + lane;
-      src = p.arena + static_cast<size_t>(w.table[blk].off256) * 256 + (is_v ? kRowBytes : 0);
+      uint32_t off = c.off256;                                  // (page-list reads: one block)
+      if constexpr (!SPARSE) off = w.table[c.first + lane].off256;
+      src = p.arena + static_cast<size_t>(off) * 256 + (is_v ? kRowBytes : 0);
     }
     if (lane == 0) mbar_expect_tx(bar, static_cast<uint32_t>(nrows) * kRowBytes);
     __syncwarp();
