@@ -26,6 +26,7 @@ constexpr int kTargetWarps = 148 * kDecodeCtasPerSm * kDecodeWarps;   // one res
 // Page-list reads: a stream's pages are split over whole CTAs, as many as fill the GPU once (at most 8)
 int sparse_ctas_per_stream(int n_streams) { return std::max(1, std::min(8, 148 / std::max(n_streams, 1))); }
 constexpr size_t kMinWarpCost = 1000;     // do not split below about one block per warp
+constexpr int kObserveOverlap = 64;      // CTAs of an observing read up to which its finish overlaps it although there are residual rows
 constexpr size_t kClusterMore = 850;      // what a cluster's warps may get beyond what they would of the whole GPU
 constexpr size_t kClusterMoreAlone = 400; // the same where there is one head group only
 constexpr size_t kFineRows = 48;          // rows of partial results per head group up to which warps get less than a block
@@ -1927,7 +1928,7 @@ int decode_impl(gkv_cache* c, int32_t layer, const void* q, const int32_t* page_
     o.res_cap = c->res_cap;
     o.err_stride = c->max_blocks;
     o.scale = c->scale;
-    CK(c, launch_observe_finish(o, !L.has_residual, st));
+    CK(c, launch_observe_finish(o, !L.has_residual || n_ctas <= kObserveOverlap, st));
   }
   return GKV_OK;
 }

@@ -211,7 +211,7 @@ constexpr uint32_t kStatusInternal = 2u;   // an index check failed inside a ker
 cudaError_t launch_decode(const DecodeParams& p, int n_ctas, bool overlap, cudaStream_t st);
 int decode_max_clusters(int ctas);          // clusters of that many decode CTAs that the GPU holds at once
 cudaError_t launch_units(UnitsParams p, int n_streams, int max_units, cudaStream_t st);
-cudaError_t launch_observe_finish(const ObserveParams& p, bool overlap, cudaStream_t st);      // overlap: not where there are residual rows
+cudaError_t launch_observe_finish(const ObserveParams& p, bool overlap, cudaStream_t st);      // overlap: see the kernel's comment
 cudaError_t launch_encode(const EncodeParams& p, cudaStream_t st);
 cudaError_t launch_ingest(const EncodeParams& p, cudaStream_t st);   // every job reads the bf16 input rows; 16-byte aligned inputs
 cudaError_t launch_stats(const StatsParams& p, cudaStream_t st);
