@@ -445,7 +445,7 @@ __device__ __forceinline__ bool load_item_sparse(WarpCtx& w, int pos, Cursor& c)
   }
   // pos == item_end (also after skipped entries): the tail, one 16-token tile each for the head group's last four warps
   const int tail_tile = p.warps_per_stream - 1 - w.sparse_rank;
-  if (pos == w.item_end && static_cast<unsigned>(tail_tile) < static_cast<unsigned>((p.n_tail + 15) >> 4)) {
+  if (pos == w.item_end && tail_tile < 4 && 16 * tail_tile < p.n_tail) {
     const TableEntry e = table[p.n_closed];
     c.item = pos;
     c.sub = 0;
@@ -479,9 +479,9 @@ __device__ __forceinline__ bool load_item_sparse(WarpCtx& w, int pos, Cursor& c)
   return true;
 }
 
-// Page-list reads: is the page of token `tok` in the stream's ascending list?  (Out of line, and pointers and tests of the page walk
-// made where they are used: the kernel is short of registers, and what it spilled in its step loop cost lists of many small pages
-// 10 %: 64 streams of 100,000 tokens, 6250 pages each of 16 tokens, 262 -> 237 us a call.)
+// Page-list reads: is the page of token `tok` in the stream's ascending list?  (Out of line, and the page walk's table pointer
+// made where it is used: the kernel is short of registers, and what it spilled in its step loop cost lists of many small pages
+// 10 %: 64 streams of 100,000 tokens, 6250 pages each of 16 tokens, 262 -> 235 us a call.)
 __device__ __noinline__ bool page_listed(const DecodeParams& p, int stream, int tok) {
   const int32_t* list = p.page_idx + static_cast<size_t>(stream) * p.n_sel;
   const int page = tok / p.page_tokens;
