@@ -1048,10 +1048,9 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   uint32_t pf[4] = {0, 0, 0, 0};
 
   // Software pipeline over steps: while step k is computed, step k + 1 is in flight.  The query is staged while the first
-  // step's bytes are on their way: for full reads in front of the loop, at the price of a second copy of the cursor and
-  // copy code, because the staging inside the loop, in a first round on an empty pseudo-unit (level 0), slows every other round
-  // (64 streams of 32,700 tokens 71.1 -> 66.9 us a call, of 100,000 193 -> 183); page-list reads, which walk a few steps per
-  // warp and are short of registers, keep the pseudo-unit.
+  // step's bytes are on their way, in front of the loop, at the price of a second copy of the cursor and copy code: staged
+  // inside the loop, in a first round on an empty pseudo-unit, it slows every other round (64 streams of 32,700 tokens 71.1 -> 66.9 us
+  // a call, of 100,000 193 -> 183; by page list, a quarter of the 64-token pages of 100,000 tokens 132.3 -> 128.3).
   Cursor cur;
   cur.item = first - 1;
   cur.first = 0;
@@ -1063,16 +1062,10 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   cur.tmask = 0;
   cur.off256 = 0;
   cur.resmask = 0;
-  int sidx = 1;
-  bool have = true;
-  if constexpr (!SPARSE) {
-    have = advance<SPARSE>(w, cur);
-    sidx = 0;
-    if (have) issue_step<SPARSE>(w, cur, 0);
-    stage_query(w, qv);
-  } else {
-    stage_query(w, qv);
-  }
+  int sidx = 0;
+  bool have = advance<SPARSE>(w, cur);
+  if (have) issue_step<SPARSE>(w, cur, 0);
+  stage_query(w, qv);
   uint32_t phase = 0;             // bit s = parity to wait for on stage s
   bool failed = false;
   float mass_l = 0.f, mass_m = kNegInf;     // (l, m) when the current block began
@@ -1080,38 +1073,36 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
     Cursor nxt = cur;
     const bool more = advance<SPARSE>(w, nxt);
     if (more) issue_step<SPARSE>(w, nxt, sidx ^ 1);
-    if (!SPARSE || cur.level != 0) {
-      // bounded wait for this step's bytes
-      int spins = 0;
-      while (!mbar_try_wait(w.bar0 + 8 * sidx, (phase >> sidx) & 1u)) {
-        if (++spins > kWaitSpins) {
-          failed = true;
-          break;
-        }
+    // bounded wait for this step's bytes
+    int spins = 0;
+    while (!mbar_try_wait(w.bar0 + 8 * sidx, (phase >> sidx) & 1u)) {
+      if (++spins > kWaitSpins) {
+        failed = true;
+        break;
       }
-      if (__any_sync(kFull, failed)) break;
-      phase ^= 1u << sidx;
-      if constexpr (MASS) {
-        if (cur.sub == 0) {
-          mass_l = st.l;
-          mass_m = st.m;
-        }
-      }
-      compute_step<SPARSE, MASS>(w, cur, sidx, st, pf);
-      if constexpr (MASS) {
-        // A block (or the partial block) is done: what it added to the lane's running sum is the
-        // sum now minus the sum at its start brought to the current max.
-        if (cur.sub == cur.nsub - 1 && cur.level != 1 && cur.level != 17) {
-          float d0 = st.l - ((mass_m == kNegInf) ? 0.f : mass_l * fast_exp2(mass_m - st.m));
-#pragma unroll
-          for (int d = 4; d <= 16; d <<= 1) d0 += __shfl_xor_sync(kFull, d0, d);
-          if (lane < 4)
-            p.mass_raw[(static_cast<size_t>(w.stream) * p.mass_stride + cur.first) * kMaxHeadsPerKv + w.head0 + lane] =
-                make_float2(st.m, fmaxf(d0, 0.f));
-        }
-      }
-      __syncwarp();
     }
+    if (__any_sync(kFull, failed)) break;
+    phase ^= 1u << sidx;
+    if constexpr (MASS) {
+      if (cur.sub == 0) {
+        mass_l = st.l;
+        mass_m = st.m;
+      }
+    }
+    compute_step<SPARSE, MASS>(w, cur, sidx, st, pf);
+    if constexpr (MASS) {
+      // A block (or the partial block) is done: what it added to the lane's running sum is the
+      // sum now minus the sum at its start brought to the current max.
+      if (cur.sub == cur.nsub - 1 && cur.level != 1 && cur.level != 17) {
+        float d0 = st.l - ((mass_m == kNegInf) ? 0.f : mass_l * fast_exp2(mass_m - st.m));
+#pragma unroll
+        for (int d = 4; d <= 16; d <<= 1) d0 += __shfl_xor_sync(kFull, d0, d);
+        if (lane < 4)
+          p.mass_raw[(static_cast<size_t>(w.stream) * p.mass_stride + cur.first) * kMaxHeadsPerKv + w.head0 + lane] =
+              make_float2(st.m, fmaxf(d0, 0.f));
+      }
+    }
+    __syncwarp();
     cur = nxt;
     have = more;
     sidx ^= 1;
