@@ -42,11 +42,9 @@ UNIT = "ctx tokens/s"
 NOMINAL_HBM_GBS = 8000.0
 FALLBACK_HBM_GBS = 6650.0
 
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch of the workload's dominant kernel from an ncu
-# capture (profiles/ holds the summaries); None = not captured for that workload.
-# dram__bytes_read.sum + dram__bytes_write.sum of one launch of the dominant kernel (ncu captures
-# summarised under profiles/): config 2 330.0 MB read + 3.8 MB written, config 4 386.4 + 6.7 MB
-DRAM_TRAFFIC_PER_LAUNCH = {"cfg2_llama8b_append": 333.8e6, "cfg4_mla_1m": 382.3e6}
+# DRAM bytes read and written by one launch of the workload's dominant kernel (dram__bytes.sum of the ncu captures
+# summarised under profiles/); None = not captured for that workload.
+DRAM_TRAFFIC_PER_LAUNCH = {"cfg2_llama8b_append": 335.4e6, "cfg4_mla_1m": 383.4e6}
 
 
 def dominant_kernel(w) -> str:

@@ -5,7 +5,7 @@
 // The arithmetic of every stored bit is the one of the block encoder used for demotions:
 //   s = fp16((max - min) / (2^b - 1)), z = fp16(min) (saturating), code = clamp(rint((x - z) * (1 / s)), 0, 2^b - 1)
 //   centroid = bf16(sequential fp32 sum over the 64 tokens * 1/64)
-// (clamping before the rounding gives the same integer: both bounds are integers).  What differs
+// (the codes are clamped behind the rounding: both bounds are integers, so the order does not matter).  What differs
 // is how the work is laid out.  The packed codes are stored in the order of the attention
 // kernel's tensor-core fragments, so the block is read from shared memory with ldmatrix, which
 // hands every lane exactly the values whose codes it has to pack: keys as the A fragment of a
@@ -17,9 +17,11 @@
 // group by one lane and handed to the others.
 //
 // One CTA (8 warps: 4 for keys, 4 for values) per block, four CTAs per SM, which take turns loading and encoding; the next
-// block's rows are on their way to L2 while the current one is encoded.  Bound by instruction issue (14.8 instructions
-// per value and lane, 63 % of the issue slots; 22 and three double-buffered CTAs per SM before packed fp32 arithmetic):
-// 8192 blocks of the staircase mixture 109 us (117 before), 24,528 in one launch 273 us, 45 us at the measured copy bandwidth.
+// block's rows are on their way to L2 while the current one is encoded.  No single limit: 14.8 instructions per value and lane
+// take 63 % of the issue slots and 38 % of the memory's rate, and the warps that wait do so in like parts for their turn, for the
+// barriers between loading and encoding, for shared memory and for the packed fp32 pipe (22 instructions and three
+// double-buffered CTAs per SM before packed arithmetic).  8192 blocks of the staircase mixture 109 us (117 before; 351 MB, 54 us
+// at the measured copy bandwidth), 24,528 in one launch 273 us (1.05 GB, 161 us).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 

@@ -22,8 +22,8 @@ struct alignas(16) TableEntry {
 // lists, all of one stream; `stream` is the index of the warp's head group (up to four query heads of
 // one KV head): stream * head_groups + group number.  A unit is one item or a run of consecutive centroid blocks:
 // `first item | run << 24`.  Items: [0, n_closed) closed blocks, n_closed = tail block,
-// n_closed + 1 + j = residual group j (16 residual rows each).  (The MLA kernel uses the same
-// struct per CTA with item_begin / item_end as a plain item range.)
+// n_closed + 1 + j = residual group j (16 residual rows each).  (The MLA kernel uses the same struct for every quad of warps,
+// four to a CTA, with item_begin / item_end as positions in quarter items: 4 * item + quarter.)
 struct alignas(16) WarpDesc {
   int32_t stream;      // -1 = idle warp
   int32_t item_begin;
