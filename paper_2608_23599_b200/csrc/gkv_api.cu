@@ -26,7 +26,8 @@ constexpr int kTargetWarps = 148 * kDecodeCtasPerSm * kDecodeWarps;   // one res
 // Page-list reads: a stream's pages are split over whole CTAs, as many as fill the GPU once (at most 8)
 int sparse_ctas_per_stream(int n_streams) { return std::max(1, std::min(8, 148 / std::max(n_streams, 1))); }
 constexpr size_t kMinWarpCost = 1000;     // do not split below about one block per warp
-constexpr int kObserveOverlap = 64;      // CTAs of an observing read up to which its finish overlaps it although there are residual rows
+constexpr int kObserveOverlap = 64;       // CTAs of an observing read up to which its finish overlaps it whatever its residual rows
+constexpr int kObserveRows = 500;         // residual rows of a stream, and a tenth of all, up to which it overlaps any
 constexpr size_t kClusterMore = 850;      // what a cluster's warps may get beyond what they would of the whole GPU
 constexpr size_t kClusterMoreAlone = 400; // the same where there is one head group only
 constexpr size_t kFineRows = 48;          // rows of partial results per head group up to which warps get less than a block
@@ -697,6 +698,16 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   }
   L.n_warps = static_cast<int>(align_up(w, kDecodeWarps));
   L.desc_dirty = false;
+}
+
+// So few exact residual rows that an observing read's finish overlaps the read whatever it leaves of the GPU.
+bool few_residual_rows(const gkv_cache* c, const LayerState& L) {
+  int total = 0, most = 0;
+  for (int s = 0; L.has_residual && s < c->n_streams; ++s) {
+    total += L.res_count_h[s];
+    most = std::max(most, L.res_count_h[s]);
+  }
+  return total <= 10 * kObserveRows && most <= kObserveRows;
 }
 
 // Cost of a unit of the layer's lists, by class.
@@ -1928,7 +1939,7 @@ int decode_impl(gkv_cache* c, int32_t layer, const void* q, const int32_t* page_
     o.res_cap = c->res_cap;
     o.err_stride = c->max_blocks;
     o.scale = c->scale;
-    CK(c, launch_observe_finish(o, !L.has_residual || n_ctas <= kObserveOverlap, st));
+    CK(c, launch_observe_finish(o, n_ctas <= kObserveOverlap || few_residual_rows(c, L), st));
   }
   return GKV_OK;
 }

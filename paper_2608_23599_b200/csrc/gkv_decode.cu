@@ -1507,12 +1507,14 @@ __device__ __forceinline__ void finish_certificate(const ObserveParams& p, int h
 // What an observing read leaves to do: CTAs [0, n_cert) make one query head's certificate each, the others
 // finish the block masses.  Bound by latency: both parts read what the decode launch has just written, so they
 // share one launch, which overlaps that launch's tail (with two launches one after the other and no
-// overlap an observing call over 8200 tokens of 16 streams took 28.9 us, with this one 21.2).  Not where there are residual
+// overlap an observing call over 8200 tokens of 16 streams took 28.9 us, with this one 21.2).  Not where there are many residual
 // rows and the read fills the GPU: an overlapped launch's CTAs crowd the first SMs that the decode kernel leaves, whose L1 is what
 // its 225 KB of shared memory left over, and the rows' pairs, looked up block by block, live off L1: 52,000 rows of 64 streams of
 // 8200 tokens 99 us a call overlapped, 30 not; 105,000 rows of 32 streams of 32,700 tokens 113 and 38.  SMs that the read leaves idle
 // have all of theirs, 16 streams of 4000 tokens 21.8 overlapped, 24.7 not, and up to 64 CTAs (kObserveOverlap) that was the faster
 // at every size; with 96 a call of 96 streams was 24.7 and 25.9 at 4000 tokens, but 45.2 and 26.4 where it writes certificates.
+// Few rows (up to 500 a stream and 5000 in all, kObserveRows) are no matter: 24 streams of 6154 tokens with 1 % of them 16.0 us a call
+// overlapped, 18.5 not; 4 streams of 26,569 tokens with eight query heads and 3 %, 800 rows each, 38.9 and 28.5.
 __global__ void __launch_bounds__(kObsThreads) observe_finish_kernel(const __grid_constant__ ObserveParams p) {
   asm volatile("griddepcontrol.wait;\n" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
