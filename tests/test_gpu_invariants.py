@@ -334,6 +334,35 @@ def test_long_context_lists(n_closed, levels):
         assert float((out - listed).norm() / listed.norm()) < 1e-4
 
 
+# ---- the finish of an observing read ---------------------------------------------------------------------------
+@pytest.mark.parametrize("n_kv,n_res", [(9, 500), (9, 501), (10, 500), (11, 455)])
+def test_observing_read_of_a_full_gpu_with_residual_rows(n_kv, n_res):
+    """On both sides of the lines (500 rows of a stream, 5000 in all) beyond which the finish waits for the read's end: calls
+    one behind another, without a wait between them, give the same bits as one alone, and every stream's masses add up
+    to 1 (fp32 sums of 158 positive masses of relative error 1e-3 at most: 2e-3)."""
+    B = _binding()
+    T = 10_033
+    w = _gqa(T, 1, n_kv, 4, policy=W.POLICY_STAIRCASE, stair_tokens=(64, 0, -1, 0), residual_fraction=(n_res + 0.5) / T)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n_res)
+    k = torch.randn((1, T, n_kv, 128), generator=gen, device="cuda").to(torch.bfloat16)
+    mass = torch.softmax(torch.randn((1, n_kv, T), generator=gen, device="cuda"), -1)
+    g = B.Cache(B.config_from_workload(w))
+    g.gkv_append_demote(0, k, k, token_mass=mass)
+    q = torch.randn((1, n_kv * 4, 128), generator=gen, device="cuda").to(torch.bfloat16)
+    out = torch.empty((1, n_kv * 4, 128), device="cuda")
+    m = [torch.full((1, n_kv, -(-T // 64)), -1.0, device="cuda") for _ in range(5)]
+    c = [torch.full((1, n_kv * 4), -1.0, device="cuda") for _ in range(5)]
+    for i in range(5):
+        g.gkv_decode_attn_observe(0, q, out, None, m[i], c[i])
+        if i == 0:
+            torch.cuda.synchronize()
+    assert [len(g.gkv_debug_export_residual(0, 0, h)) for h in range(n_kv)] == [n_res] * n_kv
+    assert g.gkv_debug_export_units(0)[:, 0].max() >= 65 * 16
+    assert torch.allclose(m[0].sum(-1), torch.ones((), device="cuda"), atol=2e-3) and float(m[0].min()) >= 0.0
+    assert all(torch.equal(m[0], x) for x in m[1:]) and all(torch.equal(c[0], x) for x in c[1:]) and float(c[0].min()) > 0.0
+
+
 # ---- page-locked host memory -----------------------------------------------------------------------------------
 def _centroid_cache(B, layers, batch, ctx):
     return B.Cache(B.make_config(layers, batch, 32, 8, 128, 128, ctx, stair_tokens=(0, 0, 0, 0)))
