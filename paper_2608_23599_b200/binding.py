@@ -62,6 +62,7 @@ class GkvError(RuntimeError):
 
 
 _lib = None
+_call = None       # the extension that makes a decode step's calls (csrc/gkv_call.cpp)
 
 
 def lib_path() -> str:
@@ -70,7 +71,7 @@ def lib_path() -> str:
 
 def load():
     """Load libgkv.so (building it is the job of ``build()`` / ``__graft_entry__.build``)."""
-    global _lib
+    global _lib, _call
     if _lib is not None:
         return _lib
     path = lib_path()
@@ -109,7 +110,10 @@ def load():
     for name in EXPORTS:
         if name != "gkv_strerror":
             getattr(lib, name).restype = C.c_int
-    _lib = lib
+    from . import _gkv_call
+    _gkv_call.bind(*(C.cast(f, vp).value for f in (lib.gkv_append_demote, lib.gkv_decode_attn, lib.gkv_decode_attn_observe,
+                                                   lib.gkv_quest_select)))
+    _lib, _call = lib, _gkv_call
     return lib
 
 
@@ -150,7 +154,8 @@ def _ptr(t) -> Optional[int]:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # torch.cuda.current_stream().cuda_stream without the Stream object in between
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _check(rc: int, what: str, allow=()):
@@ -245,20 +250,26 @@ class Cache:
         if level_plan is not None:
             self._plan_keep = level_plan = level_plan.astype("int8", copy=False)
             plan_ptr = level_plan.ctypes.data
-        return _check(load().gkv_append_demote(self.handle, layer, _ptr(k_new), _ptr(v_new), n_new,
-                                               _ptr(token_mass), plan_ptr, self._st()),
-                      "gkv_append_demote", allow=(ERR_RANGE, ERR_BUDGET))
+        rc = _call.append(self.handle, layer, k_new, v_new, n_new, token_mass, plan_ptr, self._st())
+        if rc is NotImplemented:
+            rc = load().gkv_append_demote(self.handle, layer, _ptr(k_new), _ptr(v_new), n_new, _ptr(token_mass), plan_ptr, self._st())
+        return rc if rc == OK else _check(rc, "gkv_append_demote", allow=(ERR_RANGE, ERR_BUDGET))
 
     def gkv_decode_attn(self, layer, q, out, lse=None, page_idx=None, n_sel=0):
-        return _check(load().gkv_decode_attn(self.handle, layer, _ptr(q), _ptr(page_idx), n_sel, _ptr(out),
-                                             _ptr(lse), self._st()), "gkv_decode_attn")
+        rc = _call.decode(self.handle, layer, q, page_idx, n_sel, out, lse, self._st())
+        if rc is NotImplemented:
+            rc = load().gkv_decode_attn(self.handle, layer, _ptr(q), _ptr(page_idx), n_sel, _ptr(out), _ptr(lse), self._st())
+        return rc if rc == OK else _check(rc, "gkv_decode_attn")
 
     def gkv_decode_attn_observe(self, layer, q, out, lse=None, block_mass=None, certificate=None):
         """Full-context decode that also observes the attention mass of every block and updates the
         cache's running masses (block_mass: device fp32 [batch][n_kv_heads][ceil(ctx / 64)] or None;
         certificate: device fp32 [batch][n_q_heads] or None, the error certificate of this query)."""
-        return _check(load().gkv_decode_attn_observe(self.handle, layer, _ptr(q), _ptr(out), _ptr(lse), _ptr(block_mass),
-                                                     _ptr(certificate), self._st()), "gkv_decode_attn_observe")
+        rc = _call.observe(self.handle, layer, q, out, lse, block_mass, certificate, self._st())
+        if rc is NotImplemented:
+            rc = load().gkv_decode_attn_observe(self.handle, layer, _ptr(q), _ptr(out), _ptr(lse), _ptr(block_mass),
+                                                _ptr(certificate), self._st())
+        return rc if rc == OK else _check(rc, "gkv_decode_attn_observe")
 
     def gkv_debug_export_bounds(self, layer):
         """Per-block certificate bounds as numpy [batch][n_kv_heads][n_closed][4] (kappa, delta, max |v|, 0)."""
@@ -311,10 +322,14 @@ class Cache:
         return out
 
     def gkv_quest_select(self, layer, q, budget_tokens, page_idx_out) -> int:
-        n = C.c_int32(0)
-        _check(load().gkv_quest_select(self.handle, layer, _ptr(q), budget_tokens, _ptr(page_idx_out), C.byref(n),
-                                       self._st()), "gkv_quest_select")
-        return n.value
+        res = _call.select(self.handle, layer, q, budget_tokens, page_idx_out, self._st())
+        if res is NotImplemented:
+            n = C.c_int32(0)
+            rc = load().gkv_quest_select(self.handle, layer, _ptr(q), budget_tokens, _ptr(page_idx_out), C.byref(n), self._st())
+            res = rc, n.value
+        if res[0] != OK:
+            _check(res[0], "gkv_quest_select")
+        return res[1]
 
     def gkv_quest_select_static(self, layer, q, budget_tokens, page_idx_out) -> int:
         """gkv_quest_select with its score scratch in the library's fixed device array: for callers

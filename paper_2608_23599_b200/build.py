@@ -4,10 +4,13 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libgkv.so")
+CALL_SOURCE = os.path.join(CSRC, "gkv_call.cpp")         # the binding's extension: a decode step's calls without ctypes
+CALL_LIB = os.path.join(HERE, "_gkv_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["gkv_api.cu", "gkv_decode.cu", "gkv_units.cu", "gkv_pack.cu", "gkv_ingest.cu", "gkv_quest.cu", "gkv_rdplan.cu", "gkv_mla.cu", "gkv_mla_decode.cu"]
 HEADERS = ["gkv_internal.h", "gkv_layout.cuh", "gkv_mla.h", os.path.join("..", "..", "include", "gkv.h")]
 NVCC_FLAGS = [
@@ -22,11 +25,10 @@ def _nvcc() -> str:
 
 
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS] + [os.path.abspath(__file__)]
-    return any(os.path.getmtime(d) > t for d in deps)
+    def stale(lib, deps):
+        return not os.path.exists(lib) or any(os.path.getmtime(d) > os.path.getmtime(lib) for d in deps)
+    own = os.path.abspath(__file__)
+    return stale(LIB, [os.path.join(CSRC, s) for s in SOURCES + HEADERS] + [own]) or stale(CALL_LIB, [CALL_SOURCE, own])
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -51,6 +53,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError(f"nvcc failed on {src}")
     cmd = [_nvcc(), "-shared", "-o", LIB, *objs, "-Xcompiler", "-fPIC", "-lpthread"]
     subprocess.run(cmd, check=True)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", f"-I{sysconfig.get_path('include')}",
+                    CALL_SOURCE, "-o", CALL_LIB], check=True)
     return LIB
 
 
