@@ -12,8 +12,8 @@
 // [16 tokens x 16 channels] tile, values as the A fragment of the transposed tile.  A lane then
 // builds its 32-bit code words in registers and stores them with 8- or 16-byte stores; nothing is
 // exchanged through shared memory except the per-token error sums of the two key warps that share
-// a token.  Group minima / maxima are taken on packed bf16 pairs (exact) with three shuffles over
-// the eight lanes that share a group; the division for scale and reciprocal is done once per
+// a token.  Group minima / maxima are taken on packed bf16 pairs (exact), joined over the eight lanes that
+// share a group by exchanges that halve what a lane carries; the division for scale and reciprocal is done once per
 // group by one lane and handed to the others.
 //
 // One CTA (8 warps: 4 for keys, 4 for values) per block, four CTAs per SM, which take turns loading and encoding; the next
@@ -21,7 +21,8 @@
 // take 63 % of the issue slots and 38 % of the memory's rate, and the warps that wait do so in like parts for their turn, for the
 // barriers between loading and encoding, for shared memory and for the packed fp32 pipe (22 instructions and three
 // double-buffered CTAs per SM before packed arithmetic).  8192 blocks of the staircase mixture 109 us (117 before; 351 MB, 54 us
-// at the measured copy bandwidth), 24,528 in one launch 273 us (1.05 GB, 161 us).
+// at the measured copy bandwidth), 24,528 in one launch 273 us (1.05 GB, 161 us); extremes by halving exchanges (14 shuffles for a warp's
+// groups instead of 48) and parameters kept as fp32 pairs take another 7 % off: prompts of 2 x 32,768 blocks 1264 -> 1199 us a pass.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -36,7 +37,7 @@ constexpr int kInTensor = kBlock * kInRow;        // 17408
 constexpr int kInBuf = 2 * kInTensor;             // keys, values
 constexpr int kInThreads = 256;
 constexpr int kInCtas = 4;                         // CTAs per SM
-constexpr int kInSmem = kInBuf + (256 + 128 + 16) * static_cast<int>(sizeof(float)) + 8 * 32 * 16;   // + the warps' group parameters
+constexpr int kInSmem = kInBuf + (256 + 128 + 16) * static_cast<int>(sizeof(float)) + 8 * 64 * 16;   // + the warps' group parameters
 constexpr float kMagic = 12582912.f;              // 1.5 * 2^23: x + kMagic rounds x to an integer (ties to even)
 constexpr uint32_t kMagicBits = 0x4B400000u;
 constexpr uint32_t kFullI = 0xffffffffu;
@@ -183,9 +184,15 @@ __device__ __forceinline__ uint4 i_pack_params(const GroupParams& g0, const Grou
 }
 __device__ __forceinline__ float i_h_lo(uint32_t u) { return __half2float(__ushort_as_half(static_cast<unsigned short>(u & 0xffffu))); }
 __device__ __forceinline__ float i_h_hi(uint32_t u) { return __half2float(__ushort_as_half(static_cast<unsigned short>(u >> 16))); }
-__device__ __forceinline__ PairParams i_pair_params(const uint4& P, uint64_t one) {
-  const uint32_t a = P.x ^ 0x80008000u, b = P.z ^ 0x80008000u;
-  return PairParams{i_pair(i_h_lo(a), i_h_lo(b)), i_pair(i_h_hi(a), i_h_hi(b)), i_pair(__uint_as_float(P.y), __uint_as_float(P.w)), one};
+// The same for the packed arithmetic, as fp32, so that nothing is converted for every register that uses them: two 16-byte records,
+// {-scale, -scale, -zero, -zero} and {reciprocal, reciprocal, -, -}.
+__device__ __forceinline__ void i_put_pair_params(uint4* at, const GroupParams& g0, const GroupParams& g1) {
+  at[0] = make_uint4(__float_as_uint(-g0.s), __float_as_uint(-g1.s), __float_as_uint(-g0.z), __float_as_uint(-g1.z));
+  *reinterpret_cast<uint2*>(at + 1) = make_uint2(__float_as_uint(g0.inv), __float_as_uint(g1.inv));
+}
+__device__ __forceinline__ PairParams i_pair_params(const uint4* at, uint64_t one) {
+  const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(at);
+  return PairParams{a.x, a.y, *reinterpret_cast<const unsigned long long*>(at + 1), one};
 }
 
 // Keys of one half (32 tokens) x 64 channels.  ldmatrix hands a lane, per 16-token tile and slice of
@@ -280,30 +287,41 @@ __device__ __noinline__ bool ingest_keys_wide(uint32_t tile_k, uint8_t* half_bas
   return g0.range || g1.range;
 }
 
+// Extremes of eight pairs over the eight lanes r that hold parts of them; lane r gets pair r's.  Every exchange halves what a
+// lane still carries: 14 shuffles, where reducing each pair in all lanes takes 48.
+__device__ __forceinline__ void i_extremes(uint32_t (&mn)[8], uint32_t (&mx)[8], int lane, uint32_t& my_mn, uint32_t& my_mx) {
+#pragma unroll
+  for (int n = 4; n > 0; n >>= 1) {                 // n pairs stay: lane bit 4, 3, 2 = bit 2, 1, 0 of r
+    const bool up = (lane & (4 * n)) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      mn[i] = i_min2(up ? mn[i + n] : mn[i], __shfl_xor_sync(kFullI, up ? mn[i] : mn[i + n], 4 * n));
+      mx[i] = i_max2(up ? mx[i + n] : mx[i], __shfl_xor_sync(kFullI, up ? mx[i] : mx[i + n], 4 * n));
+    }
+  }
+  my_mn = mn[0];
+  my_mx = mx[0];
+}
+
 template <int BITS>
 __device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base, int half, int chh, int lane, uint4* prm, uint64_t one, float (&e)[2][2]) {
   const int r = lane >> 2, c4 = lane & 3, mi = lane >> 3;
   const uint32_t ld = tile_k + (32 * half + (mi & 1) * 8 + (lane & 7)) * kInRow + (64 * chh + (mi >> 1) * 8) * 2;
-  uint32_t my_mn = 0u, my_mx = 0u;
-#pragma unroll 1
-  for (int sl = 0; sl < 4; ++sl) {
-    uint32_t x0[4], x1[4];
-    i_ldm4(ld + sl * 32, x0);
-    i_ldm4(ld + 16 * kInRow + sl * 32, x1);
+  uint32_t my_mn, my_mx;
+  {
+    uint32_t mn[8], mx[8];
 #pragma unroll
-    for (int ah = 0; ah < 2; ++ah) {
-      uint32_t mn = i_min2(i_min2(x0[2 * ah], x0[2 * ah + 1]), i_min2(x1[2 * ah], x1[2 * ah + 1]));
-      uint32_t mx = i_max2(i_max2(x0[2 * ah], x0[2 * ah + 1]), i_max2(x1[2 * ah], x1[2 * ah + 1]));
+    for (int sl = 0; sl < 4; ++sl) {
+      uint32_t x0[4], x1[4];
+      i_ldm4(ld + sl * 32, x0);
+      i_ldm4(ld + 16 * kInRow + sl * 32, x1);
 #pragma unroll
-      for (int d = 4; d <= 16; d <<= 1) {
-        mn = i_min2(mn, __shfl_xor_sync(kFullI, mn, d));
-        mx = i_max2(mx, __shfl_xor_sync(kFullI, mx, d));
-      }
-      if (r == 2 * sl + ah) {
-        my_mn = mn;
-        my_mx = mx;
+      for (int ah = 0; ah < 2; ++ah) {
+        mn[2 * sl + ah] = i_min2(i_min2(x0[2 * ah], x0[2 * ah + 1]), i_min2(x1[2 * ah], x1[2 * ah + 1]));
+        mx[2 * sl + ah] = i_max2(i_max2(x0[2 * ah], x0[2 * ah + 1]), i_max2(x1[2 * ah], x1[2 * ah + 1]));
       }
     }
+    i_extremes(mn, mx, lane, my_mn, my_mx);
   }
   const GroupParams g0 = i_params<BITS>(i_lo(my_mn), i_lo(my_mx)), g1 = i_params<BITS>(i_hi(my_mn), i_hi(my_mx));
   if (__any_sync(kFullI, g0.range || g1.range)) return ingest_keys_wide<BITS>(tile_k, half_base, half, chh, lane, prm, e);
@@ -315,7 +333,7 @@ __device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base,
     rec[0] = static_cast<uint32_t>(g0.z_bits) | (static_cast<uint32_t>(g1.z_bits) << 16);
     rec[4] = static_cast<uint32_t>(g0.s_bits) | (static_cast<uint32_t>(g1.s_bits) << 16);
   }
-  prm[r * 4 + c4] = i_pack_params(g0, g1);
+  i_put_pair_params(prm + (r * 4 + c4) * 2, g0, g1);
   __syncwarp();
   constexpr int SL = BITS == 2 ? 2 : 1;             // slices that fill whole words
   uint64_t err[2][2] = {{0ull, 0ull}, {0ull, 0ull}};      // [tile][a & 1], the lane's two channels side by side
@@ -330,8 +348,7 @@ __device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base,
       i_ldm4(ld + 16 * kInRow + sl * 32, x[1]);
 #pragma unroll
       for (int ah = 0; ah < 2; ++ah) {
-        const uint4 P = prm[(2 * sl + ah) * 4 + c4];
-        const PairParams g = i_pair_params(P, one);
+        const PairParams g = i_pair_params(prm + ((2 * sl + ah) * 4 + c4) * 2, one);
         const int wi = BITS == 8 ? ah : 0;
 #pragma unroll
         for (int t = 0; t < 2; ++t)
@@ -462,26 +479,21 @@ template <int BITS>
 __device__ __forceinline__ bool ingest_values(uint32_t ld, uint8_t* vp, uint8_t* codes, int lane, uint4* prm, uint64_t one, float (&e)[2][2],
                                               float (&n)[2][2]) {
   const int r = lane >> 2, c4 = lane & 3;
-  uint32_t my_mn = 0u, my_mx = 0u;
-#pragma unroll 1
-  for (int g = 0; g < 4; ++g) {
-    uint32_t x0[4], x1[4];
-    i_ldm4t(ld + g * 64, x0);
-    i_ldm4t(ld + g * 64 + 32, x1);
+  uint32_t my_mn, my_mx;
+  {
+    uint32_t mn[8], mx[8];
 #pragma unroll
-    for (int ah = 0; ah < 2; ++ah) {
-      uint32_t mn = i_min2(i_min2(x0[2 * ah], x0[2 * ah + 1]), i_min2(x1[2 * ah], x1[2 * ah + 1]));
-      uint32_t mx = i_max2(i_max2(x0[2 * ah], x0[2 * ah + 1]), i_max2(x1[2 * ah], x1[2 * ah + 1]));
+    for (int g = 0; g < 4; ++g) {
+      uint32_t x0[4], x1[4];
+      i_ldm4t(ld + g * 64, x0);
+      i_ldm4t(ld + g * 64 + 32, x1);
 #pragma unroll
-      for (int d = 4; d <= 16; d <<= 1) {
-        mn = i_min2(mn, __shfl_xor_sync(kFullI, mn, d));
-        mx = i_max2(mx, __shfl_xor_sync(kFullI, mx, d));
-      }
-      if (r == 2 * g + ah) {
-        my_mn = mn;
-        my_mx = mx;
+      for (int ah = 0; ah < 2; ++ah) {
+        mn[2 * g + ah] = i_min2(i_min2(x0[2 * ah], x0[2 * ah + 1]), i_min2(x1[2 * ah], x1[2 * ah + 1]));
+        mx[2 * g + ah] = i_max2(i_max2(x0[2 * ah], x0[2 * ah + 1]), i_max2(x1[2 * ah], x1[2 * ah + 1]));
       }
     }
+    i_extremes(mn, mx, lane, my_mn, my_mx);
   }
   const GroupParams g0 = i_params<BITS>(i_lo(my_mn), i_lo(my_mx)), g1 = i_params<BITS>(i_hi(my_mn), i_hi(my_mx));
   if (__any_sync(kFullI, g0.range || g1.range)) return ingest_values_wide<BITS>(ld, vp, codes, lane, prm, e, n);
@@ -492,7 +504,7 @@ __device__ __forceinline__ bool ingest_values(uint32_t ld, uint8_t* vp, uint8_t*
     *reinterpret_cast<uint32_t*>(p16 + (c4 * 4 + g) * 4 + ah * 2) = static_cast<uint32_t>(g0.s_bits) | (static_cast<uint32_t>(g1.s_bits) << 16);
     *reinterpret_cast<uint32_t*>(p16 + 64 + (g * 4 + c4) * 4 + ah * 2) = static_cast<uint32_t>(g0.z_bits) | (static_cast<uint32_t>(g1.z_bits) << 16);
   }
-  prm[r * 4 + c4] = i_pack_params(g0, g1);
+  i_put_pair_params(prm + (r * 4 + c4) * 2, g0, g1);
   __syncwarp();
   uint64_t err[2] = {0ull, 0ull}, nrm[2] = {0ull, 0ull};      // [a >> 1], the lane's two tokens side by side
 #pragma unroll 1
@@ -503,8 +515,7 @@ __device__ __forceinline__ bool ingest_values(uint32_t ld, uint8_t* vp, uint8_t*
     uint32_t w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int ah = 0; ah < 2; ++ah) {
-      const uint4 P = prm[(2 * g + ah) * 4 + c4];
-      const PairParams pp = i_pair_params(P, one);
+      const PairParams pp = i_pair_params(prm + ((2 * g + ah) * 4 + c4) * 2, one);
 #pragma unroll
       for (int ss = 0; ss < 2; ++ss) {
         // word of (slice 2 g + ss, a): 8 bits: 4 g + 2 ss + (a >> 1), 4 bits: 2 g + ss, 2 bits: g
@@ -547,10 +558,10 @@ __global__ void __launch_bounds__(kInThreads, kInCtas) ingest_kernel(const __gri
   float* cen = reinterpret_cast<float*>(ism + kInBuf);          // [2][128] centroid of keys, of values
   float* kd2 = cen + 256;                                       // [2 channel halves][64 tokens]
   float* red = kd2 + 128;                                       // [4 value warps][2]: max error, max norm (squared)
-  uint4* prm_all = reinterpret_cast<uint4*>(red + 16);          // [8 warps][8 pairs][4 lanes c4]
+  uint4* prm_all = reinterpret_cast<uint4*>(red + 16);          // [8 warps][8 pairs][4 lanes c4][2]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int r = lane >> 2, c4 = lane & 3, mi = lane >> 3;
-  uint4* prm = prm_all + warp * 32;
+  uint4* prm = prm_all + warp * 64;
   const uint32_t tile_s = i_u32(ism);
   const size_t row_stride = static_cast<size_t>(p.n_kv_heads) * kD;      // elements between two tokens of a stream
   const float one_f = __int_as_float(0x3f800000 + (p.n_jobs >> 31));     // n_jobs is not negative

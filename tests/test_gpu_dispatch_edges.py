@@ -207,3 +207,23 @@ def test_caches_of_two_threads_hand_on_their_host_blocks():
     assert not errors, errors
     for key, want in alone.items():
         assert torch.equal(got[key], want), key
+
+
+@pytest.mark.parametrize("T", [2, 17, 64 + 16, 3 * 64 + 33, 9 * 64 + 63])
+def test_latent_steps_of_one_to_four_units(T):
+    """148 sequences, so that one CTA walks a whole sequence: random levels put one to four units of a kind into a step of the
+    read kernel, switch between code and row operands, and end with a tail of one to four units."""
+    B = _binding()
+    w = W.Workload("edge_mla", 61, 1, 148, 16, 1, 576, 512, T, T + 64, v_aliases_k=1, n_outlier=8, outlier_gain=6.0, n_heavy=0,
+                   softmax_scale=1.0 / 192 ** 0.5, policy=W.POLICY_EXTERNAL)
+    oc = O.GradedCache(U.oracle_config(w))
+    g = B.Cache(B.config_from_workload(w))
+    data = W.make_layer(w, 0, "cpu")
+    rs = np.random.RandomState(T)
+    plan = rs.choice(np.array([16, 8, 8, 4, 4, 1], dtype=np.int8), size=(w.batch, 1, T // 64))
+    U.ingest_both(w, 0, data, oc, g, level_plan=plan)
+    out, lse, o_out, o_lse = U.decode_both(oc, g, 0, data["q"])
+    U.assert_outputs_close(out, o_out, f"latent steps T {T}")
+    assert np.max(np.abs(lse.cpu().numpy() - o_lse)) < 5e-3
+    assert g.gkv_bits_report(0).resident_bits == oc.bits_report(0)["resident_bits"]
+    g.close()
