@@ -1252,17 +1252,17 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
       }
       if (end - begin > 1) {
         // The CTA that delivers the head group's last row normalises and writes the output: the rows are
-        // published by the fence that thread 0 issues behind the barrier, and read back through L2.  Nobody
-        // waits for anybody; the order of summation is the row order, whichever CTA does it.
+        // published and the others' seen through the ticket that thread 0 takes behind the barrier, and read back through L2.  Nobody
+        // waits for anybody; the order of summation is the row order, whichever CTA does it.  (One read-modify-write that releases and
+        // acquires; with a fence on either side of it and a third behind the reset a call over 16,384 tokens of one sequence, 34 rows to a head
+        // group, took 11.9 us instead of 11.5.)
         __syncthreads();
         if (threadIdx.x == 0) {
-          __threadfence();
-          const bool is_last = atomicAdd(&p.tickets[sid], 1) == end - begin - 1;
+          int before;                               // releases the rows, acquires the others'
+          asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;\n" : "=r"(before) : "l"(p.tickets + sid) : "memory");
+          const bool is_last = before == end - begin - 1;
           s_group[4 * kDecodeWarps] = is_last;
-          if (is_last) {
-            p.tickets[sid] = 0;                   // ready for the next launch
-            __threadfence();
-          }
+          if (is_last) p.tickets[sid] = 0;          // ready for the next launch
         }
         __syncthreads();
         if (s_group[4 * kDecodeWarps]) {

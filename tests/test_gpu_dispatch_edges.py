@@ -227,3 +227,25 @@ def test_latent_steps_of_one_to_four_units(T):
     assert np.max(np.abs(lse.cpu().numpy() - o_lse)) < 5e-3
     assert g.gkv_bits_report(0).resident_bits == oc.bits_report(0)["resident_bits"]
     g.close()
+
+
+def _mixed_plan(w, seed, levels=(16, 8, 4, 2, 1)):
+    rs = np.random.RandomState(seed)
+    return rs.choice(np.array(levels, dtype=np.int8), size=(w.batch, w.n_kv_heads, w.ctx // 64))
+
+
+@pytest.mark.parametrize("T", [2048 + 5, 33000, 66000, 140000])
+def test_final_merge_of_a_few_to_many_rows(T):
+    """One stream over the whole GPU: its partial rows are merged 32 at a time, in one pass or several."""
+    B = _binding()
+    w = _gqa(T, group=3, policy=W.POLICY_EXTERNAL)
+    data = W.make_layer(w, 0, "cpu")
+    ocache, g = O.GradedCache(U.oracle_config(w)), B.Cache(B.config_from_workload(w))
+    U.ingest_both(w, 0, data, ocache, g, level_plan=_mixed_plan(w, T, (16, 8, 4, 4, 2)))
+    out, lse, o_out, o_lse = U.decode_both(ocache, g, 0, data["q"])
+    U.assert_outputs_close(out, o_out, f"T {T}")
+    assert np.max(np.abs(lse.cpu().numpy() - o_lse)) < 5e-3
+    again = torch.empty_like(out)
+    g.gkv_decode_attn(0, data["q"].to(g.device), again)
+    torch.cuda.synchronize()
+    assert torch.equal(out, again)
