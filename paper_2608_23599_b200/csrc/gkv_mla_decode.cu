@@ -917,24 +917,26 @@ __global__ void __launch_bounds__(kMThreads, 1) mla_decode_kernel(const __grid_c
   if (warp == 0) m_tmem_dealloc(tmem, kMTmemCols);
 }
 
-// Merge the partial rows of a stream's CTAs (at most kMlaMaxRows).  One block per (stream, head, slice of 64 value
-// channels).  Thread i holds row i's (m, l): maximum, weights and denominator are block reductions; then warp v
-// sums the rows v, v + 16, ... of the slice, two channels a lane, and the warps' sums are added in warp order, so
+// Merge the partial rows of a stream's CTAs (at most kMlaMaxRows).  One block per (stream, head, slice of SLICE value
+// channels).  Thread i holds row i's (m, l): maximum, weights and denominator are block reductions; then the row group v
+// sums the rows v, v + kGroups, ... of the slice, two channels a thread, and the groups' sums are added in their order, so
 // the result is bitwise reproducible.  Bound by latency (4.9 MB of partial rows, in L2): two dependent rounds of
 // loads.  (Before, every thread swept all the maxima and one thread added up the denominator: 7 us behind the read for
 // 148 rows.)
-constexpr int kCombSlice = 64, kCombThreads = 512, kCombWarps = kCombThreads / 32;
+constexpr int kCombThreads = 512, kCombWarps = kCombThreads / 32;
 static_assert(kMlaMaxRows <= kCombThreads, "one thread per partial row");
+template <int SLICE>
 __global__ void __launch_bounds__(kCombThreads) mla_combine_kernel(const float* partial, const StreamParts* parts, float* out,
                                                                    float* lse) {
-  __shared__ float sm_red[kCombWarps], sm_l[kCombWarps], sm_w[kCombThreads], sm_acc[kCombWarps][kCombSlice];
-  // launched with programmatic stream serialisation: the launch overlaps the decode kernel's tail, the
-  // partial rows are touched only after that kernel has completed
+  constexpr int kPairs = SLICE / 2, kGroups = kCombThreads / kPairs;
+  __shared__ float sm_red[kCombWarps], sm_l[kCombWarps], sm_w[kCombThreads], sm_acc[kGroups][SLICE];
   const int stream = blockIdx.x, h = blockIdx.y, slice = blockIdx.z, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  // launched with programmatic stream serialisation: the launch overlaps the decode kernel's tail, the
+  // partial rows are touched only after that kernel has completed (where they lie was settled before it began)
   const int begin = parts[stream].begin, n = parts[stream].end - begin;
   const float* base = partial + static_cast<size_t>(begin) * kMlaPartialFloats + h * (kMlaDv + 2);
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   float2 ml = make_float2(kMNegInf, 0.f);
   if (tid < n) ml = __ldcg(reinterpret_cast<const float2*>(base + static_cast<size_t>(tid) * kMlaPartialFloats));
   float M = ml.x;
@@ -952,26 +954,26 @@ __global__ void __launch_bounds__(kCombThreads) mla_combine_kernel(const float* 
   for (int d = 16; d > 0; d >>= 1) L += __shfl_xor_sync(kMFull, L, d);
   if (lane == 0) sm_l[warp] = L;
   __syncthreads();
-  const float* col = base + 2 + slice * kCombSlice + 2 * lane;
+  const int group = tid / kPairs, pair = tid % kPairs;
+  const float* col = base + 2 + slice * SLICE + 2 * pair;
   float a0 = 0.f, a1 = 0.f;
 #pragma unroll 5
-  for (int i = warp; i < n; i += kCombWarps) {
+  for (int i = group; i < n; i += kGroups) {
     const float2 v = __ldcg(reinterpret_cast<const float2*>(col + static_cast<size_t>(i) * kMlaPartialFloats));
     a0 = fmaf(sm_w[i], v.x, a0);
     a1 = fmaf(sm_w[i], v.y, a1);
   }
-  *reinterpret_cast<float2*>(&sm_acc[warp][2 * lane]) = make_float2(a0, a1);
+  *reinterpret_cast<float2*>(&sm_acc[group][2 * pair]) = make_float2(a0, a1);
   __syncthreads();
-  if (tid < kCombSlice) {
+  if (tid < SLICE) {
     float tot = 0.f;
     L = 0.f;
 #pragma unroll
-    for (int w = 0; w < kCombWarps; ++w) {
-      tot += sm_acc[w][tid];
-      L += sm_l[w];
-    }
+    for (int w = 0; w < kGroups; ++w) tot += sm_acc[w][tid];
+#pragma unroll
+    for (int w = 0; w < kCombWarps; ++w) L += sm_l[w];
     const size_t hq = static_cast<size_t>(stream) * kMlaHeads + h;
-    out[hq * kMlaDv + slice * kCombSlice + tid] = (L > 0.f) ? tot / L : 0.f;
+    out[hq * kMlaDv + slice * SLICE + tid] = (L > 0.f) ? tot / L : 0.f;
     if (lse && slice == 0 && tid == 0) lse[hq] = (L > 0.f) ? (M + log2f(L)) * 0.6931471805599453f : kMNegInf;
   }
 }
@@ -996,13 +998,23 @@ cudaError_t launch_mla_decode(const MlaDecodeParams& p, int n_ctas, const Stream
   cfg.numAttrs = 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, mla_decode_kernel, p);
   if (e != cudaSuccess) return e;
+  // Slices as narrow as one wave of blocks allows (an SM holds four; the read leaves them no room beside its own CTA): a second wave
+  // begins when the first one has gone through both rounds of loads.  Eight sequences of 8191 tokens, 1024 blocks of 64 channels: 4 us
+  // from the last row to the last output, the call 28.1 us.
   cudaLaunchConfig_t cc = {};
-  cc.gridDim = dim3(n_streams, kMlaHeads, kMlaDv / kCombSlice);
   cc.blockDim = dim3(kCombThreads);
   cc.stream = st;
   cc.attrs = attr;
   cc.numAttrs = 1;
-  return cudaLaunchKernelEx(&cc, mla_combine_kernel, static_cast<const float*>(p.partial), parts, out, lse);
+  auto combine = [&](auto kernel, int slice) {
+    cc.gridDim = dim3(n_streams, kMlaHeads, kMlaDv / slice);
+    return cudaLaunchKernelEx(&cc, kernel, static_cast<const float*>(p.partial), parts, out, lse);
+  };
+  const int wave = 4 * 148 / kMlaHeads;      // (stream, slice) pairs
+  if (n_streams * 8 <= wave) return combine(mla_combine_kernel<64>, 64);
+  if (n_streams * 4 <= wave) return combine(mla_combine_kernel<128>, 128);
+  if (n_streams * 2 <= wave) return combine(mla_combine_kernel<256>, 256);
+  return combine(mla_combine_kernel<512>, 512);
 }
 
 }  // namespace gkv

@@ -249,3 +249,18 @@ def test_final_merge_of_a_few_to_many_rows(T):
     g.gkv_decode_attn(0, data["q"].to(g.device), again)
     torch.cuda.synchronize()
     assert torch.equal(out, again)
+
+
+@pytest.mark.parametrize("batch", [4, 5, 10, 18, 19])
+def test_latent_batches_around_the_slices_of_the_merge(batch):
+    """The merge of the CTAs' rows takes 64, 128, 256 or 512 channels to a block, by the number of sequences."""
+    B = _binding()
+    T = 64 * 9 + 33
+    w = W.Workload("edge_latent", 61, 1, batch, 16, 1, 576, 512, T, T + 128, v_aliases_k=1, stair_tokens=(128, 128, 192, 0),
+                   softmax_scale=1.0 / 192.0 ** 0.5, n_outlier=8, outlier_gain=6.0, n_heavy=0)
+    data = W.make_layer(w, 0, "cpu")
+    ocache, g = O.GradedCache(U.oracle_config(w)), B.Cache(B.config_from_workload(w))
+    U.ingest_both(w, 0, data, ocache, g)
+    out, lse, o_out, o_lse = U.decode_both(ocache, g, 0, data["q"])
+    U.assert_outputs_close(out, o_out, f"latent batch {batch}")
+    assert np.max(np.abs(lse.cpu().numpy() - o_lse)) < 5e-3
