@@ -22,9 +22,12 @@
 // barriers between loading and encoding, for shared memory and for the packed fp32 pipe (22 instructions and three
 // double-buffered CTAs per SM before packed arithmetic).  8192 blocks of the staircase mixture 109 us (117 before; 351 MB, 54 us
 // at the measured copy bandwidth), 24,528 in one launch 273 us (1.05 GB, 161 us); extremes by halving exchanges (14 shuffles for a warp's
-// groups instead of 48) and parameters kept as fp32 pairs take another 7 % off: prompts of 2 x 32,768 blocks 1264 -> 1199 us a pass.
+// groups instead of 48) and parameters kept as fp32 pairs take another
+// 7 % off, no clamping where no code can leave its range 2 %: prompts of 2 x 32,768 blocks 1264 -> 1199 -> 1183 us a pass.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "gkv_internal.h"
 #include "gkv_mla.h"
@@ -99,6 +102,13 @@ __device__ __forceinline__ GroupParams i_params(float mn, float mx) {
   return g;
 }
 
+// No value of the group needs its code clamped: scaling and rounding are monotone, so the codes of the extremes bound all.
+template <int BITS>
+__device__ __forceinline__ bool i_unclamped(const GroupParams& g, float mn, float mx) {
+  const float lo = __fadd_rn(__fmul_rn(__fsub_rn(mn, g.z), g.inv), kMagic), hi = __fadd_rn(__fmul_rn(__fsub_rn(mx, g.z), g.inv), kMagic);
+  return lo >= kMagic && hi <= kMagic + static_cast<float>((1 << BITS) - 1);
+}
+
 // bit position of code (slice s, register a, half hlf) inside its 32-bit word (value codes: the fields
 // of registers 1 and 2 change places, see gkv_layout.cuh)
 template <int BITS>
@@ -158,19 +168,24 @@ struct PairParams {
 // point, which parameters inside the fp16 range imply (the inputs are bf16: their spacing bounds the rounding of the zero
 // point by 16 steps, and a rounded scale is at least half of the unrounded one): the codes are clamped as 16-bit
 // integers, both at once, behind the rounding, and go into their word with one multiply-add.  14 instructions for two
-// values, where clamping each as fp32 and taking the magic constants off the word takes 22.
+// values, where clamping each as fp32 and taking the magic constants off the word takes 22; 11 without CLAMP, for groups whose
+// extremes round to codes in range (i_unclamped): then the rounded number less the magic constant is the code.
 // The magic constant is added by a multiply-add with a 1 that the compiler cannot see: it joins a packed multiplication and a
 // packed addition into one operation, which would round the scaled value once instead of twice and move codes.
-template <int BITS>
+template <int BITS, bool CLAMP>
 __device__ __forceinline__ void i_quant_pair(uint64_t X, const PairParams& g, int b0, uint32_t& word, uint64_t& e) {
   constexpr uint32_t qmax = (1u << BITS) - 1u;
   const uint64_t magic = i_pair(kMagic, kMagic), unmagic = i_pair(-kMagic, -kMagic);
   float r0, r1;
-  i_halves(i_fma2(i_mul2(i_add2(X, g.nz), g.inv), g.one, magic), r0, r1);
+  uint64_t r = i_fma2(i_mul2(i_add2(X, g.nz), g.inv), g.one, magic);
+  i_halves(r, r0, r1);
   uint32_t c = __byte_perm(__float_as_uint(r0), __float_as_uint(r1), 0x5410);
-  c = __vimin_s16x2_relu(c, qmax | (qmax << 16));                     // max(min(c, qmax), 0)
+  if constexpr (CLAMP) {
+    c = __vimin_s16x2_relu(c, qmax | (qmax << 16));                   // max(min(c, qmax), 0)
+    r = i_pair(__uint_as_float(__byte_perm(c, kMagicBits, 0x7610)), __uint_as_float(__byte_perm(c, kMagicBits, 0x7632)));
+  }
   word += c << b0;
-  const uint64_t code = i_add2(i_pair(__uint_as_float(__byte_perm(c, kMagicBits, 0x7610)), __uint_as_float(__byte_perm(c, kMagicBits, 0x7632))), unmagic);
+  const uint64_t code = i_add2(r, unmagic);
   const uint64_t d = i_add2(X, i_fma2(code, g.ns, g.nz));             // x - (code s + z)
   e = i_fma2(d, d, e);
 }
@@ -335,8 +350,10 @@ __device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base,
   }
   i_put_pair_params(prm + (r * 4 + c4) * 2, g0, g1);
   __syncwarp();
+  const bool unclamped = __all_sync(kFullI, i_unclamped<BITS>(g0, i_lo(my_mn), i_lo(my_mx)) && i_unclamped<BITS>(g1, i_hi(my_mn), i_hi(my_mx)));
   constexpr int SL = BITS == 2 ? 2 : 1;             // slices that fill whole words
   uint64_t err[2][2] = {{0ull, 0ull}, {0ull, 0ull}};      // [tile][a & 1], the lane's two channels side by side
+  auto encode = [&](auto clamp) {
 #pragma unroll 1
   for (int u = 0; u < 4 / SL; ++u) {
     uint32_t w[2][2] = {{0u, 0u}, {0u, 0u}};        // [tile][word]: 8 bits: one word per a >> 1; else one word
@@ -354,7 +371,7 @@ __device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base,
         for (int t = 0; t < 2; ++t)
 #pragma unroll
           for (int al = 0; al < 2; ++al)
-            i_quant_pair<BITS>(i_pair_bf16(x[t][2 * ah + al]), g, i_bit<BITS>(ss, 2 * ah + al, 0), w[t][wi], err[t][al]);
+            i_quant_pair<BITS, decltype(clamp)::value>(i_pair_bf16(x[t][2 * ah + al]), g, i_bit<BITS>(ss, 2 * ah + al, 0), w[t][wi], err[t][al]);
       }
     }
 #pragma unroll
@@ -370,6 +387,9 @@ __device__ __forceinline__ bool ingest_keys(uint32_t tile_k, uint8_t* half_base,
       }
     }
   }
+  };
+  if (unclamped) encode(std::false_type{});
+  else encode(std::true_type{});
 #pragma unroll
   for (int t = 0; t < 2; ++t)
 #pragma unroll
@@ -506,7 +526,9 @@ __device__ __forceinline__ bool ingest_values(uint32_t ld, uint8_t* vp, uint8_t*
   }
   i_put_pair_params(prm + (r * 4 + c4) * 2, g0, g1);
   __syncwarp();
+  const bool unclamped = __all_sync(kFullI, i_unclamped<BITS>(g0, i_lo(my_mn), i_lo(my_mx)) && i_unclamped<BITS>(g1, i_hi(my_mn), i_hi(my_mx)));
   uint64_t err[2] = {0ull, 0ull}, nrm[2] = {0ull, 0ull};      // [a >> 1], the lane's two tokens side by side
+  auto encode = [&](auto clamp) {
 #pragma unroll 1
   for (int g = 0; g < 4; ++g) {
     uint32_t x[2][4];
@@ -523,7 +545,7 @@ __device__ __forceinline__ bool ingest_values(uint32_t ld, uint8_t* vp, uint8_t*
 #pragma unroll
         for (int al = 0; al < 2; ++al) {
           const uint64_t X = i_pair_bf16(x[ss][2 * ah + al]);
-          i_quant_pair<BITS>(X, pp, i_bit_v<BITS>(ss, 2 * ah + al, 0), w[wi], err[ah]);
+          i_quant_pair<BITS, decltype(clamp)::value>(X, pp, i_bit_v<BITS>(ss, 2 * ah + al, 0), w[wi], err[ah]);
           nrm[ah] = i_fma2(X, X, nrm[ah]);
         }
       }
@@ -537,6 +559,9 @@ __device__ __forceinline__ bool ingest_values(uint32_t ld, uint8_t* vp, uint8_t*
       *reinterpret_cast<uint32_t*>(codes + lane * 16 + g * 4) = w[0];
     }
   }
+  };
+  if (unclamped) encode(std::false_type{});
+  else encode(std::true_type{});
 #pragma unroll
   for (int ah = 0; ah < 2; ++ah) {
     i_halves(err[ah], e[ah][0], e[ah][1]);

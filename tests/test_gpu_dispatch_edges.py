@@ -264,3 +264,18 @@ def test_latent_batches_around_the_slices_of_the_merge(batch):
     out, lse, o_out, o_lse = U.decode_both(ocache, g, 0, data["q"])
     U.assert_outputs_close(out, o_out, f"latent batch {batch}")
     assert np.max(np.abs(lse.cpu().numpy() - o_lse)) < 5e-3
+
+
+@pytest.mark.parametrize("spread", [1.0, 3e-5, 2e-6])
+def test_bulk_encoder_with_and_without_codes_to_clamp(spread):
+    """Groups whose scale is a subnormal fp16 number, rounded by up to a half, have values beyond the last code; the others do not
+    and take the shorter arithmetic.  Every rung, stored bits against the oracle's."""
+    B = _binding()
+    T = 64 * 12
+    w = _gqa(T, n_kv=2, policy=W.POLICY_EXTERNAL)
+    data = W.make_layer(w, 0, "cpu")
+    for name in ("k", "v"):
+        data[name][:, T // 3:] *= spread           # (mixed: a warp takes one form or the other for all its groups)
+    ocache, g = O.GradedCache(U.oracle_config(w)), B.Cache(B.config_from_workload(w))
+    U.ingest_both(w, 0, data, ocache, g, level_plan=np.tile(np.array([8, 4, 2], dtype=np.int8), (1, 2, 4)))
+    U.assert_state_equal(ocache, g, 0)
