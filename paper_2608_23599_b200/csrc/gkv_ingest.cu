@@ -17,13 +17,11 @@
 // group by one lane and handed to the others.
 //
 // One CTA (8 warps: 4 for keys, 4 for values) per block, four CTAs per SM, which take turns loading and encoding; the next
-// block's rows are on their way to L2 while the current one is encoded.  No single limit: 14.8 instructions per value and lane
-// take 63 % of the issue slots and 38 % of the memory's rate, and the warps that wait do so in like parts for their turn, for the
-// barriers between loading and encoding, for shared memory and for the packed fp32 pipe (22 instructions and three
-// double-buffered CTAs per SM before packed arithmetic).  8192 blocks of the staircase mixture 109 us (117 before; 351 MB, 54 us
-// at the measured copy bandwidth), 24,528 in one launch 273 us (1.05 GB, 161 us); extremes by halving exchanges (14 shuffles for a warp's
-// groups instead of 48) and parameters kept as fp32 pairs take another
-// 7 % off, no clamping where no code can leave its range 2 %: prompts of 2 x 32,768 blocks 1264 -> 1199 -> 1183 us a pass.
+// block's rows are on their way to L2 while the current one is encoded.  No single limit: 11.8 instructions per value and lane
+// take 56 % of the issue slots and 42 % of the memory's rate, and the warps that wait do so for the barriers between loading and
+// encoding, for shared memory, for their turn, for instructions and for the packed fp32 pipe.  24,528 blocks of the staircase mixture in
+// one launch 250 us (1.05 GB, 161 us at the measured copy bandwidth); 273 with extremes reduced in all lanes, parameters converted at every
+// use and every code clamped (14.8 instructions), 22 instructions and three double-buffered CTAs per SM before packed arithmetic.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
