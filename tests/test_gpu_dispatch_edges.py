@@ -279,3 +279,45 @@ def test_bulk_encoder_with_and_without_codes_to_clamp(spread):
     ocache, g = O.GradedCache(U.oracle_config(w)), B.Cache(B.config_from_workload(w))
     U.ingest_both(w, 0, data, ocache, g, level_plan=np.tile(np.array([8, 4, 2], dtype=np.int8), (1, 2, 4)))
     U.assert_state_equal(ocache, g, 0)
+
+
+@pytest.mark.parametrize("level", [8, 4, 2])
+@pytest.mark.parametrize("share", [1 / 4096, 0.02])
+def test_bulk_encoder_keeps_a_nan_to_itself(level, share):
+    """NaN among ordinary values (alone in a warp's tile, or many): the extremes pass over it and its code is 0.  Codes, scales and zero points
+    against the same rows 4 bytes off, which go through the encoder of demotions; the codes of all numbers also against the
+    quantiser's rule."""
+    B = _binding()
+    T = 64 * 6
+    w = _gqa(T, n_kv=2, policy=W.POLICY_EXTERNAL)
+    rs = np.random.RandomState(level)
+    plan = np.full((1, 2, T // 64), level, dtype=np.int8)
+    rows, caches = {}, []
+    for name in ("k", "v"):
+        x = rs.randn(T, 2, 128).astype(np.float32)
+        x[rs.rand(*x.shape) < share] = np.nan
+        x[5, 0, 2] = x[6, 1, 3] = x[69, 0, 5] = np.nan          # either half of a register
+        x[:, :, 8] *= -1e4                                      # a neighbour far from the others
+        x[128:160, 0, 40] = np.nan                              # a group of nothing else
+        rows[name] = torch.from_numpy(x).to(torch.bfloat16).reshape(1, T, 2, 128)
+    for shift in (0, 2):
+        g = B.Cache(B.config_from_workload(w))
+        args = []
+        for name in ("k", "v"):
+            flat = torch.zeros(T * 256 + 8, dtype=torch.bfloat16, device=g.device)
+            flat[shift: shift + T * 256] = rows[name].to(g.device).reshape(-1)
+            args.append(flat[shift: shift + T * 256].view(1, T, 2, 128))
+        g.gkv_append_demote(0, *args, level_plan=plan)
+        caches.append(g)
+    for h in range(2):
+        for blk in range(T // 64):
+            for which, name in ((B.TENSOR_K, "k"), (B.TENSOR_V, "v")):
+                got, want = (g.gkv_debug_export_block(0, 0, h, blk, which) for g in caches)
+                for part in ("scale", "zero", "codes"):
+                    assert np.array_equal(got[part], want[part]), (name, h, blk, part)
+                s, z = (got[part].view(np.float16).astype(np.float32) for part in ("scale", "zero"))
+                x = rows[name][0, 64 * blk: 64 * blk + 64, h].float().numpy()
+                s, z = (np.repeat(p, 32, axis=0 if name == "k" else 1) for p in (s, z))
+                with np.errstate(divide="ignore", invalid="ignore"):
+                    code = np.clip(np.rint((x - z) * np.where(s > 0, np.float32(1) / s, np.float32(0))), 0, 2 ** level - 1)
+                assert np.array_equal(got["codes"], np.where(np.isnan(x), 0, code)), (name, h, blk)
