@@ -12,7 +12,7 @@ LIB = os.path.join(HERE, "libgkv.so")
 CALL_SOURCE = os.path.join(CSRC, "gkv_call.cpp")         # the binding's extension: a decode step's calls without ctypes
 CALL_LIB = os.path.join(HERE, "_gkv_call" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["gkv_api.cu", "gkv_decode.cu", "gkv_units.cu", "gkv_pack.cu", "gkv_ingest.cu", "gkv_quest.cu", "gkv_rdplan.cu", "gkv_mla.cu", "gkv_mla_decode.cu"]
-HEADERS = ["gkv_internal.h", "gkv_layout.cuh", "gkv_mla.h", os.path.join("..", "..", "include", "gkv.h")]
+HEADERS = ["gkv_internal.h", "gkv_exchange.h", "gkv_layout.cuh", "gkv_mla.h", os.path.join("..", "..", "include", "gkv.h")]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",

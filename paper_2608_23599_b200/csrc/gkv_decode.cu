@@ -28,6 +28,7 @@
 
 #include <atomic>
 
+#include "gkv_exchange.h"
 #include "gkv_internal.h"
 
 namespace gkv {
@@ -110,6 +111,13 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
       : "memory");
   return ok != 0;
 }
+struct ExchangeIo {
+  uint32_t bar;
+  uint32_t* status;
+  __device__ __forceinline__ bool poll() const { return mbar_try_wait_cluster(bar, 0); }
+  __device__ __forceinline__ void report() const { atomicOr(status, kStatusInternal); }
+  __device__ __forceinline__ void meet() const { asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory"); }
+};
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&a)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3])
@@ -978,10 +986,7 @@ __device__ __forceinline__ void stage_query(const WarpCtx& w, const uint32_t (&q
   __syncwarp();
 }
 
-// What the CTAs of a cluster send one another lies behind the merge's words: an mbarrier, kExchangeFloats accumulators (shares are
-// rounded up, so a little more than one per channel and head), a pair per CTA and head.
-constexpr int kExchangeOffset = (4 * kDecodeWarps + 2) * 4, kExchangeFloats = kHeadsPerWarp * kD + kMaxCluster;
-constexpr int kExchangeBytes = 8 + kExchangeFloats * 4 + kMaxCluster * kHeadsPerWarp * 8;
+constexpr int kExchangeOffset = (4 * kDecodeWarps + 2) * 4;      // of a cluster's exchange, behind the merge's words
 
 template <bool SPARSE, bool MASS>
 __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_kernel(const __grid_constant__ DecodeParams p) {
@@ -1033,10 +1038,9 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   if (p.cluster > 1) {
     if (threadIdx.x == 0) {
       const uint32_t x_bar = smem_u32(s_group) + kExchangeOffset;
-      const int share = (kHeadsPerWarp * kD + p.cluster - 1) / p.cluster, rank = static_cast<int>(cluster_rank());
       mbar_init(x_bar, 1);
       asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-      mbar_expect_tx(x_bar, static_cast<uint32_t>(p.cluster * (min(share, kHeadsPerWarp * kD - rank * share) * 4 + kHeadsPerWarp * 8)));
+      mbar_expect_tx(x_bar, static_cast<uint32_t>(exchange_bytes_expected(p.cluster, static_cast<int>(cluster_rank()))));
     }
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
@@ -1239,20 +1243,14 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
     // in 12 streams of three heads, eight CTAs each, stay at 8.1).
     asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
     const uint32_t x_bar = smem_u32(s_group) + kExchangeOffset, x_acc = x_bar + 8, x_ml = x_acc + kExchangeFloats * 4;
-    const int share = (kHeadsPerWarp * kD + p.cluster - 1) / p.cluster, rank = static_cast<int>(cluster_rank());
+    const int share = exchange_share(p.cluster), rank = static_cast<int>(cluster_rank());
     {
       const int e = head * kD + chan, owner = e / share;
-      send_f32(cluster_addr(x_acc + (rank * share + e - owner * share) * 4, owner), acc, cluster_addr(x_bar, owner));
+      send_f32(cluster_addr(x_acc + exchange_slot(share, rank, e) * 4, owner), acc, cluster_addr(x_bar, owner));
       if ((warp & 3) == 0 && lane < p.cluster)
         send_2f32(cluster_addr(x_ml + (rank * kHeadsPerWarp + head) * 8, lane), M, L, cluster_addr(x_bar, lane));
     }
-    int spins = 0;
-    while (!mbar_try_wait_cluster(x_bar, 0)) {
-      if (++spins > kWaitSpins) {
-        if (lane == 0) atomicOr(p.status, kStatusInternal);
-        break;
-      }
-    }
+    const int rows_in = await_exchange(ExchangeIo{x_bar, p.status}, kWaitSpins) ? p.cluster : 0;      // (none: an empty result)
     const int e = rank * share + threadIdx.x;
     if (static_cast<int>(threadIdx.x) < share && e < n_heads * kD) {
       const int h = e / kD, ch = e - h * kD;
@@ -1263,8 +1261,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
       float ca[kMaxCluster];
 #pragma unroll
       for (int c = 0; c < kMaxCluster; ++c) {            // all loads first: 8 CTAs 16.68 -> 16.22 us for two reads
-        ml[c] = c < p.cluster ? ml_of[c * kHeadsPerWarp] : make_float2(kNegInf, 0.f);
-        ca[c] = c < p.cluster ? acc_of[c * share] : 0.f;
+        ml[c] = c < rows_in ? ml_of[c * kHeadsPerWarp] : make_float2(kNegInf, 0.f);
+        ca[c] = c < rows_in ? acc_of[c * share] : 0.f;
       }
       M = kNegInf;
 #pragma unroll
