@@ -1382,11 +1382,12 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
 
 }  // namespace
 
-size_t decode_smem_bytes() {
-  // per warp: pipeline stages, their mbarriers, the query fragments (2 KiB as bf16, 2 KiB as fp16) and four words for the merge; a flag;
-  // the exchange of a cluster
-  return static_cast<size_t>(kDecodeWarps) * (kStages * kStageBytes + kStages * sizeof(uint64_t) + 2 * 2048 + 4 * sizeof(int)) + 2 * sizeof(int) + kExchangeBytes;
-}
+// per warp: pipeline stages, their mbarriers, the query fragments (2 KiB as bf16, 2 KiB as fp16) and four words for the merge; a flag;
+// the exchange of a cluster
+constexpr size_t kDecodeSmem = static_cast<size_t>(kDecodeWarps) * (kStages * (kStageBytes + sizeof(uint64_t)) + 2 * 2048) + kExchangeOffset + kExchangeBytes;
+static_assert(kDecodeSmem <= 227 * 1024, "more shared memory than an SM has for one CTA");
+static_assert(kExchangeOffset % 8 == 0, "the exchange begins with an mbarrier");
+size_t decode_smem_bytes() { return kDecodeSmem; }
 
 namespace {
 cudaError_t configure_decode() {
@@ -1568,7 +1569,7 @@ __device__ __forceinline__ void finish_certificate(const ObserveParams& p, int h
 // share one launch, which overlaps that launch's tail (with two launches one after the other and no
 // overlap an observing call over 8200 tokens of 16 streams took 28.9 us, with this one 21.2).  Not where there are many residual
 // rows and the read fills the GPU: an overlapped launch's CTAs crowd the first SMs that the decode kernel leaves, whose L1 is what
-// its 225 KB of shared memory left over, and the rows' pairs, looked up block by block, live off L1: 52,000 rows of 64 streams of
+// its 227 KB of shared memory leave over, and the rows' pairs, looked up block by block, live off L1: 52,000 rows of 64 streams of
 // 8200 tokens 99 us a call overlapped, 30 not; 105,000 rows of 32 streams of 32,700 tokens 113 and 38.  SMs that the read leaves idle
 // have all of theirs, 16 streams of 4000 tokens 21.8 overlapped, 24.7 not, and up to 64 CTAs (kObserveOverlap) that was the faster
 // at every size; with 96 a call of 96 streams was 24.7 and 25.9 at 4000 tokens, but 45.2 and 26.4 where it writes certificates.
