@@ -1,4 +1,5 @@
-"""ctypes binding of libgkv.so: the same names as include/gkv.h, argument marshalling only.
+"""Binding of libgkv.so: the same names as include/gkv.h, argument marshalling only (by ctypes; a decode step's calls by the
+extension csrc/gkv_call.cpp).
 
 Every step of the path runs in the CUDA kernels behind the C ABI.  PyTorch is used for device
 memory (the arena, inputs, outputs) and for the current CUDA stream.  If the library is missing
@@ -70,14 +71,14 @@ def lib_path() -> str:
 
 
 def load():
-    """Load libgkv.so (building it is the job of ``build()`` / ``__graft_entry__.build``)."""
+    """Load libgkv.so and the extension (building them is the job of ``build()`` / ``__graft_entry__.build``)."""
     global _lib, _call
     if _lib is not None:
         return _lib
-    path = lib_path()
-    if not os.path.exists(path):
-        raise FileNotFoundError(f"{path} is missing: run `python -m paper_2608_23599_b200.build` first")
-    lib = C.CDLL(path)
+    for path in (lib_path(), _build.CALL_LIB):
+        if not os.path.exists(path):
+            raise FileNotFoundError(f"{path} is missing: run `python -m paper_2608_23599_b200.build` first")
+    lib = C.CDLL(lib_path())
     vp, i32, sz = C.c_void_p, C.c_int32, C.c_size_t
     lib.gkv_query_arena_bytes.argtypes = [C.POINTER(GkvConfig), C.POINTER(sz)]
     lib.gkv_create.argtypes = [C.POINTER(GkvConfig), vp, sz, C.POINTER(vp)]
