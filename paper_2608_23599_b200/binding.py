@@ -113,7 +113,7 @@ def load():
             getattr(lib, name).restype = C.c_int
     from . import _gkv_call
     _gkv_call.bind(*(C.cast(f, vp).value for f in (lib.gkv_append_demote, lib.gkv_decode_attn, lib.gkv_decode_attn_observe,
-                                                   lib.gkv_quest_select)))
+                                                   lib.gkv_quest_select)), vp)
     _lib, _call = lib, _gkv_call
     return lib
 

@@ -1,7 +1,7 @@
 // The calls of a decode step without ctypes: a Python extension that takes the arguments of the binding's methods
 // (tensors, device addresses or None), makes the pointers of them and calls the C ABI with the interpreter lock released, as ctypes
-// does.  An argument of a type that ctypes might still convert (or refuse) is not judged here: the function returns
-// NotImplemented and the binding goes through ctypes.
+// does.  An argument that it cannot convert is not judged here: the function returns NotImplemented and the binding goes through
+// ctypes, which converts it or raises what it always raised.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <stdint.h>
@@ -17,44 +17,49 @@ decltype(&gkv_decode_attn_observe) f_observe = nullptr;
 decltype(&gkv_quest_select) f_select = nullptr;
 PyObject* s_data_ptr = nullptr;      // "data_ptr"
 PyObject* s_value = nullptr;         // "value"
+PyObject* void_p = nullptr;          // ctypes.c_void_p
 
-bool as_address(PyObject* o, void** out) {
-  if (o == Py_None) {
-    *out = nullptr;
-    return true;
-  }
-  PyObject* v = nullptr;
-  if (!PyLong_Check(o)) {
-    v = PyObject_CallMethodNoArgs(o, s_data_ptr);
-    if (!v) return false;
-    o = v;
-  }
-  *out = reinterpret_cast<void*>(static_cast<uintptr_t>(PyLong_AsUnsignedLongLongMask(o)));
-  Py_XDECREF(v);
+// an int or None
+bool as_plain(PyObject* o, void** out) {
+  if (o != Py_None && !PyLong_Check(o)) return false;
+  *out = o == Py_None ? nullptr : reinterpret_cast<void*>(static_cast<uintptr_t>(PyLong_AsUnsignedLongLongMask(o)));
   return !PyErr_Occurred();
 }
-// a ctypes.c_void_p or None
-bool as_handle(PyObject* o, gkv_cache** out) {
-  *out = nullptr;
-  if (o == Py_None) return true;
-  PyObject* v = PyObject_GetAttr(o, s_value);
+// an int, None, or a tensor
+bool as_address(PyObject* o, void** out) {
+  if (o == Py_None || PyLong_Check(o)) return as_plain(o, out);
+  PyObject* v = PyObject_CallMethodNoArgs(o, s_data_ptr);
   if (!v) return false;
-  void* p = nullptr;
-  const bool ok = as_address(v, &p);
+  const bool ok = as_plain(v, out);
   Py_DECREF(v);
+  return ok;
+}
+// a ctypes.c_void_p, an int or None
+bool as_handle(PyObject* o, gkv_cache** out) {
+  void* p = nullptr;
+  bool ok;
+  if (reinterpret_cast<PyObject*>(Py_TYPE(o)) == void_p) {
+    PyObject* v = PyObject_GetAttr(o, s_value);
+    if (!v) return false;
+    ok = as_plain(v, &p);
+    Py_DECREF(v);
+  } else {
+    ok = as_plain(o, &p);
+  }
   *out = static_cast<gkv_cache*>(p);
   return ok;
 }
-// false without an exception: not an int
 bool as_int(PyObject* o, int32_t* out) {
   if (!PyLong_Check(o)) return false;
   *out = static_cast<int32_t>(PyLong_AsUnsignedLongMask(o));
   return !PyErr_Occurred();
 }
-// a cudaStream_t as an int, or None
-bool as_stream(PyObject* o, void** out) { return (o == Py_None || PyLong_Check(o)) && as_address(o, out); }
+// An exception of the conversion is raised again, or not, by the binding's second attempt (an interrupt is not one).
 PyObject* refuse() {
-  if (PyErr_Occurred()) return nullptr;
+  if (PyErr_Occurred()) {
+    if (!PyErr_ExceptionMatches(PyExc_Exception)) return nullptr;
+    PyErr_Clear();
+  }
   Py_RETURN_NOTIMPLEMENTED;
 }
 bool want(Py_ssize_t n, Py_ssize_t need) {
@@ -63,12 +68,14 @@ bool want(Py_ssize_t n, Py_ssize_t need) {
   return false;
 }
 
-// bind(append, decode, observe, select): addresses
+// bind(append, decode, observe, select, c_void_p): addresses, and ctypes' type of a handle
 PyObject* py_bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
   void* p[4];
-  if (!want(n, 4)) return nullptr;
+  if (!want(n, 5)) return nullptr;
   for (int i = 0; i < 4; ++i)
-    if (!as_address(a[i], &p[i])) return nullptr;
+    if (!as_plain(a[i], &p[i])) return PyErr_Occurred() ? nullptr : PyErr_Format(PyExc_TypeError, "an address is needed");
+  Py_INCREF(a[4]);
+  Py_XSETREF(void_p, a[4]);
   f_append = reinterpret_cast<decltype(f_append)>(p[0]);
   f_decode = reinterpret_cast<decltype(f_decode)>(p[1]);
   f_observe = reinterpret_cast<decltype(f_observe)>(p[2]);
@@ -81,8 +88,9 @@ PyObject* py_append(PyObject*, PyObject* const* a, Py_ssize_t n) {
   gkv_cache* h;
   int32_t layer, n_new;
   void *k, *v, *mass, *plan, *st;
-  if (!want(n, 8) || !as_handle(a[0], &h) || !as_int(a[1], &layer) || !as_address(a[2], &k) || !as_address(a[3], &v) || !as_int(a[4], &n_new) ||
-      !as_address(a[5], &mass) || !as_address(a[6], &plan) || !as_stream(a[7], &st))
+  if (!want(n, 8)) return nullptr;
+  if (!as_handle(a[0], &h) || !as_int(a[1], &layer) || !as_address(a[2], &k) || !as_address(a[3], &v) || !as_int(a[4], &n_new) ||
+      !as_address(a[5], &mass) || !as_address(a[6], &plan) || !as_plain(a[7], &st))
     return refuse();
   int rc;
   Py_BEGIN_ALLOW_THREADS
@@ -96,8 +104,9 @@ PyObject* py_decode(PyObject*, PyObject* const* a, Py_ssize_t n) {
   gkv_cache* h;
   int32_t layer, n_sel;
   void *q, *pages, *out, *lse, *st;
-  if (!want(n, 8) || !as_handle(a[0], &h) || !as_int(a[1], &layer) || !as_address(a[2], &q) || !as_address(a[3], &pages) || !as_int(a[4], &n_sel) ||
-      !as_address(a[5], &out) || !as_address(a[6], &lse) || !as_stream(a[7], &st))
+  if (!want(n, 8)) return nullptr;
+  if (!as_handle(a[0], &h) || !as_int(a[1], &layer) || !as_address(a[2], &q) || !as_address(a[3], &pages) || !as_int(a[4], &n_sel) ||
+      !as_address(a[5], &out) || !as_address(a[6], &lse) || !as_plain(a[7], &st))
     return refuse();
   int rc;
   Py_BEGIN_ALLOW_THREADS
@@ -111,8 +120,9 @@ PyObject* py_observe(PyObject*, PyObject* const* a, Py_ssize_t n) {
   gkv_cache* h;
   int32_t layer;
   void *q, *out, *lse, *mass, *cert, *st;
-  if (!want(n, 8) || !as_handle(a[0], &h) || !as_int(a[1], &layer) || !as_address(a[2], &q) || !as_address(a[3], &out) || !as_address(a[4], &lse) ||
-      !as_address(a[5], &mass) || !as_address(a[6], &cert) || !as_stream(a[7], &st))
+  if (!want(n, 8)) return nullptr;
+  if (!as_handle(a[0], &h) || !as_int(a[1], &layer) || !as_address(a[2], &q) || !as_address(a[3], &out) || !as_address(a[4], &lse) ||
+      !as_address(a[5], &mass) || !as_address(a[6], &cert) || !as_plain(a[7], &st))
     return refuse();
   int rc;
   Py_BEGIN_ALLOW_THREADS
@@ -126,8 +136,9 @@ PyObject* py_select(PyObject*, PyObject* const* a, Py_ssize_t n) {
   gkv_cache* h;
   int32_t layer, budget, n_sel = 0;
   void *q, *pages, *st;
-  if (!want(n, 6) || !as_handle(a[0], &h) || !as_int(a[1], &layer) || !as_address(a[2], &q) || !as_int(a[3], &budget) || !as_address(a[4], &pages) ||
-      !as_stream(a[5], &st))
+  if (!want(n, 6)) return nullptr;
+  if (!as_handle(a[0], &h) || !as_int(a[1], &layer) || !as_address(a[2], &q) || !as_int(a[3], &budget) || !as_address(a[4], &pages) ||
+      !as_plain(a[5], &st))
     return refuse();
   int rc;
   Py_BEGIN_ALLOW_THREADS
