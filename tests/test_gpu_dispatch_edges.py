@@ -1,5 +1,5 @@
 """The sizes at which a kernel or a dispatch rule changes: selection lists around the number of keys a thread
-holds, page scorer shapes, work lists that become clusters of one to eight CTAs or share CTAs, device allocator sizes,
+holds, page scorer shapes, clusters of one to eight CTAs, work lists that share CTAs, device allocator sizes,
 parameters outside the fp16 range in the bulk encoder, signed zeros in page boxes, latent batches around one wave of
 CTAs, and caches that hand their page-locked block on between threads."""
 import dataclasses
@@ -106,6 +106,55 @@ def test_work_lists_from_one_cta_to_shared_ctas(batch, n_kv, group, T):
     again = torch.empty_like(out)
     g.gkv_decode_attn(0, data["q"].to(g.device), again)
     assert torch.equal(again, out2)              # the same lists until a block closes
+
+
+@pytest.mark.parametrize("ctas", [2, 3, 4, 5, 6, 7, 8])
+@pytest.mark.parametrize("batch,group", [(2, 3), (3, 1), (2, 8)])
+def test_clusters_of_every_size(ctas, batch, group):
+    """Lists of half blocks for one warp each, so many that a head group gets a cluster of `ctas` CTAs, whose shares of the channels
+    are even for two, four and eight only: the read and the observing read, and the same bits back to back."""
+    B = _binding()
+    blocks = 8 * ctas - 6                        # two units each, and four of the tail: half a CTA below ctas * 16
+    w = _gqa(64 * blocks + 50, batch, 1, group, policy=W.POLICY_EXTERNAL)
+    data = W.make_layer(w, 0, "cpu")
+    ocache, g = O.GradedCache(U.oracle_config(w)), B.Cache(B.config_from_workload(w))
+    plan = np.random.RandomState(ctas).choice(np.array([8, 4, 2], dtype=np.int8), size=(batch, 1, blocks))
+    U.ingest_both(w, 0, data, ocache, g, level_plan=plan)
+    out, lse, o_out, o_lse = U.decode_both(ocache, g, 0, data["q"])
+    units = g.gkv_debug_export_units(0)
+    first = [units[units[:, 1] == hg, 0].min() for hg in range(batch * (1 if group <= 4 else 2))]
+    assert first == [16 * ctas * hg for hg in range(len(first))]        # a head group's warps begin with a cluster, 16 to a CTA
+    U.assert_outputs_close(out, o_out, f"{ctas} CTAs")
+    assert np.max(np.abs(lse.cpu().numpy() - o_lse)) < 5e-3
+    q = data["q"].to(g.device)
+    again = [torch.empty_like(out) for _ in range(20)]
+    for o in again:
+        g.gkv_decode_attn(0, q, o)
+    assert all(torch.equal(o, out) for o in again)
+    mass = torch.empty((batch, 1, blocks + 1), dtype=torch.float32, device=g.device)
+    g.gkv_decode_attn_observe(0, q, out, None, mass)
+    U.assert_outputs_close(out, o_out, "observing read")
+    assert np.allclose(mass.cpu().numpy().sum(-1), 1.0, atol=2e-3)
+    g.gkv_bits_report(0)                         # (raises if a wait ran out)
+
+
+@pytest.mark.parametrize("streams", [15, 22, 25, 30, 40, 74, 75])
+def test_page_lists_over_clusters_of_every_size(streams):
+    """A page list is read by as many CTAs per head group as fill the GPU once, 148 / streams and at most eight, as a cluster where it has
+    room for all."""
+    B = _binding()
+    T, n_sel = 64 * 9 + 5, 6
+    w = _gqa(T, streams, 1, 2, page_tokens=64, stair_tokens=(128, 128, 128, 64))
+    data = W.make_layer(w, 0, "cpu")
+    ocache, g = O.GradedCache(U.oracle_config(w)), B.Cache(B.config_from_workload(w))
+    U.ingest_both(w, 0, data, ocache, g)
+    rs = np.random.RandomState(streams)
+    pages = np.stack([np.sort(rs.permutation(9)[:n_sel]) for _ in range(streams)]).astype(np.int32)[:, None]
+    out, lse, o_out, o_lse = U.decode_both(ocache, g, 0, data["q"], torch.from_numpy(pages).to(g.device), n_sel,
+                                           [[pages[b, 0]] for b in range(streams)])
+    U.assert_outputs_close(out, o_out, f"{streams} streams")
+    assert np.max(np.abs(lse.cpu().numpy() - o_lse)) < 5e-3
+    g.gkv_bits_report(0)
 
 
 @pytest.mark.parametrize("batch,T", [(1, 65), (2, 333), (9, 300), (148, 70), (149, 70)])
