@@ -1034,7 +1034,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
   }
   // Clusters: each CTA gets its share of the channels from all of them, [CTA][share] accumulators and [CTA][head] pairs (m, l),
   // whose bytes complete its mbarrier; the barrier of the cluster, which is waited for in front of the first value that goes out, says that
-  // all mbarriers are set up.
+  // all mbarriers are set up.  The fence publishes them and the arrival need not release anything: where it did, clusters that fill the GPU began late
+  // (15 streams of 4800 tokens and three heads, eight CTAs each, 9.14 -> 8.85 us a call, 9.04 with the barriers and remote reads before).
   if (p.cluster > 1) {
     if (threadIdx.x == 0) {
       const uint32_t x_bar = smem_u32(s_group) + kExchangeOffset;
@@ -1043,7 +1044,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
       mbar_expect_tx(x_bar, static_cast<uint32_t>(exchange_bytes_expected(p.cluster, static_cast<int>(cluster_rank()))));
     }
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
   }
   StreamParts parts{0, 0};
   uint8_t* sbase = smem + warp * (kStages * kStageBytes);
@@ -1239,8 +1240,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
     }
     // Every value goes to the CTA that finishes its channel, which waits for the bytes of all: one trip, where a
     // barrier of the cluster with reads of the others' rows behind it and a second barrier in front of the exit took three
-    // (1000 tokens of one sequence 6.91 -> 6.43 us a call, observing reads of 8200 tokens 17.0 -> 16.4 a layer; 4805 tokens
-    // in 12 streams of three heads, eight CTAs each, stay at 8.1).
+    // (one stream of 1000 tokens and four heads 7.24 -> 6.66 us a call, 12 of 4805 tokens 9.48 -> 8.91, with three heads 8.90 -> 8.68, 64 of 2000
+    // in pairs of CTAs 12.33 -> 11.94; observing reads of 64 of 4000 20.4 -> 20.1).
     asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
     const uint32_t x_bar = smem_u32(s_group) + kExchangeOffset, x_acc = x_bar + 8, x_ml = x_acc + kExchangeFloats * 4;
     const int share = exchange_share(p.cluster), rank = static_cast<int>(cluster_rank());
@@ -1260,7 +1261,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, kDecodeCtasPerSm) decode_ke
       float2 ml[kMaxCluster];
       float ca[kMaxCluster];
 #pragma unroll
-      for (int c = 0; c < kMaxCluster; ++c) {            // all loads first: 8 CTAs 16.68 -> 16.22 us for two reads
+      for (int c = 0; c < kMaxCluster; ++c) {            // (all loads first)
         ml[c] = c < rows_in ? ml_of[c * kHeadsPerWarp] : make_float2(kNegInf, 0.f);
         ca[c] = c < rows_in ? acc_of[c * share] : 0.f;
       }
