@@ -648,10 +648,11 @@ void plan_units(gkv_cache* c, LayerState& L, bool allow_split) {
   // CTAs of its own for every head group, launched as a cluster and merged through distributed shared memory, where all
   // clusters fit the GPU at once and the most laden one's warps get little more than they would of the whole GPU: up to 0.85 of a
   // block, which takes about as long as the rows in global memory and the ticket that the cluster saves.  A single head group's rows
-  // are merged by a GPU that is otherwise done: 0.4 of a block.  Clusters and shared CTAs, us a call (more, in blocks): 4 streams of
-  // 8200 tokens 9.9 and 10.6 (0.5), 16 of 8200 11.9 and 14.1 (0.5), 24 of 16,400 19.8 and 20.8 (0.6), 64 of 8200 23.1 and 25.0 (0.6),
-  // 12 of 16,400 15.8 and 14.8 (0.7), 16 of 16,400 17.5 and 16.5 (0.9), 8 of 32,700 with eight query heads each 29.9 and 24.7
-  // (1.9); one stream of 8200 10.3 and 9.1 (0.5).
+  // are merged by a GPU that is otherwise done: 0.4 of a block.  Clusters and shared CTAs over 4-bit blocks, us a call (more, in blocks):
+  // 4 streams of 8200 tokens 10.1 and 10.3 (0.5), 16 of 8200 11.3 and 12.4 (0.5), 24 of 16,400 20.8 and 22.1 (0.6), 64 of 8200 23.9 and 25.4
+  // (0.5), 12 of 16,400 14.8 and 15.7 (0.7), 64 of 12,000 31.8 and 33.5 (0.8), 8 of 12,000 12.0 and 11.8 (0.8; 11.7 and 13.9 over a mixture of
+  // rungs), 16 of 16,400 17.6 and 17.4 (0.9), 64 of 16,400 40.7 and 39.2 (1.1), 8 of 16,400 14.7 and 12.8 (1.1), 8 of 32,700 with eight query heads
+  // each 29.9 and 24.2 (1.9); one stream of 7000 8.3 and 8.6 (0.4), of 8200 9.6 and 8.8 (0.5).
   L.cluster = 0;
   if (c->n_hgroups <= 148) {
     int most = 0;                              // warps of the most laden stream

@@ -998,9 +998,11 @@ cudaError_t launch_mla_decode(const MlaDecodeParams& p, int n_ctas, const Stream
   cfg.numAttrs = 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, mla_decode_kernel, p);
   if (e != cudaSuccess) return e;
-  // Slices as narrow as one wave of blocks allows (an SM holds four; the read leaves them no room beside its own CTA): a second wave
-  // begins when the first one has gone through both rounds of loads.  Eight sequences of 8191 tokens, 1024 blocks of 64 channels: 4 us
-  // from the last row to the last output, the call 28.1 us (26.2 in one wave).
+  // Slices as narrow as one wave of blocks allows (an SM holds four; the read leaves them no room beside its own CTA), whole rows beyond 37 streams: a
+  // second wave begins when the first one has gone through both rounds of loads, and a block more costs more than a pair of channels more per
+  // thread.  Sequences of 2500 tokens, us a call with 64, 128, 256 and 512 channels: 4 sequences 14.6, 15.2, 16.0, 18.6; 5 16.4, 15.8, 16.7,
+  // 18.6; 9 19.8, 18.1, 18.5, 19.8; 10 21.3, 20.0, 19.4, 20.4; 18 29.0, 26.1, 24.4, 25.0; 19 31.1, 27.9, 26.7, 26.7; 24 35.4, 31.2, 29.7, 29.0;
+  // 64 79.6, 69.1, 63.7, 61.1 (8191 tokens: 173, 162, 157, 154); 148 156, 133, 121, 116.
   cudaLaunchConfig_t cc = {};
   cc.blockDim = dim3(kCombThreads);
   cc.stream = st;
