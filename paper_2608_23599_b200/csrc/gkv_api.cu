@@ -546,7 +546,7 @@ bool rd_allocate_streams(const gkv_config& c, const float* mass, const float* ra
 // mixed workload, measured on B200 by timing every step of individual warps of the config-2 launch
 // (in units where a 4-bit block is 1000): an exact block 1590, 8-bit 1070, 4-bit 1000, 2-bit 1015, a
 // centroid block 47 (a run of 16 costs 745).  Bytes are the wrong weight: below 8 bits the kernel
-// is bound by instruction issue and a block costs the same whatever its code width.
+// waits for its own instructions and a block costs the same whatever its code width.
 constexpr size_t kCost16 = 1590, kCost8 = 1070, kCost4 = 1000, kCost2 = 1015, kCost1 = 47;
 constexpr size_t kCostTail = 800;            // mid-fill estimate (its size changes every step)
 constexpr size_t kCostRes = 550;             // residual group of 16 exact rows

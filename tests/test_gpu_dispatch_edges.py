@@ -1,6 +1,6 @@
 """The sizes at which a kernel or a dispatch rule changes: selection lists around the number of keys a thread
 holds, page scorer shapes, clusters of one to eight CTAs, work lists that share CTAs, device allocator sizes,
-parameters outside the fp16 range in the bulk encoder, signed zeros in page boxes, latent batches around one wave of
+parameters outside the fp16 range and NaN in the bulk encoder, signed zeros in page boxes, latent batches around one wave of
 CTAs, and caches that hand their page-locked block on between threads."""
 import dataclasses
 import threading
